@@ -131,6 +131,7 @@ struct Work {
     size_t bytes = 0;
     void* X = nullptr;
     double* V = nullptr;
+    float2* yf = nullptr;        // split duals of deferred plan writes (FP32 plans)
     double* rowpart = nullptr;
     double* colpart = nullptr;
     double* rowpart2 = nullptr;
@@ -144,6 +145,9 @@ struct Work {
     size_t cpad_bytes = 0;
 };
 
+// Entries between the sets of split duals (rows of two, 16-byte starts).
+long long yf_stride(long long m, long long n) { return (m + n + 1) / 2 * 2; }
+
 size_t work_bytes(long long m, long long n, int xtype, int tile_rows, Work* w) {
     const long long ldx = (n + 3) / 4 * 4;
     const int nstrips = (int)((n + STRIP - 1) / STRIP);
@@ -154,6 +158,7 @@ size_t work_bytes(long long m, long long n, int xtype, int tile_rows, Work* w) {
     auto take = [&](size_t b) { size_t o = off; off = align_up(off + b, 256); return o; };
     const size_t oX = take((size_t)NSLOT * m * ldx * xsize_of(xtype));
     const size_t oV = take((size_t)NSLOT * 2 * (m + n) * sizeof(double));
+    const size_t oY = take(xtype == PDOT_F64 ? 0 : (size_t)YRING * yf_stride(m, n) * sizeof(float2));
     const size_t oR = take((size_t)nstrips * m * sizeof(double));
     const size_t oC = take((size_t)nchunks * ldx * sizeof(double));
     const size_t oR2 = take((size_t)nstrips * m * sizeof(double));
@@ -168,6 +173,7 @@ size_t work_bytes(long long m, long long n, int xtype, int tile_rows, Work* w) {
         char* b = (char*)w->base;
         w->X = b + oX;
         w->V = (double*)(b + oV);
+        w->yf = xtype == PDOT_F64 ? nullptr : (float2*)(b + oY);
         w->rowpart = (double*)(b + oR);
         w->colpart = (double*)(b + oC);
         w->rowpart2 = (double*)(b + oR2);
@@ -193,11 +199,11 @@ Inst make_inst(const Work& w, const void* C, int ctype, long long ldc, const dou
     I.f = f; I.g = g;
     I.X = w.X; I.xslot = w.m * w.ldx;
     I.V = w.V; I.vslot = 2 * (w.m + w.n);
+    I.yf = w.yf; I.yslot = yf_stride(w.m, w.n);
     I.rowpart = w.rowpart; I.colpart = w.colpart; I.tpart = w.tpart; I.vpart = w.vpart;
     I.rowpart2 = w.rowpart2; I.colpart2 = w.colpart2;
     I.ctrl = w.ctrl; I.ticket = w.ticket;
     I.nstrips = w.nstrips; I.nchunks = w.nchunks; I.tile_rows = w.tile_rows; I.ntiles = w.ntiles; I.nvt = w.nvt;
-    I.l2_keep_c = 0;
     return I;
 }
 
@@ -246,10 +252,12 @@ struct pdot_handle {
     int* h_status = nullptr;     // pinned [2]
     Graph chunk;                 // K x (pass, dual) + (kkt, checkvec)
     long long chunk_key[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    std::map<long long, std::pair<int, int>> tune_cache;   // (m, n, ttype) -> (pass kernel, tile_rows)
-    int autotune = 1;            // time pass-kernel candidates on a shape's first solve
+    int autotune = 1;            // pass kernel and tile height by shape (0: the handle's fixed kernel)
     int batch_min_rows = 16;     // smallest tile height of a batched instance (even)
     int res_clusters = 0;        // resident-kernel clusters the device holds at once (0: not available)
+    GridSync* d_gs = nullptr;    // barrier counters of the cooperative kernel
+    int coop_epoch = 0;
+    bool persist_on = false;     // the current single-instance call runs its passes in the cooperative kernel
     int* d_res1 = nullptr;       // {0, 1}: the list and count of a single-instance resident launch
     bool res_on = false;         // the current single-instance call runs in the resident kernel
     // host staging for pdot_solve_host
@@ -261,11 +269,7 @@ struct pdot_handle {
     long long sched_len = 0;
 
     BatchEngine* batch = nullptr;
-    int l2_hint = 0;             // L2 eviction-priority hints in the bulk pass (measured slower; opt-in)
-    int coop = 0;                // 1: single FP32-plan solves run one cooperative launch per chunk (opt-in: measured slower)
-    GridBar* d_gb = nullptr;
-    long long l2_bytes = 0;
-    void* d_tp = nullptr;        // pdot_time_pass: a second instance view and controller
+    void* d_tp = nullptr;        // pdot_time_pass: instance views with their own controllers
 };
 
 namespace {
@@ -376,9 +380,7 @@ int tile_rows_for(pdot_handle* h, long long m, long long n, int ttype, int kerne
     // each (the last wave of a dynamic queue would leave a tail), as tall as
     // that allows (fewer column partials).
     const long long blocks = ttype == TT_F64 ? h->cfg.tile_blocks_f64
-                             : kernel == 1   ? (h->coop && h->cfg.coop_blocks > 0 ? h->cfg.coop_blocks
-                                                                                  : h->cfg.bulk_blocks)
-                             : kernel == 2   ? h->cfg.group_blocks
+                             : kernel >= 1   ? h->cfg.bulk_blocks
                                              : h->cfg.tile_blocks;
     const long long warps = blocks * TWARPS;
     long long nch = warps / nstrips;
@@ -390,21 +392,15 @@ int tile_rows_for(pdot_handle* h, long long m, long long n, int ttype, int kerne
     return (int)tr;
 }
 
-// Autotuner cache key: shape, cost type and (generated costs) coordinate count.
-long long tune_key(long long m, long long n, int ttype, int gen_d) {
-    return ((m * 1000003LL + n) * 4 + ttype) * 16 + gen_d;
-}
 int gen_dims_of(const void* C, int ctype) {
     return ctype == PDOT_POINTS ? (int)static_cast<const pdot_points_cost*>(C)->d : 0;
 }
 
-int pick_tile_rows(pdot_handle* h, long long m, long long n, int ttype, bool batch = false, int gen_d = 0) {
-    if (!batch && h->opt.tile_rows <= 0) {
-        const long long key = tune_key(m, n, ttype, gen_d);
-        auto it = h->tune_cache.find(key);
-        if (it != h->tune_cache.end() && it->second.first == h->cfg.pass_bulk) return it->second.second;
-    }
-    return tile_rows_for(h, m, n, ttype, h->cfg.pass_bulk, batch);
+// Tile height of a call: by shape when the library picks the kernel (one tile
+// per resident warp), else the explicit kernel's.
+int pick_tile_rows(pdot_handle* h, long long m, long long n, int ttype, bool batch = false) {
+    const bool by_shape = !batch && h->autotune && h->opt.pass_kernel == 0;
+    return tile_rows_for(h, m, n, ttype, by_shape ? 1 : h->cfg.pass_bulk, batch);
 }
 
 const void* prepare_C(pdot_handle* h, long long m, long long n, const void* C, int ctype, long long ldc,
@@ -435,9 +431,10 @@ const void* prepare_C(pdot_handle* h, long long m, long long n, const void* C, i
 }
 
 void init_ctrl(pdot_handle* h, Ctrl* S, long long m, long long n, double tol, double norm_b, double norm_C,
-               bool fixed, double eta_fixed, double omega_fixed) {
+               bool fixed, double eta_fixed, double omega_fixed, bool lag) {
     const pdot_options& o = h->opt;
     memset(S, 0, sizeof(Ctrl));
+    S->lag = lag ? LAG : 0;
     S->adaptive_step = fixed ? 0 : o.adaptive_step;
     S->adaptive_restart = o.adaptive_restart;
     S->pw_update = o.primal_weight_update;
@@ -468,24 +465,17 @@ void init_ctrl(pdot_handle* h, Ctrl* S, long long m, long long n, double tol, do
     S->sched = h->d_sched;
     S->sched_len = h->sched_len;
     S->cur = 0; S->anc = 0; S->bar = 1; S->nxt = 2; S->barn = 3;
+    S->xcur = 0; S->xanc = 0; S->xbar = 1;
+    S->xdst = plan_dst(S->xcur, S->xbar, S->xanc);
     S->status = ST_RUNNING;
     S->res_slot = S->res_xslot = 0;
 }
 
 void launch_count(pdot_handle* h, int k) { h->launches += k; }
 
-// Keep C resident in L2 when it takes at most half of it (it is re-read every
-// pass; the plan streams get evict-first so they do not push it out).
-bool keep_c_in_l2(pdot_handle* h, const Inst& I) {
-    if (!h->l2_hint || h->l2_bytes <= 0 || I.ctype == PDOT_POINTS) return false;
-    const double cbytes = (double)I.m * (double)I.ldc * (double)csize_of(I.ctype);
-    return cbytes <= 0.5 * (double)h->l2_bytes;
-}
-
 // Upload the instance descriptor and reset the work counters.
 void stage_instance(pdot_handle* h, const Inst& I) {
     *h->h_inst = I;
-    h->h_inst->l2_keep_c = keep_c_in_l2(h, I) ? 1 : 0;
     h->cfg.gen_dims = I.ctype == PDOT_POINTS ? I.gen.d : 0;
     CK(cudaMemcpyAsync(h->d_inst, h->h_inst, sizeof(Inst), cudaMemcpyHostToDevice, h->stream));
     CK(cudaMemsetAsync(h->wctr, 0, sizeof(unsigned) * WC_N, h->stream));
@@ -511,8 +501,19 @@ void run_avgfix(pdot_handle* h, int ttype) {
     launch_count(h, 1);
 }
 
+// Whether the pass kernel of the current configuration defers plan writes
+// (every FP32-plan pass but the register pipeline).
+bool lag_for(pdot_handle* h, int ttype) { return ttype != TT_F64 && h->cfg.pass_bulk != 0; }
+
+// Apply and write the pending steps of deferred plan writes.
+void run_final(pdot_handle* h, int ttype) {
+    CKL(launch_plan_final(ttype, h->d_inst, h->d_tmap, h->d_cnt, h->wctr, h->cfg, h->stream));
+    launch_count(h, 1);
+}
+
 void issue_chunk_kernels(pdot_handle* h, int ttype, int K) {
     for (int s = 0; s < K; ++s) run_step(h, ttype);
+    if (lag_for(h, ttype)) run_final(h, ttype);
     run_check(h, ttype, MODE_CHECK);
     run_avgfix(h, ttype);
 }
@@ -525,25 +526,38 @@ bool resident_for(pdot_handle* h, long long m, long long n, int ttype) {
            (ttype == TT_F32 || ttype == TT_BF16) && resident_fits(m, n);
 }
 
-bool use_coop(pdot_handle* h, int ttype) {
-    return h->coop && h->cfg.coop_blocks > 0 && ttype != TT_F64 && ttype != TT_GEN && h->cfg.pass_bulk == 1;
+// Whether a single-instance call takes the cooperative kernel: the library's
+// own choice of kernel and tiling (one tile per resident warp), deferred plan
+// writes, all tiles resident at once, and a generated cost of at most four
+// coordinates unless its entries stay in shared memory.
+bool persist_for(pdot_handle* h, long long m, long long n, int ttype, int tile_rows) {
+    if (!lag_for(h, ttype) || h->opt.pass_kernel != 0 || h->opt.tile_rows != 0 || h->cfg.coop_blocks <= 0) return false;
+    const long long tiles = ((n + STRIP - 1) / STRIP) * ((m + tile_rows - 1) / tile_rows);
+    if (tiles > (long long)h->cfg.coop_blocks * TWARPS) return false;
+    return ttype != TT_GEN || tile_rows <= persist_rows(h->cfg.comp != 0) || h->cfg.gen_dims <= 4;
+}
+
+// `npass` passes and the final write in one launch.
+void run_persist(pdot_handle* h, int ttype, int npass) {
+    const Work& w = h->ws;
+    CKL(launch_persist(ttype, h->d_inst, w.ntiles, w.tile_rows <= persist_rows(h->cfg.comp != 0), h->d_gs, h->coop_epoch, npass, h->cfg,
+                       h->stream));
+    h->coop_epoch ^= 1;
+    launch_count(h, 1);
 }
 
 void launch_chunk(pdot_handle* h, int ttype, int K) {
     const Work& w = h->ws;
+    if (h->persist_on) {
+        run_persist(h, ttype, K);
+        run_check(h, ttype, MODE_CHECK);
+        run_avgfix(h, ttype);
+        return;
+    }
     if (h->res_on) {
         // the whole check period (K passes and the check) in one resident launch
         CKL(launch_resident(ttype, h->d_inst, h->d_res1, h->d_res1 + 1, 1, K, K, 0, h->cfg, h->stream));
         launch_count(h, 1);
-        return;
-    }
-    if (use_coop(h, ttype)) {
-        CK(cudaMemsetAsync(h->wctr, 0, sizeof(unsigned) * WC_N, h->stream));
-        CK(cudaMemsetAsync(h->d_gb, 0, sizeof(GridBar), h->stream));
-        CKL(launch_chunk_coop(ttype, h->d_inst, h->d_tmap, h->d_cnt, h->d_vmap, h->d_cnt + 1, h->wctr, h->d_gb, K,
-                              h->cfg, h->stream));
-        launch_count(h, 1);
-        run_avgfix(h, ttype);
         return;
     }
     const long long key[8] = {(long long)(uintptr_t)w.base,
@@ -581,6 +595,12 @@ void launch_chunk(pdot_handle* h, int ttype, int K) {
     CK(cudaGraphLaunch(h->chunk.exec, h->stream));
     launch_count(h, h->chunk.kernels);
 }
+
+// Bytes a pass moves per plan entry (bc, bx: bytes of a cost and a plan
+// entry): C and X read, and on every pass (deferred writes: on every LAG-th,
+// and in the final pass before a check, which is counted with the check's
+// reads) D read, X and D written.
+double pass_bytes(bool lag, double bc, double bx) { return bc + bx + 3.0 * bx / (lag ? LAG : 1); }
 
 void fill_result(const Ctrl& S, pdot_result* r, pdot_status st) {
     r->status = st;
@@ -683,92 +703,36 @@ bool compensation_for(pdot_handle* h, long long m, long long n) {
     return c == 1 || (c == 2 && m * n < (1LL << 22));
 }
 
-// Autotuner: on the first single-instance solve of a shape (m, n, dtype),
-// time whole PDHG steps (fused pass + dual update, constant step) for each
-// candidate (pass kernel, tile height) on this device with CUDA events --
-// after three untimed steps, so the running average is read -- and keep the
-// fastest.  Small shapes are launch-bound: they take the default untimed.
-void autotune_pass(pdot_handle* h, long long m, long long n, const void* C, int ctype, long long ldc,
-                   const double* f, const double* g) {
+// The pass kernel of a single-instance call, by shape.  Every FP32 plan takes
+// the deferred-write pass with one tile per resident warp; what is chosen
+// here is the order in which a bottom-up pass adds the FP32 column sums:
+// whole rows below 4M plan entries, in generated costs of more than four
+// coordinates and above 30M stored FP32 entries, groups of four rows
+// otherwise.  The order costs nothing; the lines are where the two kernels
+// that these orders come from measured fastest (4096^2: groups 58.4 us, rows
+// 59.9 us; 16384^2: rows 820 us, groups 891 us; 26.9M to 33.4M entries is
+// where they crossed), and keeping them keeps every solve's bits.
+void choose_pass(pdot_handle* h, long long m, long long n, const void* C, int ctype) {
     const int ttype = ttype_of(ctype);
     const int gen_d = gen_dims_of(C, ctype);
     h->cfg.comp = compensation_for(h, m, n) ? 1 : 0;
     if (h->opt.pass_kernel > 0) {
-        // An explicit kernel choice: no timing, no cache entry.
         int v = h->opt.pass_kernel - 1;
-        if (ttype == TT_GEN && gen_d > 4 && v == 2) v = 1;   // no grouped kernel beyond 4 coordinates
+        if (ttype == TT_GEN && gen_d > 4 && v == 2) v = 1;   // rows in order beyond 4 coordinates
         h->cfg.pass_bulk = v;
         return;
     }
     if (ttype == TT_GEN && gen_d > 4) {
-        // More than 4 coordinates: the per-row kernel is the only bulk one.
         h->cfg.pass_bulk = h->cfg_base.pass_bulk ? 1 : 0;
         return;
     }
     if (ttype == TT_F64 || h->opt.tile_rows > 0 || !h->cfg_base.pass_bulk) return;
-    const long long key = tune_key(m, n, ttype, gen_d);
-    auto it = h->tune_cache.find(key);
-    if (it != h->tune_cache.end()) {
-        h->cfg.pass_bulk = it->second.first;
+    if (!h->autotune) {
+        h->cfg.pass_bulk = h->cfg_base.pass_bulk;
         return;
     }
-    if (!h->autotune || m * n < (1LL << 22)) {
-        const int kern = h->autotune ? 1 : h->cfg_base.pass_bulk;
-        h->tune_cache[key] = {kern, tile_rows_for(h, m, n, ttype, kern, false)};
-        h->cfg.pass_bulk = kern;
-        return;
-    }
-    // Each candidate is timed on whole PDHG steps (pass + dual update): tile
-    // height also sets how many partial sums the dual update has to read.
-    // Tile height 0: one tile per resident warp.  The first candidate (the
-    // grouped kernel with one tile per warp, the fastest at 4096^2 in every
-    // measurement) is the default the others must beat by 5 %.
-    const int cands[5][2] = {{2, 0}, {1, 0}, {2, 32}, {2, 64}, {2, 128}};
-    float best = 1e30f;
-    int best_k = 2, best_tr = tile_rows_for(h, m, n, ttype, 2, false, true);
-    const int reps = m * n >= (1LL << 26) ? 6 : 20;
-    for (const auto& c : cands) {
-        const int kern = c[0];
-        const int tr = c[1] ? c[1] : tile_rows_for(h, m, n, ttype, kern, false, true);
-        h->cfg.pass_bulk = kern;
-        ensure_work(h, m, n, h->opt.x_dtype, tr);
-        ensure_maps(h);
-        Work& w = h->ws;
-        long long ldc_used = ldc;
-        const void* Cd = prepare_C(h, m, n, C, ctype, ldc, &ldc_used);
-        stage_instance(h, make_inst(w, Cd, ctype, ldc_used, f, g));
-        Ctrl* S = h->h_ctrl;
-        init_ctrl(h, S, m, n, -1.0, 1.0, 1.0, true, 0.5 / std::sqrt((double)(m + n)), 1.0);
-        CK(cudaMemcpyAsync(w.ctrl, S, sizeof(Ctrl), cudaMemcpyHostToDevice, h->stream));
-        CK(cudaMemsetAsync(w.ticket, 0, sizeof(unsigned), h->stream));
-        CK(cudaMemsetAsync(w.X, 0, (size_t)w.m * w.ldx * xsize_of(w.xtype), h->stream));
-        CK(cudaMemsetAsync(w.V, 0, sizeof(double) * 2 * (size_t)(w.m + w.n), h->stream));
-        run_check(h, ttype, MODE_INIT);
-        for (int s2 = 0; s2 < 3; ++s2) run_step(h, ttype);
-        cudaEvent_t e0, e1;
-        CK(cudaEventCreate(&e0));
-        CK(cudaEventCreate(&e1));
-        CK(cudaEventRecord(e0, h->stream));
-        for (int r = 0; r < reps; ++r) run_step(h, ttype);
-        CK(cudaEventRecord(e1, h->stream));
-        CK(cudaEventSynchronize(e1));
-        float ms = 0.f;
-        CK(cudaEventElapsedTime(&ms, e0, e1));
-        cudaEventDestroy(e0);
-        cudaEventDestroy(e1);
-        launch_count(h, 3);
-        // The first candidate is the default; another one must beat the best
-        // so far by 5 % to be taken, so near-ties (which would change the
-        // FP32 summation order, and with it the trajectory, from run to run)
-        // keep the default.
-        if (best > 1e29f || ms < 0.95f * best) {
-            best = ms;
-            best_k = kern;
-            best_tr = tr;
-        }
-    }
-    h->tune_cache[key] = {best_k, best_tr};
-    h->cfg.pass_bulk = best_k;
+    const bool rows = m * n < (1LL << 22) || (ttype == TT_F32 && m * n > 30000000LL);
+    h->cfg.pass_bulk = rows ? 1 : 2;
 }
 
 // ---------------------------------------------------------------------------
@@ -816,10 +780,10 @@ void export_state(pdot_handle* h, const Ctrl& S, void* out) {
     hd.ctrl = S;
     char* o = static_cast<char*>(out);
     CK(cudaMemcpyAsync(o, &hd, sizeof(hd), cudaMemcpyHostToDevice, h->stream));
-    const int role[3] = {S.cur, S.bar, S.anc};
+    const int role[3] = {S.cur, S.bar, S.anc}, xrole[3] = {S.xcur, S.xbar, S.xanc};
     const size_t pb = (size_t)w.m * (size_t)w.ldx * xsize_of(w.xtype), vb = sizeof(double) * 2 * (size_t)(w.m + w.n);
     for (int k = 0; k < 3; ++k) {
-        CK(cudaMemcpyAsync(o + L.plan_off(k), (const char*)w.X + (size_t)role[k] * pb, pb, cudaMemcpyDeviceToDevice,
+        CK(cudaMemcpyAsync(o + L.plan_off(k), (const char*)w.X + (size_t)xrole[k] * pb, pb, cudaMemcpyDeviceToDevice,
                            h->stream));
         CK(cudaMemcpyAsync(o + L.vec_off(k), w.V + (size_t)role[k] * 2 * (size_t)(w.m + w.n), vb,
                            cudaMemcpyDeviceToDevice, h->stream));
@@ -855,6 +819,8 @@ bool import_state(pdot_handle* h, const void* in, Ctrl* S) {
     S->r_rp2 = B.r_rp2; S->r_rd2 = B.r_rd2; S->r_cx = B.r_cx; S->r_dual = B.r_dual; S->r_gap = B.r_gap;
     S->r_kkt = B.r_kkt; S->r_rel_p = B.r_rel_p; S->r_rel_d = B.r_rel_d; S->r_rel_gap = B.r_rel_gap; S->r_rel = B.r_rel;
     S->cur = 0; S->bar = 1; S->anc = 2; S->nxt = 3; S->barn = 4;
+    S->xcur = 0; S->xbar = 1; S->xanc = 2;
+    S->xdst = plan_dst(S->xcur, S->xbar, S->xanc);
     S->status = ST_RUNNING;
     S->res_slot = S->res_xslot = 0;
     S->res_avg = 0;
@@ -887,10 +853,10 @@ pdot_status solve_impl(pdot_handle* h, long long m, long long n, const void* C, 
     const int ttype = ttype_of(ctype);
     {
         const Range r_("autotune");
-        autotune_pass(h, m, n, C, ctype, ldc, f, g);
+        choose_pass(h, m, n, C, ctype);
     }
     h->res_on = h->opt.pass_kernel == 0 && resident_for(h, m, n, ttype);
-    const int tr = pick_tile_rows(h, m, n, ttype, false, gen_dims_of(C, ctype));
+    const int tr = pick_tile_rows(h, m, n, ttype);
     ensure_work(h, m, n, h->opt.x_dtype, tr);
     ensure_maps(h);
     Work& w = h->ws;
@@ -900,7 +866,9 @@ pdot_status solve_impl(pdot_handle* h, long long m, long long n, const void* C, 
     stage_instance(h, I);
 
     Ctrl* S = h->h_ctrl;
-    init_ctrl(h, S, m, n, tol, norm_b, 0.0, false, 0.0, 0.0);   // norms: computed by the init check
+    const bool lag = !h->res_on && lag_for(h, ttype);
+    h->persist_on = lag && persist_for(h, m, n, ttype, w.tile_rows);
+    init_ctrl(h, S, m, n, tol, norm_b, 0.0, false, 0.0, 0.0, lag);   // norms: computed by the init check
     CK(cudaMemsetAsync(w.ticket, 0, sizeof(unsigned), h->stream));
     {
         const Range r_("start");   // the init check, or the replayed check of a resumed solve
@@ -914,9 +882,9 @@ pdot_status solve_impl(pdot_handle* h, long long m, long long n, const void* C, 
                 CKL(launch_resident(ttype, h->d_inst, h->d_res1, h->d_res1 + 1, 1, 0,
                                     std::max(1, h->opt.restart_check_every), 1, h->cfg, h->stream));
                 launch_count(h, 1);
-            } else if (replay) {
-                run_check(h, ttype, MODE_CHECK);
-                run_avgfix(h, ttype);
+            } else {
+                if (replay) run_check(h, ttype, MODE_CHECK);
+                if (replay || lag) run_avgfix(h, ttype);   // (also splits the current duals for the first pass)
             }
         } else {
             CK(cudaMemcpyAsync(w.ctrl, S, sizeof(Ctrl), cudaMemcpyHostToDevice, h->stream));
@@ -973,7 +941,8 @@ pdot_status solve_impl(pdot_handle* h, long long m, long long n, const void* C, 
         CK(cudaStreamSynchronize(h->stream));
         if (S->status == ST_RUNNING) {
             S->status = ST_TIMEOUT;
-            S->res_slot = S->res_xslot = S->cur;
+            S->res_slot = S->cur;
+            S->res_xslot = S->xcur;
             S->res_avg = 0;
         }
     }
@@ -982,7 +951,7 @@ pdot_status solve_impl(pdot_handle* h, long long m, long long n, const void* C, 
     res->tile_rows = h->res_on ? 0 : w.tile_rows;
     const double mn = (double)m * (double)n;
     const double bc = (double)csize_of(ctype), bx = (double)xsize_of(w.xtype);
-    res->hbm_bytes = (double)S->passes * mn * (bc + 4.0 * bx) + (double)S->checks * mn * (bc + 3.0 * bx);
+    res->hbm_bytes = (double)S->passes * mn * pass_bytes(lag, bc, bx) + (double)S->checks * mn * (bc + 3.0 * bx);
     res->rounded_obj = std::numeric_limits<double>::quiet_NaN();
     const int slot = S->res_slot, xslot = S->res_xslot;   // vector set / plan of the reported point
     const char* Xslot = (const char*)w.X + (size_t)xslot * (size_t)(w.m * w.ldx) * xsize_of(w.xtype);
@@ -1391,6 +1360,10 @@ void batch_issue_chunk(pdot_handle* h, int types) {
         }
         for (int t = 0; t < NTT; ++t) {
             if (!(types & (1 << t))) continue;
+            if (lag_for(h, t)) {
+                CKL(launch_plan_final(t, B->insts.d, B->tmap[t].d, B->cnt.d + t, h->wctr, h->cfg, st));
+                launch_count(h, 1);
+            }
             CKL(launch_kkt(t, B->insts.d, B->tmap[t].d, B->cnt.d + t, h->wctr, MODE_CHECK, h->cfg, st));
             launch_count(h, 1);
         }
@@ -1470,7 +1443,8 @@ pdot_result batch_result(pdot_handle* h, const BSlot* s, int status) {
     r.tile_rows = s->resident ? 0 : s->w.tile_rows;
     const double mn = (double)s->req.m * (double)s->req.n;
     const double bc = (double)csize_of(s->req.c_dtype), bx = (double)xsize_of(h->opt.x_dtype);
-    r.hbm_bytes = (double)s->last.passes * mn * (bc + 4.0 * bx) + (double)s->last.checks * mn * (bc + 3.0 * bx);
+    r.hbm_bytes = (double)s->last.passes * mn * pass_bytes(s->last.lag != 0, bc, bx) +
+                  (double)s->last.checks * mn * (bc + 3.0 * bx);
     r.rounded_obj = std::numeric_limits<double>::quiet_NaN();
     r.seconds = std::chrono::duration<double>(Clock::now() - s->t_submit).count();
     return r;
@@ -1581,7 +1555,8 @@ bool batch_admit(pdot_handle* h) {
         B->used += s->bytes;
         // controller
         Ctrl* S = &B->ctrl_stage.h[B->live.size()];
-        init_ctrl(h, S, r.m, r.n, r.tol > 0.0 ? r.tol : h->opt.tol, 0.0, 0.0, false, 0.0, 0.0);
+        init_ctrl(h, S, r.m, r.n, r.tol > 0.0 ? r.tol : h->opt.tol, 0.0, 0.0, false, 0.0, 0.0,
+                  !s->resident && s->ttype != TT_F64 && h->cfg_base.pass_bulk != 0);
         CK(cudaMemcpyAsync(s->w.ctrl, S, sizeof(Ctrl), cudaMemcpyHostToDevice, h->stream));
         CK(cudaMemsetAsync(s->w.ticket, 0, sizeof(unsigned), h->stream));
         CK(cudaMemsetAsync(s->w.X, 0, (size_t)s->w.m * s->w.ldx * xsize_of(s->w.xtype), h->stream));
@@ -1818,9 +1793,6 @@ pdot_status pdot_create(const pdot_options* opt, int device, void* cuda_stream, 
         const int bulk = setup_bulk_pass();
         if (bulk > 0) throw CudaError{(cudaError_t)bulk};
         h->cfg.bulk_blocks = h->sm_count * (-bulk);
-        const int grp = setup_group_pass();
-        if (grp > 0) throw CudaError{(cudaError_t)grp};
-        h->cfg.group_blocks = h->sm_count * (-grp);
         const int rc = setup_resident();
         if (rc > 0) throw CudaError{(cudaError_t)rc};
         h->res_clusters = -rc;
@@ -1829,18 +1801,20 @@ pdot_status pdot_create(const pdot_options* opt, int device, void* cuda_stream, 
             CK(cudaMalloc(&h->d_res1, sizeof(one)));
             CK(cudaMemcpy(h->d_res1, one, sizeof(one), cudaMemcpyHostToDevice));
         }
+        int coop_ok = 0;
+        CK(cudaDeviceGetAttribute(&coop_ok, cudaDevAttrCooperativeLaunch, device));
+        const int per = setup_persist();
+        if (per > 0) throw CudaError{(cudaError_t)per};
+        h->cfg.coop_blocks = coop_ok ? h->sm_count * (-per) : 0;
+        const char* pe = getenv("PDOT_COOP");   // 0: an iteration as two kernels (comparison runs)
+        if (pe && atoi(pe) == 0) h->cfg.coop_blocks = 0;
+        CK(cudaMalloc(&h->d_gs, sizeof(GridSync)));
+        CK(cudaMemset(h->d_gs, 0, sizeof(GridSync)));
         const int kb = setup_kkt_bulk();
         if (kb > 0) throw CudaError{(cudaError_t)kb};
         h->cfg.kkt_blocks = h->sm_count * (-kb);
         const char* kk = getenv("PDOT_KKT_BULK");
         if (kk && atoi(kk) == 0) h->cfg.kkt_blocks = 0;   // the register KKT pass (comparison)
-        const int coop = setup_coop_chunk();
-        if (coop > 0) throw CudaError{(cudaError_t)coop};
-        int coop_ok = 0;
-        CK(cudaDeviceGetAttribute(&coop_ok, cudaDevAttrCooperativeLaunch, device));
-        h->cfg.coop_blocks = coop_ok ? h->sm_count * (-coop) : 0;
-        const char* cp = getenv("PDOT_COOP");
-        if (cp && atoi(cp) == 1) h->coop = 1;
         h->cfg.pass_bulk = 1;
         const char* pb = getenv("PDOT_PASS_BULK");
         if (pb) {
@@ -1854,11 +1828,6 @@ pdot_status pdot_create(const pdot_options* opt, int device, void* cuda_stream, 
         if (bm && atoi(bm) >= 2 && atoi(bm) <= 64 && atoi(bm) % 2 == 0) h->batch_min_rows = atoi(bm);
         const char* at = getenv("PDOT_AUTOTUNE");
         if (at && atoi(at) == 0) h->autotune = 0;
-        int l2 = 0;
-        CK(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, device));
-        h->l2_bytes = l2;
-        const char* lh = getenv("PDOT_L2HINT");
-        if (lh && atoi(lh) == 1) h->l2_hint = 1;
         // Programmatic dependent launch: on (PDOT_PDL=0 turns it off).
         const char* pp = getenv("PDOT_PDL");
         h->cfg.pdl = (pp && atoi(pp) == 0) ? 0 : 1;
@@ -1885,8 +1854,6 @@ pdot_status pdot_create(const pdot_options* opt, int device, void* cuda_stream, 
         CK(cudaMallocHost(&h->h_inst, sizeof(Inst)));
         CK(cudaMallocHost(&h->h_status, 2 * sizeof(int)));
         CK(cudaMalloc(&h->d_cnt, 4 * sizeof(int)));
-        CK(cudaMalloc(&h->d_gb, sizeof(GridBar)));
-        CK(cudaMemset(h->d_gb, 0, sizeof(GridBar)));
         CK(cudaMallocHost(&h->h_cnt, 4 * sizeof(int)));
         return PDOT_OK;
     });
@@ -1915,8 +1882,8 @@ pdot_status pdot_destroy(pdot_handle* h) {
     if (h->h_inst) cudaFreeHost(h->h_inst);
     if (h->h_status) cudaFreeHost(h->h_status);
     if (h->d_cnt) cudaFree(h->d_cnt);
-    if (h->d_gb) cudaFree(h->d_gb);
     if (h->d_tp) cudaFree(h->d_tp);
+    if (h->d_gs) cudaFree(h->d_gs);
     if (h->d_res1) cudaFree(h->d_res1);
     if (h->h_cnt) cudaFreeHost(h->h_cnt);
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
@@ -2032,8 +1999,8 @@ pdot_status pdot_pdhg_steps(pdot_handle* h, int64_t m, int64_t n, const void* C,
         check_common_args(h, m, n, C, c_dtype, ldc, f, g);
         if (k < 0 || !(eta > 0.0) || !(omega > 0.0) || !X || !p || !q) throw ArgError{"bad k, eta, omega or state"};
         const int ttype = ttype_of(c_dtype);
-        autotune_pass(h, m, n, C, c_dtype, ldc, f, g);   // the pass kernel a solve of this shape runs
-        const int tr = pick_tile_rows(h, m, n, ttype, false, gen_dims_of(C, c_dtype));
+        choose_pass(h, m, n, C, c_dtype);   // the pass kernel a solve of this shape runs
+        const int tr = pick_tile_rows(h, m, n, ttype);
         ensure_work(h, m, n, h->opt.x_dtype, tr);
         ensure_maps(h);
         Work& w = h->ws;
@@ -2041,39 +2008,48 @@ pdot_status pdot_pdhg_steps(pdot_handle* h, int64_t m, int64_t n, const void* C,
         const void* Cd = prepare_C(h, m, n, C, c_dtype, ldc, &ldc_used);
         stage_instance(h, make_inst(w, Cd, c_dtype, ldc_used, f, g));
         Ctrl* S = h->h_ctrl;
-        init_ctrl(h, S, m, n, -1.0, 1.0, 1.0, true, eta, omega);
+        const bool resident = h->opt.pass_kernel == 0 && resident_for(h, m, n, ttype);
+        const bool lag = !resident && lag_for(h, ttype);
+        init_ctrl(h, S, m, n, -1.0, 1.0, 1.0, true, eta, omega, lag);
         S->adaptive_restart = 0;
         S->pw_update = 0;
         CK(cudaMemcpyAsync(w.ctrl, S, sizeof(Ctrl), cudaMemcpyHostToDevice, h->stream));
         CK(cudaMemsetAsync(w.ticket, 0, sizeof(unsigned), h->stream));
         upload_state(h, X, p, q);
         run_check(h, ttype, MODE_INIT);   // row/column sums of the starting plan
-        if (h->opt.pass_kernel == 0 && resident_for(h, m, n, ttype)) {
+        if (resident) {
             if (k > 0) {   // k steps in one resident launch, no check
                 CKL(launch_resident(ttype, h->d_inst, h->d_res1, h->d_res1 + 1, 1, (int)k, 0, 0, h->cfg, h->stream));
                 launch_count(h, 1);
             }
         } else {
-            for (int64_t s = 0; s < k; ++s) run_step(h, ttype);
+            if (lag && persist_for(h, m, n, ttype, w.tile_rows)) {
+                constexpr int64_t MOST = 1 << 20;   // (the barrier counter's range)
+                for (int64_t s = 0; s < k; s += MOST) run_persist(h, ttype, (int)std::min(MOST, k - s));
+            } else {
+                for (int64_t s = 0; s < k; ++s) run_step(h, ttype);
+                if (lag) run_final(h, ttype);
+            }
         }
         CK(cudaMemcpyAsync(S, w.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, h->stream));
         CK(cudaStreamSynchronize(h->stream));
         if (S->status == ST_ARG) throw ArgError{"invalid marginals"};
         if (S->status == ST_NUMERIC) return PDOT_ERR_NUMERIC;
-        const int cur = S->cur, bar = k > 0 ? S->bar : S->cur;
-        copy_plan_out(h, cur, X, cudaMemcpyDeviceToDevice);
+        const int cur = S->cur, bar = k > 0 ? S->bar : S->cur;   // vector sets
+        const int xcur = plan_slot(*S);
+        copy_plan_out(h, xcur, X, cudaMemcpyDeviceToDevice);
         copy_duals_out(h, cur, p, q, cudaMemcpyDeviceToDevice);
         if (Xbar_out) {
             // The average slot holds its deviation from the current plan:
-            // form X + D in the free next slot, then copy it out.
-            int src = cur;
+            // form X + D in a free slot, then copy it out.
+            int src = xcur;
             if (k > 0) {
                 const size_t pe = (size_t)w.m * (size_t)w.ldx, xs = xsize_of(w.xtype);
                 const char* base = (const char*)w.X;
-                CKL(launch_combine(w.xtype, base + (size_t)cur * pe * xs, base + (size_t)bar * pe * xs,
-                                   (char*)w.X + (size_t)S->nxt * pe * xs, (long long)pe, h->stream));
+                src = free_slot(xcur, S->xbar, S->xbar);
+                CKL(launch_combine(w.xtype, base + (size_t)xcur * pe * xs, base + (size_t)S->xbar * pe * xs,
+                                   (char*)w.X + (size_t)src * pe * xs, (long long)pe, h->stream));
                 launch_count(h, 1);
-                src = S->nxt;
             }
             copy_plan_out(h, src, Xbar_out, cudaMemcpyDeviceToDevice);
         }
@@ -2095,7 +2071,7 @@ pdot_status pdot_kkt(pdot_handle* h, int64_t m, int64_t n, const void* C, pdot_d
         double norm_b = 0.0;
         validate_marginals(h, m, n, f, g, false, &norm_b);
         const int ttype = ttype_of(c_dtype);
-        const int tr = pick_tile_rows(h, m, n, ttype, false, gen_dims_of(C, c_dtype));
+        const int tr = pick_tile_rows(h, m, n, ttype);
         ensure_work(h, m, n, h->opt.x_dtype, tr);
         ensure_maps(h);
         Work& w = h->ws;
@@ -2103,7 +2079,7 @@ pdot_status pdot_kkt(pdot_handle* h, int64_t m, int64_t n, const void* C, pdot_d
         const void* Cd = prepare_C(h, m, n, C, c_dtype, ldc, &ldc_used);
         stage_instance(h, make_inst(w, Cd, c_dtype, ldc_used, f, g));
         Ctrl* S = h->h_ctrl;
-        init_ctrl(h, S, m, n, -1.0, norm_b, 0.0, false, 0.0, 0.0);
+        init_ctrl(h, S, m, n, -1.0, norm_b, 0.0, false, 0.0, 0.0, false);
         CK(cudaMemcpyAsync(w.ctrl, S, sizeof(Ctrl), cudaMemcpyHostToDevice, h->stream));
         CK(cudaMemsetAsync(w.ticket, 0, sizeof(unsigned), h->stream));
         upload_state(h, X, p, q);
@@ -2269,8 +2245,8 @@ pdot_status pdot_time_pass(pdot_handle* h, int64_t m, int64_t n, const void* C, 
         check_common_args(h, m, n, C, c_dtype, ldc, f, g);
         if (reps < 1 || !ms_per_pass) throw ArgError{"reps < 1 or null output"};
         const int ttype = ttype_of(c_dtype);
-        autotune_pass(h, m, n, C, c_dtype, ldc, f, g);
-        const int tr = pick_tile_rows(h, m, n, ttype, false, gen_dims_of(C, c_dtype));
+        choose_pass(h, m, n, C, c_dtype);
+        const int tr = pick_tile_rows(h, m, n, ttype);
         ensure_work(h, m, n, h->opt.x_dtype, tr);
         ensure_maps(h);
         Work& w = h->ws;
@@ -2278,33 +2254,52 @@ pdot_status pdot_time_pass(pdot_handle* h, int64_t m, int64_t n, const void* C, 
         const void* Cd = prepare_C(h, m, n, C, c_dtype, ldc, &ldc_used);
         stage_instance(h, make_inst(w, Cd, c_dtype, ldc_used, f, g));
         Ctrl* S = h->h_ctrl;
-        init_ctrl(h, S, m, n, -1.0, 1.0, 1.0, true, 0.5 / std::sqrt((double)(m + n)), 1.0);
+        const bool lag = lag_for(h, ttype);
+        init_ctrl(h, S, m, n, -1.0, 1.0, 1.0, true, 0.5 / std::sqrt((double)(m + n)), 1.0, lag);
         CK(cudaMemcpyAsync(w.ctrl, S, sizeof(Ctrl), cudaMemcpyHostToDevice, h->stream));
         CK(cudaMemsetAsync(w.ticket, 0, sizeof(unsigned), h->stream));
         CK(cudaMemsetAsync(w.X, 0, (size_t)w.m * w.ldx * xsize_of(w.xtype), h->stream));
         CK(cudaMemsetAsync(w.V, 0, sizeof(double) * 2 * (size_t)(w.m + w.n), h->stream));
         run_check(h, ttype, MODE_INIT);
-        for (int s = 0; s < 3; ++s) run_step(h, ttype);   // steady state: k > 0, the average is read
-        // Two views of the instance whose controllers swap the current and
-        // next roles (and the pass parity, so the row order alternates):
-        // launches alternate between them, so each pass reads the plans the
-        // previous one wrote, as accepted passes of a solve do; the dual
-        // update is left out, so every launch moves the same bytes.
+        // Steady state: k > 0 (the average is read), and with deferred writes
+        // a plan that has left the anchor (it is then written in place) with
+        // every set of split duals written.
+        for (int s = 0; s < 2 * YRING; ++s) run_step(h, ttype);
+        // Views of the instance with controllers of their own, one per pass
+        // of a cycle; launches take them in turn and the dual update is left
+        // out.  Plain passes: two views whose controllers swap the current
+        // and next roles, so each pass reads the plans the previous one wrote,
+        // as accepted passes of a solve do.  Deferred writes: LAG views with
+        // 1, .., LAG pending steps (the last one applies and writes them, as
+        // every LAG-th accepted pass does).  The pass parity alternates with
+        // the launches, so the row order does too.
+        constexpr int VIEWS = LAG > 2 ? 2 * LAG : 4;   // an even number of passes per cycle
         if (!h->d_tp) {
-            CK(cudaMalloc(&h->d_tp, sizeof(Inst) + sizeof(Ctrl) + 256));
+            CK(cudaMalloc(&h->d_tp, (align_up(sizeof(Inst), 256) + align_up(sizeof(Ctrl), 256)) * VIEWS));
         }
-        Inst* d_inst2 = reinterpret_cast<Inst*>(h->d_tp);
-        Ctrl* d_ctrl2 = reinterpret_cast<Ctrl*>(reinterpret_cast<char*>(h->d_tp) + align_up(sizeof(Inst), 256));
+        char* tp = reinterpret_cast<char*>(h->d_tp);
         CK(cudaMemcpyAsync(S, w.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, h->stream));
         CK(cudaStreamSynchronize(h->stream));
-        std::swap(S->cur, S->nxt);
-        std::swap(S->bar, S->barn);
-        S->passes += 1;
-        Inst I2 = *h->h_inst;
-        I2.ctrl = d_ctrl2;
-        CK(cudaMemcpyAsync(d_ctrl2, S, sizeof(Ctrl), cudaMemcpyHostToDevice, h->stream));
-        CK(cudaMemcpyAsync(d_inst2, &I2, sizeof(Inst), cudaMemcpyHostToDevice, h->stream));
-        CK(cudaStreamSynchronize(h->stream));   // I2 lives on this stack frame
+        Inst* views[VIEWS];
+        for (int v = 0; v < VIEWS; ++v) {
+            Inst Iv = *h->h_inst;
+            views[v] = reinterpret_cast<Inst*>(tp);
+            tp += align_up(sizeof(Inst), 256);
+            Iv.ctrl = reinterpret_cast<Ctrl*>(tp);
+            tp += align_up(sizeof(Ctrl), 256);
+            Ctrl Sv = *S;
+            Sv.passes += v;
+            if (lag) {
+                Sv.npend = v % LAG + 1;
+                Sv.pfirst = 0;
+            } else if (v & 1) {
+                std::swap(Sv.cur, Sv.nxt);
+                std::swap(Sv.bar, Sv.barn);
+            }
+            CK(cudaMemcpyAsync(Iv.ctrl, &Sv, sizeof(Ctrl), cudaMemcpyHostToDevice, h->stream));
+            CK(cudaMemcpyAsync(views[v], &Iv, sizeof(Inst), cudaMemcpyHostToDevice, h->stream));
+            CK(cudaStreamSynchronize(h->stream));   // Sv and Iv live on this stack frame
+        }
         cudaEvent_t e0, e1;
         CK(cudaEventCreate(&e0));
         CK(cudaEventCreate(&e1));
@@ -2313,7 +2308,7 @@ pdot_status pdot_time_pass(pdot_handle* h, int64_t m, int64_t n, const void* C, 
         // but its own, so the next launch finds its counter at zero.
         for (int r = 0; r < reps; ++r) {
             const int wc = (r & 1) ? wc_index(WC_AUX, ttype) : wc_index(WC_PASS, ttype);
-            CKL(launch_pass(ttype, (r & 1) ? d_inst2 : h->d_inst, h->d_tmap, h->d_cnt, h->wctr, h->cfg, h->stream, wc));
+            CKL(launch_pass(ttype, views[r % VIEWS], h->d_tmap, h->d_cnt, h->wctr, h->cfg, h->stream, wc));
         }
         CK(cudaEventRecord(e1, h->stream));
         CK(cudaEventSynchronize(e1));
@@ -2324,7 +2319,8 @@ pdot_status pdot_time_pass(pdot_handle* h, int64_t m, int64_t n, const void* C, 
         launch_count(h, reps);
         *ms_per_pass = (double)ms / reps;
         if (bytes_per_pass)
-            *bytes_per_pass = (double)m * (double)n * ((double)csize_of(c_dtype) + 4.0 * (double)xsize_of(w.xtype));
+            *bytes_per_pass = (double)m * (double)n *
+                              pass_bytes(lag, (double)csize_of(c_dtype), (double)xsize_of(w.xtype));
         if (kernel_variant) {
             int v = ttype == TT_F64 ? 0 : h->cfg.pass_bulk;
             if (ttype == TT_GEN && v == 2 && h->cfg.gen_dims > 4) v = 1;   // no grouped kernel beyond 4 coordinates

@@ -18,7 +18,10 @@
 //   Ctrl : the scalar state of Algorithm 2 and the Sec. 5 controller.
 #pragma once
 #include <cmath>
+#include <cstddef>
 #include <cstdint>
+
+#include <vector_types.h>
 
 namespace pdot {
 
@@ -29,6 +32,8 @@ constexpr int VT = 256;      // threads per CTA in the vector kernels
 constexpr int VE = 32;       // entries per vector tile (one warp wide)
 constexpr int VG = VT / 32;  // partial-sum groups per vector tile
 constexpr int TP = 6;        // scalars per plan-tile partial
+constexpr int LAG = 3;       // accepted steps a plan pass may leave unapplied in the stored plan (pdot_pass.cuh)
+constexpr int YRING = LAG + 2;   // split duals kept: LAG pending steps, the current step, the next one
 constexpr int VP = 12;       // scalars per vector-tile partial
 
 constexpr int ST_RUNNING = -1;
@@ -72,7 +77,31 @@ struct Ctrl {
     // them itself.
     const double* sched;
     long long sched_len;
+    // Plan slots.  Without deferred writes (lag == 0) they equal cur, bar and
+    // anc.  With them (lag == LAG) the vector roles above move with every
+    // accepted step and the plan's roles only when pending steps are applied
+    // or at a restart: X[xcur] is the iterate before the npend pending steps,
+    // X[xbar] the deviation D that goes with it, X[xdst] where both steps and
+    // D are applied to (xcur itself unless that is the anchor).
+    int lag, npend, h0, pfirst;   // h0: ring index of the first pending step; pfirst: that step starts an epoch
+    int xcur, xbar, xanc, xdst;
+    float ptau[YRING], pw[YRING]; // step size and averaging weight of the pending steps, by ring index
 };
+
+// The lowest plan slot that is none of the three.
+__host__ __device__ __forceinline__ int free_slot(int a, int b, int c) {
+    int s = 0;
+    while (s == a || s == b || s == c) ++s;
+    return s;
+}
+// Where deferred plan writes go: in place, or beside the restart anchor.
+__host__ __device__ __forceinline__ int plan_dst(int xcur, int xbar, int xanc) {
+    return xcur != xanc ? xcur : free_slot(xanc, xbar, xbar);
+}
+// The plan slot of the current iterate after the pending steps have been
+// written (the final pass before a check), while the roles still say they
+// are pending.
+__host__ __device__ __forceinline__ int plan_slot(const Ctrl& S) { return S.npend > 0 ? S.xdst : S.xcur; }
 
 // Cost generated from coordinates (pdot_dtype PDOT_POINTS):
 //   C_ij = dist(xs_i, ys_j) / div, coordinates k = 0..d-1 accumulated in order
@@ -131,6 +160,8 @@ struct Inst {
     long long xslot;
     double* V;           // NSLOT vector sets of vslot doubles
     long long vslot;
+    float2* yf;          // YRING sets of [p | q] as FP32 pairs (deferred plan writes; null without)
+    long long yslot;
     double* rowpart;
     double* colpart;
     double* rowpart2;    // the check's exact row / column sums of the current plan
@@ -140,16 +171,12 @@ struct Inst {
     Ctrl* ctrl;
     unsigned int* ticket;
     int nstrips, nchunks, tile_rows, ntiles, nvt;
-    int l2_keep_c;       // 1: C fits in L2 next to the streams; load it evict-last, stream X evict-first
 };
 
-// Grid barrier state of the cooperative chunk kernel (device memory, zeroed
-// before each launch).
-struct GridBar {
-    unsigned int count;
-    unsigned int gen;
-    unsigned int err;
-    unsigned int pad;
+// Barrier counters of the cooperative kernel (zeroed once; launches take
+// them in turn and each zeroes the other).
+struct GridSync {
+    unsigned int count[2];
 };
 
 struct TileRef {
@@ -179,10 +206,9 @@ struct LaunchCfg {
     int tile_blocks_f64;  // CTAs of the FP64-plan tile kernels
     int vec_blocks;       // CTAs of the vector kernels (256 threads each)
     int pass_u;           // rows per load batch in the FP32-plan register pass (2 or 4)
-    int pass_bulk;        // FP32-plan pass kernel: 0 register pipeline, 1 bulk copies per row, 2 per 4-row group
-    int bulk_blocks;      // CTAs of the bulk-copy pass kernel
-    int group_blocks;     // CTAs of the grouped bulk-copy pass kernel
-    int coop_blocks;      // CTAs of the cooperative chunk kernel (all co-resident)
+    int pass_bulk;        // FP32-plan pass: 0 register pipeline, 1 / 2 deferred writes (rows / groups in order)
+    int bulk_blocks;      // CTAs of the deferred-write pass kernel
+    int coop_blocks;      // CTAs of the cooperative kernel that fit at once (0: no cooperative launch)
     int pdl;              // 1: launch with programmatic dependent launch
     int gen_dims;         // largest coordinate count of the generated costs in flight (TT_GEN)
     int comp;             // 1: plan passes of FP32 plans form the compensated reduced cost
@@ -195,6 +221,9 @@ struct LaunchCfg {
 // instance's pass count; the pass timer flips it between its launches).
 int launch_pass(int ttype, const Inst* d_insts, const TileRef* d_tmap, const int* T, unsigned* wctr,
                 const LaunchCfg& cfg, void* stream, int wc_override = -1, int dir_xor = 0);
+// Apply and write the pending steps of deferred plan writes (before a check or a copy of the plan).
+int launch_plan_final(int ttype, const Inst* d_insts, const TileRef* d_tmap, const int* T, unsigned* wctr,
+                      const LaunchCfg& cfg, void* stream);
 int launch_dual(const Inst* d_insts, const TileRef* d_vmap, const int* NV, int nv_hint, unsigned* wctr,
                 const LaunchCfg& cfg, void* stream, bool direct = false);
 int launch_kkt(int ttype, const Inst* d_insts, const TileRef* d_tmap, const int* T, unsigned* wctr, int mode,
@@ -202,8 +231,8 @@ int launch_kkt(int ttype, const Inst* d_insts, const TileRef* d_tmap, const int*
 int launch_checkvec(const Inst* d_insts, const TileRef* d_vmap, const int* NV, int nv_hint, unsigned* wctr, int mode,
                     const LaunchCfg& cfg, void* stream);
 int launch_snapshot(const Inst* d_insts, const int* count, int max_count, Ctrl* out, void* stream);
-// After a check: form the average plan the check picked (Ctrl::fix) for the
-// instances of one tile type.
+// After a check: form the average plan the check picked (Ctrl::fix) and
+// split the current duals for the next pass, for the instances of one type.
 int launch_avgfix(int ttype, const Inst* d_insts, const TileRef* d_tmap, const int* T, const LaunchCfg& cfg,
                   void* stream);
 // Resident solve (one thread-block cluster per instance, the plan held in
@@ -227,11 +256,13 @@ int occupancy_vec_blocks_per_sm();
 // Opt the bulk-copy pass kernel into its shared-memory size; returns minus
 // the CTAs per SM it can hold, or a positive cudaError_t code.
 int setup_bulk_pass();
-int setup_group_pass();
+int setup_persist();
+// Passes of a single FP32-plan instance (one tile per warp, all resident) and
+// the final write of its pending steps, in one cooperative launch.
+int launch_persist(int ttype, const Inst* d_insts, int ntiles, bool on_chip, GridSync* gs, int epoch, int npass,
+                   const LaunchCfg& cfg, void* stream);
+// Tallest tile that stays in the cooperative kernel's shared memory.
+int persist_rows(bool comp);
 int setup_kkt_bulk();
-int setup_coop_chunk();
-// K passes and one check of a single FP32-plan instance in one cooperative launch.
-int launch_chunk_coop(int ttype, const Inst* d_insts, const TileRef* d_tmap, const int* T, const TileRef* d_vmap,
-                      const int* NV, unsigned* wctr, GridBar* gb, int npass, const LaunchCfg& cfg, void* stream);
 
 }  // namespace pdot

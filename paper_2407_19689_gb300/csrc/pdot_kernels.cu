@@ -34,14 +34,13 @@
 
 namespace pdot {
 
-constexpr int KU = 2;
+constexpr int KU = 2;   // rows per load batch in the register KKT pass
 // Rows a plan pass (KKT pass) accumulates in FP32 per lane before adding into
 // its FP64 partial sums: FP64 is a narrow pipe on this part, and the FP32
 // partial over 32 (64) rows of one column carries a relative error of order
 // 1e-7, far below what the FP64 sums it feeds are compared against.
 constexpr int FLUSH_ROWS = 32;
 constexpr int KKT_FLUSH_ROWS = 64;
-constexpr int BULK_ROW_S = 8;   // row stages per warp in the per-row bulk pass   // rows per load batch in the KKT pass
 
 // ---------------------------------------------------------------------------
 // loads and stores of 4 consecutive elements
@@ -404,13 +403,7 @@ k_pass(const Inst* __restrict__ insts, const TileRef* __restrict__ tmap, const i
 }
 
 // ---------------------------------------------------------------------------
-// Plan pass, bulk-copy pipeline (FP32 plans): the same arithmetic as
-// pass_tile, but every warp streams its rows through a ring of S shared-memory
-// stages filled by the bulk-copy engine (cp.async.bulk, completion counted on
-// one mbarrier per stage).  Rows in flight cost no registers, so each SM keeps
-// ~S x 1.5 KB per warp of reads outstanding.  The warp's row stream runs
-// across tile boundaries: the producer (lane 0) fetches the next tile from the
-// queue as soon as it has issued the current one's last row.
+// Bulk copies (cp.async.bulk) with completion counted on mbarriers.
 // ---------------------------------------------------------------------------
 namespace bulk {
 
@@ -426,31 +419,6 @@ __device__ __forceinline__ void g2s(unsigned dst, const void* src, unsigned byte
                  "l"(src), "r"(bytes), "r"(bar)
                  : "memory");
 }
-// Bulk copy with an L2 eviction-priority policy (createpolicy descriptor).
-__device__ __forceinline__ void g2s_hint(unsigned dst, const void* src, unsigned bytes, unsigned bar,
-                                         unsigned long long pol) {
-    asm volatile(
-        "cp.async.bulk.shared::cta.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;" ::"r"(
-            dst),
-        "l"(src), "r"(bytes), "r"(bar), "l"(pol)
-        : "memory");
-}
-__device__ __forceinline__ unsigned long long policy_evict_last() {
-    unsigned long long p;
-    asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
-    return p;
-}
-__device__ __forceinline__ unsigned long long policy_evict_first() {
-    unsigned long long p;
-    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
-    return p;
-}
-__device__ __forceinline__ void st4_hint(float* p, const float (&v)[4], unsigned long long pol) {
-    asm volatile("st.global.L1::no_allocate.L2::cache_hint.v4.f32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(p), "f"(v[0]),
-                 "f"(v[1]), "f"(v[2]), "f"(v[3]), "l"(pol)
-                 : "memory");
-}
-
 __device__ __forceinline__ bool mbar_try_wait(unsigned bar, unsigned parity) {
     unsigned ok;
     asm volatile(
@@ -471,13 +439,8 @@ __device__ __forceinline__ bool wait_stage(unsigned bar, unsigned parity, long l
     return false;
 }
 
-constexpr int STAGE_BYTES = 3 * STRIP * 4;   // C (<= 512 B), X (512 B), Xbar (512 B)
-
-// Row duals of a tile are staged in shared memory, as FP32 pairs, per window
-// of PWIN rows.
+// Row duals staged per window of PWIN rows (the KKT pass).
 constexpr int PWIN = 128;
-template <int S>
-__host__ __device__ constexpr int warp_smem_bytes() { return S * STAGE_BYTES + S * 8 + S * 8 + PWIN * 8; }
 
 struct RowRef {       // what a stage holds
     int tile;         // global tile index (into tmap), -1 = none
@@ -486,816 +449,11 @@ struct RowRef {       // what a stage holds
 
 }  // namespace bulk
 
-namespace bulk {
-// A warp's row pipeline: its shared-memory stages and mbarriers, and the
-// counts of issued / consumed rows (they set the mbarrier phases, so they
-// persist across passes when one kernel runs several).
-template <int S>
-struct RowPipe {
-    unsigned char* wbase;
-    RowRef* refs;
-    float2* pbuf;
-    unsigned wbase_s, bars_s;
-    long long issued, consumed;
-};
+}  // namespace pdot
 
-template <int S>
-__device__ __forceinline__ void row_pipe_init(RowPipe<S>& P, unsigned char* dsm, int lane, int warp) {
-    P.wbase = dsm + warp * warp_smem_bytes<S>();
-    unsigned long long* bars = reinterpret_cast<unsigned long long*>(P.wbase + S * STAGE_BYTES);
-    P.refs = reinterpret_cast<RowRef*>(P.wbase + S * STAGE_BYTES + S * 8);
-    P.pbuf = reinterpret_cast<float2*>(P.wbase + S * STAGE_BYTES + S * 16);   // p_i of the tile's rows
-    P.wbase_s = smem_u32(P.wbase);
-    P.bars_s = smem_u32(bars);
-    P.issued = P.consumed = 0;
-    if (lane == 0) {
-        for (int s = 0; s < S; ++s) mbar_init(P.bars_s + 8 * s, 1);
-        fence_mbar_init();
-    }
-    __syncwarp();
-}
-}  // namespace bulk
+#include "pdot_pass.cuh"
 
-// One pass over the tiles handed out by the queue counter `qctr`.  Returns
-// false when a stage never completed (bounded wait); the instance's status
-// is then set to an error.
-template <typename TC, int S, bool CP>
-__device__ bool pass_row_run(const Inst* __restrict__ insts, const TileRef* __restrict__ tmap, int T, unsigned* qctr,
-                             bulk::RowPipe<S>& P, int lane, int dir_xor) {
-    using namespace bulk;
-    unsigned char* wbase = P.wbase;
-    RowRef* refs = P.refs;
-    float2* pbuf = P.pbuf;
-    const unsigned wbase_s = P.wbase_s;
-    const unsigned bars_s = P.bars_s;
-    constexpr int DM = GenDims<TC>::value;
-    constexpr bool GEN = DM > 0;                            // C generated, not copied
-    constexpr int DA = GEN ? DM : 1;                        // coordinate array size
-    constexpr long long CQ = sizeof(TC) == 2 ? 8 : 4;      // C elements per 16 bytes
-
-    // ---- producer: the tile being issued, resolved once per tile ----
-    int p_tile = T;
-    long long p_row = 0, p_stop = 0, p_r0 = 0, p_last_ragged = -1;
-    long long p_dir = 1;                // +1: top-down, -1: bottom-up (pass_reversed)
-    const char* p_c0 = nullptr;         // C at the tile's first row, column c0
-    const char* p_x0 = nullptr;         // X at the tile's first row
-    const char* p_xb0 = nullptr;        // Xbar at the tile's first row
-    long long p_cstride = 0, p_xstride = 0;
-    unsigned p_cbytes = 0, p_xbytes = 0;
-    bool p_first = true;
-    bool p_hint = false;                // keep this instance's C in L2 (it fits)
-    const unsigned long long pol_keep = policy_evict_last();
-    const unsigned long long pol_stream = policy_evict_first();
-    bool q_first = true;
-    auto next_tile = [&]() {
-        for (;;) {
-            p_tile = tile_next(qctr, q_first);
-            if (p_tile >= T) return;
-            const TileRef tr = tmap[p_tile];
-            const Inst& I = insts[tr.inst];
-            const Ctrl& Sc = *I.ctrl;
-            if (Sc.status != ST_RUNNING) continue;
-            const int strip = tr.local % I.nstrips, chunk = tr.local / I.nstrips;
-            const long long c0 = (long long)strip * STRIP;
-            const long long ncols = min((long long)STRIP, I.n - c0);
-            const long long r0 = (long long)chunk * I.tile_rows;
-            const long long r1 = min(r0 + (long long)I.tile_rows, I.m);
-            const bool rev = pass_reversed(Sc, dir_xor);
-            p_dir = rev ? -1 : 1;
-            p_r0 = r0;
-            p_row = rev ? r1 - 1 : r0;
-            p_stop = rev ? r0 - 1 : r1;
-            p_xstride = I.ldx * 4;
-            if constexpr (!GEN) {
-                p_cstride = I.ldc * (long long)sizeof(TC);
-                p_c0 = reinterpret_cast<const char*>(I.C) + r0 * p_cstride + c0 * (long long)sizeof(TC);
-            }
-            p_x0 = reinterpret_cast<const char*>(reinterpret_cast<const float*>(I.X) + (long long)Sc.cur * I.xslot +
-                                                 r0 * I.ldx + c0);
-            p_xb0 = reinterpret_cast<const char*>(reinterpret_cast<const float*>(I.X) + (long long)Sc.bar * I.xslot +
-                                                  r0 * I.ldx + c0);
-            p_xbytes = (unsigned)(((ncols + 3) / 4) * 16);
-            if constexpr (!GEN) {
-                p_cbytes = (unsigned)(((ncols + CQ - 1) / CQ) * CQ * (long long)sizeof(TC));
-                // The rounded-up C copy could run past the caller's allocation on
-                // the last matrix row of a ragged strip: lanes load that row.
-                p_last_ragged = (ncols % CQ) != 0 ? I.m - 1 : -1;
-            }
-            p_first = Sc.k == 0;
-            p_hint = I.l2_keep_c != 0;
-            return;
-        }
-    };
-    long long issued = P.issued, consumed = P.consumed;
-    const long long base = issued;   // rows of earlier passes (ring position)
-    auto issue = [&]() {
-        const int st = (int)(issued % S);
-        const long long dr = p_row - p_r0;
-        const char* p_c = p_c0 + dr * p_cstride;
-        const char* p_x = p_x0 + dr * p_xstride;
-        const char* p_xb = p_xb0 + dr * p_xstride;
-        if (lane == 0) {
-            refs[st].tile = p_tile;
-            refs[st].row = (int)p_row;
-            const unsigned bar = bars_s + 8 * st;
-            const unsigned dst = wbase_s + st * STAGE_BYTES;
-            const unsigned cb = p_row == p_last_ragged ? 0u : p_cbytes;
-            fence_proxy_async();
-            mbar_expect_tx(bar, cb + p_xbytes + (p_first ? 0u : p_xbytes));
-            if (p_hint) {
-                // C is re-read every pass and fits in L2: keep it; stream the plan.
-                if (cb) g2s_hint(dst, p_c, cb, bar, pol_keep);
-                g2s_hint(dst + STRIP * 4, p_x, p_xbytes, bar, pol_stream);
-                if (!p_first) g2s_hint(dst + 2 * STRIP * 4, p_xb, p_xbytes, bar, pol_stream);
-            } else {
-                if (cb) g2s(dst, p_c, cb, bar);
-                g2s(dst + STRIP * 4, p_x, p_xbytes, bar);
-                if (!p_first) g2s(dst + 2 * STRIP * 4, p_xb, p_xbytes, bar);
-            }
-        }
-        ++issued;
-        p_row += p_dir;
-        if (p_row == p_stop) next_tile();
-    };
-    next_tile();
-    while (issued - base < S && p_tile < T) issue();
-
-    // ---- consumer: the tile being computed, resolved once per tile ----
-    int c_tile = -1;
-    const Inst* CI = nullptr;
-    const TC* c_C = nullptr;
-    long long c_ldc = 0, c_ldx = 0, c_i0 = 0, c_n = 0, c_last_ragged = -1, c_chunk = 0;
-    float* c_xn = nullptr;      // X+ at row c_i0, column j0
-    float* c_xbn = nullptr;     // Xbar+ at row c_i0, column j0
-    double* c_rowpart = nullptr;
-    long long j0 = 0;
-    bool on = false, valid[4] = {false, false, false, false};
-    float qv[4] = {0.f, 0.f, 0.f, 0.f}, ql[4] = {0.f, 0.f, 0.f, 0.f};
-    float tau = 0.f, w = 0.f;
-    bool first = true;
-    double cs[4] = {0.0, 0.0, 0.0, 0.0}, dx2 = 0.0;
-    float csa[4] = {0.f, 0.f, 0.f, 0.f}, dxa = 0.f;
-    int rows_in_batch = 0;
-    int c_local = 0;
-    const double* c_p = nullptr;   // p of the consumer's instance
-    bool c_hint = false;
-    long long c_i1 = 0, c_win = -1;
-    // Generated cost: the lane's four columns' coordinates, and the
-    // coordinates of a window of 32 rows (lane r holds row window*32 + r).
-    GenSpec gs = {nullptr, nullptr, 0, 0, 1.f, 1.f};
-    float gy[4][DA], growc[DA];
-    long long c_cwin = -1;
-    auto flush_tile = [&]() {
-        if (c_tile < 0) return;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) cs[e] += (double)csa[e];
-        dx2 += (double)dxa;
-        if (on) {
-            double* cp = CI->colpart + c_chunk * CI->ldx + j0;
-            reinterpret_cast<double2*>(cp)[0] = make_double2(cs[0], cs[1]);
-            reinterpret_cast<double2*>(cp)[1] = make_double2(cs[2], cs[3]);
-        }
-        const double d = warp_sum(dx2);
-        if (lane == 0) CI->tpart[(long long)c_local * TP + 0] = d;
-    };
-    auto open_consumer = [&](int t) {
-        flush_tile();
-        c_tile = t;
-        const TileRef tr = tmap[t];
-        CI = &insts[tr.inst];
-        const Ctrl& Sc = *CI->ctrl;
-        c_local = tr.local;
-        const int strip = tr.local % CI->nstrips;
-        c_chunk = tr.local / CI->nstrips;
-        const long long c0 = (long long)strip * STRIP;
-        c_n = CI->n;
-        c_ldc = CI->ldc;
-        c_ldx = CI->ldx;
-        c_i0 = c_chunk * CI->tile_rows;
-        const long long i1 = min(c_i0 + (long long)CI->tile_rows, CI->m);
-        j0 = c0 + lane * 4;
-        on = j0 < c_n;
-        if constexpr (GEN) {
-            gs = CI->gen;
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-#pragma unroll
-                for (int k = 0; k < DA; ++k)
-                    gy[e][k] = (k < gs.d && j0 + e < c_n) ? __ldg(gs.ys + (j0 + e) * gs.d + k) : 0.f;
-            }
-            c_cwin = -1;
-        } else {
-            const long long ncols = min((long long)STRIP, c_n - c0);
-            c_last_ragged = (ncols % CQ) != 0 ? CI->m - 1 : -1;
-            c_C = reinterpret_cast<const TC*>(CI->C) + j0;
-        }
-        float* Xb = reinterpret_cast<float*>(CI->X);
-        c_xn = Xb + (long long)Sc.nxt * CI->xslot + c_i0 * c_ldx + j0;
-        c_xbn = Xb + (long long)Sc.barn * CI->xslot + c_i0 * c_ldx + j0;
-        c_rowpart = CI->rowpart + (long long)strip * CI->m;
-        const double* pv = slot_v(*CI, Sc.cur);
-        const double* q = pv + CI->m;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            valid[e] = j0 + e < c_n;
-            split_dual(valid[e] ? q[j0 + e] : 0.0, qv[e], ql[e]);
-        }
-        tau = (float)Sc.tau;
-        w = (float)Sc.wavg;
-        first = Sc.k == 0;
-        c_p = pv;
-        c_i1 = i1;
-        c_hint = CI->l2_keep_c != 0;
-        c_win = -1;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) { cs[e] = 0.0; csa[e] = 0.f; }
-        dx2 = 0.0;
-        dxa = 0.f;
-        rows_in_batch = 0;
-    };
-
-    bool failed = false;
-    while (consumed < issued) {
-        const int st = (int)(consumed % S);
-        if (!wait_stage(bars_s + 8 * st, (unsigned)((consumed / S) & 1))) { failed = true; break; }
-        const RowRef ref = refs[st];
-        if (ref.tile != c_tile) open_consumer(ref.tile);
-        const long long i = ref.row;
-        const long long di = i - c_i0;
-        const unsigned char* stage = wbase + st * STAGE_BYTES;
-        float c[4], x[4], xb[4];
-        if constexpr (GEN) {
-            // Every lane takes part in the shuffles (lanes past n included).
-            const long long cw = di >> 5;
-            if (cw != c_cwin) {
-                const long long r = c_i0 + cw * 32 + lane;
-#pragma unroll
-                for (int k = 0; k < DA; ++k)
-                    growc[k] = (k < gs.d && r < c_i1) ? __ldg(gs.xs + r * gs.d + k) : 0.f;
-                c_cwin = cw;
-            }
-            // gen_cost with the coordinate loop outermost (one shuffle per
-            // coordinate, four accumulators) and the distance kind resolved
-            // once per row: the same operations per entry.
-            const int src = (int)(di & 31);
-            float acc[4] = {0.f, 0.f, 0.f, 0.f};
-            if (gs.kind == GK_L1) {
-#pragma unroll
-                for (int k = 0; k < DA; ++k) {
-                    if (k < gs.d) {
-                        const float xk = __shfl_sync(0xffffffffu, growc[k], src);
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) acc[e] = acc[e] + fabsf(xk - gy[e][k]);
-                    }
-                }
-            } else if (gs.kind == GK_LINF) {
-#pragma unroll
-                for (int k = 0; k < DA; ++k) {
-                    if (k < gs.d) {
-                        const float xk = __shfl_sync(0xffffffffu, growc[k], src);
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) acc[e] = fmaxf(acc[e], fabsf(xk - gy[e][k]));
-                    }
-                }
-            } else {
-#pragma unroll
-                for (int k = 0; k < DA; ++k) {
-                    if (k < gs.d) {
-                        const float xk = __shfl_sync(0xffffffffu, growc[k], src);
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const float t = xk - gy[e][k];
-                            acc[e] = fmaf(t, t, acc[e]);
-                        }
-                    }
-                }
-                if (gs.kind == GK_L2) {
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) acc[e] = sqrtf(acc[e]);
-                }
-            }
-#pragma unroll
-            for (int e = 0; e < 4; ++e) c[e] = gen_div(acc[e], gs.div, gs.inv);
-        }
-        if (on) {
-            if constexpr (GEN) {
-            } else if (i != c_last_ragged) {
-                if (sizeof(TC) == 4) {
-                    const float4 t = *reinterpret_cast<const float4*>(stage + lane * 16);
-                    c[0] = t.x; c[1] = t.y; c[2] = t.z; c[3] = t.w;
-                } else {
-                    const uint2 t = *reinterpret_cast<const uint2*>(stage + lane * 8);
-                    c[0] = bf16_bits_to_f32(t.x & 0xffffu);
-                    c[1] = bf16_bits_to_f32(t.x >> 16);
-                    c[2] = bf16_bits_to_f32(t.y & 0xffffu);
-                    c[3] = bf16_bits_to_f32(t.y >> 16);
-                }
-            } else {
-                ldc4_tail<float>(c_C + i * c_ldc, c_n - j0, c);
-            }
-            const float4 tx = *reinterpret_cast<const float4*>(stage + STRIP * 4 + lane * 16);
-            x[0] = tx.x; x[1] = tx.y; x[2] = tx.z; x[3] = tx.w;
-            if (!first) {
-                const float4 tb = *reinterpret_cast<const float4*>(stage + 2 * STRIP * 4 + lane * 16);
-                xb[0] = tb.x; xb[1] = tb.y; xb[2] = tb.z; xb[3] = tb.w;
-            } else {
-                xb[0] = xb[1] = xb[2] = xb[3] = 0.f;
-            }
-        } else {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) { c[e] = GEN ? c[e] : 0.f; x[e] = 0.f; xb[e] = 0.f; }
-        }
-        // Row duals are staged in shared memory per window of PWIN rows
-        // instead of one dependent global load per row.
-        const long long win = di / PWIN;
-        if (win != c_win) {
-            const long long r0 = c_i0 + win * PWIN;
-            const long long r1 = min(r0 + (long long)PWIN, c_i1);
-            __syncwarp();
-            for (long long r = r0 + lane; r < r1; r += 32) {
-                float h, l;
-                split_dual(c_p[r], h, l);
-                pbuf[r - r0] = make_float2(h, l);
-            }
-            __syncwarp();
-            c_win = win;
-        }
-        const float2 pv = pbuf[di - win * PWIN];
-        // The stage has been read: release it to the producer.
-        __syncwarp();
-        ++consumed;
-        if (p_tile < T) issue();
-
-        float xn[4], xbn[4], rs = 0.f;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const float R = reduced_cost(c[e], pv.x, pv.y, qv[e], ql[e], CP);
-            float v = x[e] - tau * R;
-            v = v > 0.f ? v : 0.f;
-            v = valid[e] ? v : 0.f;
-            const float d = v - x[e];
-            dxa += d * d;
-            rs += d;                                              // row / column sums of X+ - X
-            csa[e] += d;
-            xn[e] = v;
-            xbn[e] = avg_dev_next(xb[e], d, w, first);
-        }
-        if (on) {
-            if (c_hint) {
-                st4_hint(c_xn + di * c_ldx, xn, pol_stream);
-                st4_hint(c_xbn + di * c_ldx, xbn, pol_stream);
-            } else {
-                st4(c_xn + di * c_ldx, xn);
-                st4(c_xbn + di * c_ldx, xbn);
-            }
-        }
-        rs = warp_sum(rs);
-        if (lane == 0) c_rowpart[i] = (double)rs;
-        if (++rows_in_batch == FLUSH_ROWS) {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) { cs[e] += (double)csa[e]; csa[e] = 0.f; }
-            dx2 += (double)dxa;
-            dxa = 0.f;
-            rows_in_batch = 0;
-        }
-    }
-    if (!failed) {
-        flush_tile();
-    } else if (lane == 0) {
-        // A stage never completed: report it and stop (bounded, never a trap).
-        const int t = refs[(int)(consumed % S)].tile;
-        atomicExch(&insts[tmap[t].inst].ctrl->status, ST_DEVICE);
-    }
-    // Drain: wait (bounded) for every copy still in flight.
-    while (consumed < issued) {
-        const int st = (int)(consumed % S);
-        wait_stage(bars_s + 8 * st, (unsigned)((consumed / S) & 1));
-        ++consumed;
-    }
-    P.issued = issued;
-    P.consumed = consumed;
-    return !failed;
-}
-
-template <typename TC, int S, bool CP>
-__global__ void __launch_bounds__(TWARPS * 32, 2)
-k_pass_bulk(const Inst* __restrict__ insts, const TileRef* __restrict__ tmap, const int* __restrict__ Tp,
-            unsigned* wctr, int wc, int dir_xor) {
-    // Setup that does not depend on the preceding kernel (tile count and maps
-    // are host-written; shared-memory barriers are local) runs before the wait.
-    const int T = *Tp;
-    extern __shared__ __align__(128) unsigned char dsm[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    bulk::RowPipe<S> P;
-    bulk::row_pipe_init<S>(P, dsm, lane, warp);
-    prefetch_first_tile(insts, tmap, T);
-    pdl_enter();
-    reset_other_counters(wctr, wc);
-    pass_row_run<TC, S, CP>(insts, tmap, T, &wctr[wc], P, lane, dir_xor);
-    pdl_release();
-}
-
-// ---------------------------------------------------------------------------
-// Plan pass, grouped bulk-copy pipeline (default for FP32 plans).  Like
-// k_pass_bulk, but a stage holds a group of up to R consecutive rows of one
-// tile: one mbarrier wait and one bookkeeping step per group, the group's
-// 3R row copies issued by 3R lanes at once, and the R row sums reduced by a
-// multi-row butterfly (6 shuffles for 4 rows instead of 20).
-// ---------------------------------------------------------------------------
-namespace bulk {
-
-struct GroupRef {
-    int tile;     // global tile index
-    int row0;     // first matrix row of the group
-    int count;    // rows in the group (1..R)
-    int pad;
-};
-
-template <int R, int S>
-__host__ __device__ constexpr int warp_smem_bytes_g() { return S * R * STAGE_BYTES + S * 8 + S * 16 + PWIN * 8; }
-
-// Sum v[r] over the 32 lanes for R = 4 rows with 6 shuffles.  The total of
-// row r ends in lanes 8r .. 8r+7.
-__device__ __forceinline__ float rows4_sum(const float (&v)[4], int lane) {
-    const bool hi16 = lane & 16;
-    const float s0 = __shfl_xor_sync(0xffffffffu, hi16 ? v[0] : v[2], 16);
-    const float s1 = __shfl_xor_sync(0xffffffffu, hi16 ? v[1] : v[3], 16);
-    const float a0 = (hi16 ? v[2] : v[0]) + s0;   // row 0 (low half) / row 2 (high half)
-    const float a1 = (hi16 ? v[3] : v[1]) + s1;   // row 1 / row 3
-    const bool hi8 = lane & 8;
-    const float t = __shfl_xor_sync(0xffffffffu, hi8 ? a0 : a1, 8);
-    float b = (hi8 ? a1 : a0) + t;
-    b += __shfl_xor_sync(0xffffffffu, b, 4);
-    b += __shfl_xor_sync(0xffffffffu, b, 2);
-    b += __shfl_xor_sync(0xffffffffu, b, 1);
-    return b;
-}
-
-}  // namespace bulk
-
-template <typename TC, int S, bool CP>
-__global__ void __launch_bounds__(TWARPS * 32, 2)
-k_pass_group(const Inst* __restrict__ insts, const TileRef* __restrict__ tmap, const int* __restrict__ Tp,
-             unsigned* wctr, int wc, int dir_xor) {
-    using namespace bulk;
-    constexpr int R = 4;
-    const int T = *Tp;   // host-written: read before the wait (see k_pass_bulk)
-    prefetch_first_tile(insts, tmap, T);
-    pdl_enter();
-    reset_other_counters(wctr, wc);
-    extern __shared__ __align__(128) unsigned char dsm[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    unsigned char* wbase = dsm + warp * warp_smem_bytes_g<R, S>();
-    unsigned long long* bars = reinterpret_cast<unsigned long long*>(wbase + S * R * STAGE_BYTES);
-    GroupRef* refs = reinterpret_cast<GroupRef*>(wbase + S * R * STAGE_BYTES + S * 8);
-    float2* pbuf = reinterpret_cast<float2*>(wbase + S * R * STAGE_BYTES + S * 24);
-    const unsigned wbase_s = smem_u32(wbase);
-    const unsigned bars_s = smem_u32(bars);
-    if (lane == 0) {
-        for (int s = 0; s < S; ++s) mbar_init(bars_s + 8 * s, 1);
-        fence_mbar_init();
-    }
-    __syncwarp();
-    constexpr int DM = GenDims<TC>::value;
-    constexpr bool GEN = DM > 0;                         // C generated, not copied
-    constexpr int DA = GEN ? DM : 1;                     // coordinate array size
-    constexpr long long CQ = sizeof(TC) == 2 ? 8 : 4;   // C elements per 16 bytes
-
-    // ---- producer: a tile's R-row groups, walked in either order (pass_reversed) ----
-    int p_tile = T;
-    long long p_r0 = 0, p_r1 = 0, p_G = 0, p_gi = 0, p_last_ragged = -1;
-    bool p_rev = false;
-    const char* p_c0 = nullptr;         // C, X, Xbar at the tile's first row
-    const char* p_x0 = nullptr;
-    const char* p_xb0 = nullptr;
-    long long p_cstride = 0, p_xstride = 0;
-    unsigned p_cbytes = 0, p_xbytes = 0;
-    bool p_first = true;
-    bool q_first = true;
-    auto next_tile = [&]() {
-        for (;;) {
-            p_tile = tile_next(&wctr[wc], q_first);
-            if (p_tile >= T) return;
-            const TileRef tr = tmap[p_tile];
-            const Inst& I = insts[tr.inst];
-            const Ctrl& Sc = *I.ctrl;
-            if (Sc.status != ST_RUNNING) continue;
-            const int strip = tr.local % I.nstrips, chunk = tr.local / I.nstrips;
-            const long long c0 = (long long)strip * STRIP;
-            const long long ncols = min((long long)STRIP, I.n - c0);
-            p_r0 = (long long)chunk * I.tile_rows;
-            p_r1 = min(p_r0 + (long long)I.tile_rows, I.m);
-            p_G = (p_r1 - p_r0 + R - 1) / R;
-            p_gi = 0;
-            p_rev = pass_reversed(Sc, dir_xor);
-            p_xstride = I.ldx * 4;
-            if constexpr (!GEN) {
-                p_cstride = I.ldc * (long long)sizeof(TC);
-                p_c0 = reinterpret_cast<const char*>(I.C) + p_r0 * p_cstride + c0 * (long long)sizeof(TC);
-            }
-            p_x0 = reinterpret_cast<const char*>(reinterpret_cast<const float*>(I.X) + (long long)Sc.cur * I.xslot +
-                                                 p_r0 * I.ldx + c0);
-            p_xb0 = reinterpret_cast<const char*>(reinterpret_cast<const float*>(I.X) + (long long)Sc.bar * I.xslot +
-                                                  p_r0 * I.ldx + c0);
-            p_xbytes = (unsigned)(((ncols + 3) / 4) * 16);
-            if constexpr (!GEN) {
-                p_cbytes = (unsigned)(((ncols + CQ - 1) / CQ) * CQ * (long long)sizeof(TC));
-                p_last_ragged = (ncols % CQ) != 0 ? I.m - 1 : -1;
-            }
-            p_first = Sc.k == 0;
-            return;
-        }
-    };
-    long long issued = 0, consumed = 0;   // in groups
-    auto issue = [&]() {
-        const int st = (int)(issued % S);
-        const long long p_row = p_r0 + R * (p_rev ? p_G - 1 - p_gi : p_gi);   // the group's first row
-        const int g = (int)min((long long)R, p_r1 - p_row);
-        const long long dr = p_row - p_r0;
-        const char* p_c = p_c0 + dr * p_cstride;
-        const char* p_x = p_x0 + dr * p_xstride;
-        const char* p_xb = p_xb0 + dr * p_xstride;
-        const unsigned bar = bars_s + 8 * st;
-        const unsigned dst = wbase_s + st * (R * STAGE_BYTES);
-        // The C copy of the last matrix row of a ragged strip is skipped (lanes load it).
-        const bool skip_c = p_last_ragged >= p_row && p_last_ragged < p_row + g;
-        const unsigned bytes = (unsigned)g * (p_cbytes + p_xbytes + (p_first ? 0u : p_xbytes)) - (skip_c ? p_cbytes : 0u);
-        if (lane == 0) {
-            refs[st].tile = p_tile;
-            refs[st].row0 = (int)p_row;
-            refs[st].count = g;
-            fence_proxy_async();
-            mbar_expect_tx(bar, bytes);
-        }
-        __syncwarp();
-        // Lane k copies array (k % 3) of row (k / 3): 3g copies issued at once.
-        if (lane < 3 * g) {
-            const int r = lane / 3, arr = lane % 3;
-            const unsigned d = dst + r * STAGE_BYTES + arr * (STRIP * 4);
-            fence_proxy_async();   // this lane's copy follows the warp's generic reads of the stage
-            if (arr == 0) {
-                if constexpr (!GEN) {
-                    if (!(skip_c && p_row + r == p_last_ragged)) g2s(d, p_c + r * p_cstride, p_cbytes, bar);
-                }
-            } else if (arr == 1) {
-                g2s(d, p_x + r * p_xstride, p_xbytes, bar);
-            } else if (!p_first) {
-                g2s(d, p_xb + r * p_xstride, p_xbytes, bar);
-            }
-        }
-        ++issued;
-        if (++p_gi == p_G) next_tile();
-    };
-    next_tile();
-    while (issued < S && p_tile < T) issue();
-
-    // ---- consumer ----
-    int c_tile = -1;
-    const Inst* CI = nullptr;
-    const TC* c_C = nullptr;
-    long long c_ldc = 0, c_ldx = 0, c_i0 = 0, c_n = 0, c_last_ragged = -1, c_chunk = 0;
-    float* c_xn = nullptr;
-    float* c_xbn = nullptr;
-    double* c_rowpart = nullptr;
-    long long j0 = 0;
-    bool on = false, valid[4] = {false, false, false, false};
-    float qv[4] = {0.f, 0.f, 0.f, 0.f}, ql[4] = {0.f, 0.f, 0.f, 0.f};
-    float tau = 0.f, w = 0.f;
-    bool first = true;
-    double cs[4] = {0.0, 0.0, 0.0, 0.0}, dx2 = 0.0;
-    float csa[4] = {0.f, 0.f, 0.f, 0.f}, dxa = 0.f;
-    int rows_in_batch = 0;
-    int c_local = 0;
-    const double* c_p = nullptr;
-    long long c_i1 = 0, c_win = -1;
-    // Generated cost: the lane's four columns' coordinates, and a 32-row
-    // window of row coordinates (lane r holds row window * 32 + r).
-    GenSpec gs = {nullptr, nullptr, 0, 0, 1.f, 1.f};
-    float gy[4][DA], growc[DA];
-    long long c_cwin = -1;
-    auto flush_tile = [&]() {
-        if (c_tile < 0) return;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) cs[e] += (double)csa[e];
-        dx2 += (double)dxa;
-        if (on) {
-            double* cp = CI->colpart + c_chunk * CI->ldx + j0;
-            reinterpret_cast<double2*>(cp)[0] = make_double2(cs[0], cs[1]);
-            reinterpret_cast<double2*>(cp)[1] = make_double2(cs[2], cs[3]);
-        }
-        const double d = warp_sum(dx2);
-        if (lane == 0) CI->tpart[(long long)c_local * TP + 0] = d;
-    };
-    auto open_consumer = [&](int t) {
-        flush_tile();
-        c_tile = t;
-        const TileRef tr = tmap[t];
-        CI = &insts[tr.inst];
-        const Ctrl& Sc = *CI->ctrl;
-        c_local = tr.local;
-        const int strip = tr.local % CI->nstrips;
-        c_chunk = tr.local / CI->nstrips;
-        const long long c0 = (long long)strip * STRIP;
-        c_n = CI->n;
-        c_ldc = CI->ldc;
-        c_ldx = CI->ldx;
-        c_i0 = c_chunk * CI->tile_rows;
-        c_i1 = min(c_i0 + (long long)CI->tile_rows, CI->m);
-        j0 = c0 + lane * 4;
-        on = j0 < c_n;
-        if constexpr (GEN) {
-            gs = CI->gen;
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-#pragma unroll
-                for (int k = 0; k < DA; ++k)
-                    gy[e][k] = (k < gs.d && j0 + e < c_n) ? __ldg(gs.ys + (j0 + e) * gs.d + k) : 0.f;
-            }
-            c_cwin = -1;
-        } else {
-            const long long ncols = min((long long)STRIP, c_n - c0);
-            c_last_ragged = (ncols % CQ) != 0 ? CI->m - 1 : -1;
-            c_C = reinterpret_cast<const TC*>(CI->C) + j0;
-        }
-        float* Xb = reinterpret_cast<float*>(CI->X);
-        c_xn = Xb + (long long)Sc.nxt * CI->xslot + c_i0 * c_ldx + j0;
-        c_xbn = Xb + (long long)Sc.barn * CI->xslot + c_i0 * c_ldx + j0;
-        c_rowpart = CI->rowpart + (long long)strip * CI->m;
-        c_p = slot_v(*CI, Sc.cur);
-        const double* q = c_p + CI->m;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            valid[e] = j0 + e < c_n;
-            split_dual(valid[e] ? q[j0 + e] : 0.0, qv[e], ql[e]);
-        }
-        tau = (float)Sc.tau;
-        w = (float)Sc.wavg;
-        first = Sc.k == 0;
-        c_win = -1;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) { cs[e] = 0.0; csa[e] = 0.f; }
-        dx2 = 0.0;
-        dxa = 0.f;
-        rows_in_batch = 0;
-    };
-
-    bool failed = false;
-    while (consumed < issued) {
-        const int st = (int)(consumed % S);
-        if (!wait_stage(bars_s + 8 * st, (unsigned)((consumed / S) & 1))) { failed = true; break; }
-        const GroupRef ref = refs[st];
-        if (ref.tile != c_tile) open_consumer(ref.tile);
-        const unsigned char* stage = wbase + st * (R * STAGE_BYTES);
-        float rsv[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            rsv[r] = 0.f;
-            if (r >= ref.count) continue;
-            const long long i = ref.row0 + r;
-            const long long di = i - c_i0;
-            const unsigned char* rst = stage + r * STAGE_BYTES;
-            // Row duals staged per window of PWIN rows.
-            const long long win = di / PWIN;
-            if (win != c_win) {
-                const long long r0 = c_i0 + win * PWIN;
-                const long long r1 = min(r0 + (long long)PWIN, c_i1);
-                __syncwarp();
-                for (long long rr = r0 + lane; rr < r1; rr += 32) {
-                    float h, l;
-                    split_dual(c_p[rr], h, l);
-                    pbuf[rr - r0] = make_float2(h, l);
-                }
-                __syncwarp();
-                c_win = win;
-            }
-            const float2 pv = pbuf[di - win * PWIN];
-            float c[4], x[4], xb[4];
-            if constexpr (GEN) {
-                // Same operations as gen_cost; every lane takes part in the shuffles.
-                const long long cw = di >> 5;
-                if (cw != c_cwin) {
-                    const long long rr = c_i0 + cw * 32 + lane;
-#pragma unroll
-                    for (int k = 0; k < DA; ++k)
-                        growc[k] = (k < gs.d && rr < c_i1) ? __ldg(gs.xs + rr * gs.d + k) : 0.f;
-                    c_cwin = cw;
-                }
-                const int src = (int)(di & 31);
-                float acc[4] = {0.f, 0.f, 0.f, 0.f};
-                if (gs.kind == GK_L1) {
-#pragma unroll
-                    for (int k = 0; k < DA; ++k) {
-                        if (k < gs.d) {
-                            const float xk = __shfl_sync(0xffffffffu, growc[k], src);
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) acc[e] = acc[e] + fabsf(xk - gy[e][k]);
-                        }
-                    }
-                } else if (gs.kind == GK_LINF) {
-#pragma unroll
-                    for (int k = 0; k < DA; ++k) {
-                        if (k < gs.d) {
-                            const float xk = __shfl_sync(0xffffffffu, growc[k], src);
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) acc[e] = fmaxf(acc[e], fabsf(xk - gy[e][k]));
-                        }
-                    }
-                } else {
-#pragma unroll
-                    for (int k = 0; k < DA; ++k) {
-                        if (k < gs.d) {
-                            const float xk = __shfl_sync(0xffffffffu, growc[k], src);
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                const float t = xk - gy[e][k];
-                                acc[e] = fmaf(t, t, acc[e]);
-                            }
-                        }
-                    }
-                    if (gs.kind == GK_L2) {
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) acc[e] = sqrtf(acc[e]);
-                    }
-                }
-#pragma unroll
-                for (int e = 0; e < 4; ++e) c[e] = gen_div(acc[e], gs.div, gs.inv);
-            }
-            if (on) {
-                if constexpr (GEN) {
-                } else if (i != c_last_ragged) {
-                    if (sizeof(TC) == 4) {
-                        const float4 t = *reinterpret_cast<const float4*>(rst + lane * 16);
-                        c[0] = t.x; c[1] = t.y; c[2] = t.z; c[3] = t.w;
-                    } else {
-                        const uint2 t = *reinterpret_cast<const uint2*>(rst + lane * 8);
-                        c[0] = bf16_bits_to_f32(t.x & 0xffffu);
-                        c[1] = bf16_bits_to_f32(t.x >> 16);
-                        c[2] = bf16_bits_to_f32(t.y & 0xffffu);
-                        c[3] = bf16_bits_to_f32(t.y >> 16);
-                    }
-                } else {
-                    ldc4_tail<float>(c_C + i * c_ldc, c_n - j0, c);
-                }
-                const float4 tx = *reinterpret_cast<const float4*>(rst + STRIP * 4 + lane * 16);
-                x[0] = tx.x; x[1] = tx.y; x[2] = tx.z; x[3] = tx.w;
-                if (!first) {
-                    const float4 tb = *reinterpret_cast<const float4*>(rst + 2 * STRIP * 4 + lane * 16);
-                    xb[0] = tb.x; xb[1] = tb.y; xb[2] = tb.z; xb[3] = tb.w;
-                } else {
-                    xb[0] = xb[1] = xb[2] = xb[3] = 0.f;
-                }
-            } else {
-#pragma unroll
-                for (int e = 0; e < 4; ++e) { c[e] = GEN ? c[e] : 0.f; x[e] = 0.f; xb[e] = 0.f; }
-            }
-            float xn[4], xbn[4], rs = 0.f;
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const float Rc = reduced_cost(c[e], pv.x, pv.y, qv[e], ql[e], CP);
-                float v = x[e] - tau * Rc;
-                v = v > 0.f ? v : 0.f;
-                v = valid[e] ? v : 0.f;
-                const float d = v - x[e];
-                dxa += d * d;
-                rs += d;                                          // row / column sums of X+ - X
-                csa[e] += d;
-                xn[e] = v;
-                xbn[e] = avg_dev_next(xb[e], d, w, first);
-            }
-            if (on) {
-                st4(c_xn + di * c_ldx, xn);
-                st4(c_xbn + di * c_ldx, xbn);
-            }
-            rsv[r] = rs;
-        }
-        // The group's stage has been read: release it and refill it.
-        __syncwarp();
-        ++consumed;
-        if (p_tile < T) issue();
-        const float tot = rows4_sum(rsv, lane);
-        if ((lane & 7) == 0 && (lane >> 3) < ref.count) c_rowpart[ref.row0 + (lane >> 3)] = (double)tot;
-        rows_in_batch += ref.count;
-        if (rows_in_batch >= FLUSH_ROWS) {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) { cs[e] += (double)csa[e]; csa[e] = 0.f; }
-            dx2 += (double)dxa;
-            dxa = 0.f;
-            rows_in_batch = 0;
-        }
-    }
-    pdl_release();
-    if (!failed) {
-        flush_tile();
-    } else if (lane == 0) {
-        const int t = refs[(int)(consumed % S)].tile;
-        atomicExch(&insts[tmap[t].inst].ctrl->status, ST_DEVICE);
-    }
-    while (consumed < issued) {
-        const int st = (int)(consumed % S);
-        wait_stage(bars_s + 8 * st, (unsigned)((consumed / S) & 1));
-        ++consumed;
-    }
-}
+namespace pdot {
 
 // ---------------------------------------------------------------------------
 // Slot bookkeeping
@@ -1310,6 +468,7 @@ __device__ __forceinline__ void assign_free(Ctrl* S, int cur, int bar, int anc) 
     S->nxt = picks[0];
     S->barn = picks[1];
 }
+
 
 // ---------------------------------------------------------------------------
 // Dual step + PDLP step-size controller
@@ -1340,6 +499,8 @@ struct StepPre {
     double eta, omega;
     long long passes, k, total, rejected;
     int cur, nxt, bar, barn, anc, adaptive_step;
+    int lag, npend, h0, xcur, xbar, xanc, xdst;
+    float tau, wavg;
 };
 __device__ __forceinline__ StepPre step_pre(const Ctrl* S) {
     StepPre P;
@@ -1355,7 +516,22 @@ __device__ __forceinline__ StepPre step_pre(const Ctrl* S) {
     P.barn = S->barn;
     P.anc = S->anc;
     P.adaptive_step = S->adaptive_step;
+    P.lag = S->lag;
+    P.npend = S->npend;
+    P.h0 = S->h0;
+    P.xcur = S->xcur;
+    P.xbar = S->xbar;
+    P.xanc = S->xanc;
+    P.xdst = S->xdst;
+    P.tau = (float)S->tau;
+    P.wavg = (float)S->wavg;
     return P;
+}
+
+// isfinite in integer arithmetic (an FP64 comparison takes the FP64 pipe 64
+// cycles on the controller's serial path).
+__device__ __forceinline__ bool finite_bits(double v) {
+    return (((unsigned)__double2hiint(v) >> 20) & 2047u) != 2047u;
 }
 
 // w_next: 1 / (k + 2), the averaging weight after an accepted step (computed
@@ -1384,16 +560,46 @@ __device__ void finalize_step(Ctrl* S, const StepPre& P, double dX2, double dy2,
         S->last_etabar = etabar;
         eta = eta_next;
     }
-    if (!isfinite(dX2) || !isfinite(dy2) || !isfinite(eta) || !(eta > 0.0)) {
+    if (!finite_bits(dX2) || !finite_bits(dy2) || !finite_bits(eta) || !(eta > 0.0)) {
         S->status = ST_NUMERIC;
-        S->res_slot = S->res_xslot = P.cur;
+        S->res_slot = P.cur;
         S->res_avg = 0;
+        // The current plan: with deferred writes, where this pass or the
+        // final pass has applied the pending steps.
+        S->res_xslot = !P.lag ? P.cur : P.npend ? P.xdst : P.xcur;
+        if (P.lag && P.npend == P.lag) {
+            S->xcur = P.xdst;
+            S->npend = 0;
+        }
         return;
     }
     S->fix = 0;   // the plan a restart picked has been formed before this pass
+    if (P.lag) {
+        // Deferred plan writes: this pass has applied the pending steps if
+        // there were `lag` of them; an accepted step becomes pending.
+        int np = P.npend;
+        const int c = (P.h0 + np) % YRING;   // ring index of this pass's duals
+        if (np == P.lag) {
+            np = 0;
+            S->h0 = c;
+            S->xcur = P.xdst;
+            S->xdst = plan_dst(P.xdst, P.xbar, P.xanc);
+        }
+        if (accept) {
+            if (np == 0) S->pfirst = P.k == 0;
+            S->ptau[c] = P.tau;
+            S->pw[c] = P.wavg;
+            ++np;
+        }
+        S->npend = np;
+    }
     if (accept) {
         S->cur = P.nxt;
         S->bar = P.barn;
+        if (!P.lag) {
+            S->xcur = P.nxt;
+            S->xbar = P.barn;
+        }
         assign_free(S, P.nxt, P.barn, P.anc);
         S->k = P.k + 1;
         S->wavg = w_next;
@@ -1401,9 +607,11 @@ __device__ void finalize_step(Ctrl* S, const StepPre& P, double dX2, double dy2,
     } else {
         S->rejected = P.rejected + 1;
     }
-    S->eta = eta;
-    S->tau = eta / P.omega;
-    S->sigma = eta * P.omega;
+    if (P.adaptive_step) {   // (a constant step keeps tau and sigma)
+        S->eta = eta;
+        S->tau = eta / P.omega;
+        S->sigma = eta * P.omega;
+    }
 }
 
 __device__ __forceinline__ void finalize_step(Ctrl* S, double dX2, double dy2, double inter, SchedFactors fac,
@@ -1432,6 +640,7 @@ __device__ void dual_tile(const Inst& I, Ctrl* S, int lvt, double* sgrp) {
     long long k = 0;
     double* Vn = nullptr;
     double* Vbn = nullptr;
+    float2* yfn = nullptr;
     SchedFactors fac = {0.0, 0.0};
     // The step decision's controller fields, used only by the instance's last
     // tile (lane 0 of warp 0 copies and later reads them: no barrier needed).
@@ -1449,6 +658,7 @@ __device__ void dual_tile(const Inst& I, Ctrl* S, int lvt, double* sgrp) {
         const double* Vb = slot_v(I, S->bar);
         Vn = slot_v(I, S->nxt);
         Vbn = slot_v(I, S->barn);
+        if (S->lag) yfn = I.yf + (long long)((S->h0 + S->npend + 1) % YRING) * I.yslot;
         if (row || col) {
             b = row ? I.f[idx] : I.g[idx];
             r = Vc[so];
@@ -1486,6 +696,11 @@ __device__ void dual_tile(const Inst& I, Ctrl* S, int lvt, double* sgrp) {
             const double w = wavg;
             const double yn = y + sigma * (b - (r + 2.0 * t));
             Vn[yo] = yn;
+            if (yfn) {   // the next pass reads the duals as FP32 pairs: split once here, not in every plan tile
+                float2 v;
+                split_dual(yn, v.x, v.y);
+                yfn[e] = v;
+            }
             Vn[so] = r + t;
             Vbn[yo] = k == 0 ? yn : ybar + w * (yn - ybar);
             const double dy = yn - y;
@@ -1568,9 +783,9 @@ __device__ __forceinline__ void kkt_tile(const Inst& I, const Ctrl& S, int lt, i
     const bool init = mode == MODE_INIT;
     const bool avg = !init && S.k > 0;      // the running average exists
     const bool sums = init || avg;          // exact row/col sums of X (init) or Xbar (check)
-    const TX* X = slot_x<TX>(I, S.cur);
-    const TX* Xb = slot_x<TX>(I, S.bar);
-    const TX* Xa = slot_x<TX>(I, S.anc);
+    const TX* X = slot_x<TX>(I, plan_slot(S));
+    const TX* Xb = slot_x<TX>(I, S.xbar);
+    const TX* Xa = slot_x<TX>(I, S.xanc);
     const double* p = slot_v(I, S.cur);
     const double* q = p + m;
     const double* pb = slot_v(I, S.bar);
@@ -1787,9 +1002,9 @@ k_kkt_bulk(const Inst* __restrict__ insts, const TileRef* __restrict__ tmap, con
             p_cstride = I.ldc * (long long)sizeof(TC);
             p_c0 = reinterpret_cast<const char*>(I.C) + p_r0 * p_cstride + c0 * (long long)sizeof(TC);
             const float* Xb = reinterpret_cast<const float*>(I.X);
-            p_x0 = reinterpret_cast<const char*>(Xb + (long long)Sc.cur * I.xslot + p_r0 * I.ldx + c0);
-            p_xb0 = reinterpret_cast<const char*>(Xb + (long long)Sc.bar * I.xslot + p_r0 * I.ldx + c0);
-            p_xa0 = reinterpret_cast<const char*>(Xb + (long long)Sc.anc * I.xslot + p_r0 * I.ldx + c0);
+            p_x0 = reinterpret_cast<const char*>(Xb + (long long)plan_slot(Sc) * I.xslot + p_r0 * I.ldx + c0);
+            p_xb0 = reinterpret_cast<const char*>(Xb + (long long)Sc.xbar * I.xslot + p_r0 * I.ldx + c0);
+            p_xa0 = reinterpret_cast<const char*>(Xb + (long long)Sc.xanc * I.xslot + p_r0 * I.ldx + c0);
             p_xbytes = (unsigned)(((ncols + 3) / 4) * 16);
             p_cbytes = (unsigned)(((ncols + CQ - 1) / CQ) * CQ * (long long)sizeof(TC));
             // The rounded-up C copy could run past the caller's allocation on
@@ -2052,7 +1267,21 @@ __device__ void report(Ctrl* S, const KP& k) {
 //    6 <C,X>, 7 rd2 cur, 8 <C,Xbar>, 9 rd2 avg, 10 ||X - Xa||^2, 11 ||Xbar - Xa||^2.
 // In MODE_INIT: 1 sum f, 3 sum g, 4 ||[f;g]||^2, 5 invalid marginal entries,
 //    8 ||C||_F^2.
+// Report the current iterate.
+__device__ __forceinline__ void set_result(Ctrl* S) {
+    S->res_slot = S->cur;
+    S->res_xslot = S->xcur;
+    S->res_avg = 0;
+}
+
 __device__ void finalize_check(Ctrl* S, const double* A, int mode) {
+    if (S->lag && S->npend) {
+        // The final pass before this check has applied the pending steps.
+        S->h0 = (S->h0 + S->npend) % YRING;
+        S->npend = 0;
+        S->xcur = S->xdst;
+        S->xdst = plan_dst(S->xcur, S->xbar, S->xanc);
+    }
     if (mode == MODE_INIT) {
         // Data norms for the relative measures, and the marginal checks of the ABI.
         S->norm_b = sqrt(A[4]);
@@ -2060,7 +1289,7 @@ __device__ void finalize_check(Ctrl* S, const double* A, int mode) {
         const double sf = A[1], sg = A[3];
         if (A[5] > 0.0 || !(fabs(sf - sg) <= 1e-9 * fmax(sf, 1.0))) {
             S->status = ST_ARG;
-            S->res_slot = S->res_xslot = S->cur;
+            set_result(S);
             return;
         }
     }
@@ -2072,16 +1301,15 @@ __device__ void finalize_check(Ctrl* S, const double* A, int mode) {
         // measures this check has just computed for it.
         report(S, c);
         S->status = ST_TIMEOUT;
-        S->res_slot = S->res_xslot = S->cur;
-        S->res_avg = 0;
+        set_result(S);
         return;
     }
     if (mode == MODE_INIT) {
         report(S, c);
         S->kkt0 = c.kkt;
         S->kkt_prev = c.kkt;
-        if (!isfinite(c.kkt)) { S->status = ST_NUMERIC; S->res_slot = S->res_xslot = S->cur; S->res_avg = 0; }
-        else if (c.rel <= S->tol) { S->status = ST_OK; S->res_slot = S->res_xslot = S->cur; S->res_avg = 0; }
+        if (!isfinite(c.kkt)) { S->status = ST_NUMERIC; set_result(S); }
+        else if (c.rel <= S->tol) { S->status = ST_OK; set_result(S); }
         return;
     }
     if (S->k == 0) {
@@ -2089,8 +1317,7 @@ __device__ void finalize_check(Ctrl* S, const double* A, int mode) {
         if (S->passes >= S->max_passes) {
             report(S, c);
             S->status = ST_MAX_ITER;
-            S->res_slot = S->res_xslot = S->cur;
-            S->res_avg = 0;
+            set_result(S);
         }
         return;
     }
@@ -2099,29 +1326,29 @@ __device__ void finalize_check(Ctrl* S, const double* A, int mode) {
     if (!isfinite(c.kkt) || !isfinite(b.kkt)) {
         report(S, c);
         S->status = ST_NUMERIC;
-        S->res_slot = S->res_xslot = S->cur;
-        S->res_avg = 0;
+        set_result(S);
         return;
     }
     // Restart candidate (Sec. 5): current iff its KKT is strictly smaller.
     const bool use_avg = S->adaptive_restart ? !(c.kkt < b.kkt) : true;
     const KP& kk = use_avg ? b : c;
-    const int cand = use_avg ? S->bar : S->cur;
+    const int cand = use_avg ? S->bar : S->cur;       // vector set
+    const int candx = use_avg ? S->xbar : S->xcur;    // plan slot
     report(S, kk);
     if (kk.rel <= S->tol || S->passes >= S->max_passes) {
         S->status = kk.rel <= S->tol ? ST_OK : ST_MAX_ITER;
         S->res_slot = cand;
-        S->res_xslot = cand;
+        S->res_xslot = candx;
         S->res_avg = use_avg ? 1 : 0;
         if (use_avg) {
-            // The reported plan X + D is formed into the free next slot, so
+            // The reported plan X + D is formed into a free slot, so
             // the current plan, D and the anchor stay as they are (a solve
             // stopped by its pass budget can be resumed from them).
             S->fix = 1;
-            S->fix_x = S->cur;
-            S->fix_d = S->bar;
-            S->fix_dst = S->nxt;
-            S->res_xslot = S->nxt;
+            S->fix_x = S->xcur;
+            S->fix_d = S->xbar;
+            S->fix_dst = S->lag ? free_slot(S->xcur, S->xbar, S->xanc) : S->nxt;
+            S->res_xslot = S->fix_dst;
         }
         return;
     }
@@ -2149,9 +1376,9 @@ __device__ void finalize_check(Ctrl* S, const double* A, int mode) {
         // next pass (the vector set of that slot already holds the averaged
         // duals and the exact sums of X + D).
         S->fix = 1;
-        S->fix_x = S->cur;
-        S->fix_d = cand;
-        S->fix_dst = cand;
+        S->fix_x = S->xcur;
+        S->fix_d = candx;
+        S->fix_dst = candx;
     }
     S->cur = cand;
     S->anc = cand;
@@ -2166,6 +1393,9 @@ __device__ void finalize_check(Ctrl* S, const double* A, int mode) {
         S->nxt = picks[1];
         S->barn = picks[2];
     }
+    S->xcur = S->xanc = candx;
+    S->xbar = S->lag ? free_slot(candx, candx, candx) : S->bar;
+    S->xdst = plan_dst(S->xcur, S->xbar, S->xanc);
     S->k = 0;
     S->wavg = 1.0;
     S->kkt0 = kk.kkt;
@@ -2247,6 +1477,11 @@ __device__ void checkvec_tile(const Inst& I, Ctrl* S, int lvt, int mode, double*
                 if (row) a[1] = b; else a[3] = b;
                 a[4] = b * b;
                 a[5] = (b >= 0.0 && isfinite(b)) ? 0.0 : 1.0;
+                if (S->lag) {   // the first pass's duals as FP32 pairs
+                    float2 v;
+                    split_dual(y, v.x, v.y);
+                    I.yf[(long long)S->h0 * I.yslot + e] = v;
+                }
             } else {
                 Vc[so] = s2;
                 a[0] = (s2 - b) * (s2 - b);
@@ -2317,111 +1552,15 @@ __global__ void __launch_bounds__(VT) k_checkvec(const Inst* __restrict__ insts,
 }
 
 // ---------------------------------------------------------------------------
-// Cooperative chunk kernel (single instance, FP32 plans): one launch runs K
-// passes and the check.  Each pass: the plan pass over all tiles, a grid
-// barrier, the dual update (the instance's last vector tile runs the step
-// controller), a grid barrier.  Then the KKT pass, a barrier, the check.
-// All CTAs are co-resident (cooperative launch).  The barrier is the fence +
-// atomic-arrive + fenced-spin pattern, so plain loads after it see every
-// other CTA's writes before it; its spin is bounded and sets an error flag.
-// ---------------------------------------------------------------------------
-constexpr long long BARRIER_SPIN_LIMIT = 1LL << 24;
-
-__device__ bool grid_barrier(GridBar* gb, unsigned nblocks, int* s_ok) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int ok = 1;
-        volatile unsigned* vgen = &gb->gen;
-        const unsigned gen = *vgen;
-        __threadfence();
-        const unsigned arrived = atomicAdd(&gb->count, 1u);
-        if (arrived == nblocks - 1) {
-            atomicExch(&gb->count, 0u);
-            __threadfence();
-            atomicAdd(&gb->gen, 1u);
-        } else {
-            long long it = 0;
-            while (*vgen == gen) {
-                if (++it > BARRIER_SPIN_LIMIT) {
-                    atomicExch(&gb->err, 1u);
-                    ok = 0;
-                    break;
-                }
-                __nanosleep(32);
-            }
-        }
-        __threadfence();
-        if (*(volatile unsigned*)&gb->err) ok = 0;
-        *s_ok = ok;
-    }
-    __syncthreads();
-    return *s_ok != 0;
-}
-
-template <typename TC, bool CP>
-__global__ void __launch_bounds__(TWARPS * 32, 2)
-k_chunk_coop(const Inst* __restrict__ insts, const TileRef* __restrict__ tmap, const int* __restrict__ Tp,
-             const TileRef* __restrict__ vmap, const int* __restrict__ NVp, unsigned* wctr, GridBar* gb, int npass,
-             int wc_a, int wc_b, int wc_kkt) {
-    __shared__ double sgrp[2 * VG * 32];
-    __shared__ int s_ok;
-    extern __shared__ __align__(128) unsigned char dsm[];
-    const int T = *Tp, NV = *NVp;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const unsigned G = gridDim.x;
-    bulk::RowPipe<BULK_ROW_S> P;
-    bulk::row_pipe_init<BULK_ROW_S>(P, dsm, lane, warp);
-    Ctrl* S0 = insts[0].ctrl;
-    bool ok = true;
-    for (int s = 0; s < npass && ok; ++s) {
-        // Every CTA reads the status after the same barrier: a uniform exit.
-        if (*(volatile int*)&S0->status != ST_RUNNING) break;
-        const int qc = (s & 1) ? wc_b : wc_a;
-        pass_row_run<TC, BULK_ROW_S, CP>(insts, tmap, T, &wctr[qc], P, lane, 0);
-        ok = grid_barrier(gb, G, &s_ok);
-        if (!ok) break;
-        if (blockIdx.x == 0 && threadIdx.x == 0) atomicExch(&wctr[qc], 0u);   // ready for pass s + 2
-        for (int vt = blockIdx.x; vt < NV; vt += G) {
-            const TileRef tr = vmap[vt];
-            const Inst& I = insts[tr.inst];
-            dual_tile(I, I.ctrl, tr.local, sgrp);
-        }
-        ok = grid_barrier(gb, G, &s_ok);
-    }
-    if (ok && *(volatile int*)&S0->status == ST_RUNNING) {
-        bool first = true;
-        for (;;) {
-            const int t = tile_next(&wctr[wc_kkt], first);
-            if (t >= T) break;
-            const TileRef tr = tmap[t];
-            const Inst& I = insts[tr.inst];
-            const Ctrl& S = *I.ctrl;
-            if (S.status != ST_RUNNING) continue;
-            kkt_tile<TC, float>(I, S, tr.local, lane, MODE_CHECK);
-        }
-        ok = grid_barrier(gb, G, &s_ok);
-        if (ok) {
-            for (int vt = blockIdx.x; vt < NV; vt += G) {
-                const TileRef tr = vmap[vt];
-                const Inst& I = insts[tr.inst];
-                Ctrl* S = I.ctrl;
-                if (S->status != ST_RUNNING) continue;
-                checkvec_tile(I, S, tr.local, MODE_CHECK, sgrp);
-            }
-        }
-    }
-    if (!ok && blockIdx.x == 0 && threadIdx.x == 0) atomicExch(&S0->status, ST_DEVICE);
-}
-
-// ---------------------------------------------------------------------------
 // Snapshot of every resident instance's controller (one D2H copy per chunk)
 // ---------------------------------------------------------------------------
 // ---------------------------------------------------------------------------
-// Average plan forming (after every check): where the check picked the
-// running average (a restart to it, or the reported point), write
-// X[fix_dst] = X[fix_x] + X[fix_d] -- the current plan plus the stored
-// deviation, with the rounding the checks used for the same value.  One warp
-// per plan tile; instances without a request cost one controller read.
+// After every check: where the check picked the running average (a restart to
+// it, or the reported point), write X[fix_dst] = X[fix_x] + X[fix_d] -- the
+// current plan plus the stored deviation, with the rounding the checks used
+// for the same value -- and, for deferred plan writes, split the current
+// duals for the next pass (a restart may have changed them).  One warp per
+// plan tile; the tiles of the first strip and chunk cover the duals.
 // ---------------------------------------------------------------------------
 template <typename TX>
 __global__ void __launch_bounds__(TWARPS * 32)
@@ -2433,13 +1572,32 @@ k_avgfix(const Inst* __restrict__ insts, const TileRef* __restrict__ tmap, const
     for (int t = (int)blockIdx.x * TWARPS + (int)(threadIdx.x >> 5); t < T; t += nw) {
         const TileRef tr = tmap[t];
         const Inst& I = insts[tr.inst];
-        const Ctrl& S = *I.ctrl;
-        if (!S.fix) continue;
+        Ctrl& S = *I.ctrl;
         const int strip = tr.local % I.nstrips, chunk = tr.local / I.nstrips;
         const long long j0 = (long long)strip * STRIP + lane * 4;
-        if (j0 >= I.n) continue;
         const long long i0 = (long long)chunk * I.tile_rows;
         const long long i1 = min(i0 + (long long)I.tile_rows, I.m);
+        if (S.lag) {
+            if (S.status == ST_NUMERIC && S.npend > 0) {
+                // A step with a non-finite value ended the solve: the final
+                // pass has applied the steps before it.
+                if (tr.local == 0 && lane == 0) {
+                    S.xcur = S.xdst;
+                    S.npend = 0;
+                }
+                continue;
+            }
+            if (S.status == ST_RUNNING) {
+                float2* yf = I.yf + (long long)S.h0 * I.yslot;
+                const double* y = slot_v(I, S.cur);
+                if (strip == 0)
+                    for (long long i = i0 + lane; i < i1; i += 32) split_dual(y[i], yf[i].x, yf[i].y);
+                if (chunk == 0)
+                    for (int e = 0; e < 4; ++e)
+                        if (j0 + e < I.n) split_dual(y[I.m + j0 + e], yf[I.m + j0 + e].x, yf[I.m + j0 + e].y);
+            }
+        }
+        if (!S.fix || j0 >= I.n) continue;
         const TX* Xa = slot_x<TX>(I, S.fix_x);
         const TX* Xd = slot_x<TX>(I, S.fix_d);
         TX* Xo = slot_x<TX>(I, S.fix_dst);
@@ -2504,6 +1662,8 @@ __global__ void k_watchdog_selftest(long long limit, int* status) {
 }  // namespace pdot
 
 #include "pdot_resident.cuh"
+#include "pdot_persist.cuh"
+
 
 namespace pdot {
 
@@ -2531,10 +1691,26 @@ static int launch_k(bool pdl, void (*kern)(KArgs...), unsigned grid, unsigned bl
     return err(cudaLaunchKernelEx(&c, kern, args...));
 }
 
-constexpr int BULK_S = BULK_ROW_S;
-constexpr int bulk_smem() { return TWARPS * bulk::warp_smem_bytes<BULK_S>(); }
-constexpr int GROUP_S = 2;   // stages of 4 rows: 8 rows in flight per warp
-constexpr int group_smem() { return TWARPS * bulk::warp_smem_bytes_g<4, GROUP_S>(); }
+// The pass kernel of FP32 plans with deferred writes; FINAL: apply and write
+// the pending steps only.  Generated costs take the variant with room for
+// their coordinates.
+template <bool CP, bool FINAL>
+static int launch_lag(int ttype, const Inst* d_insts, const TileRef* d_tmap, const int* T, unsigned* wctr, int wc,
+                      int dir_xor, const LaunchCfg& cfg, cudaStream_t st) {
+    const bool pdl = cfg.pdl != 0;
+    const unsigned nb = (unsigned)cfg.bulk_blocks, th = TWARPS * 32;
+    const int ro = cfg.pass_bulk == 1 ? 1 : 0;
+    constexpr int sm = lagp::smem_bytes();
+    if (ttype == TT_BF16)
+        return launch_k(pdl, k_pass_lag<unsigned short, CP, FINAL>, nb, th, sm, st, d_insts, d_tmap, T, wctr, wc, dir_xor, ro);
+    if (ttype == TT_F32)
+        return launch_k(pdl, k_pass_lag<float, CP, FINAL>, nb, th, sm, st, d_insts, d_tmap, T, wctr, wc, dir_xor, ro);
+    if (cfg.gen_dims <= 2)
+        return launch_k(pdl, k_pass_lag<GenC<2>, CP, FINAL>, nb, th, sm, st, d_insts, d_tmap, T, wctr, wc, dir_xor, ro);
+    if (cfg.gen_dims <= 4)
+        return launch_k(pdl, k_pass_lag<GenC4, CP, FINAL>, nb, th, sm, st, d_insts, d_tmap, T, wctr, wc, dir_xor, ro);
+    return launch_k(pdl, k_pass_lag<GenC8, CP, FINAL>, nb, th, sm, st, d_insts, d_tmap, T, wctr, wc, dir_xor, ro);
+}
 
 template <bool CP>
 static int launch_pass_t(int ttype, const Inst* d_insts, const TileRef* d_tmap, const int* T, unsigned* wctr,
@@ -2543,38 +1719,13 @@ static int launch_pass_t(int ttype, const Inst* d_insts, const TileRef* d_tmap, 
     const int wc = wc_override >= 0 ? wc_override : wc_index(WC_PASS, ttype);
     const bool pdl = cfg.pdl != 0;
     const unsigned tb = (unsigned)cfg.tile_blocks, th = TWARPS * 32;
-    if (ttype == TT_GEN) {
-        // Generated cost: the bulk pipelines copy X and Xbar only (the grouped
-        // one for up to 4 coordinates), or the register pipeline when the
-        // bulk kernels are switched off.
-        if (cfg.pass_bulk == 2 && cfg.gen_dims <= 4)
-            return launch_k(pdl, k_pass_group<GenC4, GROUP_S, CP>, (unsigned)cfg.group_blocks, th, group_smem(), st,
-                            d_insts, d_tmap, T, wctr, wc, dir_xor);
-        if (cfg.pass_bulk && cfg.gen_dims <= 4)
-            return launch_k(pdl, k_pass_bulk<GenC4, BULK_S, CP>, (unsigned)cfg.bulk_blocks, th, bulk_smem(), st, d_insts,
-                            d_tmap, T, wctr, wc, dir_xor);
-        if (cfg.pass_bulk)
-            return launch_k(pdl, k_pass_bulk<GenC8, BULK_S, CP>, (unsigned)cfg.bulk_blocks, th, bulk_smem(), st, d_insts,
-                            d_tmap, T, wctr, wc, dir_xor);
-        return launch_k(pdl, k_pass<GenC8, float, 2, CP>, tb, th, 0, st, d_insts, d_tmap, T, wctr, wc, dir_xor);
-    }
-    if (cfg.pass_bulk == 2 && ttype != TT_F64) {
-        if (ttype == TT_BF16)
-            return launch_k(pdl, k_pass_group<unsigned short, GROUP_S, CP>, (unsigned)cfg.group_blocks, th, group_smem(), st,
-                            d_insts, d_tmap, T, wctr, wc, dir_xor);
-        return launch_k(pdl, k_pass_group<float, GROUP_S, CP>, (unsigned)cfg.group_blocks, th, group_smem(), st, d_insts,
-                        d_tmap, T, wctr, wc, dir_xor);
-    }
-    if (cfg.pass_bulk && ttype != TT_F64) {
-        if (ttype == TT_BF16)
-            return launch_k(pdl, k_pass_bulk<unsigned short, BULK_S, CP>, (unsigned)cfg.bulk_blocks, th, bulk_smem(), st,
-                            d_insts, d_tmap, T, wctr, wc, dir_xor);
-        return launch_k(pdl, k_pass_bulk<float, BULK_S, CP>, (unsigned)cfg.bulk_blocks, th, bulk_smem(), st, d_insts,
-                        d_tmap, T, wctr, wc, dir_xor);
-    }
     if (ttype == TT_F64)
         return launch_k(pdl, k_pass<double, double, 2, CP>, (unsigned)cfg.tile_blocks_f64, th, 0, st, d_insts, d_tmap, T,
                         wctr, wc, dir_xor);
+    if (cfg.pass_bulk)
+        return launch_lag<CP, false>(ttype, d_insts, d_tmap, T, wctr, wc, dir_xor, cfg, st);
+    if (ttype == TT_GEN)
+        return launch_k(pdl, k_pass<GenC8, float, 2, CP>, tb, th, 0, st, d_insts, d_tmap, T, wctr, wc, dir_xor);
     if (ttype == TT_BF16) {
         if (cfg.pass_u == 4)
             return launch_k(pdl, k_pass<unsigned short, float, 4, CP>, tb, th, 0, st, d_insts, d_tmap, T, wctr, wc, dir_xor);
@@ -2587,6 +1738,13 @@ int launch_pass(int ttype, const Inst* d_insts, const TileRef* d_tmap, const int
                 const LaunchCfg& cfg, void* stream, int wc_override, int dir_xor) {
     if (cfg.comp) return launch_pass_t<true>(ttype, d_insts, d_tmap, T, wctr, cfg, stream, wc_override, dir_xor);
     return launch_pass_t<false>(ttype, d_insts, d_tmap, T, wctr, cfg, stream, wc_override, dir_xor);
+}
+int launch_plan_final(int ttype, const Inst* d_insts, const TileRef* d_tmap, const int* T, unsigned* wctr,
+                      const LaunchCfg& cfg, void* stream) {
+    const int wc = wc_index(WC_AUX, ttype);
+    const cudaStream_t st = (cudaStream_t)stream;
+    if (cfg.comp) return launch_lag<true, true>(ttype, d_insts, d_tmap, T, wctr, wc, 0, cfg, st);
+    return launch_lag<false, true>(ttype, d_insts, d_tmap, T, wctr, wc, 0, cfg, st);
 }
 
 int launch_dual(const Inst* d_insts, const TileRef* d_vmap, const int* NV, int nv_hint, unsigned* wctr,
@@ -2703,48 +1861,6 @@ static int setup_dyn(const void* const* fns, int nf, int bytes) {
     return -(r > 0 ? r : 1);
 }
 
-int setup_coop_chunk() {
-    const void* fns[] = {(const void*)k_chunk_coop<float, true>, (const void*)k_chunk_coop<float, false>,
-                         (const void*)k_chunk_coop<unsigned short, true>,
-                         (const void*)k_chunk_coop<unsigned short, false>};
-    return setup_dyn(fns, 4, bulk_smem());
-}
-
-int launch_chunk_coop(int ttype, const Inst* d_insts, const TileRef* d_tmap, const int* T, const TileRef* d_vmap,
-                      const int* NV, unsigned* wctr, GridBar* gb, int npass, const LaunchCfg& cfg, void* stream) {
-    cudaLaunchConfig_t c = {};
-    c.gridDim = dim3((unsigned)cfg.coop_blocks);
-    c.blockDim = dim3(TWARPS * 32);
-    c.dynamicSmemBytes = bulk_smem();
-    c.stream = (cudaStream_t)stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    c.attrs = attr;
-    c.numAttrs = 1;
-    const int wa = wc_index(WC_PASS, ttype), wb = wc_index(WC_AUX, ttype), wk = wc_index(WC_KKT, ttype);
-    cudaError_t e;
-    if (ttype == TT_BF16)
-        e = cfg.comp ? cudaLaunchKernelEx(&c, k_chunk_coop<unsigned short, true>, d_insts, d_tmap, T, d_vmap, NV, wctr,
-                                          gb, npass, wa, wb, wk)
-                     : cudaLaunchKernelEx(&c, k_chunk_coop<unsigned short, false>, d_insts, d_tmap, T, d_vmap, NV, wctr,
-                                          gb, npass, wa, wb, wk);
-    else
-        e = cfg.comp ? cudaLaunchKernelEx(&c, k_chunk_coop<float, true>, d_insts, d_tmap, T, d_vmap, NV, wctr, gb, npass,
-                                          wa, wb, wk)
-                     : cudaLaunchKernelEx(&c, k_chunk_coop<float, false>, d_insts, d_tmap, T, d_vmap, NV, wctr, gb,
-                                          npass, wa, wb, wk);
-    return err(e);
-}
-
-int setup_group_pass() {
-    const void* fns[] = {(const void*)k_pass_group<float, GROUP_S, true>, (const void*)k_pass_group<float, GROUP_S, false>,
-                         (const void*)k_pass_group<unsigned short, GROUP_S, true>,
-                         (const void*)k_pass_group<unsigned short, GROUP_S, false>,
-                         (const void*)k_pass_group<GenC4, GROUP_S, true>, (const void*)k_pass_group<GenC4, GROUP_S, false>};
-    return setup_dyn(fns, 6, group_smem());
-}
-
 // Resident kernel: its shared-memory size, and how many of its clusters the
 // device holds at once (-count; 0: cannot run, a positive value: an error).
 int setup_resident() {
@@ -2795,13 +1911,60 @@ int setup_kkt_bulk() {
     return setup_dyn(fns, 2, kkt_smem());
 }
 
+template <typename TC>
+static int setup_lag() {
+    const void* fns[] = {(const void*)k_pass_lag<TC, true, false>, (const void*)k_pass_lag<TC, false, false>,
+                         (const void*)k_pass_lag<TC, true, true>, (const void*)k_pass_lag<TC, false, true>};
+    return setup_dyn(fns, 4, lagp::smem_bytes());
+}
 int setup_bulk_pass() {
-    const void* fns[] = {(const void*)k_pass_bulk<float, BULK_S, true>, (const void*)k_pass_bulk<float, BULK_S, false>,
-                         (const void*)k_pass_bulk<unsigned short, BULK_S, true>,
-                         (const void*)k_pass_bulk<unsigned short, BULK_S, false>,
-                         (const void*)k_pass_bulk<GenC4, BULK_S, true>, (const void*)k_pass_bulk<GenC4, BULK_S, false>,
-                         (const void*)k_pass_bulk<GenC8, BULK_S, true>, (const void*)k_pass_bulk<GenC8, BULK_S, false>};
-    return setup_dyn(fns, 8, bulk_smem());   // negative: blocks per SM
+    const int r[] = {setup_lag<float>(), setup_lag<unsigned short>(), setup_lag<GenC<2>>(), setup_lag<GenC4>(),
+                     setup_lag<GenC8>()};
+    int worst = r[0];
+    for (int v : r) worst = v > worst ? v : worst;   // an error, or the fewest blocks per SM (negative)
+    return worst;
+}
+
+template <typename TC>
+static int setup_pers() {
+    const void* plain[] = {(const void*)k_persist<TC, false>};
+    const void* comp[] = {(const void*)k_persist<TC, true>};
+    const int a = setup_dyn(plain, 1, pers::Lay<false>::CTA), b = setup_dyn(comp, 1, pers::Lay<true>::CTA);
+    return a > b ? a : b;
+}
+int setup_persist() {
+    const int r[] = {setup_pers<float>(), setup_pers<unsigned short>(), setup_pers<GenC<2>>(), setup_pers<GenC4>()};
+    int worst = r[0];
+    for (int v : r) worst = v > worst ? v : worst;
+    return worst;
+}
+int persist_rows(bool comp) { return (comp ? pers::Lay<true>::NS : pers::Lay<false>::NS) * pers::R; }
+template <typename TC>
+static int launch_pers(const Inst* d_insts, int ntiles, GridSync* gs, int epoch, int npass, const LaunchCfg& cfg,
+                       cudaStream_t st) {
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3((unsigned)((ntiles + TWARPS - 1) / TWARPS));
+    c.blockDim = dim3(TWARPS * 32);
+    c.dynamicSmemBytes = cfg.comp ? pers::Lay<true>::CTA : pers::Lay<false>::CTA;
+    c.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    c.attrs = attr;
+    c.numAttrs = 1;
+    const int ro = cfg.pass_bulk == 1 ? 1 : 0;
+    return err(cfg.comp ? cudaLaunchKernelEx(&c, k_persist<TC, true>, d_insts, gs, epoch, npass, ro)
+                        : cudaLaunchKernelEx(&c, k_persist<TC, false>, d_insts, gs, epoch, npass, ro));
+}
+int launch_persist(int ttype, const Inst* d_insts, int ntiles, bool on_chip, GridSync* gs, int epoch, int npass,
+                   const LaunchCfg& cfg, void* stream) {
+    const cudaStream_t st = (cudaStream_t)stream;
+    if (ttype == TT_BF16) return launch_pers<unsigned short>(d_insts, ntiles, gs, epoch, npass, cfg, st);
+    // A generated cost whose tiles stay on the chip is computed once and then
+    // served as a stored one.
+    if (ttype == TT_F32 || on_chip) return launch_pers<float>(d_insts, ntiles, gs, epoch, npass, cfg, st);
+    if (cfg.gen_dims <= 2) return launch_pers<GenC<2>>(d_insts, ntiles, gs, epoch, npass, cfg, st);
+    return launch_pers<GenC4>(d_insts, ntiles, gs, epoch, npass, cfg, st);
 }
 
 int occupancy_vec_blocks_per_sm() {
