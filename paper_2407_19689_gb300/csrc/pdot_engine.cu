@@ -32,13 +32,11 @@
 using namespace pdot;
 
 namespace pdot {
-int launch_round_rowsum(const void* X, int xtype, long long m, long long n, long long ldx, const double* rs,
-                        const double* cs, double* rowout, double* colpart, int colparts, void* stream);
-int launch_round_write(const void* X, int xtype, long long m, long long n, long long ldx, const double* rs,
-                       const double* cs, const double* er, const double* ec, double inv_l1, void* Xout,
-                       long long ldo, const void* C, int ctype, long long ldc, const GenSpec* gen,
-                       double* objpart, int parts, void* stream);
-int launch_colreduce(const double* colpart, int parts, long long n, double* out, void* stream);
+long long round_scratch_words(long long m, long long n, int sm);
+double* round_obj_parts(double* base, long long m, long long n, int sm, long long* count);
+int launch_round(const void* X, int xtype, long long m, long long n, long long ldx, const double* f, const double* g,
+                 void* out, long long ldo, const void* C, int ctype, long long ldc, const GenSpec* gen, double* scratch,
+                 int sm, void* stream);
 int launch_dual_bound(const void* C, int ctype, long long ldc, const GenSpec* gen, const double* p,
                       const double* f, const double* g, long long m, long long n, double* colmin, int parts,
                       double* q, double* out, void* stream);
@@ -996,8 +994,7 @@ namespace {
 double round_plan_dev(pdot_handle* h, long long m, long long n, int xtype, const void* Xsrc, long long ldx,
                       const double* f, const double* g, void* X_out, const void* C, int ctype, long long ldc,
                       const GenSpec* gen) {
-    const int parts = 64;   // column-partial rows (fixed order)
-    const size_t need = sizeof(double) * (size_t)(4 * m + 4 * n + (size_t)parts * n + parts + 8);
+    const size_t need = sizeof(double) * (size_t)round_scratch_words(m, n, h->sm_count);
     if (h->round_scratch_bytes < need) {
         if (h->round_scratch) cudaFree(h->round_scratch);
         h->round_scratch = nullptr;
@@ -1005,64 +1002,27 @@ double round_plan_dev(pdot_handle* h, long long m, long long n, int xtype, const
         CK(cudaMalloc(&h->round_scratch, need));
         h->round_scratch_bytes = need;
     }
-    double* xs = h->round_scratch;      // row scales (m)
-    double* ys = xs + m;                // column scales (n)
-    double* rsum = ys + n;              // row sums (m)
-    double* csum = rsum + m;            // column sums (n)
-    double* er = csum + n;              // err_r (m)
-    double* ec = er + m;                // err_c (n)
-    double* colpart = ec + n;           // parts x n
-    double* objpart = colpart + (size_t)parts * n;
     void* out = X_out;
     void* tmp = nullptr;
     if (!out) {
         CK(cudaMalloc(&tmp, (size_t)m * n * xsize_of(xtype)));
         out = tmp;
     }
-    // 1) r = X1 -> x_i = min(f_i / r_i, 1)
-    CKL(launch_round_rowsum(Xsrc, xtype, m, n, ldx, nullptr, nullptr, rsum, colpart, parts, h->stream));
-    // 2) column sums of diag(x) X -> y_j = min(g_j / c_j, 1)
-    // 3) row and column sums of diag(x) X diag(y) -> err_r, err_c
-    // The host drives the scalar glue with tiny vector kernels inside the launcher file.
-    CKL(launch_colreduce(colpart, parts, n, csum, h->stream));
-    launch_count(h, 2);
-    // Scales are computed on the host from the sums (O(m+n), once per solve).
-    std::vector<double> hr((size_t)m), hc((size_t)n), hf((size_t)m), hg((size_t)n), hx((size_t)m), hy((size_t)n);
-    CK(cudaMemcpyAsync(hr.data(), rsum, sizeof(double) * m, cudaMemcpyDeviceToHost, h->stream));
-    CK(cudaMemcpyAsync(hf.data(), f, sizeof(double) * m, cudaMemcpyDeviceToHost, h->stream));
-    CK(cudaMemcpyAsync(hg.data(), g, sizeof(double) * n, cudaMemcpyDeviceToHost, h->stream));
-    CK(cudaStreamSynchronize(h->stream));
-    for (long long i = 0; i < m; ++i) hx[(size_t)i] = hr[(size_t)i] > 0.0 ? std::min(hf[(size_t)i] / hr[(size_t)i], 1.0) : 1.0;
-    CK(cudaMemcpyAsync(xs, hx.data(), sizeof(double) * m, cudaMemcpyHostToDevice, h->stream));
-    CKL(launch_round_rowsum(Xsrc, xtype, m, n, ldx, xs, nullptr, rsum, colpart, parts, h->stream));
-    CKL(launch_colreduce(colpart, parts, n, csum, h->stream));
-    launch_count(h, 2);
-    CK(cudaMemcpyAsync(hc.data(), csum, sizeof(double) * n, cudaMemcpyDeviceToHost, h->stream));
-    CK(cudaStreamSynchronize(h->stream));
-    for (long long j = 0; j < n; ++j) hy[(size_t)j] = hc[(size_t)j] > 0.0 ? std::min(hg[(size_t)j] / hc[(size_t)j], 1.0) : 1.0;
-    CK(cudaMemcpyAsync(ys, hy.data(), sizeof(double) * n, cudaMemcpyHostToDevice, h->stream));
-    CKL(launch_round_rowsum(Xsrc, xtype, m, n, ldx, xs, ys, rsum, colpart, parts, h->stream));
-    CKL(launch_colreduce(colpart, parts, n, csum, h->stream));
-    launch_count(h, 2);
-    CK(cudaMemcpyAsync(hr.data(), rsum, sizeof(double) * m, cudaMemcpyDeviceToHost, h->stream));
-    CK(cudaMemcpyAsync(hc.data(), csum, sizeof(double) * n, cudaMemcpyDeviceToHost, h->stream));
-    CK(cudaStreamSynchronize(h->stream));
-    double l1 = 0.0;
-    for (long long i = 0; i < m; ++i) { hr[(size_t)i] = hf[(size_t)i] - hr[(size_t)i]; l1 += std::fabs(hr[(size_t)i]); }
-    for (long long j = 0; j < n; ++j) hc[(size_t)j] = hg[(size_t)j] - hc[(size_t)j];
-    CK(cudaMemcpyAsync(er, hr.data(), sizeof(double) * m, cudaMemcpyHostToDevice, h->stream));
-    CK(cudaMemcpyAsync(ec, hc.data(), sizeof(double) * n, cudaMemcpyHostToDevice, h->stream));
-    const double inv_l1 = l1 > 0.0 ? 1.0 / l1 : 0.0;
-    // 4) X_feas = diag(x) X diag(y) + err_r err_c^T / ||err_r||_1, and <C, X_feas>
-    CKL(launch_round_write(Xsrc, xtype, m, n, ldx, xs, ys, er, ec, inv_l1, out, n, C, ctype, ldc, gen, objpart,
-                           parts, h->stream));
-    launch_count(h, 1);
-    std::vector<double> ho((size_t)parts);
-    CK(cudaMemcpyAsync(ho.data(), objpart, sizeof(double) * parts, cudaMemcpyDeviceToHost, h->stream));
-    CK(cudaStreamSynchronize(h->stream));
-    if (tmp) cudaFree(tmp);
+    CKL(launch_round(Xsrc, xtype, m, n, ldx, f, g, out, n, C, ctype, ldc, gen, h->round_scratch, h->sm_count, h->stream));
+    launch_count(h, 5);
     double obj = 0.0;
-    for (int k = 0; k < parts; ++k) obj += ho[(size_t)k];
+    if (C || ctype == PDOT_POINTS) {
+        long long count = 0;
+        const double* d = round_obj_parts(h->round_scratch, m, n, h->sm_count, &count);
+        std::vector<double> ho((size_t)count);
+        CK(cudaMemcpyAsync(ho.data(), d, sizeof(double) * ho.size(), cudaMemcpyDeviceToHost, h->stream));
+        CK(cudaStreamSynchronize(h->stream));
+        for (double v : ho) obj += v;
+    }
+    if (tmp) {
+        CK(cudaStreamSynchronize(h->stream));
+        cudaFree(tmp);
+    }
     return obj;
 }
 }  // namespace

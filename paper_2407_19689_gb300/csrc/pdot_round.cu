@@ -1,9 +1,33 @@
 // pdot_round.cu -- Algorithm 3 of arXiv 2407.19689 (rounding onto the
-// transportation polytope, after Altschuler et al.) on the device.
-// Runs once per solve, so the kernels are plain and order-deterministic:
-// row sums by one warp per row, column sums by fixed row groups, and a final
-// write of diag(x) X diag(y) + err_r err_c^T / ||err_r||_1 with <C, X_feas>.
+// transportation polytope, after Altschuler et al.) and the weak-duality
+// bound, on the device.
+//
+// Rounding: with x = min(f / X1, 1), y = min(g / (diag(x) X)^T 1, 1), the plan
+// diag(x) X diag(y) + err_r err_c^T / ||err_r||_1.  Four sweeps over X, each
+// sum in a fixed order:
+//   rows   r = X1 -> x
+//   cols   c = (diag(x) X)^T 1, by row groups, then one thread per column adds
+//          the groups -> y and err_c = g - y c (the column sums of
+//          diag(x) X diag(y) are y_j c_j: no sweep of their own)
+//   rows   X y -> err_r = f - x (X y); the last block adds ||err_r||_1
+//   write  the plan, and <C, plan> when a cost is given
+// All scalars stay on the device: the old form copied them to the host and
+// back three times and took the write through 64 blocks (1313 us at 4096 x
+// 4096, FP32; here 64 us; 2 x 67 MB take 20 us).
+//
+// FP64 is a narrow pipe on this part (two lanes per cycle and SM: one FP64
+// operation per entry of a 4096 x 4096 plan takes 27 us), so FP32 plans are
+// summed as unevaluated FP32 pairs: Knuth's TwoSum keeps each addition's
+// rounding error, an FMA each product's, and the pairs are added up in FP64
+// at the end of a lane's run.  Scales are kept as FP32 pairs too (48 bits).
+// The sums' error (about 1e-13) stays far below the FP32 rounding of the
+// written entries; measured against 64 bits the plan's error is unchanged
+// (2.5e-8).  Sums of 1e30 and more, or not finite, switch the sweeps to FP64
+// arithmetic, so no range is lost.  FP64 plans use FP64 throughout.
 #include <cuda_runtime.h>
+
+#include <cstdint>
+#include <type_traits>
 
 #include "pdot_internal.h"
 
@@ -11,48 +35,321 @@ namespace pdot {
 
 namespace {
 
-template <typename TX>
-__device__ __forceinline__ double scaled(const TX* X, long long ldx, long long i, long long j, const double* rs,
-                                         const double* cs) {
-    double v = (double)X[i * ldx + j];
-    if (rs) v *= rs[i];
-    if (cs) v *= cs[j];
-    return v;
-}
+constexpr int RB = 256;           // threads per block
+constexpr int RPARTS = 64;        // most row groups of the column sums
+constexpr int RU = 4;             // rows a thread of the write has in flight
+constexpr int RROWS = 64;         // rows whose scales a block of the write holds at a time
+constexpr double RWIDE = 1e30;    // row sums from here on: FP64 arithmetic
 
-// rowout[i] = sum_j rs_i X_ij cs_j   (one warp per row)
-template <typename TX>
-__global__ void k_round_rows(const TX* X, long long m, long long n, long long ldx, const double* rs,
-                             const double* cs, double* rowout) {
-    const long long row = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (row >= m) return;
+// A scale as the sweeps use it: an FP32 pair for FP32 plans (FP64 bits in the
+// same eight bytes where the plan's sums need FP64 arithmetic), FP64 otherwise.
+template <typename T>
+struct __align__(8) Scale {
+    float h, l;
+    __device__ __forceinline__ void set(double v) {
+        h = (float)v;
+        l = (float)(v - (double)h);
+    }
+    __device__ __forceinline__ void set(double v, bool wide) {
+        set(v);
+        if (wide) {
+            h = __int_as_float(__double2hiint(v));
+            l = __int_as_float(__double2loint(v));
+        }
+    }
+    __device__ __forceinline__ double wide() const { return __hiloint2double(__float_as_int(h), __float_as_int(l)); }
+};
+template <>
+struct Scale<double> {
+    double v;
+    __device__ __forceinline__ void set(double w, bool = false) { v = w; }
+    __device__ __forceinline__ double wide() const { return v; }
+};
+
+// Running sum: FP32 pair (value plus the additions' errors) or FP64.
+template <typename T>
+struct __align__(8) Acc {
+    float s = 0.f, e = 0.f;
+    __device__ __forceinline__ void two_sum(float x) {
+        const float t = s + x, b = t - s;
+        e += (s - (t - b)) + (x - b);
+        s = t;
+    }
+    __device__ __forceinline__ void add(float x) { two_sum(x); }
+    __device__ __forceinline__ void add(float x, const Scale<float>& w) {
+        const float p = x * w.h;
+        e += fmaf(x, w.l, fmaf(x, w.h, -p));
+        two_sum(p);
+    }
+    __device__ __forceinline__ void merge(const Acc& o) {
+        two_sum(o.s);
+        e += o.e;
+    }
+    __device__ __forceinline__ Acc shfl_xor(int m) const {
+        Acc r;
+        r.s = __shfl_xor_sync(0xffffffffu, s, m);
+        r.e = __shfl_xor_sync(0xffffffffu, e, m);
+        return r;
+    }
+    __device__ __forceinline__ double get() const { return (double)s + (double)e; }
+    // The errors folded into the value, before they grow in number.
+    __device__ __forceinline__ void fold() {
+        const float t = s + e;
+        e = (s - t) + e;
+        s = t;
+    }
+};
+template <>
+struct __align__(8) Acc<double> {
     double s = 0.0;
-    for (long long j = lane; j < n; j += 32) s += scaled(X, ldx, row, j, rs, cs);
+    __device__ __forceinline__ void merge(const Acc& o) { s += o.s; }
+    __device__ __forceinline__ Acc shfl_xor(int m) const {
+        Acc r;
+        r.s = __shfl_xor_sync(0xffffffffu, s, m);
+        return r;
+    }
+    __device__ __forceinline__ void fold() {}
+    __device__ __forceinline__ void add(double x) { s += x; }
+    __device__ __forceinline__ void add(double x, const Scale<double>& w) { s = fma(x, w.v, s); }
+    __device__ __forceinline__ double get() const { return s; }
+};
+
+template <typename T>
+__device__ __forceinline__ void warp_merge(Acc<T>& a) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) a.merge(a.shfl_xor(o));
+}
+__device__ __forceinline__ double warp_add(double s) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) rowout[row] = s;
+    return s;
 }
 
-// colpart[g][j] = sum over rows i of group g of rs_i X_ij cs_j
-template <typename TX>
-__global__ void k_round_cols(const TX* X, long long m, long long n, long long ldx, const double* rs,
-                             const double* cs, double* colpart, int parts) {
-    const long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+// Four consecutive entries (VEC: 16-byte aligned rows), `cnt` of which exist.
+template <typename T, bool VEC>
+__device__ __forceinline__ void load4(const T* p, long long cnt, T (&v)[4]) {
+    if (VEC && cnt >= 4) {
+        if constexpr (sizeof(T) == 4) {
+            const float4 t = *reinterpret_cast<const float4*>(p);
+            v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+        } else {
+            const double2 a = reinterpret_cast<const double2*>(p)[0], b = reinterpret_cast<const double2*>(p)[1];
+            v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+        }
+    } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) v[e] = e < cnt ? p[e] : T(0);
+    }
+}
+
+// Sweep by rows: a block has RB / 32 warps, WPR of which share RPW rows
+// (every entry's scale is then read once for RPW rows).  WEIGHTED: sum_j X_ij
+// y_j -> out = err_r, and the last block the inverse of ||err_r||_1; else sum_j
+// X_ij -> out.  A lane's four entries are consecutive (16-byte loads), or 32
+// columns apart where rows are not aligned and where scales are read (their
+// loads then are consecutive over the lanes).
+template <typename T, bool VEC, int WPR, int RPW, bool WEIGHTED>
+__global__ void __launch_bounds__(RB) k_round_rows(const T* __restrict__ X, long long m, long long n, long long ldx,
+                                                   const double* __restrict__ f, const Scale<T>* __restrict__ ys,
+                                                   const double* __restrict__ xs, double* out, double* inv_l1,
+                                                   unsigned* state) {
+    constexpr int RPB = (RB / 32) / WPR * RPW;
+    constexpr bool V4 = VEC && !WEIGHTED;
+    __shared__ Acc<T> part[RB / 32][RPW];
+    __shared__ double red[RB / 32];
+    __shared__ unsigned last;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const long long i0 = (long long)blockIdx.x * RPB + warp / WPR * RPW;
+    const bool wide = sizeof(T) == 4 && WEIGHTED && state[1] != 0u;
+    const int w0 = (warp % WPR) * 128, step = 128 * WPR;
+    Acc<T> a[RPW][2];
+    const T* row[RPW];
+#pragma unroll
+    for (int u = 0; u < RPW; ++u) row[u] = X + (i0 + u < m ? i0 + u : 0) * ldx + (V4 ? lane * 4 : lane);
+    auto chunk = [&](long long j0, auto tail_c) {
+        constexpr bool TAIL = decltype(tail_c)::value;
+        Scale<T> y[4];
+        if (WEIGHTED) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const long long j = j0 + e * 32 + lane;
+                y[e] = ys[!TAIL || j < n ? j : n - 1];
+            }
+        }
+        T v[RPW][4];
+#pragma unroll
+        for (int u = 0; u < RPW; ++u) {
+            if (V4) {
+                load4<T, true>(row[u] + j0, TAIL ? n - j0 - lane * 4 : 4, v[u]);
+            } else {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) v[u][e] = !TAIL || j0 + e * 32 + lane < n ? row[u][j0 + e * 32] : T(0);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < RPW; ++u) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                if (WEIGHTED) a[u][e & 1].add(v[u][e], y[e]);
+                else a[u][e & 1].add(v[u][e]);
+            }
+        }
+    };
+    if (!wide) {
+        constexpr int UN = RPW == 1 ? 8 : 2;   // chunks in flight
+        long long j0 = w0;
+        int run = 0;
+        for (; j0 + (UN - 1) * step + 128 <= n; j0 += UN * step) {
+#pragma unroll
+            for (int k = 0; k < UN; ++k) chunk(j0 + k * step, std::false_type());
+            if (++run == 8) {   // long rows
+                run = 0;
+#pragma unroll
+                for (int u = 0; u < RPW; ++u) { a[u][0].fold(); a[u][1].fold(); }
+            }
+        }
+        for (; j0 < n; j0 += step) chunk(j0, std::true_type());
+    }
+#pragma unroll
+    for (int u = 0; u < RPW; ++u) {
+        a[u][0].merge(a[u][1]);
+        warp_merge(a[u][0]);
+        if (WPR > 1 && lane == 0) part[warp][u] = a[u][0];
+    }
+    if (WPR > 1) {
+        __syncthreads();
+        if (warp % WPR == 0) {
+#pragma unroll
+            for (int u = 0; u < RPW; ++u)
+                for (int w = 1; w < WPR; ++w) a[u][0].merge(part[warp + w][u]);
+        }
+    }
+    if (warp % WPR == 0) {
+#pragma unroll
+        for (int u = 0; u < RPW; ++u) {
+            const long long i = i0 + u;
+            if (i >= m) break;
+            // Sums that leave FP32's range: again, in FP64 by one warp.
+            const bool big = sizeof(T) == 4 && (wide || (!WEIGHTED && !(fabsf((float)a[u][0].s) < (float)RWIDE)));
+            double sum = 0.0;
+            if (big) {
+                for (long long j = lane; j < n; j += 32)
+                    sum += WEIGHTED ? (double)X[i * ldx + j] * ys[j].wide() : (double)X[i * ldx + j];
+                sum = warp_add(sum);
+            }
+            if (lane == 0) {
+                if (!big) sum = a[u][0].get();
+                if (!WEIGHTED) {
+                    out[i] = sum;
+                    if (big) atomicOr(state + 1, 1u);
+                } else {
+                    out[i] = f[i] - xs[i] * sum;
+                }
+            }
+        }
+    }
+    if (!WEIGHTED) return;
+    // The last block adds |err_r| (each thread a strided run, then in order).
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(state, 1u) == gridDim.x - 1 ? 1u : 0u;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    double l1 = 0.0;
+    for (long long r = threadIdx.x; r < m; r += RB) l1 += fabs(__ldcg(out + r));
+    l1 = warp_add(l1);
+    if (lane == 0) red[warp] = l1;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        l1 = 0.0;
+        for (int w = 0; w < RB / 32; ++w) l1 += red[w];
+        *inv_l1 = l1 > 0.0 ? 1.0 / l1 : 0.0;
+    }
+}
+
+// The sweeps' FP64 forms for FP32 plans whose sums leave FP32's range, out of
+// line: they would only take registers from the others.
+template <typename T>
+__device__ __noinline__ void cols_wide(const T* X, long long r0, long long r1, long long ldx, const double* f,
+                                       const double* r_sum, long long n, long long j, long long es, double* part) {
+    for (int e = 0; e < 4; ++e) {
+        if (j + e * es >= n) break;
+        double c = 0.0;
+        for (long long i = r0; i < r1; ++i)
+            c += (double)X[i * ldx + j + e * es] * (r_sum[i] > 0.0 ? fmin(f[i] / r_sum[i], 1.0) : 1.0);
+        part[j + e * es] = c;
+    }
+}
+
+// x_i = min(f_i / r_i, 1) (a zero sum keeps scale 1; the blocks of the first
+// columns write it), and colpart[g][j] = sum over the rows i of group g of
+// x_i X_ij: four columns per thread.
+template <typename T, bool VEC>
+__global__ void __launch_bounds__(RB) k_round_cols(const T* __restrict__ X, long long m, long long n, long long ldx,
+                                                   const double* __restrict__ f, const double* __restrict__ r_sum, double* xs,
+                                                   Acc<T>* __restrict__ colpart, int parts, const unsigned* __restrict__ state) {
+    const long long j = VEC ? ((long long)blockIdx.x * RB + threadIdx.x) * 4 : (long long)blockIdx.x * RB * 4 + threadIdx.x;
+    constexpr long long ES = VEC ? 1 : RB;   // distance of a thread's columns
     const int grp = blockIdx.y;
-    if (j >= n) return;
     const long long r0 = m * grp / parts, r1 = m * (grp + 1) / parts;
-    double s = 0.0;
-    for (long long i = r0; i < r1; ++i) s += scaled(X, ldx, i, j, rs, cs);
-    colpart[(long long)grp * n + j] = s;
+    const bool wide = sizeof(T) == 4 && state[1] != 0u;
+    __shared__ Scale<T> sx[64];
+    if (wide && j < n) cols_wide(X, r0, r1, ldx, f, r_sum, n, j, ES, reinterpret_cast<double*>(colpart) + (long long)grp * n);
+    Acc<T> a[4];
+    for (long long b = r0; b < r1; b += 64) {
+        const int cnt = (int)(b + 64 < r1 ? 64 : r1 - b);
+        __syncthreads();
+        if ((int)threadIdx.x < cnt) {
+            const double s = r_sum[b + threadIdx.x];
+            const double x = s > 0.0 ? fmin(f[b + threadIdx.x] / s, 1.0) : 1.0;
+            sx[threadIdx.x].set(x);
+            if (blockIdx.x == 0) xs[b + threadIdx.x] = x;
+        }
+        __syncthreads();
+        if (j >= n || wide) continue;
+#pragma unroll 8
+        for (int r = 0; r < cnt; ++r) {
+            const T* row = X + (b + r) * ldx + j;
+            T v[4];
+            if (VEC) {
+                load4<T, true>(row, n - j, v);
+            } else {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) v[e] = j + e * ES < n ? row[e * ES] : T(0);
+            }
+            const Scale<T> w = sx[r];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) a[e].add(v[e], w);
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) a[e].fold();
+    }
+    if (j >= n || wide) return;
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+        if (j + e * ES < n) colpart[(long long)grp * n + j + e * ES] = a[e];
 }
 
-__global__ void k_colreduce(const double* colpart, int parts, long long n, double* out) {
+// c_j = the groups' sums -> y_j, err_c.
+template <typename T>
+__global__ void k_round_colscale(const Acc<T>* __restrict__ colpart, int parts, long long n, const double* __restrict__ g,
+                                 Scale<T>* ys, Scale<T>* ec, const unsigned* __restrict__ state) {
+    const bool wide = sizeof(T) == 4 && state[1] != 0u;
     const long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= n) return;
-    double s = 0.0;
-    for (int g = 0; g < parts; ++g) s += colpart[(long long)g * n + j];
-    out[j] = s;
+    double c = 0.0;
+    if (wide) {
+        for (int k = 0; k < parts; ++k) c += *reinterpret_cast<const double*>(colpart + (long long)k * n + j);
+    } else {
+        Acc<T> a;
+#pragma unroll 16
+        for (int k = 0; k < parts; ++k) a.merge(colpart[(long long)k * n + j]);
+        c = a.get();
+    }
+    const double y = c > 0.0 ? fmin(g[j] / c, 1.0) : 1.0;
+    ys[j].set(y, wide);
+    ec[j].set(g[j] - y * c, wide);
 }
 
 // Cost entry (i, j) for the objective of the rounded plan: a stored matrix
@@ -63,45 +360,160 @@ struct StoredCost {
     long long ldc;
     __device__ __forceinline__ bool on() const { return C != nullptr; }
     __device__ __forceinline__ double operator()(long long i, long long j) const { return (double)C[i * ldc + j]; }
+    __device__ __forceinline__ float f32(long long i, long long j) const { return (float)C[i * ldc + j]; }
 };
 struct PointsCost {
     GenSpec g;
     __device__ __forceinline__ bool on() const { return true; }
-    __device__ __forceinline__ double operator()(long long i, long long j) const {
-        return (double)gen_cost(g.kind, g.d, g.xs + i * g.d, g.ys + j * g.d, g.div, g.inv);
+    __device__ __forceinline__ float f32(long long i, long long j) const {
+        return gen_cost(g.kind, g.d, g.xs + i * g.d, g.ys + j * g.d, g.div, g.inv);
     }
+    __device__ __forceinline__ double operator()(long long i, long long j) const { return (double)f32(i, j); }
 };
 
-template <typename TX, typename CA>
-__global__ void k_round_write(const TX* X, long long m, long long n, long long ldx, const double* rs,
-                              const double* cs, const double* er, const double* ec, double inv_l1, TX* out,
-                              long long ldo, CA C, double* objpart, int parts) {
-    __shared__ double red[32];
-    const int grp = blockIdx.x;
-    const long long r0 = m * grp / parts, r1 = m * (grp + 1) / parts;
+// The entry x y v + a e of the rounded plan (a = err_r / ||err_r||_1), rounded
+// once to the plan's type.
+__device__ __forceinline__ float rounded(float v, const Scale<float>& x, const Scale<float>& y, const Scale<float>& a,
+                                         const Scale<float>& e) {
+    const float t = v * x.h;
+    const float tl = fmaf(v, x.l, fmaf(v, x.h, -t));
+    const float p = t * y.h;
+    const float pl = fmaf(tl, y.h, fmaf(t, y.l, fmaf(t, y.h, -p)));
+    const float c = a.h * e.h;
+    const float cl = fmaf(a.l, e.h, fmaf(a.h, e.l, fmaf(a.h, e.h, -c)));
+    const float s = p + c, b = s - p;
+    return s + (((p - (s - b)) + (c - b)) + (pl + cl));
+}
+__device__ __forceinline__ double rounded(double v, const Scale<double>& x, const Scale<double>& y, const Scale<double>& a,
+                                          const Scale<double>& e) {
+    return fma(v * x.v, y.v, a.v * e.v);
+}
+
+template <typename T, typename CA>
+__device__ __noinline__ double write_wide(const T* X, long long r0, long long r1, long long ldx, const double* xs,
+                                          const Scale<T>* ys, const double* er, const Scale<T>* ec, double inv, T* out,
+                                          long long ldo, const CA& C, long long n, long long j, long long es) {
     double obj = 0.0;
     for (long long i = r0; i < r1; ++i) {
-        for (long long j = threadIdx.x; j < n; j += blockDim.x) {
-            const double v = scaled(X, ldx, i, j, rs, cs) + er[i] * ec[j] * inv_l1;
-            const TX vo = (TX)v;
-            out[i * ldo + j] = vo;
-            if (C.on()) obj += C(i, j) * (double)vo;
+        for (int e = 0; e < 4; ++e) {
+            const long long c = j + e * es;
+            if (c >= n) break;
+            const T w = (T)((double)X[i * ldx + c] * xs[i] * ys[c].wide() + er[i] * ec[c].wide() * inv);
+            out[i * ldo + c] = w;
+            if (C.on()) obj += C(i, c) * (double)w;
         }
     }
+    return obj;
+}
+
+template <typename T, bool VEC, typename CA>
+__global__ void __launch_bounds__(RB) k_round_write(const T* X, long long m, long long n, long long ldx,
+                                                    const double* __restrict__ xs, const Scale<T>* __restrict__ ys,
+                                                    const double* __restrict__ er, const Scale<T>* __restrict__ ec,
+                                                    const double* __restrict__ inv_l1, T* out, long long ldo, CA C,
+                                                    double* objpart, const unsigned* __restrict__ state) {
+    __shared__ double red[RB / 32];
+    __shared__ Scale<T> sx[RROWS], sa[RROWS];
+    const long long j = VEC ? ((long long)blockIdx.x * RB + threadIdx.x) * 4 : (long long)blockIdx.x * RB * 4 + threadIdx.x;
+    constexpr long long ES = VEC ? 1 : RB;
+    const int grp = blockIdx.y, parts = gridDim.y;
+    const long long r0 = m * grp / parts, r1 = m * (grp + 1) / parts;
+    const double inv = *inv_l1;
+    const bool wide = sizeof(T) == 4 && state[1] != 0u;
+    double obj = 0.0;
+    if (wide) {
+        if (j < n) obj = write_wide(X, r0, r1, ldx, xs, ys, er, ec, inv, out, ldo, C, n, j, ES);
+    } else {
+        auto load = [&](long long i, T (&v)[4]) {
+            const T* row = X + i * ldx + j;
+            if (VEC) {
+                load4<T, true>(row, n - j, v);
+            } else {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) obj += __shfl_xor_sync(0xffffffffu, obj, o);
+                for (int e = 0; e < 4; ++e) v[e] = j + e * ES < n ? row[e * ES] : T(0);
+            }
+        };
+        Scale<T> y[4], e4[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const bool in = j + e * ES < n;
+            y[e] = ys[in ? j + e * ES : 0];
+            e4[e] = ec[in ? j + e * ES : 0];
+        }
+        for (long long b = r0; b < r1; b += RROWS) {
+            const int cnt = (int)(b + RROWS < r1 ? RROWS : r1 - b);
+            // RU rows are read before the ones before them are written (out may
+            // be X itself: an entry is read and written by one thread).
+            T v[RU][4];
+            if (j < n) {
+#pragma unroll
+                for (int u = 0; u < RU; ++u)
+                    if (u < cnt) load(b + u, v[u]);
+            }
+            __syncthreads();
+            if ((int)threadIdx.x < cnt) {   // the rows' scales
+                sx[threadIdx.x].set(xs[b + threadIdx.x]);
+                sa[threadIdx.x].set(er[b + threadIdx.x] * inv);
+            }
+            __syncthreads();
+            if (j >= n) continue;
+            Acc<T> acc;
+            for (int rb = 0; rb < cnt; rb += RU) {
+#pragma unroll
+                for (int u = 0; u < RU; ++u) {
+                    const int r = rb + u;
+                    if (r >= cnt) break;
+                    const Scale<T> x = sx[r], a = sa[r];
+                    T w[4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) w[e] = rounded(v[u][e], x, y[e], a, e4[e]);
+                    if (r + RU < cnt) load(b + r + RU, v[u]);
+                    T* o = out + (b + r) * ldo + j;
+                    if (VEC && j + 4 <= n) {
+                        if constexpr (sizeof(T) == 4) {
+                            *reinterpret_cast<float4*>(o) = make_float4(w[0], w[1], w[2], w[3]);
+                        } else {
+                            reinterpret_cast<double2*>(o)[0] = make_double2(w[0], w[1]);
+                            reinterpret_cast<double2*>(o)[1] = make_double2(w[2], w[3]);
+                        }
+                    } else {
+#pragma unroll
+                        for (int e = 0; e < 4; ++e)
+                            if (j + e * ES < n) o[e * ES] = w[e];
+                    }
+                    if (C.on()) {
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            if (j + e * ES >= n) continue;
+                            if constexpr (sizeof(T) == 4) {
+                                Scale<float> k;
+                                k.h = C.f32(b + r, j + e * ES);
+                                k.l = 0.f;
+                                acc.add(w[e], k);
+                            } else {
+                                obj += C(b + r, j + e * ES) * w[e];
+                            }
+                        }
+                    }
+                }
+            }
+            if (sizeof(T) == 4) obj += acc.get();
+        }
+    }
+    if (!C.on()) return;
+    obj = warp_add(obj);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = obj;
     __syncthreads();
     if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
-        objpart[grp] = s;
+        double t = 0.0;
+        for (int w = 0; w < RB / 32; ++w) t += red[w];
+        objpart[(long long)blockIdx.y * gridDim.x + blockIdx.x] = t;
     }
 }
 
 struct Bf16 {
     unsigned short b;
-    __device__ operator double() const { return (double)__uint_as_float(((unsigned)b) << 16); }
+    __device__ operator float() const { return __uint_as_float(((unsigned)b) << 16); }
 };
 
 // Weak-duality bound of Eq. (1) from a row dual p (no counterpart in the
@@ -179,48 +591,110 @@ int launch_dual_bound(const void* C, int ctype, long long ldc, const GenSpec* ge
     return (int)cudaGetLastError();
 }
 
-int launch_round_rowsum(const void* X, int xtype, long long m, long long n, long long ldx, const double* rs,
-                        const double* cs, double* rowout, double* colpart, int parts, void* stream) {
-    const cudaStream_t st = (cudaStream_t)stream;
-    const dim3 rb((unsigned)((m + 7) / 8));
-    const dim3 cb((unsigned)((n + 255) / 256), (unsigned)parts);
-    if (xtype == 2) {
-        k_round_rows<double><<<rb, 256, 0, st>>>((const double*)X, m, n, ldx, rs, cs, rowout);
-        k_round_cols<double><<<cb, 256, 0, st>>>((const double*)X, m, n, ldx, rs, cs, colpart, parts);
-    } else {
-        k_round_rows<float><<<rb, 256, 0, st>>>((const float*)X, m, n, ldx, rs, cs, rowout);
-        k_round_cols<float><<<cb, 256, 0, st>>>((const float*)X, m, n, ldx, rs, cs, colpart, parts);
-    }
+namespace {
+
+// Scratch of a rounding, in doubles (scales take one each).
+struct RoundScratch {
+    double *rs, *xs, *er, *ys, *ec, *colpart, *inv, *obj;
+    unsigned* state;   // ticket; 1: a row sum needs FP64 arithmetic
+    long long words;
+};
+int round_parts(long long m, long long n, int sm) {
+    // Row groups: enough blocks for four per SM, of at least 16 rows.
+    const long long cb = (n + 4 * RB - 1) / (4 * RB);
+    long long p = (4LL * sm + cb - 1) / cb;
+    if (p > (m + 15) / 16) p = (m + 15) / 16;
+    if (p > 65535) p = 65535;
+    return (int)(p < 1 ? 1 : p);
+}
+RoundScratch round_scratch(double* base, long long m, long long n, int sm) {
+    const int parts = round_parts(m, n, sm);
+    const int cparts = parts < RPARTS ? parts : RPARTS;
+    const long long cb = (n + 4 * RB - 1) / (4 * RB);
+    RoundScratch r;
+    r.rs = base;
+    r.xs = r.rs + m;
+    r.er = r.xs + m;
+    r.ys = r.er + m;
+    r.ec = r.ys + n;
+    r.colpart = r.ec + n;
+    r.inv = r.colpart + (long long)cparts * n;
+    r.state = reinterpret_cast<unsigned*>(r.inv + 1);
+    r.obj = r.inv + 2;
+    r.words = 3 * m + (2 + (long long)cparts) * n + 2 + cb * parts;
+    return r;
+}
+
+template <typename T, bool VEC, typename CA>
+int run_round(const T* X, long long m, long long n, long long ldx, const double* f, const double* g, T* out, long long ldo,
+              CA C, const RoundScratch& w, int sm, cudaStream_t st) {
+    double* xs = w.xs;
+    Scale<T>* ys = reinterpret_cast<Scale<T>*>(w.ys);
+    Scale<T>* ec = reinterpret_cast<Scale<T>*>(w.ec);
+    const int parts = round_parts(m, n, sm), cparts = parts < RPARTS ? parts : RPARTS;
+    const unsigned cb = (unsigned)((n + 4 * RB - 1) / (4 * RB));
+    const cudaError_t e = cudaMemsetAsync(w.state, 0, 2 * sizeof(unsigned), st);
+    if (e != cudaSuccess) return (int)e;
+    // By rows: a block per row where there are few rows, else a warp per row
+    // (the weighted sweep: four rows per warp where that leaves eight warps per
+    // SM, for one read of the columns' scales).
+    Acc<T>* cpart = reinterpret_cast<Acc<T>*>(w.colpart);
+    const bool few = m < 16LL * sm && n >= 1024;
+    if (few)
+        k_round_rows<T, VEC, 8, 1, false><<<(unsigned)m, RB, 0, st>>>(X, m, n, ldx, f, nullptr, nullptr, w.rs, nullptr, w.state);
+    else
+        k_round_rows<T, VEC, 1, 1, false><<<(unsigned)((m + 7) / 8), RB, 0, st>>>(X, m, n, ldx, f, nullptr, nullptr, w.rs,
+                                                                                  nullptr, w.state);
+    k_round_cols<T, VEC><<<dim3(cb, (unsigned)cparts), RB, 0, st>>>(X, m, n, ldx, f, w.rs, xs, cpart, cparts, w.state);
+    k_round_colscale<T><<<(unsigned)((n + 63) / 64), 64, 0, st>>>(cpart, cparts, n, g, ys, ec, w.state);
+    if (few && m >= 4LL * sm)
+        k_round_rows<T, VEC, 8, 4, true><<<(unsigned)((m + 3) / 4), RB, 0, st>>>(X, m, n, ldx, f, ys, xs, w.er, w.inv, w.state);
+    else if (few)
+        k_round_rows<T, VEC, 8, 1, true><<<(unsigned)m, RB, 0, st>>>(X, m, n, ldx, f, ys, xs, w.er, w.inv, w.state);
+    else if (m < 64LL * sm && n >= 1024)
+        k_round_rows<T, VEC, 4, 4, true><<<(unsigned)((m + 7) / 8), RB, 0, st>>>(X, m, n, ldx, f, ys, xs, w.er, w.inv, w.state);
+    else
+        k_round_rows<T, VEC, 1, 4, true><<<(unsigned)((m + 31) / 32), RB, 0, st>>>(X, m, n, ldx, f, ys, xs, w.er, w.inv, w.state);
+    k_round_write<T, VEC, CA><<<dim3(cb, (unsigned)parts), RB, 0, st>>>(X, m, n, ldx, xs, ys, w.er, ec, w.inv, out, ldo, C,
+                                                                        w.obj, w.state);
     return (int)cudaGetLastError();
 }
 
-int launch_colreduce(const double* colpart, int parts, long long n, double* out, void* stream) {
-    k_colreduce<<<(unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream>>>(colpart, parts, n, out);
-    return (int)cudaGetLastError();
+template <typename T, typename CA>
+int run_round_v(const T* X, long long m, long long n, long long ldx, const double* f, const double* g, T* out, long long ldo,
+                CA C, const RoundScratch& w, int sm, cudaStream_t st) {
+    // 16-byte accesses where the rows of both plans start on 16-byte boundaries.
+    const long long q = 16 / (long long)sizeof(T);
+    const bool vec = reinterpret_cast<uintptr_t>(X) % 16 == 0 && reinterpret_cast<uintptr_t>(out) % 16 == 0 &&
+                     ldx % q == 0 && ldo % q == 0;
+    return vec ? run_round<T, true>(X, m, n, ldx, f, g, out, ldo, C, w, sm, st)
+               : run_round<T, false>(X, m, n, ldx, f, g, out, ldo, C, w, sm, st);
 }
 
-int launch_round_write(const void* X, int xtype, long long m, long long n, long long ldx, const double* rs,
-                       const double* cs, const double* er, const double* ec, double inv_l1, void* Xout,
-                       long long ldo, const void* C, int ctype, long long ldc, const GenSpec* gen,
-                       double* objpart, int parts, void* stream) {
+}  // namespace
+
+// Doubles of scratch a rounding takes, and the objective partials in it.
+long long round_scratch_words(long long m, long long n, int sm) { return round_scratch(nullptr, m, n, sm).words; }
+double* round_obj_parts(double* base, long long m, long long n, int sm, long long* count) {
+    *count = (n + 4 * RB - 1) / (4 * RB) * round_parts(m, n, sm);
+    return round_scratch(base, m, n, sm).obj;
+}
+
+// Algorithm 3 on X (m x n, leading dimension ldx) into out (ldo); with a cost,
+// the partials of <C, out> too.
+int launch_round(const void* X, int xtype, long long m, long long n, long long ldx, const double* f, const double* g,
+                 void* out, long long ldo, const void* C, int ctype, long long ldc, const GenSpec* gen, double* scratch,
+                 int sm, void* stream) {
     const cudaStream_t st = (cudaStream_t)stream;
-    if (xtype == 2) {
-        k_round_write<double><<<parts, 256, 0, st>>>((const double*)X, m, n, ldx, rs, cs, er, ec, inv_l1,
-                                                     (double*)Xout, ldo,
-                                                     StoredCost<double>{(const double*)C, ldc}, objpart, parts);
-    } else if (ctype == 3) {
-        k_round_write<float><<<parts, 256, 0, st>>>((const float*)X, m, n, ldx, rs, cs, er, ec, inv_l1,
-                                                    (float*)Xout, ldo, PointsCost{*gen}, objpart, parts);
-    } else if (ctype == 1) {
-        k_round_write<float><<<parts, 256, 0, st>>>((const float*)X, m, n, ldx, rs, cs, er, ec, inv_l1,
-                                                    (float*)Xout, ldo, StoredCost<Bf16>{(const Bf16*)C, ldc},
-                                                    objpart, parts);
-    } else {
-        k_round_write<float><<<parts, 256, 0, st>>>((const float*)X, m, n, ldx, rs, cs, er, ec, inv_l1,
-                                                    (float*)Xout, ldo, StoredCost<float>{(const float*)C, ldc},
-                                                    objpart, parts);
-    }
-    return (int)cudaGetLastError();
+    const RoundScratch w = round_scratch(scratch, m, n, sm);
+    if (xtype == 2)
+        return run_round_v((const double*)X, m, n, ldx, f, g, (double*)out, ldo, StoredCost<double>{(const double*)C, ldc}, w,
+                           sm, st);
+    if (ctype == 3) return run_round_v((const float*)X, m, n, ldx, f, g, (float*)out, ldo, PointsCost{*gen}, w, sm, st);
+    if (ctype == 1)
+        return run_round_v((const float*)X, m, n, ldx, f, g, (float*)out, ldo, StoredCost<Bf16>{(const Bf16*)C, ldc}, w, sm,
+                           st);
+    return run_round_v((const float*)X, m, n, ldx, f, g, (float*)out, ldo, StoredCost<float>{(const float*)C, ldc}, w, sm, st);
 }
 
 }  // namespace pdot
