@@ -37,9 +37,10 @@ double* round_obj_parts(double* base, long long m, long long n, int sm, long lon
 int launch_round(const void* X, int xtype, long long m, long long n, long long ldx, const double* f, const double* g,
                  void* out, long long ldo, const void* C, int ctype, long long ldc, const GenSpec* gen, double* scratch,
                  int sm, void* stream);
+long long bound_scratch_bytes(long long n);
 int launch_dual_bound(const void* C, int ctype, long long ldc, const GenSpec* gen, const double* p,
-                      const double* f, const double* g, long long m, long long n, double* colmin, int parts,
-                      double* q, double* out, void* stream);
+                      const double* f, const double* g, long long m, long long n, void* scratch, double* q_out,
+                      double** value, int sm, void* stream);
 }  // namespace pdot
 
 namespace {
@@ -2079,8 +2080,7 @@ pdot_status pdot_dual_bound(pdot_handle* h, int64_t m, int64_t n, const void* C,
         CK(cudaSetDevice(h->device));
         check_common_args(h, m, n, C, c_dtype, ldc, f, g);
         if (!p || !lower) throw ArgError{"null p or lower"};
-        const int parts = (int)std::min<long long>(64, m);   // row groups of the column minima
-        const size_t need = sizeof(double) * ((size_t)parts * (size_t)n + (size_t)n + 8);
+        const size_t need = (size_t)bound_scratch_bytes(n);
         if (h->round_scratch_bytes < need) {
             if (h->round_scratch) cudaFree(h->round_scratch);
             h->round_scratch = nullptr;
@@ -2088,16 +2088,15 @@ pdot_status pdot_dual_bound(pdot_handle* h, int64_t m, int64_t n, const void* C,
             CK(cudaMalloc(&h->round_scratch, need));
             h->round_scratch_bytes = need;
         }
-        double* colmin = h->round_scratch;
-        double* q = colmin + (size_t)parts * (size_t)n;
-        double* val = q + n;
+        double* val = nullptr;
         GenSpec gs{};
         if (c_dtype == PDOT_POINTS) gs = gen_spec_of(C);
-        CKL(launch_dual_bound(C, (int)c_dtype, ldc, &gs, p, f, g, m, n, colmin, parts, q, val, h->stream));
-        launch_count(h, 3);
-        if (q_out) CK(cudaMemcpyAsync(q_out, q, sizeof(double) * (size_t)n, cudaMemcpyDeviceToDevice, h->stream));
-        CK(cudaMemcpyAsync(lower, val, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+        CKL(launch_dual_bound(C, (int)c_dtype, ldc, &gs, p, f, g, m, n, h->round_scratch, q_out, &val, h->sm_count, h->stream));
+        launch_count(h, c_dtype == PDOT_F64 ? 2 : 3);
+        double* hv = reinterpret_cast<double*>(h->h_status);   // (pinned, 8 bytes)
+        CK(cudaMemcpyAsync(hv, val, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
         CK(cudaStreamSynchronize(h->stream));
+        *lower = *hv;
         return PDOT_OK;
     });
 }

@@ -25,6 +25,7 @@
 // (2.5e-8).  Sums of 1e30 and more, or not finite, switch the sweeps to FP64
 // arithmetic, so no range is lost.  FP64 plans use FP64 throughout.
 #include <cuda_runtime.h>
+#include <math_constants.h>
 
 #include <cstdint>
 #include <type_traits>
@@ -352,6 +353,11 @@ __global__ void k_round_colscale(const Acc<T>* __restrict__ colpart, int parts, 
     ec[j].set(g[j] - y * c, wide);
 }
 
+struct Bf16 {
+    unsigned short b;
+    __device__ operator float() const { return __uint_as_float(((unsigned)b) << 16); }
+};
+
 // Cost entry (i, j) for the objective of the rounded plan: a stored matrix
 // (null: no objective) or the generated cost.
 template <typename TC>
@@ -511,83 +517,233 @@ __global__ void __launch_bounds__(RB) k_round_write(const T* X, long long m, lon
     }
 }
 
-struct Bf16 {
-    unsigned short b;
-    __device__ operator float() const { return __uint_as_float(((unsigned)b) << 16); }
-};
-
 // Weak-duality bound of Eq. (1) from a row dual p (no counterpart in the
 // paper; it certifies a result): q_j = min_i (C_ij - p_i) is the largest
-// column dual with p_i + q_j <= C_ij for all i, and f^T p + g^T q <= OPT.
-// colmin[grp][j] = min over the rows of group grp (one thread per column, so
-// a warp reads 32 consecutive entries of a row).  The minimum is exact, so
-// the result does not depend on the grouping.
-template <typename CA>
-__global__ void k_cmin_cols(CA C, const double* p, long long m, long long n, double* colmin, int parts) {
-    const long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int grp = blockIdx.y;
+// column dual with p_i + q_j <= C_ij for all i, and f^T p + g^T q <= OPT.  The
+// minimum is exact, so the result does not depend on the grouping.
+//
+// FP64 C: one sweep.  Otherwise the difference, the comparison and the
+// conversion in FP64 would bound the sweep (106 us at 4096 x 4096): a first
+// sweep takes the minimum of C - RN32(p) in FP32, a second one forms the FP64
+// difference only where the FP32 one is within its rounding error of that
+// minimum -- a handful of entries per column (two sweeps, 42 us).  |RN32(c - RN32(p)) - (c - p)| is
+// at most 2^-24 (|p| + |c - p|) (and 2^-149 below the normal range), so the
+// entry that attains the minimum lies within 2^-22 (max|p| + |min|) + 2^-125.
+// Row duals of 1e30 and more make every entry a candidate.
+__device__ __forceinline__ unsigned key32(float v) {   // order-preserving
+    const unsigned u = __float_as_uint(v);
+    return u & 0x80000000u ? ~u : u | 0x80000000u;
+}
+__device__ __forceinline__ float unkey32(unsigned k) { return __uint_as_float(k & 0x80000000u ? k & 0x7fffffffu : ~k); }
+__device__ __forceinline__ unsigned long long key64(double v) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(v);
+    return u >> 63 ? ~u : u | 0x8000000000000000ull;
+}
+__device__ __forceinline__ double unkey64(unsigned long long k) {
+    return __longlong_as_double((long long)(k >> 63 ? k & 0x7fffffffffffffffull : ~k));
+}
+
+// Four cost entries of a row (columns j + e ES).
+template <bool VEC, typename CA>
+__device__ __forceinline__ void cost4(const CA& C, long long i, long long j, long long es, long long n, float (&c)[4]) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) c[e] = j + e * es < n ? C.f32(i, j + e * es) : 0.f;
+}
+template <bool VEC>
+__device__ __forceinline__ void cost4(const StoredCost<float>& C, long long i, long long j, long long es, long long n,
+                                      float (&c)[4]) {
+    if (VEC) {
+        load4<float, true>(C.C + i * C.ldc + j, n - j, c);
+    } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) c[e] = j + e * es < n ? C.f32(i, j + e * es) : 0.f;
+    }
+}
+template <bool VEC>
+__device__ __forceinline__ void cost4(const StoredCost<Bf16>& C, long long i, long long j, long long es, long long n,
+                                      float (&c)[4]) {
+    if (VEC && j + 4 <= n) {
+        const uint2 t = *reinterpret_cast<const uint2*>(C.C + i * C.ldc + j);
+        c[0] = __uint_as_float(t.x << 16); c[1] = __uint_as_float(t.x & 0xffff0000u);
+        c[2] = __uint_as_float(t.y << 16); c[3] = __uint_as_float(t.y & 0xffff0000u);
+    } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) c[e] = j + e * es < n ? C.f32(i, j + e * es) : 0.f;
+    }
+}
+
+// EXACT false: qmin[j] <- min of the FP32 differences (as keys), pmax <- the
+// complement of the bits of max |RN32(p)| (all of these start as all ones).  EXACT true: qkey[j] <- min of the FP64 differences of
+// the candidates.
+template <bool EXACT, bool VEC, typename CA>
+__global__ void __launch_bounds__(RB) k_bound_cols(CA C, const double* __restrict__ p, long long m, long long n,
+                                                   unsigned* qmin, unsigned* pmax, unsigned long long* qkey) {
+    const long long j = VEC ? ((long long)blockIdx.x * RB + threadIdx.x) * 4 : (long long)blockIdx.x * RB * 4 + threadIdx.x;
+    constexpr long long ES = VEC ? 1 : RB;
+    const long long r0 = m * blockIdx.y / gridDim.y, r1 = m * (blockIdx.y + 1) / gridDim.y;
+    __shared__ float sp[64];
+    float lim[4];
+    double best[4];
+    bool any[4] = {false, false, false, false};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        lim[e] = CUDART_INF_F;
+        best[e] = CUDART_INF;
+        if (EXACT && j + e * ES < n) {
+            const float v = unkey32(qmin[j + e * ES]), pm = __uint_as_float(~*pmax);
+            lim[e] = pm < 1e30f ? v + (0x1p-22f * (pm + fabsf(v)) + 0x1p-125f) : CUDART_NAN_F;
+        }
+    }
+    float pm = 0.f;
+    for (long long b = r0; b < r1; b += 64) {
+        const int cnt = (int)(b + 64 < r1 ? 64 : r1 - b);
+        __syncthreads();
+        if ((int)threadIdx.x < cnt) {
+            sp[threadIdx.x] = (float)p[b + threadIdx.x];
+            pm = fmaxf(pm, fabsf(sp[threadIdx.x]));
+        }
+        __syncthreads();
+        if (j >= n) continue;
+#pragma unroll 8
+        for (int r = 0; r < cnt; ++r) {
+            float c[4];
+            cost4<VEC>(C, b + r, j, ES, n, c);
+            const float ph = sp[r];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float t = c[e] - ph;
+                if (!EXACT) {
+                    lim[e] = fminf(lim[e], t);
+                } else if (!(t > lim[e])) {   // (also where the limit is not a number)
+                    const double d = (double)c[e] - p[b + r];
+                    any[e] = true;
+                    if (d < best[e]) best[e] = d;
+                }
+            }
+        }
+    }
+    if (!EXACT && blockIdx.x == 0 && threadIdx.x < 64) {
+        // (NaN duals leave the maximum alone: their differences are never minima)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) pm = fmaxf(pm, __shfl_xor_sync(0xffffffffu, pm, o));
+        if ((threadIdx.x & 31) == 0) atomicMin(pmax, ~__float_as_uint(pm));
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        if (j + e * ES >= n) continue;
+        if (!EXACT) atomicMin(qmin + j + e * ES, key32(lim[e]));
+        else if (any[e]) atomicMin(qkey + j + e * ES, key64(best[e]));
+    }
+}
+
+__global__ void __launch_bounds__(RB) k_bound_cols64(StoredCost<double> C, const double* __restrict__ p, long long m,
+                                                     long long n, unsigned long long* qkey) {
+    const long long j = (long long)blockIdx.x * RB + threadIdx.x;
     if (j >= n) return;
-    const long long r0 = m * grp / parts, r1 = m * (grp + 1) / parts;
-    double v = __longlong_as_double(0x7ff0000000000000LL);   // +inf: an empty group
+    const long long r0 = m * blockIdx.y / gridDim.y, r1 = m * (blockIdx.y + 1) / gridDim.y;
+    double v = CUDART_INF;
+#pragma unroll 8
     for (long long i = r0; i < r1; ++i) {
         const double t = C(i, j) - p[i];
         if (t < v) v = t;
     }
-    colmin[(long long)grp * n + j] = v;
+    atomicMin(qkey + j, key64(v));
 }
 
-__global__ void k_cmin_reduce(const double* colmin, int parts, long long n, double* q) {
-    const long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= n) return;
-    double v = colmin[j];
-    for (int g = 1; g < parts; ++g) {
-        const double t = colmin[(long long)g * n + j];
-        if (t < v) v = t;
-    }
-    q[j] = v;
-}
-
-// out[0] = f^T p + g^T q: one block, fixed-order strided sums, then a tree.
-__global__ void k_dual_value(const double* f, const double* p, long long m, const double* g, const double* q,
-                             long long n, double* out) {
-    __shared__ double red[1024];
+// q from its keys (into q_out, where wanted) and out[0] = f^T p + g^T q: fixed
+// runs per block, the last block adds the blocks' sums in order.  ticket starts
+// as all ones.
+__global__ void __launch_bounds__(RB) k_bound_value(const double* __restrict__ f, const double* __restrict__ p, long long m,
+                                                    const double* __restrict__ g,
+                                                    const unsigned long long* __restrict__ qkey, double* q_out, long long n,
+                                                    double* part, double* out, unsigned* ticket) {
+    __shared__ double red[RB / 32];
+    __shared__ unsigned last;
     double s = 0.0;
-    for (long long i = threadIdx.x; i < m; i += blockDim.x) s += f[i] * p[i];
-    for (long long j = threadIdx.x; j < n; j += blockDim.x) s += g[j] * q[j];
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int w = blockDim.x >> 1; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-        __syncthreads();
+    for (long long e = (long long)blockIdx.x * RB + threadIdx.x; e < m + n; e += (long long)gridDim.x * RB) {
+        if (e < m) {
+            s = fma(f[e], p[e], s);
+        } else {
+            const double q = unkey64(qkey[e - m]);
+            if (q_out) q_out[e - m] = q;
+            s = fma(g[e - m], q, s);
+        }
     }
-    if (threadIdx.x == 0) out[0] = red[0];
+    s = warp_add(s);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        s = 0.0;
+        for (int w = 0; w < RB / 32; ++w) s += red[w];
+        part[blockIdx.x] = s;
+        __threadfence();
+        last = atomicAdd(ticket, 1u) + 1u == gridDim.x - 1 ? 1u : 0u;
+    }
+    __syncthreads();
+    if (!last || threadIdx.x >= 32) return;
+    __threadfence();
+    s = 0.0;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += 32) s += __ldcg(part + b);
+    s = warp_add(s);
+    if (threadIdx.x == 0) out[0] = s;
 }
 
 template <typename CA>
-void launch_cmin(CA C, const double* p, long long m, long long n, double* colmin, int parts, cudaStream_t st) {
-    const dim3 cb((unsigned)((n + 255) / 256), (unsigned)parts);
-    k_cmin_cols<CA><<<cb, 256, 0, st>>>(C, p, m, n, colmin, parts);
+void launch_bound_cols(CA C, bool vec, const double* p, long long m, long long n, unsigned* qmin, unsigned* pmax,
+                       unsigned long long* qkey, int sm, cudaStream_t st) {
+    // Row groups: four blocks per SM, of at least 16 rows.
+    const long long cb = (n + 4 * RB - 1) / (4 * RB);
+    long long parts = (4LL * sm + cb - 1) / cb;
+    if (parts > (m + 15) / 16) parts = (m + 15) / 16;
+    if (parts > 65535) parts = 65535;
+    const dim3 grid((unsigned)cb, (unsigned)parts);
+    if (vec) {
+        k_bound_cols<false, true, CA><<<grid, RB, 0, st>>>(C, p, m, n, qmin, pmax, qkey);
+        k_bound_cols<true, true, CA><<<grid, RB, 0, st>>>(C, p, m, n, qmin, pmax, qkey);
+    } else {
+        k_bound_cols<false, false, CA><<<grid, RB, 0, st>>>(C, p, m, n, qmin, pmax, qkey);
+        k_bound_cols<true, false, CA><<<grid, RB, 0, st>>>(C, p, m, n, qmin, pmax, qkey);
+    }
 }
+
+constexpr int BOUND_BLOCKS = 64;
 
 }  // namespace
 
-// The bound above: q (n) and out[0] = f^T p + g^T q.  colmin: parts x n
-// scratch, 1 <= parts <= m.  ctype: 0 FP32, 1 BF16, 2 FP64 (row-major with
-// leading dimension ldc), 3 generated (gen).
+// Scratch of the bound in bytes: the keys, the FP32 minima, max |p| and the
+// ticket (all ones at the start), the block sums, the value.
+long long bound_scratch_bytes(long long n) { return 8 * n + 4 * ((n + 1) / 2 * 2) + 8 + 8 * (BOUND_BLOCKS + 1); }
+
+// The bound above: q_out (n, or null) and *value = f^T p + g^T q.
+// ctype: 0 FP32, 1 BF16, 2 FP64 (row-major with leading dimension ldc), 3
+// generated (gen).
 int launch_dual_bound(const void* C, int ctype, long long ldc, const GenSpec* gen, const double* p,
-                      const double* f, const double* g, long long m, long long n, double* colmin, int parts,
-                      double* q, double* out, void* stream) {
+                      const double* f, const double* g, long long m, long long n, void* scratch, double* q_out,
+                      double** value, int sm, void* stream) {
     const cudaStream_t st = (cudaStream_t)stream;
-    if (ctype == 3)
-        launch_cmin(PointsCost{*gen}, p, m, n, colmin, parts, st);
-    else if (ctype == 2)
-        launch_cmin(StoredCost<double>{(const double*)C, ldc}, p, m, n, colmin, parts, st);
-    else if (ctype == 1)
-        launch_cmin(StoredCost<Bf16>{(const Bf16*)C, ldc}, p, m, n, colmin, parts, st);
-    else
-        launch_cmin(StoredCost<float>{(const float*)C, ldc}, p, m, n, colmin, parts, st);
-    k_cmin_reduce<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(colmin, parts, n, q);
-    k_dual_value<<<1, 1024, 0, st>>>(f, p, m, g, q, n, out);
+    unsigned long long* qkey = static_cast<unsigned long long*>(scratch);
+    unsigned* qmin = reinterpret_cast<unsigned*>(qkey + n);
+    unsigned* pmax = qmin + (n + 1) / 2 * 2;
+    double* part = reinterpret_cast<double*>(pmax + 2);
+    *value = part + BOUND_BLOCKS;
+    const cudaError_t e = cudaMemsetAsync(scratch, 0xff, (size_t)(reinterpret_cast<char*>(part) - static_cast<char*>(scratch)), st);
+    if (e != cudaSuccess) return (int)e;
+    const bool a16 = reinterpret_cast<uintptr_t>(C) % 16 == 0;
+    if (ctype == 3) {
+        launch_bound_cols(PointsCost{*gen}, false, p, m, n, qmin, pmax, qkey, sm, st);
+    } else if (ctype == 2) {
+        long long parts = 64 < m ? 64 : m;
+        k_bound_cols64<<<dim3((unsigned)((n + RB - 1) / RB), (unsigned)parts), RB, 0, st>>>(
+            StoredCost<double>{(const double*)C, ldc}, p, m, n, qkey);
+    } else if (ctype == 1) {
+        launch_bound_cols(StoredCost<Bf16>{(const Bf16*)C, ldc}, a16 && ldc % 4 == 0, p, m, n, qmin, pmax, qkey, sm, st);
+    } else {
+        launch_bound_cols(StoredCost<float>{(const float*)C, ldc}, a16 && ldc % 4 == 0, p, m, n, qmin, pmax, qkey, sm, st);
+    }
+    // One block per 256 entries where that is fewer.
+    long long vb = (m + n + RB - 1) / RB;
+    if (vb > BOUND_BLOCKS) vb = BOUND_BLOCKS;
+    k_bound_value<<<(unsigned)vb, RB, 0, st>>>(f, p, m, g, qkey, q_out, n, part, *value, pmax + 1);
     return (int)cudaGetLastError();
 }
 
