@@ -244,6 +244,7 @@ struct pdot_handle {
     TileRef* d_tmap = nullptr;
     TileRef* d_vmap = nullptr;
     size_t tmap_cap = 0, vmap_cap = 0;
+    int cnt_tiles = -1, cnt_vec = -1;   // counts now in d_cnt
     int* d_cnt = nullptr;        // [0] plan tiles, [1] vector tiles of the single-instance path
     int* h_cnt = nullptr;        // pinned staging
     Ctrl* h_ctrl = nullptr;      // pinned
@@ -303,29 +304,31 @@ void ensure_work(pdot_handle* h, long long m, long long n, int xtype, int tile_r
     CK(cudaMemsetAsync(w.ticket, 0, sizeof(unsigned), h->stream));
 }
 
+// The single instance's maps: entry t is {0, t}, so they are written when they
+// grow, and the counts when they change.
 void ensure_maps(pdot_handle* h) {
     const Work& w = h->ws;
-    if ((size_t)w.ntiles > h->tmap_cap) {
-        if (h->d_tmap) cudaFree(h->d_tmap);
-        h->d_tmap = nullptr;
-        CK(cudaMalloc(&h->d_tmap, sizeof(TileRef) * (size_t)w.ntiles));
-        h->tmap_cap = (size_t)w.ntiles;
-    }
-    if ((size_t)w.nvt > h->vmap_cap) {
-        if (h->d_vmap) cudaFree(h->d_vmap);
-        h->d_vmap = nullptr;
-        CK(cudaMalloc(&h->d_vmap, sizeof(TileRef) * (size_t)w.nvt));
-        h->vmap_cap = (size_t)w.nvt;
-    }
-    std::vector<TileRef> tm((size_t)w.ntiles), vm((size_t)w.nvt);
-    for (int t = 0; t < w.ntiles; ++t) tm[(size_t)t] = TileRef{0, t};
-    for (int t = 0; t < w.nvt; ++t) vm[(size_t)t] = TileRef{0, t};
-    CK(cudaMemcpyAsync(h->d_tmap, tm.data(), sizeof(TileRef) * tm.size(), cudaMemcpyHostToDevice, h->stream));
-    CK(cudaMemcpyAsync(h->d_vmap, vm.data(), sizeof(TileRef) * vm.size(), cudaMemcpyHostToDevice, h->stream));
+    auto grow = [&](TileRef*& d, size_t& cap, size_t need) {
+        if (need <= cap) return;
+        if (d) cudaFree(d);
+        d = nullptr;
+        cap = 0;
+        CK(cudaMalloc(&d, sizeof(TileRef) * need));
+        std::vector<TileRef> v(need);
+        for (size_t t = 0; t < need; ++t) v[t] = TileRef{0, (int)t};
+        CK(cudaMemcpyAsync(d, v.data(), sizeof(TileRef) * need, cudaMemcpyHostToDevice, h->stream));
+        CK(cudaStreamSynchronize(h->stream));   // v is pageable and goes out of scope
+        cap = need;
+    };
+    grow(h->d_tmap, h->tmap_cap, (size_t)w.ntiles);
+    grow(h->d_vmap, h->vmap_cap, (size_t)w.nvt);
+    if (h->cnt_tiles == w.ntiles && h->cnt_vec == w.nvt) return;
+    CK(cudaStreamSynchronize(h->stream));       // an earlier copy may still read the staging words
     h->h_cnt[0] = w.ntiles;
     h->h_cnt[1] = w.nvt;
     CK(cudaMemcpyAsync(h->d_cnt, h->h_cnt, 2 * sizeof(int), cudaMemcpyHostToDevice, h->stream));
-    CK(cudaStreamSynchronize(h->stream));   // vectors above are pageable and go out of scope
+    h->cnt_tiles = w.ntiles;
+    h->cnt_vec = w.nvt;
 }
 
 void validate_marginals(pdot_handle* h, long long m, long long n, const double* f, const double* g, bool host,
@@ -650,12 +653,13 @@ void copy_duals_out(pdot_handle* h, int slot, double* p_out, double* q_out, cuda
     if (q_out) CK(cudaMemcpyAsync(q_out, V + w.m, sizeof(double) * (size_t)w.n, kind, h->stream));
 }
 
-// Upload a dense m x n plan and its duals into slot 0.
+// Upload a dense m x n plan (null: the caller's is read in place) and its
+// duals into slot 0.
 void upload_state(pdot_handle* h, const void* X, const double* p, const double* q) {
     const Work& w = h->ws;
     const size_t xs = xsize_of(w.xtype);
-    CK(cudaMemsetAsync(w.X, 0, (size_t)w.m * w.ldx * xs, h->stream));
-    CK(cudaMemcpy2DAsync(w.X, (size_t)w.ldx * xs, X, (size_t)w.n * xs, (size_t)w.n * xs, (size_t)w.m,
+    if (X && w.ldx != w.n) CK(cudaMemsetAsync(w.X, 0, (size_t)w.m * w.ldx * xs, h->stream));   // (the padding)
+    if (X) CK(cudaMemcpy2DAsync(w.X, (size_t)w.ldx * xs, X, (size_t)w.n * xs, (size_t)w.n * xs, (size_t)w.m,
                          cudaMemcpyDeviceToDevice, h->stream));
     CK(cudaMemsetAsync(w.V, 0, sizeof(double) * 2 * (size_t)(w.m + w.n), h->stream));
     CK(cudaMemcpyAsync(w.V, p, sizeof(double) * (size_t)w.m, cudaMemcpyDeviceToDevice, h->stream));
@@ -830,7 +834,7 @@ bool import_state(pdot_handle* h, const void* in, Ctrl* S) {
 void upload_start(pdot_handle* h, const pdot_start* st) {
     const Work& w = h->ws;
     const size_t xs = xsize_of(w.xtype);
-    CK(cudaMemsetAsync(w.X, 0, (size_t)w.m * w.ldx * xs, h->stream));
+    if (!(st && st->X0) || w.ldx != w.n) CK(cudaMemsetAsync(w.X, 0, (size_t)w.m * w.ldx * xs, h->stream));
     CK(cudaMemsetAsync(w.V, 0, sizeof(double) * 2 * (size_t)(w.m + w.n), h->stream));
     if (st && st->X0)
         CK(cudaMemcpy2DAsync(w.X, (size_t)w.ldx * xs, st->X0, (size_t)w.n * xs, (size_t)w.n * xs, (size_t)w.m,
@@ -2029,8 +2033,7 @@ pdot_status pdot_kkt(pdot_handle* h, int64_t m, int64_t n, const void* C, pdot_d
         CK(cudaSetDevice(h->device));
         check_common_args(h, m, n, C, c_dtype, ldc, f, g);
         if (!X || !p || !q || !out) throw ArgError{"null X, p, q or out"};
-        double norm_b = 0.0;
-        validate_marginals(h, m, n, f, g, false, &norm_b);
+        // (The init check tests the marginals on the device.)
         const int ttype = ttype_of(c_dtype);
         const int tr = pick_tile_rows(h, m, n, ttype);
         ensure_work(h, m, n, h->opt.x_dtype, tr);
@@ -2038,12 +2041,17 @@ pdot_status pdot_kkt(pdot_handle* h, int64_t m, int64_t n, const void* C, pdot_d
         Work& w = h->ws;
         long long ldc_used = ldc;
         const void* Cd = prepare_C(h, m, n, C, c_dtype, ldc, &ldc_used);
-        stage_instance(h, make_inst(w, Cd, c_dtype, ldc_used, f, g));
+        Inst I = make_inst(w, Cd, c_dtype, ldc_used, f, g);
+        // The check only reads the plan: the caller's own where its rows have
+        // the workspace's layout (no padding, 16-byte starts).
+        const bool in_place = w.ldx == n && (uintptr_t)X % 16 == 0;
+        if (in_place) I.X = const_cast<void*>(X);
+        stage_instance(h, I);
         Ctrl* S = h->h_ctrl;
-        init_ctrl(h, S, m, n, -1.0, norm_b, 0.0, false, 0.0, 0.0, false);
+        init_ctrl(h, S, m, n, -1.0, 0.0, 0.0, false, 0.0, 0.0, false);
         CK(cudaMemcpyAsync(w.ctrl, S, sizeof(Ctrl), cudaMemcpyHostToDevice, h->stream));
         CK(cudaMemsetAsync(w.ticket, 0, sizeof(unsigned), h->stream));
-        upload_state(h, X, p, q);
+        upload_state(h, in_place ? nullptr : X, p, q);
         run_check(h, ttype, MODE_INIT);
         CK(cudaMemcpyAsync(S, w.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, h->stream));
         CK(cudaStreamSynchronize(h->stream));

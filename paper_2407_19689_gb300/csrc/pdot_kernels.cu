@@ -929,18 +929,18 @@ k_kkt(const Inst* __restrict__ insts, const TileRef* __restrict__ tmap, const in
 }
 
 // ---------------------------------------------------------------------------
-// KKT pass, bulk-copy pipeline (FP32 plans with a stored FP32 or BF16 cost):
-// the arithmetic of kkt_tile, with each warp streaming its tile's rows of C,
-// X, Xbar and the restart anchor through KS shared-memory stages filled by
-// cp.async.bulk (completion counted on one mbarrier per stage, bounded wait),
-// so a warp keeps KS rows of four arrays in flight without holding them in
-// registers.  The FP32 accumulators are added into FP64 every 16 rows.
+// KKT pass, copy pipeline (FP32 plans with a stored FP32 or BF16 cost): the
+// arithmetic of kkt_tile, with each warp streaming its tile's rows of C, X, D
+// and the restart anchor through KS shared-memory stages.  Every lane copies
+// the 16 bytes it reads itself (cp.async; by bulk copies the rows took 40
+// cycles each of an SM's copy engine: this kernel at 4096 x 4096 74 us, here 61).
+// The FP32 accumulators are added into FP64 every 64 rows.
 // ---------------------------------------------------------------------------
 constexpr int KS = 4;                     // stages per warp (two CTAs per SM: 64 rows of 4 arrays in flight)
 constexpr int KSTAGE = 4 * STRIP * 4;     // C (<= 512 B), X, Xbar, anchor (512 B each)
 constexpr int KACC = TP + 8;              // FP64 accumulators per lane kept in shared memory (6 scalars, 2 x 4 columns)
 __host__ __device__ constexpr int kkt_warp_smem() {
-    return KS * KSTAGE + KS * 8 + KS * 8 + bulk::PWIN * 8 + KACC * 32 * 8;
+    return KS * KSTAGE + KS * 16 + bulk::PWIN * 8 + KACC * 32 * 8;
 }
 constexpr int kkt_smem() { return TWARPS * kkt_warp_smem(); }
 
@@ -953,35 +953,25 @@ k_kkt_bulk(const Inst* __restrict__ insts, const TileRef* __restrict__ tmap, con
     extern __shared__ __align__(128) unsigned char dsm[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     unsigned char* wbase = dsm + warp * kkt_warp_smem();
-    unsigned long long* bars = reinterpret_cast<unsigned long long*>(wbase + KS * KSTAGE);
-    RowRef* refs = reinterpret_cast<RowRef*>(wbase + KS * KSTAGE + KS * 8);
+    RowRef* refs = reinterpret_cast<RowRef*>(wbase + KS * KSTAGE);
     float2* pbuf = reinterpret_cast<float2*>(wbase + KS * KSTAGE + KS * 16);   // (p_i, pbar_i) of a row window
     // The lane's FP64 accumulators (kept out of registers): [k * 32 + lane],
     // k < TP the tile scalars, then 4 column sums (average / initial plan), 4
     // column sums (current plan).
     double* sacc = reinterpret_cast<double*>(wbase + KS * KSTAGE + KS * 16 + bulk::PWIN * 8);
     const unsigned wbase_s = smem_u32(wbase);
-    const unsigned bars_s = smem_u32(bars);
-    if (lane == 0) {
-        for (int s = 0; s < KS; ++s) mbar_init(bars_s + 8 * s, 1);
-        fence_mbar_init();
-    }
-    __syncwarp();
     prefetch_first_tile(insts, tmap, T);
     pdl_enter();
     reset_other_counters(wctr, wc);
     const bool init = mode == MODE_INIT;
-    constexpr long long CQ = sizeof(TC) == 2 ? 8 : 4;   // C elements per 16 bytes
 
     // ---- producer ----
     int p_tile = T;
-    long long p_row = 0, p_end = 0, p_r0 = 0, p_last_ragged = -1;
-    const char* p_c0 = nullptr;     // C, X, Xbar, anchor at the tile's first row
-    const char* p_x0 = nullptr;
-    const char* p_xb0 = nullptr;
-    const char* p_xa0 = nullptr;
-    long long p_cstride = 0, p_xstride = 0;
-    unsigned p_cbytes = 0, p_xbytes = 0;
+    int p_row = 0, p_end = 0, p_last = -1;
+    const TC* p_c = nullptr;        // this lane's columns of C and X in the row to copy; D and the anchor as offsets from X
+    const float* p_x = nullptr;
+    long long p_cstride = 0, p_xstride = 0, p_db = 0, p_da = 0;
+    unsigned p_cb = 0, p_xb = 0;    // bytes of C and X this lane has in a row
     bool p_avg = false;
     bool q_first = true;
     auto next_tile = [&]() {
@@ -992,24 +982,23 @@ k_kkt_bulk(const Inst* __restrict__ insts, const TileRef* __restrict__ tmap, con
             const Inst& I = insts[tr.inst];
             const Ctrl& Sc = *I.ctrl;
             if (Sc.status != ST_RUNNING) continue;
-            const int strip = tr.local % I.nstrips, chunk = tr.local / I.nstrips;
+            const unsigned strip = (unsigned)tr.local % (unsigned)I.nstrips, chunk = (unsigned)tr.local / (unsigned)I.nstrips;
             const long long c0 = (long long)strip * STRIP;
-            const long long ncols = min((long long)STRIP, I.n - c0);
-            p_r0 = (long long)chunk * I.tile_rows;
-            p_row = p_r0;
-            p_end = min(p_r0 + (long long)I.tile_rows, I.m);
-            p_xstride = I.ldx * 4;
-            p_cstride = I.ldc * (long long)sizeof(TC);
-            p_c0 = reinterpret_cast<const char*>(I.C) + p_r0 * p_cstride + c0 * (long long)sizeof(TC);
+            const int mine = (int)min(4LL, I.n - c0 - lane * 4);   // columns of this lane (<= 0: none)
+            const long long j = c0 + (mine > 0 ? lane * 4 : 0);
+            p_row = (int)chunk * I.tile_rows;
+            p_end = min(p_row + I.tile_rows, (int)I.m);
+            p_xstride = I.ldx;
+            p_cstride = I.ldc;
+            p_c = reinterpret_cast<const TC*>(I.C) + p_row * p_cstride + j;
             const float* Xb = reinterpret_cast<const float*>(I.X);
-            p_x0 = reinterpret_cast<const char*>(Xb + (long long)plan_slot(Sc) * I.xslot + p_r0 * I.ldx + c0);
-            p_xb0 = reinterpret_cast<const char*>(Xb + (long long)Sc.xbar * I.xslot + p_r0 * I.ldx + c0);
-            p_xa0 = reinterpret_cast<const char*>(Xb + (long long)Sc.xanc * I.xslot + p_r0 * I.ldx + c0);
-            p_xbytes = (unsigned)(((ncols + 3) / 4) * 16);
-            p_cbytes = (unsigned)(((ncols + CQ - 1) / CQ) * CQ * (long long)sizeof(TC));
-            // The rounded-up C copy could run past the caller's allocation on
-            // the last matrix row of a ragged strip: lanes load that row.
-            p_last_ragged = (ncols % CQ) != 0 ? I.m - 1 : -1;
+            const int sx = plan_slot(Sc);
+            p_x = Xb + (long long)sx * I.xslot + p_row * p_xstride + j;
+            p_db = (long long)(Sc.xbar - sx) * I.xslot;
+            p_da = (long long)(Sc.xanc - sx) * I.xslot;
+            p_xb = mine > 0 ? 16u : 0u;
+            p_cb = mine > 0 ? (unsigned)mine * (unsigned)sizeof(TC) : 0u;
+            p_last = mine < 4 ? (int)I.m - 1 : -1;   // the row whose padding may be past the allocation
             p_avg = !init && Sc.k > 0;
             return;
         }
@@ -1017,21 +1006,21 @@ k_kkt_bulk(const Inst* __restrict__ insts, const TileRef* __restrict__ tmap, con
     long long issued = 0, consumed = 0;
     auto issue = [&]() {
         const int st = (int)(issued % KS);
-        const long long dr = p_row - p_r0;
+        const unsigned dst = wbase_s + st * KSTAGE + (unsigned)lane * 16u;
+        const bool off = p_xb == 0u;
+        lagp::cp16z(dst + STRIP * 4, p_x, off);
+        if (p_avg) lagp::cp16z(dst + 2 * STRIP * 4, p_x + p_db, off);
+        if (!init) lagp::cp16z(dst + 3 * STRIP * 4, p_x + p_da, off);
+        if constexpr (sizeof(TC) == 4) lagp::cp16(dst, p_c, p_row == p_last ? p_cb : p_xb);
+        else lagp::cp8(dst - lane * 8u, p_c, p_row == p_last ? p_cb : p_xb / 2u);
+        lagp::cp_commit();
         if (lane == 0) {
             refs[st].tile = p_tile;
-            refs[st].row = (int)p_row;
-            const unsigned bar = bars_s + 8 * st;
-            const unsigned dst = wbase_s + st * KSTAGE;
-            const unsigned cb = p_row == p_last_ragged ? 0u : p_cbytes;
-            fence_proxy_async();
-            mbar_expect_tx(bar, cb + p_xbytes + (p_avg ? p_xbytes : 0u) + (init ? 0u : p_xbytes));
-            if (cb) g2s(dst, p_c0 + dr * p_cstride, cb, bar);
-            g2s(dst + STRIP * 4, p_x0 + dr * p_xstride, p_xbytes, bar);
-            if (p_avg) g2s(dst + 2 * STRIP * 4, p_xb0 + dr * p_xstride, p_xbytes, bar);
-            if (!init) g2s(dst + 3 * STRIP * 4, p_xa0 + dr * p_xstride, p_xbytes, bar);
+            refs[st].row = p_row;
         }
         ++issued;
+        p_x += p_xstride;
+        p_c += p_cstride;
         if (++p_row >= p_end) next_tile();
     };
     next_tile();
@@ -1040,8 +1029,7 @@ k_kkt_bulk(const Inst* __restrict__ insts, const TileRef* __restrict__ tmap, con
     // ---- consumer ----
     int c_tile = -1, c_local = 0;
     const Inst* CI = nullptr;
-    const TC* c_C = nullptr;
-    long long c_ldc = 0, c_i0 = 0, c_i1 = 0, c_n = 0, c_last_ragged = -1, c_chunk = 0, c_win = -1, j0 = 0;
+    long long c_i0 = 0, c_i1 = 0, c_n = 0, c_chunk = 0, c_win = -1, j0 = 0;
     bool on = false, c_avg = false, valid[4] = {false, false, false, false};
     float qv[4] = {0.f, 0.f, 0.f, 0.f}, qbv[4] = {0.f, 0.f, 0.f, 0.f};
     const double* c_p = nullptr;
@@ -1050,16 +1038,23 @@ k_kkt_bulk(const Inst* __restrict__ insts, const TileRef* __restrict__ tmap, con
     double* c_rowpart2 = nullptr;
     float t[TP], csa[4], csa2[4];
     int rows_in_batch = 0;
+    bool flushed = false;
     auto flush_acc = [&]() {
 #pragma unroll
-        for (int k = 0; k < TP; ++k) { sacc[k * 32 + lane] += (double)t[k]; t[k] = 0.f; }
+        for (int k = 0; k < TP; ++k) {
+            const double v = lagp::widen(t[k]);
+            sacc[k * 32 + lane] = flushed ? sacc[k * 32 + lane] + v : v;
+            t[k] = 0.f;
+        }
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            sacc[(TP + e) * 32 + lane] += (double)csa[e];
-            sacc[(TP + 4 + e) * 32 + lane] += (double)csa2[e];
+            const double v = lagp::widen(csa[e]), v2 = lagp::widen(csa2[e]);
+            sacc[(TP + e) * 32 + lane] = flushed ? sacc[(TP + e) * 32 + lane] + v : v;
+            sacc[(TP + 4 + e) * 32 + lane] = flushed ? sacc[(TP + 4 + e) * 32 + lane] + v2 : v2;
             csa[e] = 0.f;
             csa2[e] = 0.f;
         }
+        flushed = true;
         rows_in_batch = 0;
     };
     auto flush_tile = [&]() {
@@ -1078,6 +1073,7 @@ k_kkt_bulk(const Inst* __restrict__ insts, const TileRef* __restrict__ tmap, con
         }
 #pragma unroll
         for (int k = 0; k < TP; ++k) {
+            if (init ? k > 2 : (!c_avg && (k == 2 || k == 3 || k == 5))) continue;   // not read by the check
             const double a = warp_sum(sacc[k * 32 + lane]);
             if (lane == 0) CI->tpart[(long long)c_local * TP + k] = a;
         }
@@ -1093,14 +1089,10 @@ k_kkt_bulk(const Inst* __restrict__ insts, const TileRef* __restrict__ tmap, con
         c_chunk = tr.local / CI->nstrips;
         const long long c0 = (long long)strip * STRIP;
         c_n = CI->n;
-        c_ldc = CI->ldc;
         c_i0 = c_chunk * CI->tile_rows;
         c_i1 = min(c_i0 + (long long)CI->tile_rows, CI->m);
         j0 = c0 + lane * 4;
         on = j0 < c_n;
-        const long long ncols = min((long long)STRIP, c_n - c0);
-        c_last_ragged = (ncols % CQ) != 0 ? CI->m - 1 : -1;
-        c_C = reinterpret_cast<const TC*>(CI->C) + j0;
         c_avg = !init && Sc.k > 0;
         c_p = slot_v(*CI, Sc.cur);
         c_pb = slot_v(*CI, Sc.bar);
@@ -1115,8 +1107,7 @@ k_kkt_bulk(const Inst* __restrict__ insts, const TileRef* __restrict__ tmap, con
         c_rowpart = CI->rowpart + (long long)strip * CI->m;
         c_rowpart2 = CI->rowpart2 + (long long)strip * CI->m;
         c_win = -1;
-#pragma unroll
-        for (int k = 0; k < KACC; ++k) sacc[k * 32 + lane] = 0.0;
+        flushed = false;
 #pragma unroll
         for (int k = 0; k < TP; ++k) t[k] = 0.f;
 #pragma unroll
@@ -1124,10 +1115,15 @@ k_kkt_bulk(const Inst* __restrict__ insts, const TileRef* __restrict__ tmap, con
         rows_in_batch = 0;
     };
 
-    bool failed = false;
     while (consumed < issued) {
         const int st = (int)(consumed % KS);
-        if (!wait_stage(bars_s + 8 * st, (unsigned)((consumed / KS) & 1))) { failed = true; break; }
+        // The oldest row's copies (wait_group counts the newer ones).
+        const long long newer = issued - consumed - 1;
+        if (newer >= 3) lagp::cp_wait<3>();
+        else if (newer == 2) lagp::cp_wait<2>();
+        else if (newer == 1) lagp::cp_wait<1>();
+        else lagp::cp_wait<0>();
+        __syncwarp();
         const RowRef ref = refs[st];
         if (ref.tile != c_tile) open_consumer(ref.tile);
         const long long i = ref.row;
@@ -1135,19 +1131,15 @@ k_kkt_bulk(const Inst* __restrict__ insts, const TileRef* __restrict__ tmap, con
         const unsigned char* stage = wbase + st * KSTAGE;
         float c[4], x[4], xb[4], xa[4];
         if (on) {
-            if (i != c_last_ragged) {
-                if (sizeof(TC) == 4) {
-                    const float4 v = *reinterpret_cast<const float4*>(stage + lane * 16);
-                    c[0] = v.x; c[1] = v.y; c[2] = v.z; c[3] = v.w;
-                } else {
-                    const uint2 v = *reinterpret_cast<const uint2*>(stage + lane * 8);
-                    c[0] = bf16_bits_to_f32(v.x & 0xffffu);
-                    c[1] = bf16_bits_to_f32(v.x >> 16);
-                    c[2] = bf16_bits_to_f32(v.y & 0xffffu);
-                    c[3] = bf16_bits_to_f32(v.y >> 16);
-                }
+            if (sizeof(TC) == 4) {
+                const float4 v = *reinterpret_cast<const float4*>(stage + lane * 16);
+                c[0] = v.x; c[1] = v.y; c[2] = v.z; c[3] = v.w;
             } else {
-                ldc4_tail<float>(c_C + i * c_ldc, c_n - j0, c);
+                const uint2 v = *reinterpret_cast<const uint2*>(stage + lane * 8);
+                c[0] = bf16_bits_to_f32(v.x & 0xffffu);
+                c[1] = bf16_bits_to_f32(v.x >> 16);
+                c[2] = bf16_bits_to_f32(v.y & 0xffffu);
+                c[3] = bf16_bits_to_f32(v.y >> 16);
             }
             const float4 vx = *reinterpret_cast<const float4*>(stage + STRIP * 4 + lane * 16);
             x[0] = vx.x; x[1] = vx.y; x[2] = vx.z; x[3] = vx.w;
@@ -1209,26 +1201,16 @@ k_kkt_bulk(const Inst* __restrict__ insts, const TileRef* __restrict__ tmap, con
         }
         if (init || c_avg) {
             rs = warp_sum(rs);
-            if (lane == 0) c_rowpart[i] = (double)rs;
+            if (lane == 0) c_rowpart[i] = lagp::widen(rs);
         }
         if (!init) {
             rs2 = warp_sum(rs2);
-            if (lane == 0) c_rowpart2[i] = (double)rs2;
+            if (lane == 0) c_rowpart2[i] = lagp::widen(rs2);
         }
         if (++rows_in_batch == KKT_FLUSH_ROWS) flush_acc();
     }
     pdl_release();
-    if (!failed) {
-        flush_tile();
-    } else if (lane == 0) {
-        const int tt = refs[(int)(consumed % KS)].tile;
-        atomicExch(&insts[tmap[tt].inst].ctrl->status, ST_DEVICE);
-    }
-    while (consumed < issued) {   // drain: wait (bounded) for every copy still in flight
-        const int st = (int)(consumed % KS);
-        wait_stage(bars_s + 8 * st, (unsigned)((consumed / KS) & 1));
-        ++consumed;
-    }
+    flush_tile();
 }
 
 // ---------------------------------------------------------------------------
@@ -1274,7 +1256,9 @@ __device__ __forceinline__ void set_result(Ctrl* S) {
     S->res_avg = 0;
 }
 
-__device__ void finalize_check(Ctrl* S, const double* A, int mode) {
+// pre: the measures of the current point and of the average, where the caller
+// has formed them (kkt_parts of the same sums).
+__device__ void finalize_check(Ctrl* S, const double* A, int mode, const KP* pre = nullptr) {
     if (S->lag && S->npend) {
         // The final pass before this check has applied the pending steps.
         S->h0 = (S->h0 + S->npend) % YRING;
@@ -1294,7 +1278,8 @@ __device__ void finalize_check(Ctrl* S, const double* A, int mode) {
         }
     }
     KP c;
-    kkt_parts(S, A[0], A[7], A[6], A[2], c);
+    if (pre) c = pre[0];
+    else kkt_parts(S, A[0], A[7], A[6], A[2], c);
     S->checks += 1;
     if (mode == MODE_CHECK && S->stop_req) {
         // Stopped by the host (time limit): the current iterate, with the
@@ -1322,7 +1307,8 @@ __device__ void finalize_check(Ctrl* S, const double* A, int mode) {
         return;
     }
     KP b;
-    kkt_parts(S, A[1], A[9], A[8], A[3], b);
+    if (pre) b = pre[1];
+    else kkt_parts(S, A[1], A[9], A[8], A[3], b);
     if (!isfinite(c.kkt) || !isfinite(b.kkt)) {
         report(S, c);
         S->status = ST_NUMERIC;
@@ -1405,45 +1391,24 @@ __device__ void finalize_check(Ctrl* S, const double* A, int mode) {
     S->sigma = S->eta * S->omega;
 }
 
-// Fixed-order sums of entry `idx` over two partial sets at once (A: the
-// average's, or the plan's at the initial check; B: the current plan's):
-// group g (warp g) adds partials g, g + VG, ... of each set, then warp 0
-// combines the VG group sums in order.  One block barrier; the results are
-// valid in warp 0.
-__device__ __forceinline__ void group_sum2(const double* pa, const double* pb, long long stride, int count,
-                                           long long idx, bool active, bool use_a, bool use_b, double* sgrp,
-                                           double& sa, double& sb) {
-    const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
-    double a = 0.0, b = 0.0;
-    if (active) {
-#pragma unroll 4
-        for (int k = grp; k < count; k += VG) {
-            if (use_a) a += pa[(long long)k * stride + idx];
-            if (use_b) b += pb[(long long)k * stride + idx];
-        }
-    }
-    sgrp[grp * 32 + lane] = a;
-    sgrp[(VG + grp) * 32 + lane] = b;
-    __syncthreads();
-    sa = 0.0;
-    sb = 0.0;
-    if (grp == 0) {
-#pragma unroll
-        for (int g2 = 0; g2 < VG; ++g2) {
-            sa += sgrp[g2 * 32 + lane];
-            sb += sgrp[(VG + g2) * 32 + lane];
-        }
-    }
-}
-
 // One vector tile of the check: the exact row / column sums (both partial
-// sets in one phase), then warp 0 alone forms the residual, dual-objective and
-// distance terms, adds the tile partials of the plan pass, reduces the twelve
-// scalars with shuffles and takes the instance's ticket; the last tile runs
-// the restart / termination logic.  FP64 stays on one warp (a narrow pipe on
-// this part) and only one block barrier is on the path.  sgrp: 2 VG x 32
-// doubles.
-__device__ void checkvec_tile(const Inst& I, Ctrl* S, int lvt, int mode, double* sgrp) {
+// sets: A the plan's at the initial check, the average's at a check; B the
+// current plan's, which the passes carry forward by sums of changes between
+// checks), the residual, dual-objective and distance terms, the plan tiles'
+// partials, twelve scalars and the instance's ticket; the last tile runs the
+// restart / termination logic.  Group g (warp g) adds partials g, g + VG, ...
+// of each set, warp 0 combines the groups in order.  FP64 takes 64 cycles per
+// warp instruction on each of an SM's four schedulers, so the sums over the
+// plan tiles, the twelve reductions, the last tile's and the two points'
+// measures are spread over the warps (all on one warp: 24 us at 4096 x 4096; here 18).
+struct CheckShared {
+    double grp[2 * VG * 32];
+    double a[VP][32];
+    double tot[VP];
+    KP kp[2];
+    int last;
+};
+__device__ void checkvec_tile(const Inst& I, Ctrl* S, int lvt, int mode, CheckShared& sh) {
     const long long m = I.m, n = I.n;
     const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
     const long long e = (long long)lvt * VE + lane;
@@ -1451,19 +1416,41 @@ __device__ void checkvec_tile(const Inst& I, Ctrl* S, int lvt, int mode, double*
     const bool avg = !init && S->k > 0;
     const bool row = e < m, col = !row && e < m + n;
     const long long idx = row ? e : e - m;          // i or j
-    double s = 0.0, s2 = 0.0;
-    // A: the plan's sums at the initial check, the average's at a check;
-    // B: the current plan's exact sums (the passes carry them forward by sums
-    // of changes between checks).
-    group_sum2(row ? I.rowpart : I.colpart, row ? I.rowpart2 : I.colpart2, row ? m : I.ldx,
-               row ? I.nstrips : I.nchunks, idx, row || col, init || avg, !init, sgrp, s, s2);
+    {
+        const double* pa = row ? I.rowpart : I.colpart;
+        const double* pb = row ? I.rowpart2 : I.colpart2;
+        const long long stride = row ? m : I.ldx;
+        const int count = row ? I.nstrips : I.nchunks;
+        double a = 0.0, b = 0.0;
+        if (row || col) {
+#pragma unroll 4
+            for (int k = grp; k < count; k += VG) {
+                if (init || avg) a += pa[(long long)k * stride + idx];
+                if (!init) b += pb[(long long)k * stride + idx];
+            }
+        }
+        sh.grp[grp * 32 + lane] = a;
+        sh.grp[(VG + grp) * 32 + lane] = b;
+    }
+    if (grp >= 1 && grp <= TP) {   // the plan tiles' scalars: one per warp
+        const int k = grp - 1;
+        const int t0 = (int)((long long)I.ntiles * lvt / I.nvt), t1 = (int)((long long)I.ntiles * (lvt + 1) / I.nvt);
+        double a = 0.0;
+        for (int t = t0 + lane; t < t1; t += 32) a += I.tpart[(long long)t * TP + k];
+        sh.a[6 + k][lane] = a;
+    }
+    __syncthreads();
     if (grp == 0) {
+        double s = 0.0, s2 = 0.0;
+#pragma unroll
+        for (int g2 = 0; g2 < VG; ++g2) {
+            if (init || avg) s += sh.grp[g2 * 32 + lane];
+            if (!init) s2 += sh.grp[(VG + g2) * 32 + lane];
+        }
         double* Vc = slot_v(I, S->cur);
         double* Vb = slot_v(I, S->bar);
         const double* Va = slot_v(I, S->anc);
-        double a[VP];
-#pragma unroll
-        for (int k = 0; k < VP; ++k) a[k] = 0.0;
+        double a[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
         if (row || col) {
             const long long yo = row ? idx : m + idx;                   // offset of p_i / q_j in a vector set
             const long long so = row ? m + n + idx : 2 * m + n + idx;   // offset of r_i / c_j
@@ -1497,47 +1484,42 @@ __device__ void checkvec_tile(const Inst& I, Ctrl* S, int lvt, int mode, double*
                 }
             }
         }
-        const long long T = I.ntiles;
-        const long long t0 = T * lvt / I.nvt, t1 = T * (lvt + 1) / I.nvt;
-        for (long long t = t0 + lane; t < t1; t += 32) {
 #pragma unroll
-            for (int k = 0; k < TP; ++k) a[6 + k] += I.tpart[t * TP + k];
+        for (int k = 0; k < 6; ++k) sh.a[k][lane] = a[k];
+    }
+    __syncthreads();
+    for (int k = grp; k < VP; k += VG) {
+        const double t = warp_sum(sh.a[k][lane]);
+        if (lane == 0) I.vpart[(long long)lvt * VP + k] = t;
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) sh.last = ticket_arrive(I.ticket) == (unsigned)(I.nvt - 1) ? 1 : 0;
+    __syncthreads();
+    if (sh.last) {
+        for (int k = grp; k < VP; k += VG) {
+            double t = 0.0;
+            for (int v = lane; v < I.nvt; v += 32) t += __ldcg(I.vpart + (long long)v * VP + k);
+            t = warp_sum(t);
+            if (lane == 0) sh.tot[k] = t;
         }
-#pragma unroll
-        for (int k = 0; k < VP; ++k) a[k] = warp_sum(a[k]);
-        unsigned old = 0;
-        if (lane == 0) {
-            double* vp = I.vpart + (long long)lvt * VP;
-#pragma unroll
-            for (int k = 0; k < VP; ++k) vp[k] = a[k];
-            old = ticket_arrive(I.ticket);
+        __syncthreads();
+        if (!init) {
+            if (threadIdx.x == 0) kkt_parts(S, sh.tot[0], sh.tot[7], sh.tot[6], sh.tot[2], sh.kp[0]);
+            if (threadIdx.x == 32) kkt_parts(S, sh.tot[1], sh.tot[9], sh.tot[8], sh.tot[3], sh.kp[1]);
+            __syncthreads();
         }
-        old = __shfl_sync(0xffffffffu, old, 0);
-        __syncwarp();
-        if (old == (unsigned)(I.nvt - 1)) {
-            double b[VP];
-#pragma unroll
-            for (int k = 0; k < VP; ++k) b[k] = 0.0;
-            for (int v = lane; v < I.nvt; v += 32) {
-                const double* vp = I.vpart + (long long)v * VP;
-#pragma unroll
-                for (int k = 0; k < VP; ++k) b[k] += __ldcg(vp + k);
-            }
-#pragma unroll
-            for (int k = 0; k < VP; ++k) b[k] = warp_sum(b[k]);
-            if (lane == 0) {
-                *I.ticket = 0u;
-                finalize_check(S, b, mode);
-            }
+        if (threadIdx.x == 0) {
+            *I.ticket = 0u;
+            finalize_check(S, sh.tot, mode, init ? nullptr : sh.kp);
         }
     }
-    __syncthreads();   // sgrp is reused by the caller's next tile
 }
 
 __global__ void __launch_bounds__(VT) k_checkvec(const Inst* __restrict__ insts, const TileRef* __restrict__ vmap,
                                                  const int* __restrict__ NVp, unsigned* wctr, int mode) {
     // One CTA per vector tile (no work queue): the grid covers the tile count.
-    __shared__ double sgrp[2 * VG * 32];
+    __shared__ CheckShared sh;
     pdl_enter();
     // No work counter of its own, but it still resets the others for the
     // kernels that follow (block 0, before any early exit).
@@ -1548,7 +1530,7 @@ __global__ void __launch_bounds__(VT) k_checkvec(const Inst* __restrict__ insts,
     const Inst& I = insts[tr.inst];
     Ctrl* S = I.ctrl;
     if (S->status != ST_RUNNING) return;
-    checkvec_tile(I, S, tr.local, mode, sgrp);
+    checkvec_tile(I, S, tr.local, mode, sh);
 }
 
 // ---------------------------------------------------------------------------
