@@ -621,39 +621,39 @@ __device__ __forceinline__ void finalize_step(Ctrl* S, double dX2, double dy2, d
 
 // One vector tile (VE = 32 entries of [p; q]) per CTA.  All warps add the
 // FP64 partial sums of the tile's row or column sums (group g: partials g,
-// g + VG, ...); warp 0 combines the groups in order, updates the duals and
-// the averages, reduces the tile's step-size scalars with shuffles and takes
-// the instance's ticket; the last tile of an instance finishes the step.
-// Everything that does not depend on the partial sums is requested before
-// them, and only one block-wide barrier is on the path (FP64 is a narrow pipe
-// on this part: block-wide FP64 reductions cost more than they save).
-__device__ void dual_tile(const Inst& I, Ctrl* S, int lvt, double* sgrp) {
+// g + VG, ...).  FP64 takes 64 cycles per warp instruction on each of an SM's
+// four schedulers, so what follows is spread over four warps: warps 0, 1 and 3
+// combine the groups in order and form the duals and ||dy||^2, dy^T A dx, and
+// the new sums and averages; warp 2 has the tile's slice of ||dX||^2 and warp 4
+// what the controller needs besides the sums.  The instance's last tile (a
+// ticket) adds the tiles' scalars, one per warp, and runs the step controller.
+// (One warp for all of it: 19.0 us a launch with 16 uneven instances, here 16.6.)
+struct DualShared {
+    double grp[VG * 32];
+    double sum[3];
+    double w_next;
+    SchedFactors fac;
+    StepPre pre;
+    int last;
+};
+__device__ void dual_tile(const Inst& I, Ctrl* S, int lvt, DualShared& sh) {
     const long long m = I.m, n = I.n;
     const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
     const long long e = (long long)lvt * VE + lane;
     const bool row = e < m, col = !row && e < m + n;
     const long long idx = row ? e : e - m;
-    const long long yo = row ? idx : m + idx;                   // p_i or q_j
-    const long long so = row ? m + n + idx : 2 * m + n + idx;   // r_i or c_j
-    int status = ST_RUNNING;
-    double sigma = 0.0, b = 0.0, r = 0.0, y = 0.0, ybar = 0.0, wavg = 1.0, w_next = 0.5;
+    const long long so = m + n + e;                             // r_i or c_j
+    const bool upd = grp == 0 || grp == 1 || grp == 3;
+    if (S->status != ST_RUNNING) return;
+    double sigma = 0.0, b = 0.0, r = 0.0, y = 0.0, ybar = 0.0, wavg = 1.0;
     long long k = 0;
     double* Vn = nullptr;
     double* Vbn = nullptr;
     float2* yfn = nullptr;
-    SchedFactors fac = {0.0, 0.0};
-    // The step decision's controller fields, used only by the instance's last
-    // tile (lane 0 of warp 0 copies and later reads them: no barrier needed).
-    __shared__ StepPre s_pre;
-    if (grp == 0) {
-        status = S->status;
-        if (lane == 0) s_pre = step_pre(S);
+    if (upd) {
         sigma = S->sigma;
         k = S->k;
         wavg = S->wavg;
-        w_next = 1.0 / (double)(k + 2);   // used by the instance's last tile, if the step is accepted
-        // requested now, used only by the instance's last tile
-        if (S->adaptive_step) fac = sched_factors(S, S->total);
         const double* Vc = slot_v(I, S->cur);
         const double* Vb = slot_v(I, S->bar);
         Vn = slot_v(I, S->nxt);
@@ -662,80 +662,94 @@ __device__ void dual_tile(const Inst& I, Ctrl* S, int lvt, double* sgrp) {
         if (row || col) {
             b = row ? I.f[idx] : I.g[idx];
             r = Vc[so];
-            y = Vc[yo];
-            if (k != 0) ybar = Vb[yo];
+            y = Vc[e];
+            if (k != 0 && grp == 3) ybar = Vb[e];
         }
     }
     double s = 0.0;
     if (row || col) {
-        const double* part = row ? I.rowpart : I.colpart;
+        const double* part = (row ? I.rowpart : I.colpart) + idx;
         const long long stride = row ? m : I.ldx;
         const int count = row ? I.nstrips : I.nchunks;
-#pragma unroll 8
-        for (int kk = grp; kk < count; kk += VG) s += part[(long long)kk * stride + idx];
-    }
-    // This tile's slice of the plan tiles' ||X+ - X||^2 partials, requested
-    // with the partial sums above (before the barrier, off the serial path).
-    double a2 = 0.0;
-    if (grp == 0) {
-        const long long T = I.ntiles;
-        const long long t0 = T * lvt / I.nvt, t1 = T * (lvt + 1) / I.nvt;
-        for (long long tt = t0 + lane; tt < t1; tt += 32) a2 += I.tpart[tt * TP + 0];
-    }
-    sgrp[grp * 32 + lane] = s;
-    __syncthreads();
-    if (grp == 0 && status == ST_RUNNING) {
-        double t = 0.0;
+#pragma unroll 1
+        for (int kk = grp; kk < count; kk += 8 * VG) {
+            double v[8];
 #pragma unroll
-        for (int g2 = 0; g2 < VG; ++g2) t += sgrp[g2 * 32 + lane];
-        double a0 = 0.0, a1 = 0.0;   // ||dy||^2, dy^T A dx (this tile's slice; a2: ||dX||^2)
-        if (row || col) {
-            // t: this row's or column's sum of X+ - X (the pass sums the change
-            // itself, so the step-size term dy^T A dX below is not a difference
-            // of two nearly equal sums); (2X+ - X) 1 = r + 2t, X+ 1 = r + t.
-            const double w = wavg;
-            const double yn = y + sigma * (b - (r + 2.0 * t));
-            Vn[yo] = yn;
-            if (yfn) {   // the next pass reads the duals as FP32 pairs: split once here, not in every plan tile
-                float2 v;
-                split_dual(yn, v.x, v.y);
-                yfn[e] = v;
-            }
-            Vn[so] = r + t;
-            Vbn[yo] = k == 0 ? yn : ybar + w * (yn - ybar);
-            const double dy = yn - y;
-            a0 = dy * dy;
-            a1 = dy * t;
-        }
-        a0 = warp_sum(a0);
-        a1 = warp_sum(a1);
-        a2 = warp_sum(a2);
-        unsigned old = 0;
-        if (lane == 0) {
-            double* vp = I.vpart + (long long)lvt * VP;
-            vp[0] = a0; vp[1] = a1; vp[2] = a2;
-            old = ticket_arrive(I.ticket);
-        }
-        old = __shfl_sync(0xffffffffu, old, 0);
-        __syncwarp();
-        if (old == (unsigned)(I.nvt - 1)) {
-            double b0 = 0.0, b1 = 0.0, b2 = 0.0;
-            for (int v = lane; v < I.nvt; v += 32) {
-                const double* vp = I.vpart + (long long)v * VP;
-                b0 += __ldcg(vp + 0);
-                b1 += __ldcg(vp + 1);
-                b2 += __ldcg(vp + 2);
-            }
-            b0 = warp_sum(b0);
-            b1 = warp_sum(b1);
-            b2 = warp_sum(b2);
-            if (lane == 0) {
-                *I.ticket = 0u;
-                finalize_step(S, s_pre, b2, b0, b1, fac, w_next);
+            for (int u = 0; u < 8; ++u) v[u] = kk + u * VG < count ? part[(long long)(kk + u * VG) * stride] : 0.0;
+            if (kk == grp) s = v[0];
+            else s += v[0];
+#pragma unroll
+            for (int u = 1; u < 8; ++u) {
+                if (kk + u * VG >= count) break;
+                s += v[u];
             }
         }
     }
-    __syncthreads();   // sgrp is reused by the caller's next tile
+    sh.grp[grp * 32 + lane] = s;
+    double* vp = I.vpart + (long long)lvt * VP;
+    if (grp == 2) {
+        // This tile's slice of the plan tiles' ||X+ - X||^2 partials.
+        const int t0 = (int)((long long)I.ntiles * lvt / I.nvt), t1 = (int)((long long)I.ntiles * (lvt + 1) / I.nvt);
+        double a2 = 0.0;
+        for (int tt = t0 + lane; tt < t1; tt += 32) a2 += I.tpart[(long long)tt * TP];
+        a2 = warp_sum(a2);
+        if (lane == 0) vp[2] = a2;
+    }
+    __syncthreads();
+    if (upd) {
+        double t = sh.grp[lane];
+#pragma unroll
+        for (int g2 = 1; g2 < VG; ++g2) t += sh.grp[g2 * 32 + lane];
+        // t: this row's or column's sum of X+ - X (the pass sums the change
+        // itself, so the step-size term dy^T A dX below is not a difference
+        // of two nearly equal sums); (2X+ - X) 1 = r + 2t, X+ 1 = r + t.
+        const double yn = y + sigma * (b - (r + 2.0 * t));
+        const bool in = row || col;
+        if (grp == 3) {
+            if (in) {
+                Vn[so] = r + t;
+                Vbn[e] = k == 0 ? yn : ybar + wavg * (yn - ybar);
+            }
+        } else {
+            const double dy = yn - y;
+            double a = 0.0;
+            if (in) a = grp == 0 ? dy * dy : dy * t;
+            if (grp == 0 && in) {
+                Vn[e] = yn;
+                if (yfn) {   // the next pass reads the duals as FP32 pairs: split once here, not in every plan tile
+                    float2 v;
+                    split_dual(yn, v.x, v.y);
+                    yfn[e] = v;
+                }
+            }
+            a = warp_sum(a);
+            if (lane == 0) vp[grp] = a;
+        }
+    } else if (threadIdx.x == 4 * 32) {
+        // Used by the instance's last tile.  Only the step decision itself
+        // writes these fields during a dual update.
+        sh.w_next = 1.0 / (double)(S->k + 2);
+        if (S->adaptive_step) sh.fac = sched_factors(S, S->total);
+        sh.pre = step_pre(S);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) sh.last = ticket_arrive(I.ticket) == (unsigned)(I.nvt - 1) ? 1 : 0;
+    __syncthreads();
+    if (!sh.last) return;
+    if (grp < 3) {
+        double t = 0.0;
+        for (int v = lane; v < I.nvt; v += 32) {
+            const double a = __ldcg(I.vpart + (long long)v * VP + grp);
+            t = v == lane ? a : t + a;
+        }
+        t = warp_sum(t);
+        if (lane == 0) sh.sum[grp] = t;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        *I.ticket = 0u;
+        finalize_step(S, sh.pre, sh.sum[2], sh.sum[0], sh.sum[1], sh.fac, sh.w_next);
+    }
 }
 
 __global__ void __launch_bounds__(VT) k_dual(const Inst* __restrict__ insts, const TileRef* __restrict__ vmap,
@@ -743,7 +757,7 @@ __global__ void __launch_bounds__(VT) k_dual(const Inst* __restrict__ insts, con
     // One CTA per vector tile (no work queue): the grid covers the tile count.
     // direct: one instance whose vector tiles are exactly the grid (no map or
     // count to read before the work).
-    __shared__ double sgrp[VG * 32];
+    __shared__ DualShared sh;
     pdl_enter();
     // The next pass may start launching now: it waits for this grid to
     // complete before it reads anything this grid writes, and its CTAs use
@@ -762,9 +776,8 @@ __global__ void __launch_bounds__(VT) k_dual(const Inst* __restrict__ insts, con
         tr = vmap[blockIdx.x];
     }
     const Inst& I = insts[tr.inst];
-    // The instance's status is read inside (warp 0), next to the other
-    // controller fields; a finished instance's tile does nothing.
-    dual_tile(I, I.ctrl, tr.local, sgrp);
+    // (a finished instance's tile does nothing)
+    dual_tile(I, I.ctrl, tr.local, sh);
 }
 
 // ---------------------------------------------------------------------------
