@@ -539,11 +539,20 @@ bool persist_for(pdot_handle* h, long long m, long long n, int ttype, int tile_r
     return ttype != TT_GEN || tile_rows <= persist_rows(h->cfg.comp != 0) || h->cfg.gen_dims <= 4;
 }
 
+// CTAs of an instance that has the device to itself: eight tiles each (one
+// per warp), or as few as four while that needs no second CTA on an SM (64 x
+// 64: 5.7K -> 4.5K cycles per traversal; 300 x 517: 5.4K -> 4.7K.  Two CTAs on
+// an SM take turns at the controller's FP64: 4.5K -> 5.4K cycles at 300 x 517).
+int coop_ctas(pdot_handle* h, long long ntiles) {
+    const long long per = std::min<long long>(TWARPS, std::max<long long>(4, (ntiles + h->sm_count - 1) / h->sm_count));
+    return (int)((ntiles + per - 1) / per);
+}
+
 // `npass` passes and the final write in one launch.
 void run_persist(pdot_handle* h, int ttype, int npass) {
     const Work& w = h->ws;
-    CKL(launch_persist(ttype, h->d_inst, w.ntiles, w.tile_rows <= persist_rows(h->cfg.comp != 0), h->d_gs, h->coop_epoch, npass, h->cfg,
-                       h->stream));
+    CKL(launch_persist(ttype, h->d_inst, nullptr, coop_ctas(h, w.ntiles),
+                       w.tile_rows <= persist_rows(h->cfg.comp != 0), h->d_gs, h->coop_epoch, npass, h->cfg, h->stream));
     h->coop_epoch ^= 1;
     launch_count(h, 1);
 }
@@ -1040,7 +1049,9 @@ double round_plan_dev(pdot_handle* h, long long m, long long n, int xtype, const
 // multi-instance kernels: one chunk = chunk_checks x (K x (pass, dual) +
 // (kkt, checkvec)) plus a controller snapshot copied to pinned host memory,
 // captured once as a CUDA graph (tile maps and counts live in device memory,
-// so a new batch composition only rewrites those buffers).  Between chunks
+// so a new batch composition only rewrites those buffers).  Where the live
+// instances fit a few cooperative launches, a check period's passes are those
+// launches instead (batch_plan_coop).  Between chunks
 // pdot_poll retires finished instances (stream-ordered output copies and
 // frees), admits queued requests while the HBM budget and slot count allow,
 // runs their init checks, and launches the next chunk, which then overlaps
@@ -1101,6 +1112,13 @@ constexpr int CNT_VEC = NTT, CNT_INST = NTT + 1, CNT_INIT = NTT + 2, CNT_INIT_VE
               CNT_RES = 2 * NTT + 3, CNT_WORDS = 2 * NTT + 5, CNT_TIMEOUT = 14, CNT_CANCEL = 15;
 static_assert(CNT_WORDS <= CNT_TIMEOUT, "count words overlap");
 
+// Cooperative launches per check period of a batch, at most.  256 passes of
+// instances of 64 .. 2048 rows and columns, tile kernels -> cooperative: 8 of
+// them (one launch) 10.9 -> 7.0 ms, 16 (two) 17.5 -> 13.7, 48 (four or five)
+// 37.1 -> 34.1, 64 (five) 45.4 -> 43.0.  Beyond, a launch's time is that of its tiles either
+// way, and the tile kernels spread a period's tail over all instances.
+constexpr int COOP_WAVES = 5;
+
 struct BatchEngine {
     std::deque<BSlot*> queue;
     std::vector<BSlot*> live;
@@ -1112,6 +1130,15 @@ struct BatchEngine {
     DevArr<TileRef> vmap;
     DevArr<TileRef> tmap_init[NTT];
     DevArr<TileRef> vmap_init;
+    // The active tile instances' cooperative launches of a check period (empty:
+    // the tile kernels): CTAs [first, first + ctas) of `refs`.
+    struct Coop {
+        int ttype = 0, first = 0, ctas = 0;
+    };
+    std::vector<Coop> coop;
+    DevArr<CtaRef> refs;
+    GridSync* gs = nullptr;   // barrier counters, one per instance of the table
+    size_t gs_cap = 0;
     DevArr<int> rlist[2];     // resident instances with FP32 / BF16 costs (indices into insts)
     int res_grid[2] = {0, 0}; // cluster-count bound of each resident launch (bucketed)
     DevArr<Ctrl> snap[2];     // controller snapshots of the two chunks that can be in flight
@@ -1181,6 +1208,82 @@ void batch_free_slot(pdot_handle* h, BSlot* s) {
 
 // Rebuild the device-side composition: instance table, tile maps per type,
 // vector-tile map, and the init maps of freshly admitted instances.
+// The cooperative launches of a check period, when all active tile instances
+// can take that kernel and fit a few launches: each launch holds whole
+// instances, the largest first, with one CTA per eight tiles.  CTAs that are
+// left over go to the instances with the most vector tiles per CTA.
+void batch_plan_coop(pdot_handle* h, const std::vector<char>& active) {
+    BatchEngine* B = h->batch;
+    B->coop.clear();
+    const int cap = h->cfg.coop_blocks;
+    struct Part {
+        int inst, tiles, ctas, nvt;
+    };
+    struct Wave {
+        int ttype, used;
+        std::vector<Part> parts;
+    };
+    std::vector<Wave> waves;
+    std::vector<int> order;
+    for (int i = 0; i < (int)B->live.size(); ++i)
+        if (active[(size_t)i] && !B->live[(size_t)i]->resident) order.push_back(i);
+    std::stable_sort(order.begin(), order.end(),
+                     [&](int a, int b) { return B->live[(size_t)a]->w.ntiles > B->live[(size_t)b]->w.ntiles; });
+    for (int i : order) {
+        const BSlot* s = B->live[(size_t)i];
+        const int ctas = (int)((s->w.ntiles + TWARPS - 1) / TWARPS);
+        if (s->ttype == TT_F64 || h->cfg_base.pass_bulk == 0 || h->opt.pass_kernel != 0 || h->opt.tile_rows != 0 || ctas > cap ||
+            (s->ttype == TT_GEN && B->gen_dims > 4))
+            return;
+        size_t k = 0;
+        while (k < waves.size() && (waves[k].ttype != s->ttype || waves[k].used + ctas > cap)) ++k;
+        if (k == waves.size()) {
+            if (k == (size_t)COOP_WAVES) return;
+            waves.push_back(Wave{s->ttype, 0, {}});
+        }
+        waves[k].used += ctas;
+        waves[k].parts.push_back(Part{i, (int)s->w.ntiles, ctas, (int)s->w.nvt});
+    }
+    size_t total = 0;
+    for (Wave& w : waves) {
+        while (w.used < cap) {
+            Part* best = nullptr;
+            for (Part& p : w.parts)
+                if (p.ctas < p.nvt && (!best || (long long)p.nvt * best->ctas > (long long)best->nvt * p.ctas)) best = &p;
+            if (!best) break;
+            ++best->ctas;
+            ++w.used;
+        }
+        while (w.used < cap) {   // then to those with the most tiles per CTA
+            Part* best = nullptr;
+            auto per = [](const Part& p) { return (p.tiles + p.ctas - 1) / p.ctas; };
+            int need = 0;
+            for (Part& p : w.parts)
+                if (per(p) > 1 && (!best || per(p) > per(*best))) best = &p;
+            if (best) need = (best->tiles + per(*best) - 2) / (per(*best) - 1) - best->ctas;
+            if (!best || w.used + need > cap) break;
+            best->ctas += need;
+            w.used += need;
+        }
+        total += (size_t)w.used;
+    }
+    B->refs.ensure(std::max<size_t>(total, 1));
+    int at = 0;
+    for (const Wave& w : waves) {
+        B->coop.push_back(BatchEngine::Coop{w.ttype, at, w.used});
+        for (const Part& p : w.parts)
+            for (int c = 0; c < p.ctas; ++c) B->refs.h[at++] = CtaRef{p.inst, c, p.ctas};
+    }
+    if (at) CK(cudaMemcpyAsync(B->refs.d, B->refs.h, sizeof(CtaRef) * (size_t)at, cudaMemcpyHostToDevice, h->stream));
+    if (B->gs_cap < B->insts.cap) {
+        if (B->gs) CK(cudaFree(B->gs));
+        B->gs = nullptr;
+        B->gs_cap = 0;
+        CK(cudaMalloc(&B->gs, sizeof(GridSync) * B->insts.cap));
+        B->gs_cap = B->insts.cap;
+    }
+}
+
 void batch_compose(pdot_handle* h) {
     BatchEngine* B = h->batch;
     const int L = (int)B->live.size();
@@ -1250,6 +1353,7 @@ void batch_compose(pdot_handle* h) {
             if (s->fresh) B->vmap_init.h[ovi++] = TileRef{i, t};
         }
     }
+    batch_plan_coop(h, active);
     const cudaStream_t st = h->stream;
     if (L > 0) CK(cudaMemcpyAsync(B->insts.d, B->insts.h, sizeof(Inst) * (size_t)L, cudaMemcpyHostToDevice, st));
     for (int t = 0; t < NTT; ++t) {
@@ -1314,7 +1418,12 @@ void batch_issue_chunk(pdot_handle* h, int types) {
         launch_count(h, 1);
     }
     for (int c = 0; c < checks; ++c) {
-        for (int s = 0; s < K; ++s) {
+        if (!B->coop.empty()) CK(cudaMemsetAsync(B->gs, 0, sizeof(GridSync) * B->live.size(), st));
+        for (const BatchEngine::Coop& w : B->coop) {
+            CKL(launch_persist(w.ttype, B->insts.d, B->refs.d + w.first, w.ctas, false, B->gs, 0, K, h->cfg, st));
+            launch_count(h, 1);
+        }
+        for (int s = 0; s < K && B->coop.empty(); ++s) {
             for (int t = 0; t < NTT; ++t) {
                 if (!(types & (1 << t))) continue;
                 CKL(launch_pass(t, B->insts.d, B->tmap[t].d, B->cnt.d + t, h->wctr, h->cfg, st));
@@ -1325,7 +1434,7 @@ void batch_issue_chunk(pdot_handle* h, int types) {
         }
         for (int t = 0; t < NTT; ++t) {
             if (!(types & (1 << t))) continue;
-            if (lag_for(h, t)) {
+            if (lag_for(h, t) && B->coop.empty()) {
                 CKL(launch_plan_final(t, B->insts.d, B->tmap[t].d, B->cnt.d + t, h->wctr, h->cfg, st));
                 launch_count(h, 1);
             }
@@ -1358,7 +1467,7 @@ void batch_launch_chunk(pdot_handle* h) {
                                   ((long long)B->res_grid[1] << 40),
                               h->opt.restart_check_every, h->opt.chunk_checks,
                               h->cfg.comp | ((long long)B->nv_grid << 8)};
-    if (!h->opt.use_graph) {
+    if (!h->opt.use_graph || !B->coop.empty()) {   // (few launches: nothing that a graph would save)
         batch_issue_chunk(h, types);
     } else {
         if (!B->graph.exec || memcmp(key, B->graph_key, sizeof(key)) != 0) {
@@ -1650,6 +1759,8 @@ void batch_destroy(pdot_handle* h) {
     }
     B->vmap.release();
     B->vmap_init.release();
+    B->refs.release();
+    if (B->gs) cudaFree(B->gs);
     B->rlist[0].release();
     B->rlist[1].release();
     B->snap[0].release();

@@ -173,8 +173,8 @@ struct Inst {
     int nstrips, nchunks, tile_rows, ntiles, nvt;
 };
 
-// Barrier counters of the cooperative kernel (zeroed once; launches take
-// them in turn and each zeroes the other).
+// Barrier counters of the cooperative kernel, one pair per instance (zeroed
+// once; launches take them in turn and each zeroes the other).
 struct GridSync {
     unsigned int count[2];
 };
@@ -182,6 +182,12 @@ struct GridSync {
 struct TileRef {
     int inst;
     int local;
+};
+
+// A CTA of the cooperative kernel: its instance, its place among the
+// instance's CTAs, and their number.
+struct CtaRef {
+    int inst, cta, count;
 };
 
 // Plan-kernel type combinations (cost dtype / plan dtype).
@@ -257,10 +263,12 @@ int occupancy_vec_blocks_per_sm();
 // the CTAs per SM it can hold, or a positive cudaError_t code.
 int setup_bulk_pass();
 int setup_persist();
-// Passes of a single FP32-plan instance (one tile per warp, all resident) and
-// the final write of its pending steps, in one cooperative launch.
-int launch_persist(int ttype, const Inst* d_insts, int ntiles, bool on_chip, GridSync* gs, int epoch, int npass,
-                   const LaunchCfg& cfg, void* stream);
+// Passes of FP32-plan instances (one tile per warp, all resident) and the
+// final write of their pending steps, in one cooperative launch of `ctas`
+// CTAs.  refs: which instance each CTA serves (null: insts[0]); on_chip: every
+// tile stays in shared memory.
+int launch_persist(int ttype, const Inst* d_insts, const CtaRef* refs, int ctas, bool on_chip, GridSync* gs, int epoch,
+                   int npass, const LaunchCfg& cfg, void* stream);
 // Tallest tile that stays in the cooperative kernel's shared memory.
 int persist_rows(bool comp);
 int setup_kkt_bulk();

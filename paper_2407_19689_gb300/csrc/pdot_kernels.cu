@@ -619,6 +619,48 @@ __device__ __forceinline__ void finalize_step(Ctrl* S, double dX2, double dy2, d
     finalize_step(S, step_pre(S), dX2, dy2, inter, fac, w_next);
 }
 
+// Group sum of FP64 (or FP32) partials k = grp, grp + VG, ... < count in order,
+// at part + k * stride, U of them requested together.  A partial that is zero
+// in all 32 lanes is not added (it changes nothing, and an FP64 addition takes
+// 64 cycles of its scheduler): the plan of a solve is sparse, so most tiles
+// leave most columns as they were.
+__device__ __forceinline__ bool nonzero(double v) {
+    return ((unsigned)__double2hiint(v) << 1 | (unsigned)__double2loint(v)) != 0u;
+}
+__device__ __forceinline__ bool nonzero(float v) { return v != 0.f; }
+__device__ __forceinline__ double as_double(double v) { return v; }
+__device__ __forceinline__ double as_double(float v) { return lagp::widen(v); }
+// (The loads are volatile: the compiler otherwise moves each one behind the
+// test that uses it.)
+__device__ __forceinline__ double ld_part(const double* p, bool in) {
+    double v;
+    asm volatile("{ .reg .pred t; setp.ne.u32 t, %2, 0; mov.b64 %0, 0; @t ld.global.cg.f64 %0, [%1]; }"
+                 : "=d"(v) : "l"(p), "r"((unsigned)in));
+    return v;
+}
+__device__ __forceinline__ float ld_part(const float* p, bool in) {
+    float v;
+    asm volatile("{ .reg .pred t; setp.ne.u32 t, %2, 0; mov.b32 %0, 0; @t ld.global.cg.f32 %0, [%1]; }"
+                 : "=f"(v) : "l"(p), "r"((unsigned)in));
+    return v;
+}
+template <int U, typename T>
+__device__ __forceinline__ double group_sum(const T* part, int stride, int count, int grp, bool active) {
+    double s = 0.0;
+#pragma unroll 1
+    for (int k = grp; k < count; k += U * VG) {
+        T v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) v[u] = ld_part(part + (long long)(k + u * VG) * stride, active && k + u * VG < count);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (k + u * VG >= count) break;
+            if (__any_sync(0xffffffffu, nonzero(v[u]))) s += as_double(v[u]);
+        }
+    }
+    return s;
+}
+
 // One vector tile (VE = 32 entries of [p; q]) per CTA.  All warps add the
 // FP64 partial sums of the tile's row or column sums (group g: partials g,
 // g + VG, ...).  FP64 takes 64 cycles per warp instruction on each of an SM's
@@ -666,24 +708,13 @@ __device__ void dual_tile(const Inst& I, Ctrl* S, int lvt, DualShared& sh) {
             if (k != 0 && grp == 3) ybar = Vb[e];
         }
     }
+    // (a tile can hold the last rows and the first columns: two runs then)
+    const bool any_row = (long long)lvt * VE < m, any_col = (long long)lvt * VE + VE > m;
     double s = 0.0;
-    if (row || col) {
-        const double* part = (row ? I.rowpart : I.colpart) + idx;
-        const long long stride = row ? m : I.ldx;
-        const int count = row ? I.nstrips : I.nchunks;
-#pragma unroll 1
-        for (int kk = grp; kk < count; kk += 8 * VG) {
-            double v[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) v[u] = kk + u * VG < count ? part[(long long)(kk + u * VG) * stride] : 0.0;
-            if (kk == grp) s = v[0];
-            else s += v[0];
-#pragma unroll
-            for (int u = 1; u < 8; ++u) {
-                if (kk + u * VG >= count) break;
-                s += v[u];
-            }
-        }
+    if (any_row) s = group_sum<4>(I.rowpart + idx, (int)m, I.nstrips, grp, row);
+    if (any_col) {
+        const double c = group_sum<8>(I.colpart + idx, (int)I.ldx, I.nchunks, grp, col);
+        if (col) s = c;
     }
     sh.grp[grp * 32 + lane] = s;
     double* vp = I.vpart + (long long)lvt * VP;
@@ -1935,10 +1966,10 @@ int setup_persist() {
 }
 int persist_rows(bool comp) { return (comp ? pers::Lay<true>::NS : pers::Lay<false>::NS) * pers::R; }
 template <typename TC>
-static int launch_pers(const Inst* d_insts, int ntiles, GridSync* gs, int epoch, int npass, const LaunchCfg& cfg,
+static int launch_pers(const Inst* d_insts, const CtaRef* refs, int ctas, GridSync* gs, int epoch, int npass, const LaunchCfg& cfg,
                        cudaStream_t st) {
     cudaLaunchConfig_t c = {};
-    c.gridDim = dim3((unsigned)((ntiles + TWARPS - 1) / TWARPS));
+    c.gridDim = dim3((unsigned)ctas);
     c.blockDim = dim3(TWARPS * 32);
     c.dynamicSmemBytes = cfg.comp ? pers::Lay<true>::CTA : pers::Lay<false>::CTA;
     c.stream = st;
@@ -1948,18 +1979,18 @@ static int launch_pers(const Inst* d_insts, int ntiles, GridSync* gs, int epoch,
     c.attrs = attr;
     c.numAttrs = 1;
     const int ro = cfg.pass_bulk == 1 ? 1 : 0;
-    return err(cfg.comp ? cudaLaunchKernelEx(&c, k_persist<TC, true>, d_insts, gs, epoch, npass, ro)
-                        : cudaLaunchKernelEx(&c, k_persist<TC, false>, d_insts, gs, epoch, npass, ro));
+    return err(cfg.comp ? cudaLaunchKernelEx(&c, k_persist<TC, true>, d_insts, refs, gs, epoch, npass, ro)
+                        : cudaLaunchKernelEx(&c, k_persist<TC, false>, d_insts, refs, gs, epoch, npass, ro));
 }
-int launch_persist(int ttype, const Inst* d_insts, int ntiles, bool on_chip, GridSync* gs, int epoch, int npass,
-                   const LaunchCfg& cfg, void* stream) {
+int launch_persist(int ttype, const Inst* d_insts, const CtaRef* refs, int ctas, bool on_chip, GridSync* gs, int epoch,
+                   int npass, const LaunchCfg& cfg, void* stream) {
     const cudaStream_t st = (cudaStream_t)stream;
-    if (ttype == TT_BF16) return launch_pers<unsigned short>(d_insts, ntiles, gs, epoch, npass, cfg, st);
+    if (ttype == TT_BF16) return launch_pers<unsigned short>(d_insts, refs, ctas, gs, epoch, npass, cfg, st);
     // A generated cost whose tiles stay on the chip is computed once and then
     // served as a stored one.
-    if (ttype == TT_F32 || on_chip) return launch_pers<float>(d_insts, ntiles, gs, epoch, npass, cfg, st);
-    if (cfg.gen_dims <= 2) return launch_pers<GenC<2>>(d_insts, ntiles, gs, epoch, npass, cfg, st);
-    return launch_pers<GenC4>(d_insts, ntiles, gs, epoch, npass, cfg, st);
+    if (ttype == TT_F32 || on_chip) return launch_pers<float>(d_insts, refs, ctas, gs, epoch, npass, cfg, st);
+    if (cfg.gen_dims <= 2) return launch_pers<GenC<2>>(d_insts, refs, ctas, gs, epoch, npass, cfg, st);
+    return launch_pers<GenC4>(d_insts, refs, ctas, gs, epoch, npass, cfg, st);
 }
 
 int occupancy_vec_blocks_per_sm() {

@@ -190,38 +190,10 @@ __device__ __forceinline__ void dual_part(const Inst& I, const Ctrl& S, int lvt,
     const int e = lvt * VE + lane;
     const bool row = e < m, col = !row && e < m + n;
     double s = 0.0;
-    if (row) {
-        const float* part = reinterpret_cast<const float*>(I.rowpart) + e;
-        const int cnt = I.nstrips;
-#pragma unroll 1
-        for (int k = grp; k < cnt; k += 8 * VG) {
-            float v[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) v[u] = k + u * VG < cnt ? __ldcg(part + (long long)(k + u * VG) * m) : 0.f;
-            if (k == grp) s = lagp::widen(v[0]);
-            else s += lagp::widen(v[0]);
-#pragma unroll
-            for (int u = 1; u < 8; ++u) {
-                if (k + u * VG >= cnt) break;
-                s += lagp::widen(v[u]);
-            }
-        }
-    } else if (col) {
-        const double* part = I.colpart + (e - m);
-        const int cnt = I.nchunks;
-#pragma unroll 1
-        for (int k = grp; k < cnt; k += 16 * VG) {
-            double v[16];
-#pragma unroll
-            for (int u = 0; u < 16; ++u) v[u] = k + u * VG < cnt ? __ldcg(part + (long long)(k + u * VG) * I.ldx) : 0.0;
-            if (k == grp) s = v[0];
-            else s += v[0];
-#pragma unroll
-            for (int u = 1; u < 16; ++u) {
-                if (k + u * VG >= cnt) break;
-                s += v[u];
-            }
-        }
+    if (lvt * VE < m) s = group_sum<4>(reinterpret_cast<const float*>(I.rowpart) + e, m, I.nstrips, grp, row);
+    if (lvt * VE + VE > m) {
+        const double c = group_sum<16>(I.colpart + (e - m), (int)I.ldx, I.nchunks, grp, col);
+        if (col) s = c;
     }
     sgrp(grp) = s;
     if (grp == 2) {
@@ -260,12 +232,15 @@ __device__ __forceinline__ void dual_part(const Inst& I, const Ctrl& S, int lvt,
 
 }  // namespace pers
 
-// npass passes of insts[0], then the pending steps applied and written.
+// npass passes of an instance, then the pending steps applied and written.
+// refs: the instance of every CTA and its place among that instance's CTAs
+// (null: all CTAs serve insts[0]).  Instances of one launch only share the
+// launch: each has its own barrier counter.
 // TC float also serves a generated cost whose tiles stay in shared memory
 // (ctype 3: the entries are computed once, when a tile is loaded).
 template <typename TC, bool CP>
 __global__ void __launch_bounds__(TWARPS * 32, 2)
-k_persist(const Inst* __restrict__ insts, GridSync* gs, int epoch, int npass, int roworder) {
+k_persist(const Inst* __restrict__ insts, const CtaRef* __restrict__ refs, GridSync* gs, int epoch, int npass, int roworder) {
     using namespace bulk;
     using namespace pers;
     using pers::pack; using lagp::unpack; using lagp::widen;
@@ -283,22 +258,28 @@ k_persist(const Inst* __restrict__ insts, GridSync* gs, int epoch, int npass, in
     constexpr int NS = L::NS;
     extern __shared__ __align__(128) unsigned char dsm[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const unsigned G = gridDim.x;
+    __shared__ CtaRef me;
+    if (threadIdx.x == 0) me = refs == nullptr ? CtaRef{0, (int)blockIdx.x, (int)gridDim.x} : refs[blockIdx.x];
+    __syncthreads();
+    insts += me.inst;
+    gs += me.inst;
     for (int w = threadIdx.x; w < (int)(sizeof(Inst) / 4); w += blockDim.x)
         reinterpret_cast<int*>(&I)[w] = reinterpret_cast<const int*>(insts)[w];
     __syncthreads();
     for (int w = threadIdx.x; w < (int)(sizeof(Ctrl) / 4); w += blockDim.x)
         reinterpret_cast<int*>(&S)[w] = reinterpret_cast<const int*>(I.ctrl)[w];
-    unsigned* bar_count = &gs->count[epoch & 1];
-    if (blockIdx.x == 0 && threadIdx.x == 0) gs->count[(epoch & 1) ^ 1] = 0u;   // for the next launch
+    __shared__ unsigned* bar_count;
+    if (threadIdx.x == 0) bar_count = &gs->count[epoch & 1];
+    if (me.cta == 0 && threadIdx.x == 0) gs->count[(epoch & 1) ^ 1] = 0u;   // for the next launch
     __syncthreads();
     if (S.status != ST_RUNNING) return;
 
     // ---- this warp's tile ----
     unsigned char* wbase = dsm + warp * L::WARP;
     const unsigned wbase_s = smem_u32(wbase);
-    const int lt = (int)blockIdx.x * TWARPS + warp;
-    const bool active = lt < I.ntiles;
+    const int per_cta = (I.ntiles + me.count - 1) / me.count;   // at most TWARPS
+    const int lt = me.cta * per_cta + warp;
+    const bool active = warp < per_cta && lt < I.ntiles;
     const unsigned strip = (unsigned)lt % (unsigned)I.nstrips, chunk = (unsigned)lt / (unsigned)I.nstrips;
     const int n = (int)I.n, m = (int)I.m;
     const int r0 = (int)chunk * I.tile_rows;
@@ -439,7 +420,7 @@ k_persist(const Inst* __restrict__ insts, GridSync* gs, int epoch, int npass, in
     // to X and D and write both (Dg, Xg: D and the written X at the group's
     // first row); fin: no candidate.
     auto rows = [&](auto rr_c, auto rb_c, auto write_c, auto desc_c, auto mid_c, unsigned sl, int count, bool fin, float* Dg,
-                    float* Xg, float* rs) {
+                    float* Xg, const float4 (&dn)[2], float* rs) {
         constexpr int RR = decltype(rr_c)::value, RB = decltype(rb_c)::value;
         constexpr bool WRITE = decltype(write_c)::value, DESC = decltype(desc_c)::value, MID = decltype(mid_c)::value;
         constexpr int ROW0 = DESC ? R - 1 - RB : RB, DR = DESC ? -1 : 1;   // the stage's rows
@@ -447,11 +428,7 @@ k_persist(const Inst* __restrict__ insts, GridSync* gs, int epoch, int npass, in
         float4 dv[WRITE ? RR : 1];
         if (WRITE) {
 #pragma unroll
-            for (int r = 0; r < RR; ++r) {
-                const int rr = ROW0 + DR * r;
-                dv[WRITE ? r : 0] = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (rr < count && on && !dfirst) dv[WRITE ? r : 0] = __ldcg(reinterpret_cast<const float4*>(Dg + rr * ldx));
-            }
+            for (int r = 0; r < RR; ++r) dv[WRITE ? r : 0] = dn[WRITE ? r : 0];
         }
 #pragma unroll
         for (int r = 0; r < RR; ++r) {
@@ -527,18 +504,44 @@ k_persist(const Inst* __restrict__ insts, GridSync* gs, int epoch, int npass, in
         }
         sum_rows<RR, MID>(d, a, rs + RB, (DESC ? R - count : 0) - RB, (DESC ? R : count) - RB, flush_sums);
     };
-    auto group = [&](auto desc_c, auto mid_c, bool wr, unsigned sl, int count, bool fin, float* Dg, float* Xg, float* rs) {
+    // D of two rows (rb and rb + 1 in the order they are taken in).  A stored
+    // cost's are requested two rows ahead of their use: 4096 x 4096, 55.0K ->
+    // 52.4K cycles per traversal.  A generated cost and the compensated one
+    // have no registers to hold them and load them in place (they spilled, and
+    // a spilled value is read from L2 after a barrier: generated, 4096 x 4096,
+    // 88K -> 92K cycles per pass; compensated, 64 x 64, 18.0K -> 19.7K).
+    constexpr bool AHEAD = !GEN && !CP;
+    auto load_d = [&](const float* Dg, int count, int rb, bool desc, float4 (&d)[2]) {
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const int rr = desc ? R - 1 - rb - r : rb + r;
+            d[r] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (rr < count && on && !dfirst) d[r] = __ldcg(reinterpret_cast<const float4*>(Dg + rr * ldx));
+        }
+    };
+    float4 dn[2];   // (writing passes) D of the next two rows
+    // ncount, Dn: the next group's rows and D (0: none).
+    auto group = [&](auto desc_c, auto mid_c, bool wr, unsigned sl, int count, bool fin, float* Dg, float* Xg, int ncount,
+                     const float* Dn, float* rs) {
         typedef std::integral_constant<int, 0> I0;
         typedef std::integral_constant<int, 2> I2;
         typedef std::integral_constant<int, 4> I4;
+        constexpr bool DESC = decltype(desc_c)::value;
         if (!wr && CP) {   // (the compensated cost's pairs leave registers for two rows at a time)
-            rows(I2(), I0(), std::false_type(), desc_c, mid_c, sl, count, false, nullptr, nullptr, rs);
-            rows(I2(), I2(), std::false_type(), desc_c, mid_c, sl, count, false, nullptr, nullptr, rs);
+            rows(I2(), I0(), std::false_type(), desc_c, mid_c, sl, count, false, nullptr, nullptr, dn, rs);
+            rows(I2(), I2(), std::false_type(), desc_c, mid_c, sl, count, false, nullptr, nullptr, dn, rs);
         } else if (!wr) {
-            rows(I4(), I0(), std::false_type(), desc_c, mid_c, sl, count, false, nullptr, nullptr, rs);
+            rows(I4(), I0(), std::false_type(), desc_c, mid_c, sl, count, false, nullptr, nullptr, dn, rs);
         } else {
-            rows(I2(), I0(), std::true_type(), desc_c, mid_c, sl, count, fin, Dg, Xg, rs);
-            rows(I2(), I2(), std::true_type(), desc_c, mid_c, sl, count, fin, Dg, Xg, rs);
+            if (!AHEAD) load_d(Dg, count, 0, DESC, dn);
+            float4 d[2] = {dn[0], dn[1]};
+            if (AHEAD) load_d(Dg, count, 2, DESC, dn);
+            rows(I2(), I0(), std::true_type(), desc_c, mid_c, sl, count, fin, Dg, Xg, d, rs);
+            if (!AHEAD) load_d(Dg, count, 2, DESC, dn);
+            d[0] = dn[0];
+            d[1] = dn[1];
+            if (AHEAD && ncount > 0) load_d(Dn, ncount, 0, DESC, dn);
+            rows(I2(), I2(), std::true_type(), desc_c, mid_c, sl, count, fin, Dg, Xg, d, rs);
         }
     };
 
@@ -572,6 +575,7 @@ k_persist(const Inst* __restrict__ insts, GridSync* gs, int epoch, int npass, in
         const float2* py = ring >= 0 ? yf0 + ring * yslot + r0 + l_row : nullptr;
         float* rp = rowp + (desc ? R - 1 - (lane >> 3) : lane >> 3);
         unsigned st = (unsigned)g0 % NS;
+        if (AHEAD && wr) load_d(Dt + (long long)(g0 * R) * ldx, min(R, nrows - g0 * R), 0, desc, dn);
 #pragma unroll 1
         for (int t = 0, g = g0; t < NG; ++t, g += dg) {
             const int count = min(R, nrows - g * R);
@@ -590,9 +594,11 @@ k_persist(const Inst* __restrict__ insts, GridSync* gs, int epoch, int npass, in
             const unsigned sl = wbase_s + st * SB + (unsigned)lane * 16u;
             float* Dg = Dt + (long long)(g * R) * ldx;
             float* Xg = Xo + (long long)(g * R) * ldx;
-            if (!desc) group(std::false_type(), std::false_type(), wr, sl, count, fin, Dg, Xg, rsv);
-            else if (!mid) group(std::true_type(), std::false_type(), wr, sl, count, fin, Dg, Xg, rsv);
-            else group(std::true_type(), std::true_type(), wr, sl, count, fin, Dg, Xg, rsv);
+            const int ncount = t + 1 < NG ? min(R, nrows - (g + dg) * R) : 0;
+            const float* Dn = Dg + (long long)(dg * R) * ldx;
+            if (!desc) group(std::false_type(), std::false_type(), wr, sl, count, fin, Dg, Xg, ncount, Dn, rsv);
+            else if (!mid) group(std::true_type(), std::false_type(), wr, sl, count, fin, Dg, Xg, ncount, Dn, rsv);
+            else group(std::true_type(), std::true_type(), wr, sl, count, fin, Dg, Xg, ncount, Dn, rsv);
             __syncwarp();
             if (t + NS < NG) issue(g + NS * dg, st, Xt);   // (the same stage)
             lagp::cp_commit();
@@ -620,7 +626,6 @@ k_persist(const Inst* __restrict__ insts, GridSync* gs, int epoch, int npass, in
         }
     }
     bool ok = true;
-    unsigned target = 0;
     float2 pw = none;
     if (active) {
         const int h = (S.h0 + S.npend) % YRING;
@@ -628,10 +633,9 @@ k_persist(const Inst* __restrict__ insts, GridSync* gs, int epoch, int npass, in
         if (l_slot == LAG) pw = row_dual(h, (S.passes & 1) ? NG - 1 : 0);
     }
     // The CTA's first vector tile: its slice of the plan tiles' ||dX||^2.
-    const int nvt = I.nvt;
-    const int vt0 = (int)blockIdx.x;
-    const int sl0 = vt0 < nvt ? (int)((long long)I.ntiles * vt0 / nvt) : 0;
-    const int sl1 = vt0 < nvt ? (int)((long long)I.ntiles * (vt0 + 1) / nvt) : 0;
+    __shared__ int s_sl[2];
+    const int vt0 = me.cta;
+    if (threadIdx.x < 2 && vt0 < I.nvt) s_sl[threadIdx.x] = (int)((long long)I.ntiles * (vt0 + (int)threadIdx.x) / I.nvt);
     for (int ps = 0; ps < npass; ++ps) {
         if (active) {
             const float t0 = -(float)S.tau;
@@ -649,10 +653,9 @@ k_persist(const Inst* __restrict__ insts, GridSync* gs, int epoch, int npass, in
             if (lane == 0) I.tpart[(long long)lt * TP] = t;
         }
         DualPre d;
-        if (warp < 4 && vt0 < nvt) dual_pre(I, S, vt0, d);   // (arrives during the barrier)
-        target += G;
-        if (!grid_sync(bar_count, target, &s_ok)) { ok = false; break; }
-        if (vt0 < nvt) dual_part(I, S, vt0, d, sl0, sl1, dsm + L::SCR, L::WARP);
+        if (warp < 4 && vt0 < I.nvt) dual_pre(I, S, vt0, d);   // (arrives during the barrier)
+        if (!grid_sync(bar_count, (unsigned)(me.count * (2 * ps + 1)), &s_ok)) { ok = false; break; }
+        if (vt0 < I.nvt) dual_part(I, S, vt0, d, s_sl[0], s_sl[1], dsm + L::SCR, L::WARP);
         if (threadIdx.x == 5 * 32) {
             // What the controller needs besides the sums, by a warp that has
             // done its part of the dual update.
@@ -660,14 +663,13 @@ k_persist(const Inst* __restrict__ insts, GridSync* gs, int epoch, int npass, in
             s_wn = 1.0 / (double)(S.k + 2);
             s_pre = step_pre(&S);
         }
-        for (int vt = vt0 + (int)G; vt < nvt; vt += (int)G) {
+        for (int vt = vt0 + me.count; vt < I.nvt; vt += me.count) {
             __syncthreads();   // the scratch is reused
             if (warp < 4) dual_pre(I, S, vt, d);
-            dual_part(I, S, vt, d, (int)((long long)I.ntiles * vt / nvt), (int)((long long)I.ntiles * (vt + 1) / nvt), dsm + L::SCR,
+            dual_part(I, S, vt, d, (int)((long long)I.ntiles * vt / I.nvt), (int)((long long)I.ntiles * (vt + 1) / I.nvt), dsm + L::SCR,
                       L::WARP);
         }
-        target += G;
-        if (!grid_sync(bar_count, target, &s_ok)) { ok = false; break; }
+        if (!grid_sync(bar_count, (unsigned)(me.count * (2 * ps + 2)), &s_ok)) { ok = false; break; }
         // The step scalars, one warp each; meanwhile all warps request what
         // the next pass starts with, for either decision.
         const int h_old = (S.h0 + S.npend) % YRING, np_old = S.npend;
@@ -675,10 +677,18 @@ k_persist(const Inst* __restrict__ insts, GridSync* gs, int epoch, int npass, in
         const int np_base = wrote ? 0 : np_old, h_base = wrote ? h_old : S.h0;
         const long long total_old = S.total;
         if (warp < 3) {
+            const int nvt = I.nvt;
             double b = 0.0;
-            for (int v = lane; v < nvt; v += 32) {
-                const double t = __ldcg(I.vpart + (long long)v * VP + warp);
-                b = v == lane ? t : b + t;
+#pragma unroll 1
+            for (int v0 = lane; v0 - lane < nvt; v0 += 32 * 8) {
+                double t[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) t[u] = ld_part(I.vpart + (long long)(v0 + 32 * u) * VP + warp, v0 + 32 * u < nvt);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    if (v0 - lane + 32 * u >= nvt) break;
+                    b = v0 == lane && u == 0 ? t[u] : b + t[u];
+                }
             }
             b = warp_sum(b);
             if (lane == 0) s_sum[warp] = b;
@@ -719,7 +729,7 @@ k_persist(const Inst* __restrict__ insts, GridSync* gs, int epoch, int npass, in
     // The pending steps, written.
     if (ok && active && np > 0) traverse(true, pw);
     if (!ok && lane == 0) atomicExch(&I.ctrl->status, ST_DEVICE);   // a barrier gave up
-    if (blockIdx.x != 0) return;
+    if (me.cta != 0) return;
     __syncthreads();
     if (threadIdx.x == 0 && S.npend > 0) {
         S.h0 = (S.h0 + S.npend) % YRING;
