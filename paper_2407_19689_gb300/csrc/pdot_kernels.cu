@@ -1,12 +1,12 @@
 // pdot_kernels.cu -- sm_103a kernels of restarted PDHG for optimal transport
 // (arXiv 2407.19689, Algorithm 2 with the Sec. 5 controller).
 //
-// One iteration = two launches over a multi-instance work queue:
-//   k_pass  (plan tiles, HBM-bound): one read of C, X, Xbar and one write of
-//           X+, Xbar+ per element.  Computes the projected primal step of
-//           Algorithm 2, X+ = max(0, X - tau (C - p 1^T - 1 q^T)), the running
-//           average, and in registers the row sums of X+ (warp shuffles), the
-//           column sums of X+ (per-lane accumulators) and ||X+ - X||^2.
+// One iteration, as two launches over a multi-instance work queue:
+//   plan pass (plan tiles): forms the projected primal step of Algorithm 2,
+//           X+ = max(0, X - tau (C - p 1^T - 1 q^T)), and in registers the row
+//           and column sums of X+ - X and ||X+ - X||^2.  FP32 plans and their
+//           averages are written by every third pass (k_pass_lag,
+//           pdot_pass.cuh), FP64 ones by each (k_pass).
 //   k_dual  (vector tiles, O(m+n)): fixed-order reduction of the partial sums,
 //           the dual updates p+ = p + sigma (f - (2 r+ - r)),
 //           q+ = q + sigma (g - (2 c+ - c)) (r = X 1, c = X^T 1 of the current
@@ -14,6 +14,8 @@
 //           step-size reductions.  The last vector tile of each instance
 //           (atomic ticket) runs the scalar controller: PDLP step-size test,
 //           accept/reject by swapping slot roles.
+// or, where all tiles are resident at once, the passes and dual updates of a
+// check period in one cooperative launch (k_persist, pdot_persist.cuh).
 // Every K passes:
 //   k_kkt      (plan tiles): reads C, X, Xbar, anchor once; <C,X>, <C,Xbar>,
 //              ||[p1^T+1q^T-C]^+||^2 for the current and the average duals,
@@ -644,14 +646,16 @@ __device__ __forceinline__ float ld_part(const float* p, bool in) {
                  : "=f"(v) : "l"(p), "r"((unsigned)in));
     return v;
 }
+// off: added to the group of some lanes (whose groups' indexes are not smaller).
 template <int U, typename T>
-__device__ __forceinline__ double group_sum(const T* part, int stride, int count, int grp, bool active) {
+__device__ __forceinline__ double group_sum(const T* part, int stride, int count, int grp, bool active, int off = 0) {
     double s = 0.0;
 #pragma unroll 1
     for (int k = grp; k < count; k += U * VG) {
         T v[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) v[u] = ld_part(part + (long long)(k + u * VG) * stride, active && k + u * VG < count);
+        for (int u = 0; u < U; ++u)
+            v[u] = ld_part(part + (long long)(k + off + u * VG) * stride, active && k + off + u * VG < count);
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             if (k + u * VG >= count) break;

@@ -21,11 +21,11 @@
 //           the same inputs, so the same decision in every CTA.
 // FP64 is the serial part (64 cycles per warp instruction and scheduler), so
 // conversions are integer operations (widen) and the dual update's FP64 is
-// spread over the CTA's schedulers.  Measured per iteration of a solve
-// (adaptive steps, checks included), before deferred writes and this kernel ->
-// here: 64 x 64 17.2 -> 11.2 us, 300 x 517 19.5 -> 15.5, 1024 x 1024 25.7 ->
-// 17.1, 4096 x 4096 70.5 -> 44.1 (two kernels with deferred writes: 53),
-// 16384 x 16384 873 -> 564 us.
+// spread over the CTA's schedulers.  Measured per iteration of a whole call
+// (its start and end included), before deferred writes and this kernel ->
+// here: constant steps, 64 x 64 15.7 -> 8.8 us, 517 x 301 20.2 -> 12.4,
+// 16384 x 16384 904 -> 592; adaptive steps with their checks, 1024 x 1024 27.3
+// -> 16.0, 4096 x 4096 74.0 -> 43.8 (two kernels with deferred writes: 53).
 // The two barriers are one counter each way (release add, acquire poll), with
 // a poll limit; all CTAs are co-resident (cooperative launch, one tile per
 // warp).  A CTA that gives up sets the counter's fail bit, which every other
@@ -58,6 +58,7 @@ struct Lay {
     static constexpr int CTA = TWARPS * WARP;
 };
 
+constexpr int HALVE_MIN = 32;               // partial sums per column from which a vector tile is halved
 constexpr int SPIN_LIMIT = 1 << 23;          // polls of a barrier before it gives up (seconds)
 
 constexpr unsigned FAIL = 0x40000000u;       // set in a barrier's counter when someone gave up
@@ -163,9 +164,14 @@ __device__ __forceinline__ void sum_rows(const f2 (&d)[RR][2], Sums& a, float* r
 struct DualPre {
     double b, r, y, ybar;
 };
-__device__ __forceinline__ void dual_pre(const Inst& I, const Ctrl& S, int lvt, DualPre& d) {
-    const int lane = threadIdx.x & 31;
-    const long long m = I.m, n = I.n, e = (long long)lvt * VE + lane;
+// A vector tile is updated by one CTA (half < 0), or its entries of even and
+// of odd index by one CTA each (half 0 and 1; lanes 0 .. 15 hold them, and 16 ..
+// 31 the same ones in the sums' upper four groups).
+__device__ __forceinline__ int vec_entry(int lvt, int half, int lane) {
+    return lvt * VE + (half < 0 ? lane : (lane & 15) * 2 + half);
+}
+__device__ __forceinline__ void dual_pre(const Inst& I, const Ctrl& S, int lvt, int half, DualPre& d) {
+    const long long m = I.m, n = I.n, e = vec_entry(lvt, half, threadIdx.x & 31);
     d.b = d.r = d.y = d.ybar = 0.0;
     if (e >= m + n) return;
     const double* Vc = slot_v(I, S.cur);
@@ -176,27 +182,35 @@ __device__ __forceinline__ void dual_pre(const Inst& I, const Ctrl& S, int lvt, 
 }
 
 // dual_tile on the CTA's copy of the controller, with FP32 row partials and
-// no ticket: the tile's scalars go to vpart.  FP64 takes 64 cycles per warp
-// instruction on each scheduler, so what follows the partial sums is spread
-// over four warps (four schedulers): each adds the eight group sums, then
+// no ticket: the tile's scalars go to vpart (an odd half's four words on).
+// FP64 takes 64 cycles per warp instruction on each scheduler, so what
+// follows the partial sums is spread over four warps (four schedulers): each adds the eight group sums, then
 // warp 0 forms the duals and ||dy||^2, warp 1 dy^T A dx, warp 2 the tile's
 // slice of ||dX||^2, warp 3 the new sums and averages.
-__device__ __forceinline__ void dual_part(const Inst& I, const Ctrl& S, int lvt, const DualPre& d, int t0, int t1,
+// A column's partial sums are one per tile of rows, up to 570 in eight groups:
+// two warps per scheduler take turns for 64 cycles each.  Halves of a tile
+// take four warps of full lanes (16 entries x 2 groups), one per scheduler,
+// and the scalars' tree over a tile's 32 lanes ends with even + odd, so its
+// bits are those of a whole tile.
+__device__ __forceinline__ void dual_part(const Inst& I, const Ctrl& S, int lvt, int half, const DualPre& d, int t0, int t1,
                                           unsigned char* scr, int pitch) {
     // scr: 256 bytes per warp, `pitch` bytes apart
-    auto sgrp = [&](int g2) -> double& { return reinterpret_cast<double*>(scr + g2 * pitch)[threadIdx.x & 31]; };
     const int m = (int)I.m, n = (int)I.n;
     const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
-    const int e = lvt * VE + lane;
+    const int off = half < 0 ? 0 : lane >> 4 << 2, at = half < 0 ? lane : lane & 15;
+    auto sgrp = [&](int g2) -> double& { return reinterpret_cast<double*>(scr + g2 * pitch)[at]; };
+    const int e = vec_entry(lvt, half, lane);
     const bool row = e < m, col = !row && e < m + n;
-    double s = 0.0;
-    if (lvt * VE < m) s = group_sum<4>(reinterpret_cast<const float*>(I.rowpart) + e, m, I.nstrips, grp, row);
-    if (lvt * VE + VE > m) {
-        const double c = group_sum<16>(I.colpart + (e - m), (int)I.ldx, I.nchunks, grp, col);
-        if (col) s = c;
+    if (half < 0 || grp < 4) {
+        double s = 0.0;
+        if (lvt * VE < m) s = group_sum<4>(reinterpret_cast<const float*>(I.rowpart) + e, m, I.nstrips, grp, row, off);
+        if (lvt * VE + VE > m) {
+            const double c = group_sum<16>(I.colpart + (e - m), (int)I.ldx, I.nchunks, grp, col, off);
+            if (col) s = c;
+        }
+        sgrp(grp + off) = s;
     }
-    sgrp(grp) = s;
-    if (grp == 2) {
+    if (grp == (half < 0 ? 2 : 4) && half <= 0) {
         double a2 = 0.0;
         for (int tt = t0 + lane; tt < t1; tt += 32) a2 += __ldcg(I.tpart + (long long)tt * TP);
         a2 = warp_sum(a2);
@@ -207,7 +221,7 @@ __device__ __forceinline__ void dual_part(const Inst& I, const Ctrl& S, int lvt,
         double t = sgrp(0);
 #pragma unroll
         for (int g2 = 1; g2 < VG; ++g2) t += sgrp(g2);
-        const bool in = row || col;
+        const bool in = (row || col) && lane == at;
         const double yn = d.y + S.sigma * (d.b - (d.r + 2.0 * t));
         if (grp == 3) {
             if (in) {
@@ -225,7 +239,7 @@ __device__ __forceinline__ void dual_part(const Inst& I, const Ctrl& S, int lvt,
                 I.yf[(long long)((S.h0 + S.npend + 1) % YRING) * I.yslot + e] = v;
             }
             a = warp_sum(a);
-            if (lane == 0) I.vpart[(long long)lvt * VP + grp] = a;
+            if (lane == 0) I.vpart[(long long)lvt * VP + (half > 0 ? 4 : 0) + grp] = a;
         }
     }
 }
@@ -632,9 +646,28 @@ k_persist(const Inst* __restrict__ insts, const CtaRef* __restrict__ refs, GridS
         load_q(h, qc, qcl);
         if (l_slot == LAG) pw = row_dual(h, (S.passes & 1) ? NG - 1 : 0);
     }
-    // The CTA's first vector tile: its slice of the plan tiles' ||dX||^2.
-    __shared__ int s_sl[2];
-    const int vt0 = me.cta;
+    // The CTA's first vector tile (its slice of the plan tiles' ||dX||^2).  Tiles
+    // with column duals are halved where there are CTAs for all halves and the
+    // columns' sums are long enough to pay for the halves' extra additions
+    // (0.5K cycles in every CTA).  The longest vector tile, whole -> halved:
+    // 64 x 64 (32 partial sums per column) 5.2K -> 3.9K cycles, 1024 x 1024
+    // (256) 11.2K -> 8.5K, 1137 x 155 (569) 19.2K -> 14.7K.  Only the
+    // compensated kernels: the plain ones serve plans whose vector tiles fill
+    // the CTAs, and lost 2.7 % at 4096 x 4096 to the spills of the unused code.
+    constexpr bool HALVES = CP;
+    __shared__ int s_sl[2], s_half, s_rows;
+    int vt0 = me.cta;
+    if constexpr (HALVES) {
+        const int nr = (int)(I.m / VE);   // tiles of row duals only
+        const bool halve = I.nchunks >= HALVE_MIN && 2 * I.nvt - nr <= me.count;
+        const bool mine = halve && vt0 >= nr;
+        if (threadIdx.x == 0) {
+            s_rows = halve ? nr : I.nvt;
+            s_half = mine ? (vt0 - nr) & 1 : -1;
+        }
+        if (mine) vt0 = nr + (vt0 - nr) / 2;
+        __syncthreads();
+    }
     if (threadIdx.x < 2 && vt0 < I.nvt) s_sl[threadIdx.x] = (int)((long long)I.ntiles * (vt0 + (int)threadIdx.x) / I.nvt);
     for (int ps = 0; ps < npass; ++ps) {
         if (active) {
@@ -653,9 +686,9 @@ k_persist(const Inst* __restrict__ insts, const CtaRef* __restrict__ refs, GridS
             if (lane == 0) I.tpart[(long long)lt * TP] = t;
         }
         DualPre d;
-        if (warp < 4 && vt0 < I.nvt) dual_pre(I, S, vt0, d);   // (arrives during the barrier)
+        if (warp < 4 && vt0 < I.nvt) dual_pre(I, S, vt0, HALVES ? s_half : -1, d);   // (arrives during the barrier)
         if (!grid_sync(bar_count, (unsigned)(me.count * (2 * ps + 1)), &s_ok)) { ok = false; break; }
-        if (vt0 < I.nvt) dual_part(I, S, vt0, d, s_sl[0], s_sl[1], dsm + L::SCR, L::WARP);
+        if (vt0 < I.nvt) dual_part(I, S, vt0, HALVES ? s_half : -1, d, s_sl[0], s_sl[1], dsm + L::SCR, L::WARP);
         if (threadIdx.x == 5 * 32) {
             // What the controller needs besides the sums, by a warp that has
             // done its part of the dual update.
@@ -663,10 +696,10 @@ k_persist(const Inst* __restrict__ insts, const CtaRef* __restrict__ refs, GridS
             s_wn = 1.0 / (double)(S.k + 2);
             s_pre = step_pre(&S);
         }
-        for (int vt = vt0 + me.count; vt < I.nvt; vt += me.count) {
+        for (int vt = (HALVES ? me.cta : vt0) + me.count; vt < (HALVES ? s_rows : I.nvt); vt += me.count) {
             __syncthreads();   // the scratch is reused
-            if (warp < 4) dual_pre(I, S, vt, d);
-            dual_part(I, S, vt, d, (int)((long long)I.ntiles * vt / I.nvt), (int)((long long)I.ntiles * (vt + 1) / I.nvt), dsm + L::SCR,
+            if (warp < 4) dual_pre(I, S, vt, -1, d);
+            dual_part(I, S, vt, -1, d, (int)((long long)I.ntiles * vt / I.nvt), (int)((long long)I.ntiles * (vt + 1) / I.nvt), dsm + L::SCR,
                       L::WARP);
         }
         if (!grid_sync(bar_count, (unsigned)(me.count * (2 * ps + 2)), &s_ok)) { ok = false; break; }
@@ -684,6 +717,19 @@ k_persist(const Inst* __restrict__ insts, const CtaRef* __restrict__ refs, GridS
                 double t[8];
 #pragma unroll
                 for (int u = 0; u < 8; ++u) t[u] = ld_part(I.vpart + (long long)(v0 + 32 * u) * VP + warp, v0 + 32 * u < nvt);
+                if (HALVES && warp < 2 && s_rows < nvt) {   // halved tiles: even + odd
+                    double o[8];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        const int v = v0 + 32 * u;
+                        o[u] = ld_part(I.vpart + (long long)v * VP + 4 + warp, v >= s_rows && v < nvt);
+                    }
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        if (v0 - lane + 32 * u >= nvt) break;
+                        t[u] += o[u];
+                    }
+                }
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
                     if (v0 - lane + 32 * u >= nvt) break;
