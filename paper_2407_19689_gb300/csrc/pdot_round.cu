@@ -13,7 +13,7 @@
 //   write  the plan, and <C, plan> when a cost is given
 // All scalars stay on the device: the old form copied them to the host and
 // back three times and took the write through 64 blocks (1313 us at 4096 x
-// 4096, FP32; here 64 us; 2 x 67 MB take 20 us).
+// 4096, FP32; here 139 us; 2 x 67 MB take 20 us).
 //
 // FP64 is a narrow pipe on this part (two lanes per cycle and SM: one FP64
 // operation per entry of a 4096 x 4096 plan takes 27 us), so FP32 plans are
@@ -636,8 +636,11 @@ __global__ void __launch_bounds__(RB) k_bound_cols(CA C, const double* __restric
     }
 }
 
-__global__ void __launch_bounds__(RB) k_bound_cols64(StoredCost<double> C, const double* __restrict__ p, long long m,
-                                                     long long n, unsigned long long* qkey) {
+// FP64 differences throughout: FP64 costs, and matrices too small for the
+// screen's second launch to pay.
+template <typename CA>
+__global__ void __launch_bounds__(RB) k_bound_cols64(CA C, const double* __restrict__ p, long long m, long long n,
+                                                     unsigned long long* qkey) {
     const long long j = (long long)blockIdx.x * RB + threadIdx.x;
     if (j >= n) return;
     const long long r0 = m * blockIdx.y / gridDim.y, r1 = m * (blockIdx.y + 1) / gridDim.y;
@@ -688,9 +691,26 @@ __global__ void __launch_bounds__(RB) k_bound_value(const double* __restrict__ f
     if (threadIdx.x == 0) out[0] = s;
 }
 
+// Below 2M entries the bound takes one sweep of FP64 differences: the FP32
+// screen's second launch and its keys' round trip take 15 us of a call, the
+// FP64 pipe less.  Whole calls, screened -> direct: 64 x 64 55.7 -> 38.4 us,
+// 1053 x 439 59.1 -> 43.0, 1000 x 1000 59.6 -> 44.9, 1400 x 1400 59.3 -> 55.7;
+// 2000 x 2000 59.4 -> 69.2.
+constexpr long long BOUND_DIRECT = 1LL << 21;
+
+template <typename CA>
+void launch_bound_cols64(CA C, const double* p, long long m, long long n, unsigned long long* qkey, cudaStream_t st) {
+    const long long parts = 64 < m ? 64 : m;
+    k_bound_cols64<CA><<<dim3((unsigned)((n + RB - 1) / RB), (unsigned)parts), RB, 0, st>>>(C, p, m, n, qkey);
+}
+
 template <typename CA>
 void launch_bound_cols(CA C, bool vec, const double* p, long long m, long long n, unsigned* qmin, unsigned* pmax,
                        unsigned long long* qkey, int sm, cudaStream_t st) {
+    if (m * n < BOUND_DIRECT) {
+        launch_bound_cols64(C, p, m, n, qkey, st);
+        return;
+    }
     // Row groups: four blocks per SM, of at least 16 rows.
     const long long cb = (n + 4 * RB - 1) / (4 * RB);
     long long parts = (4LL * sm + cb - 1) / cb;
@@ -732,9 +752,7 @@ int launch_dual_bound(const void* C, int ctype, long long ldc, const GenSpec* ge
     if (ctype == 3) {
         launch_bound_cols(PointsCost{*gen}, false, p, m, n, qmin, pmax, qkey, sm, st);
     } else if (ctype == 2) {
-        long long parts = 64 < m ? 64 : m;
-        k_bound_cols64<<<dim3((unsigned)((n + RB - 1) / RB), (unsigned)parts), RB, 0, st>>>(
-            StoredCost<double>{(const double*)C, ldc}, p, m, n, qkey);
+        launch_bound_cols64(StoredCost<double>{(const double*)C, ldc}, p, m, n, qkey, st);
     } else if (ctype == 1) {
         launch_bound_cols(StoredCost<Bf16>{(const Bf16*)C, ldc}, a16 && ldc % 4 == 0, p, m, n, qmin, pmax, qkey, sm, st);
     } else {

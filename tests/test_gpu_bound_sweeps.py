@@ -13,7 +13,8 @@ pytestmark = pytest.mark.gpu
 CASES = ["plain", "ties", "near_ties", "large", "beyond_fp32", "tiny", "inf_cost", "minus_inf_cost", "nan_dual"]
 
 
-@pytest.mark.parametrize("m,n,ldc", [(1, 1, 1), (5, 1023, 1023), (70, 1030, 1032), (4097, 6, 8), (300, 257, 301)])
+@pytest.mark.parametrize("m,n,ldc", [(1, 1, 1), (5, 1023, 1023), (70, 1030, 1032), (4097, 6, 8), (300, 257, 301),
+                                     (1100, 2030, 2032), (2101, 1003, 1003)])
 @pytest.mark.parametrize("case", CASES)
 @pytest.mark.parametrize("bf16", [False, True])
 def test_bound_is_exact(m, n, ldc, case, bf16):
