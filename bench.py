@@ -49,7 +49,7 @@ def parse():
                     help="host cores the oracle baseline runs on, one independent copy each (0: all)")
     ap.add_argument("--no-e2e", action="store_true")
     ap.add_argument("--pass-kernel", type=int, default=0,
-                    help="plan-pass kernel (pdot_options.pass_kernel; 0: the autotuner's choice) -- for profiling")
+                    help="plan-pass kernel (pdot_options.pass_kernel; 0: chosen by shape) -- for profiling")
     ap.add_argument("--tile-rows", type=int, default=0, help="rows per plan tile (0: by shape) -- for profiling")
     ap.add_argument("--resident", type=int, default=0, choices=[0, 1],
                     help="grid workload: solve in the resident kernel where the plan fits (pdot_options.resident) "
@@ -193,7 +193,7 @@ def unit_for(grid: int, tol: float) -> str:
 def grid_config(args, world: int = 1) -> dict:
     """The workload description both arms print."""
     m = args.grid * args.grid
-    bpe = {"f32": 20, "bf16": 18, "points": 16}[args.cdtype]
+    bpe = {"f32": 12, "bf16": 10, "points": 8}[args.cdtype]
     return {"workload": f"grid{args.grid}_blobs_sqeuclid (image-like {m}x{m})", "m": m, "n": m,
             "cost_dtype": args.cdtype, "tol": args.tol, "parallelism": f"replicas x{world}",
             "l2": f"working set {m * m * bpe / 1e6:.0f} MB per pass > 126 MB L2; no flush needed"}
@@ -750,7 +750,7 @@ def run_pass_sweep(args):
                 st, ms, b, _ = pdot.pdot_time_pass(s.h, m, n, C.data_ptr(), pdot.F32, n, f.data_ptr(), g.data_ptr(),
                                                    30 if G == 64 else 10)
                 s.close()
-                row = {"m": m, "kernel": {"2": "bulk-group", "1": "bulk-row", "0": "register"}[bulk],
+                row = {"m": m, "kernel": {"2": "deferred, by fours", "1": "deferred, by rows", "0": "register"}[bulk],
                        "tile_rows": tr or "auto",
                        "us": ms * 1e3, "GBps": b / (ms * 1e-3) / 1e9, "frac": b / (ms * 1e-3) / 1e9 / peak}
                 out.append(row)
@@ -761,7 +761,7 @@ def run_pass_sweep(args):
         st, ms, b, var = pdot.pdot_time_pass(s.h, m, n, C.data_ptr(), pdot.F32, n, f.data_ptr(), g.data_ptr(),
                                              30 if G == 64 else 10)
         s.close()
-        row = {"m": m, "kernel": "compensated cost, " + {0: "register", 1: "bulk-row", 2: "bulk-group"}.get(var, "?"),
+        row = {"m": m, "kernel": "compensated cost, " + {0: "register", 1: "deferred, by rows", 2: "deferred, by fours"}.get(var, "?"),
                "tile_rows": "auto", "us": ms * 1e3,
                "GBps": b / (ms * 1e-3) / 1e9, "frac": b / (ms * 1e-3) / 1e9 / peak}
         out.append(row)
@@ -778,7 +778,7 @@ def run_pass_sweep(args):
         st, ms, b, var = pdot.pdot_time_pass(s.h, m, n, ctypes.addressof(cost), pdot.POINTS, 0, f.data_ptr(),
                                              g.data_ptr(), 30 if G == 64 else 10)
         s.close()
-        row = {"m": m, "kernel": "generated cost, " + {0: "register", 1: "bulk-row", 2: "bulk-group"}.get(var, "?"),
+        row = {"m": m, "kernel": "generated cost, " + {0: "register", 1: "deferred, by rows", 2: "deferred, by fours"}.get(var, "?"),
                "tile_rows": "auto", "us": ms * 1e3,
                "GBps": b / (ms * 1e-3) / 1e9, "frac": b / (ms * 1e-3) / 1e9 / peak}
         out.append(row)

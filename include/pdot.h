@@ -121,16 +121,17 @@ typedef struct {
                                       admission order whose per-pass plan bytes still fit this budget
                                       (large solves keep the bandwidth; small ones fill in beside them) */
     int32_t pass_kernel;           /* plan-pass kernel of single-instance calls with FP32 plans (pdot_solve,
-                                      pdot_pdhg_steps, pdot_time_pass): 0 = the autotuner's choice (default),
-                                      1 = register pipeline, 2 = bulk copies per row, 3 = bulk copies per
-                                      4-row group (generated costs with d > 4 take 2 instead).  FP64 plans
+                                      pdot_pdhg_steps, pdot_time_pass): 0 = chosen by shape (default),
+                                      1 = register pipeline, 2 / 3 = deferred plan writes, the columns' FP32
+                                      sums taken row by row / in groups of four rows (generated costs with
+                                      d > 4 take 2 instead).  FP64 plans
                                       always take the register pipeline.  Other values: PDOT_ERR_ARG */
     int32_t compensated_cost;      /* FP32 plans (reading C9): 1 = the reduced cost C - p - q is formed
                                       from the FP64 duals split into FP32 hi/lo pairs, with the rounding
                                       error of C - p_hi recovered exactly (TwoSum), so its error is
                                       relative to itself rather than to p and q (far fewer passes where
-                                      FP32 rounding would stall the solve; about 6 % more time per pass
-                                      at 4096^2, 1 % at 16384^2, none where a pass is latency-bound);
+                                      FP32 rounding would stall the solve; about 23 % more time per pass
+                                      at 4096^2, 17 % at 16384^2, little where a pass is latency-bound);
                                       0 = (C - (float)p) - (float)q; 2 (default) = 1 for instances of
                                       fewer than 4M plan entries and in the batch engine, 0 above.
                                       No effect on FP64 plans.  Other values: PDOT_ERR_ARG */
@@ -240,8 +241,8 @@ pdot_status pdot_solve(pdot_handle *h, int64_t m, int64_t n, const void *C, pdot
  *       weight and every counter.  A solve split at a stop by max_iter or
  *       time_limit_s and resumed this way takes the same passes and returns
  *       the same result, bit for bit, as the uninterrupted solve on a handle
- *       that picks the same pass kernel and tile height (the autotuner's
- *       choice is cached per handle; pass_kernel and tile_rows fix it).
+ *       with the same pass kernel and tile height (pass_kernel and tile_rows;
+ *       by default a function of the shape and the cost type).
  *       max_iter counts passes from the original start.  Overrides X0/p0/q0.
  *       A blob of another shape or type, or not written by this library:
  *       PDOT_ERR_ARG.
@@ -285,7 +286,7 @@ pdot_status pdot_solve_host(pdot_handle *h, int64_t m, int64_t n, const void *C,
  * device state (X, p, q) and overwriting it with (X^k, p^k, q^k).  The uniform
  * running averages (Xbar, pbar, qbar) of Algorithm 2 are written when the
  * pointers are non-null.  k >= 0.  The plan pass is the kernel pdot_solve runs
- * for the same shape and cost type (the autotuner's choice, or the handle's
+ * for the same shape and cost type (chosen by shape, or the handle's
  * pass_kernel option), with the same tile height.
  */
 pdot_status pdot_pdhg_steps(pdot_handle *h, int64_t m, int64_t n, const void *C, pdot_dtype c_dtype, int64_t ldc,
@@ -381,17 +382,18 @@ int64_t pdot_launch_count(pdot_handle *h);
  * passes of a solve do; the dual update is left out, so every launch moves
  * the same bytes).  *ms_per_pass receives the mean device time of one pass;
  * *bytes_per_pass (nullable) the algorithmic bytes one pass moves:
- * m n (sizeof C + 4 sizeof X) (read C, X, Xbar; write X+, Xbar+; sizeof C
- * is 0 for a generated cost);
+ * m n (sizeof C + 2 sizeof X) with deferred plan writes (read C and X; every
+ * third pass also reads Xbar and writes X+ and Xbar+), m n (sizeof C + 4
+ * sizeof X) with the register pipeline; sizeof C is 0 for a generated cost;
  * *kernel_variant (nullable) the pass kernel used for this shape: 0 register
- * pipeline, 1 bulk copies per row, 2 bulk copies per 4-row group (FP64 plans
- * always 0). */
+ * pipeline, 1 deferred writes with row-by-row sums, 2 with sums by four rows
+ * (FP64 plans always 0). */
 pdot_status pdot_time_pass(pdot_handle *h, int64_t m, int64_t n, const void *C, pdot_dtype c_dtype, int64_t ldc,
                            const double *f, const double *g, int reps, double *ms_per_pass, double *bytes_per_pass,
                            int32_t *kernel_variant);
 
 /*
- * Self-test of the failure path of the bulk-copy pass kernels: on `device`,
+ * Self-test of the failure path of the shared-memory waits: on `device`,
  * one warp waits, with their bounded wait, for a transfer that is announced on
  * a shared-memory barrier but never issued.  The wait gives up after `polls`
  * polls (1 .. 2^24) and *device_status (host memory) receives the status a

@@ -252,7 +252,7 @@ struct pdot_handle {
     int* h_status = nullptr;     // pinned [2]
     Graph chunk;                 // K x (pass, dual) + (kkt, checkvec)
     long long chunk_key[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    int autotune = 1;            // pass kernel and tile height by shape (0: the handle's fixed kernel)
+    int autotune = 1;            // order of the pass's sums and tile height by shape (0: the handle's fixed choice)
     int batch_min_rows = 16;     // smallest tile height of a batched instance (even)
     int res_clusters = 0;        // resident-kernel clusters the device holds at once (0: not available)
     GridSync* d_gs = nullptr;    // barrier counters of the cooperative kernel
@@ -358,7 +358,7 @@ void validate_marginals(pdot_handle* h, long long m, long long n, const double* 
 }
 
 // Rows per plan tile.  `kernel`: the FP32-plan pass kernel the tiles are for
-// (0 register, 1 bulk per row, 2 bulk per 4-row group).
+// (0 register, 1 / 2 deferred writes with sums by rows / by four rows).
 // split: for the grouped kernel too, one tile per resident warp instead of
 // 32-row tiles through the queue.
 int tile_rows_for(pdot_handle* h, long long m, long long n, int ttype, int kernel, bool batch, bool split = false) {
@@ -706,9 +706,9 @@ double round_plan_dev(pdot_handle* h, long long m, long long n, int xtype, const
                       const GenSpec* gen);
 
 // Compensated reduced cost (option compensated_cost; reading C9): 2 = on
-// where a pass is latency-bound (fewer than 4M plan entries, the autotuner's
-// threshold too), where it costs nothing, and off above, where it costs about
-// 6 % per pass at 4096^2.  The batch engine (many small instances) takes it
+// where a pass is latency-bound (fewer than 4M plan entries), where it costs
+// little, and off above (42.7 -> 52.7 us per pass at 4096^2, 615 -> 718 at
+// 16384^2).  The batch engine (many small instances) takes it
 // unless it is switched off.
 bool compensation_for(pdot_handle* h, long long m, long long n) {
     const int c = h->opt.compensated_cost;
@@ -1897,7 +1897,7 @@ pdot_status pdot_create(const pdot_options* opt, int device, void* cuda_stream, 
             const int v = atoi(pb);
             if (v >= 0 && v <= 2) {
                 h->cfg.pass_bulk = v;
-                h->autotune = 0;   // an explicit kernel choice disables the tuner
+                h->autotune = 0;   // an explicit choice replaces the rule
             }
         }
         const char* bm = getenv("PDOT_BATCH_MIN_ROWS");   // comparison runs only

@@ -319,8 +319,8 @@ def kernel_name(variant: int, c_dtype: int) -> str:
     if variant == 0:
         return f"k_pass<{tc}, ...> (register pipeline)"
     if variant == 1:
-        return f"k_pass_bulk<{tc}, 8> (bulk copies per row)"
-    return f"k_pass_group<{tc}, 2> (bulk copies per 4-row group)"
+        return f"k_pass_lag<{tc}> (deferred plan writes, rows in order)"
+    return f"k_pass_lag<{tc}> (deferred plan writes, rows by fours)"
 
 
 def pdot_watchdog_selftest(device: int = 0, polls: int = 4096):
