@@ -22,8 +22,12 @@
 // at the end of a lane's run.  Scales are kept as FP32 pairs too (48 bits).
 // The sums' error (about 1e-13) stays far below the FP32 rounding of the
 // written entries; measured against 64 bits the plan's error is unchanged
-// (2.5e-8).  Sums of 1e30 and more, or not finite, switch the sweeps to FP64
-// arithmetic, so no range is lost.  FP64 plans use FP64 throughout.
+// (2.5e-8).  Where FP32's range would not hold a sum or a scale, the sweeps
+// that follow take FP64 arithmetic and the FP64 scales, which are kept beside
+// the pairs: row sums of 1e30 and more or not finite, and scales below RTINY
+// that are multiplied by more than 1 (a pair's absolute error is 2^-150, so a
+// product with at most 1 is as exact as an FP32 entry can be).  FP64 plans use
+// FP64 throughout.
 #include <cuda_runtime.h>
 #include <math_constants.h>
 
@@ -41,9 +45,18 @@ constexpr int RPARTS = 64;        // most row groups of the column sums
 constexpr int RU = 4;             // rows a thread of the write has in flight
 constexpr int RROWS = 64;         // rows whose scales a block of the write holds at a time
 constexpr double RWIDE = 1e30;    // row sums from here on: FP64 arithmetic
+constexpr double RTINY = 0x1p-100;   // scales below: an FP32 pair has lost bits (its low part is subnormal from 2^-102 on)
 
-// A scale as the sweeps use it: an FP32 pair for FP32 plans (FP64 bits in the
-// same eight bytes where the plan's sums need FP64 arithmetic), FP64 otherwise.
+// Words of RoundScratch::state: the ticket; FP32's range does not hold a row
+// sum or scale (from the first sweep), a column's or the error's scale (from
+// the sweeps behind the column sums); a column's error exceeds 1.
+constexpr int RS_TICKET = 0, RS_WIDE = 1, RS_LATE = 2, RS_ERR = 3, RS_WORDS = 4;
+
+// v >= 1 (or not a number), in integer arithmetic: an FP64 comparison takes the
+// FP64 pipe.
+__device__ __forceinline__ bool from_one(double v) { return __double2hiint(v) >= 0x3ff00000; }
+
+// A scale as the sweeps use it: an FP32 pair for FP32 plans, FP64 otherwise.
 template <typename T>
 struct __align__(8) Scale {
     float h, l;
@@ -51,20 +64,11 @@ struct __align__(8) Scale {
         h = (float)v;
         l = (float)(v - (double)h);
     }
-    __device__ __forceinline__ void set(double v, bool wide) {
-        set(v);
-        if (wide) {
-            h = __int_as_float(__double2hiint(v));
-            l = __int_as_float(__double2loint(v));
-        }
-    }
-    __device__ __forceinline__ double wide() const { return __hiloint2double(__float_as_int(h), __float_as_int(l)); }
 };
 template <>
 struct Scale<double> {
     double v;
-    __device__ __forceinline__ void set(double w, bool = false) { v = w; }
-    __device__ __forceinline__ double wide() const { return v; }
+    __device__ __forceinline__ void set(double w) { v = w; }
 };
 
 // Running sum: FP32 pair (value plus the additions' errors) or FP64.
@@ -152,8 +156,8 @@ __device__ __forceinline__ void load4(const T* p, long long cnt, T (&v)[4]) {
 template <typename T, bool VEC, int WPR, int RPW, bool WEIGHTED>
 __global__ void __launch_bounds__(RB) k_round_rows(const T* __restrict__ X, long long m, long long n, long long ldx,
                                                    const double* __restrict__ f, const Scale<T>* __restrict__ ys,
-                                                   const double* __restrict__ xs, double* out, double* inv_l1,
-                                                   unsigned* state) {
+                                                   const double* __restrict__ yd, const double* __restrict__ xs, double* out,
+                                                   double* inv_l1, unsigned* state) {
     constexpr int RPB = (RB / 32) / WPR * RPW;
     constexpr bool V4 = VEC && !WEIGHTED;
     __shared__ Acc<T> part[RB / 32][RPW];
@@ -161,7 +165,7 @@ __global__ void __launch_bounds__(RB) k_round_rows(const T* __restrict__ X, long
     __shared__ unsigned last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long i0 = (long long)blockIdx.x * RPB + warp / WPR * RPW;
-    const bool wide = sizeof(T) == 4 && WEIGHTED && state[1] != 0u;
+    const bool wide = sizeof(T) == 4 && WEIGHTED && (state[RS_WIDE] | state[RS_LATE]) != 0u;
     const int w0 = (warp % WPR) * 128, step = 128 * WPR;
     Acc<T> a[RPW][2];
     const T* row[RPW];
@@ -235,14 +239,14 @@ __global__ void __launch_bounds__(RB) k_round_rows(const T* __restrict__ X, long
             double sum = 0.0;
             if (big) {
                 for (long long j = lane; j < n; j += 32)
-                    sum += WEIGHTED ? (double)X[i * ldx + j] * ys[j].wide() : (double)X[i * ldx + j];
+                    sum += WEIGHTED ? (double)X[i * ldx + j] * yd[j] : (double)X[i * ldx + j];
                 sum = warp_add(sum);
             }
             if (lane == 0) {
                 if (!big) sum = a[u][0].get();
                 if (!WEIGHTED) {
                     out[i] = sum;
-                    if (big) atomicOr(state + 1, 1u);
+                    if (big || (sizeof(T) == 4 && from_one(sum) && f[i] > 0.0 && f[i] < RTINY * sum)) atomicOr(state + RS_WIDE, 1u);
                 } else {
                     out[i] = f[i] - xs[i] * sum;
                 }
@@ -253,7 +257,7 @@ __global__ void __launch_bounds__(RB) k_round_rows(const T* __restrict__ X, long
     // The last block adds |err_r| (each thread a strided run, then in order).
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(state, 1u) == gridDim.x - 1 ? 1u : 0u;
+    if (threadIdx.x == 0) last = atomicAdd(state + RS_TICKET, 1u) == gridDim.x - 1 ? 1u : 0u;
     __syncthreads();
     if (!last) return;
     __threadfence();
@@ -266,11 +270,20 @@ __global__ void __launch_bounds__(RB) k_round_rows(const T* __restrict__ X, long
         l1 = 0.0;
         for (int w = 0; w < RB / 32; ++w) l1 += red[w];
         *inv_l1 = l1 > 0.0 ? 1.0 / l1 : 0.0;
+        red[0] = l1;
     }
+    if (sizeof(T) == 8 || state[RS_ERR] == 0u) return;
+    __syncthreads();
+    bool tiny = false;   // the scales |err_r| / ||err_r||_1 of the error term
+    for (long long r = threadIdx.x; r < m; r += RB) {
+        const double e = fabs(__ldcg(out + r));
+        tiny |= e > 0.0 && e < RTINY * red[0];
+    }
+    if (tiny) atomicOr(state + RS_LATE, 1u);
 }
 
-// The sweeps' FP64 forms for FP32 plans whose sums leave FP32's range, out of
-// line: they would only take registers from the others.
+// The sweeps' FP64 forms for FP32 plans whose sums or scales leave FP32's
+// range, out of line: they would only take registers from the others.
 template <typename T>
 __device__ __noinline__ void cols_wide(const T* X, long long r0, long long r1, long long ldx, const double* f,
                                        const double* r_sum, long long n, long long j, long long es, double* part) {
@@ -294,7 +307,7 @@ __global__ void __launch_bounds__(RB) k_round_cols(const T* __restrict__ X, long
     constexpr long long ES = VEC ? 1 : RB;   // distance of a thread's columns
     const int grp = blockIdx.y;
     const long long r0 = m * grp / parts, r1 = m * (grp + 1) / parts;
-    const bool wide = sizeof(T) == 4 && state[1] != 0u;
+    const bool wide = sizeof(T) == 4 && state[RS_WIDE] != 0u;
     __shared__ Scale<T> sx[64];
     if (wide && j < n) cols_wide(X, r0, r1, ldx, f, r_sum, n, j, ES, reinterpret_cast<double*>(colpart) + (long long)grp * n);
     Acc<T> a[4];
@@ -332,11 +345,12 @@ __global__ void __launch_bounds__(RB) k_round_cols(const T* __restrict__ X, long
         if (j + e * ES < n) colpart[(long long)grp * n + j + e * ES] = a[e];
 }
 
-// c_j = the groups' sums -> y_j, err_c.
+// c_j = the groups' sums -> y_j, err_c (FP32 plans: in FP64 too).  Bound by the
+// groups' loads: sixteen of them are requested before any is added.
 template <typename T>
-__global__ void k_round_colscale(const Acc<T>* __restrict__ colpart, int parts, long long n, const double* __restrict__ g,
-                                 Scale<T>* ys, Scale<T>* ec, const unsigned* __restrict__ state) {
-    const bool wide = sizeof(T) == 4 && state[1] != 0u;
+__global__ void __launch_bounds__(64) k_round_colscale(const Acc<T>* __restrict__ colpart, int parts, long long n, const double* __restrict__ g,
+                                 Scale<T>* ys, Scale<T>* ec, double* yd, double* ed, unsigned* state) {
+    const bool wide = sizeof(T) == 4 && state[RS_WIDE] != 0u;
     const long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= n) return;
     double c = 0.0;
@@ -344,13 +358,27 @@ __global__ void k_round_colscale(const Acc<T>* __restrict__ colpart, int parts, 
         for (int k = 0; k < parts; ++k) c += *reinterpret_cast<const double*>(colpart + (long long)k * n + j);
     } else {
         Acc<T> a;
-#pragma unroll 16
-        for (int k = 0; k < parts; ++k) a.merge(colpart[(long long)k * n + j]);
+        for (int k = 0; k < parts; k += 16) {
+            Acc<T> v[16];
+#pragma unroll
+            for (int u = 0; u < 16; ++u)
+                if (k + u < parts) v[u] = colpart[(long long)(k + u) * n + j];
+#pragma unroll
+            for (int u = 0; u < 16; ++u)
+                if (k + u < parts) a.merge(v[u]);
+        }
         c = a.get();
     }
     const double y = c > 0.0 ? fmin(g[j] / c, 1.0) : 1.0;
-    ys[j].set(y, wide);
-    ec[j].set(g[j] - y * c, wide);
+    const double e = g[j] - y * c;
+    ys[j].set(y);
+    ec[j].set(e);
+    if (sizeof(T) == 4) {
+        yd[j] = y;
+        ed[j] = e;
+        if (from_one(c) && y > 0.0 && y < RTINY) atomicOr(state + RS_LATE, 1u);
+        if (from_one(e)) atomicOr(state + RS_ERR, 1u);
+    }
 }
 
 struct Bf16 {
@@ -397,14 +425,14 @@ __device__ __forceinline__ double rounded(double v, const Scale<double>& x, cons
 
 template <typename T, typename CA>
 __device__ __noinline__ double write_wide(const T* X, long long r0, long long r1, long long ldx, const double* xs,
-                                          const Scale<T>* ys, const double* er, const Scale<T>* ec, double inv, T* out,
+                                          const double* yd, const double* er, const double* ed, double inv, T* out,
                                           long long ldo, const CA& C, long long n, long long j, long long es) {
     double obj = 0.0;
     for (long long i = r0; i < r1; ++i) {
         for (int e = 0; e < 4; ++e) {
             const long long c = j + e * es;
             if (c >= n) break;
-            const T w = (T)((double)X[i * ldx + c] * xs[i] * ys[c].wide() + er[i] * ec[c].wide() * inv);
+            const T w = (T)((double)X[i * ldx + c] * xs[i] * yd[c] + er[i] * ed[c] * inv);
             out[i * ldo + c] = w;
             if (C.on()) obj += C(i, c) * (double)w;
         }
@@ -416,6 +444,7 @@ template <typename T, bool VEC, typename CA>
 __global__ void __launch_bounds__(RB) k_round_write(const T* X, long long m, long long n, long long ldx,
                                                     const double* __restrict__ xs, const Scale<T>* __restrict__ ys,
                                                     const double* __restrict__ er, const Scale<T>* __restrict__ ec,
+                                                    const double* __restrict__ yd, const double* __restrict__ ed,
                                                     const double* __restrict__ inv_l1, T* out, long long ldo, CA C,
                                                     double* objpart, const unsigned* __restrict__ state) {
     __shared__ double red[RB / 32];
@@ -425,10 +454,10 @@ __global__ void __launch_bounds__(RB) k_round_write(const T* X, long long m, lon
     const int grp = blockIdx.y, parts = gridDim.y;
     const long long r0 = m * grp / parts, r1 = m * (grp + 1) / parts;
     const double inv = *inv_l1;
-    const bool wide = sizeof(T) == 4 && state[1] != 0u;
+    const bool wide = sizeof(T) == 4 && (state[RS_WIDE] | state[RS_LATE]) != 0u;
     double obj = 0.0;
     if (wide) {
-        if (j < n) obj = write_wide(X, r0, r1, ldx, xs, ys, er, ec, inv, out, ldo, C, n, j, ES);
+        if (j < n) obj = write_wide(X, r0, r1, ldx, xs, yd, er, ed, inv, out, ldo, C, n, j, ES);
     } else {
         auto load = [&](long long i, T (&v)[4]) {
             const T* row = X + i * ldx + j;
@@ -769,8 +798,8 @@ namespace {
 
 // Scratch of a rounding, in doubles (scales take one each).
 struct RoundScratch {
-    double *rs, *xs, *er, *ys, *ec, *colpart, *inv, *obj;
-    unsigned* state;   // ticket; 1: a row sum needs FP64 arithmetic
+    double *rs, *xs, *er, *ys, *ec, *yd, *ed, *colpart, *inv, *obj;   // yd, ed: ys and ec in FP64
+    unsigned* state;
     long long words;
 };
 int round_parts(long long m, long long n, int sm) {
@@ -791,11 +820,13 @@ RoundScratch round_scratch(double* base, long long m, long long n, int sm) {
     r.er = r.xs + m;
     r.ys = r.er + m;
     r.ec = r.ys + n;
-    r.colpart = r.ec + n;
+    r.yd = r.ec + n;
+    r.ed = r.yd + n;
+    r.colpart = r.ed + n;
     r.inv = r.colpart + (long long)cparts * n;
     r.state = reinterpret_cast<unsigned*>(r.inv + 1);
-    r.obj = r.inv + 2;
-    r.words = 3 * m + (2 + (long long)cparts) * n + 2 + cb * parts;
+    r.obj = r.inv + 1 + (RS_WORDS + 1) / 2;
+    r.words = 3 * m + (4 + (long long)cparts) * n + 1 + (RS_WORDS + 1) / 2 + cb * parts;
     return r;
 }
 
@@ -807,7 +838,7 @@ int run_round(const T* X, long long m, long long n, long long ldx, const double*
     Scale<T>* ec = reinterpret_cast<Scale<T>*>(w.ec);
     const int parts = round_parts(m, n, sm), cparts = parts < RPARTS ? parts : RPARTS;
     const unsigned cb = (unsigned)((n + 4 * RB - 1) / (4 * RB));
-    const cudaError_t e = cudaMemsetAsync(w.state, 0, 2 * sizeof(unsigned), st);
+    const cudaError_t e = cudaMemsetAsync(w.state, 0, RS_WORDS * sizeof(unsigned), st);
     if (e != cudaSuccess) return (int)e;
     // By rows: a block per row where there are few rows, else a warp per row
     // (the weighted sweep: four rows per warp where that leaves eight warps per
@@ -815,21 +846,21 @@ int run_round(const T* X, long long m, long long n, long long ldx, const double*
     Acc<T>* cpart = reinterpret_cast<Acc<T>*>(w.colpart);
     const bool few = m < 16LL * sm && n >= 1024;
     if (few)
-        k_round_rows<T, VEC, 8, 1, false><<<(unsigned)m, RB, 0, st>>>(X, m, n, ldx, f, nullptr, nullptr, w.rs, nullptr, w.state);
+        k_round_rows<T, VEC, 8, 1, false><<<(unsigned)m, RB, 0, st>>>(X, m, n, ldx, f, nullptr, nullptr, nullptr, w.rs, nullptr, w.state);
     else
-        k_round_rows<T, VEC, 1, 1, false><<<(unsigned)((m + 7) / 8), RB, 0, st>>>(X, m, n, ldx, f, nullptr, nullptr, w.rs,
-                                                                                  nullptr, w.state);
+        k_round_rows<T, VEC, 1, 1, false><<<(unsigned)((m + 7) / 8), RB, 0, st>>>(X, m, n, ldx, f, nullptr, nullptr, nullptr,
+                                                                                  w.rs, nullptr, w.state);
     k_round_cols<T, VEC><<<dim3(cb, (unsigned)cparts), RB, 0, st>>>(X, m, n, ldx, f, w.rs, xs, cpart, cparts, w.state);
-    k_round_colscale<T><<<(unsigned)((n + 63) / 64), 64, 0, st>>>(cpart, cparts, n, g, ys, ec, w.state);
+    k_round_colscale<T><<<(unsigned)((n + 63) / 64), 64, 0, st>>>(cpart, cparts, n, g, ys, ec, w.yd, w.ed, w.state);
     if (few && m >= 4LL * sm)
-        k_round_rows<T, VEC, 8, 4, true><<<(unsigned)((m + 3) / 4), RB, 0, st>>>(X, m, n, ldx, f, ys, xs, w.er, w.inv, w.state);
+        k_round_rows<T, VEC, 8, 4, true><<<(unsigned)((m + 3) / 4), RB, 0, st>>>(X, m, n, ldx, f, ys, w.yd, xs, w.er, w.inv, w.state);
     else if (few)
-        k_round_rows<T, VEC, 8, 1, true><<<(unsigned)m, RB, 0, st>>>(X, m, n, ldx, f, ys, xs, w.er, w.inv, w.state);
+        k_round_rows<T, VEC, 8, 1, true><<<(unsigned)m, RB, 0, st>>>(X, m, n, ldx, f, ys, w.yd, xs, w.er, w.inv, w.state);
     else if (m < 64LL * sm && n >= 1024)
-        k_round_rows<T, VEC, 4, 4, true><<<(unsigned)((m + 7) / 8), RB, 0, st>>>(X, m, n, ldx, f, ys, xs, w.er, w.inv, w.state);
+        k_round_rows<T, VEC, 4, 4, true><<<(unsigned)((m + 7) / 8), RB, 0, st>>>(X, m, n, ldx, f, ys, w.yd, xs, w.er, w.inv, w.state);
     else
-        k_round_rows<T, VEC, 1, 4, true><<<(unsigned)((m + 31) / 32), RB, 0, st>>>(X, m, n, ldx, f, ys, xs, w.er, w.inv, w.state);
-    k_round_write<T, VEC, CA><<<dim3(cb, (unsigned)parts), RB, 0, st>>>(X, m, n, ldx, xs, ys, w.er, ec, w.inv, out, ldo, C,
+        k_round_rows<T, VEC, 1, 4, true><<<(unsigned)((m + 31) / 32), RB, 0, st>>>(X, m, n, ldx, f, ys, w.yd, xs, w.er, w.inv, w.state);
+    k_round_write<T, VEC, CA><<<dim3(cb, (unsigned)parts), RB, 0, st>>>(X, m, n, ldx, xs, ys, w.er, ec, w.yd, w.ed, w.inv, out, ldo, C,
                                                                         w.obj, w.state);
     return (int)cudaGetLastError();
 }

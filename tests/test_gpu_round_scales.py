@@ -1,0 +1,44 @@
+"""Rounding of FP32 plans whose scales leave the range of an FP32 pair: row
+scales f_i / (X 1)_i, column scales and error scales far below FP32's smallest
+numbers, with entries so large that the products are ordinary numbers."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2407_19689_gb300 import pdot
+
+pytestmark = pytest.mark.gpu
+
+
+def _case(kind, m, n):
+    r = np.random.default_rng(m + n)
+    X = r.uniform(0.5, 1.5, (m, n)).astype(np.float32).astype(np.float64)
+    f, g = r.uniform(0.5, 1.5, m), r.uniform(0.5, 1.5, n)
+    f, g = f / f.sum(), g / g.sum()
+    if kind == "rows":          # all row scales about 1e-46
+        X, f, g = X * 1e22, f * 1e-24, g * 1e-24
+    elif kind == "one_row":     # one row scale of about 1e-46, beside ordinary ones
+        f[m // 2] *= 1e-46
+    elif kind == "columns":     # all column scales but one about 1e-46
+        X, f, g = X * 1e22, f * 1e22, g * 1e-24
+        g[n // 2] = f.sum()
+    elif kind == "errors":      # err_r of one row against all: about 1e-45
+        X, f, g = X * 1e-30, f * 1e-25, g * 1e20
+        f[m // 2] = 1e20
+    X = X.astype(np.float32).astype(np.float64)
+    return X, f, g
+
+
+@pytest.mark.parametrize("kind", ["rows", "one_row", "columns", "errors"])
+@pytest.mark.parametrize("m,n", [(6, 6), (70, 1030), (2500, 36)])
+def test_round_with_tiny_scales(kind, m, n):
+    X, f, g = _case(kind, m, n)
+    want = oracle.round_plan(X, f, g)
+    s = pdot.Solver(device=0)
+    got = s.round(torch.tensor(X, device="cuda:0", dtype=torch.float32), f, g).double().cpu().numpy()
+    s.close()
+    # Every entry is the FP64 one rounded once (2^-24, or half of the smallest
+    # FP32 number); the sums behind it differ by about 1e-12 of their terms'.
+    scale = np.minimum(np.abs(want).max(axis=1, keepdims=True), np.abs(want).max(axis=0, keepdims=True))
+    assert (np.abs(got - want) <= 1e-7 * scale + 1e-45).all()
