@@ -542,6 +542,7 @@ __device__ __forceinline__ bool finite_bits(double v) {
 __device__ void finalize_step(Ctrl* S, const StepPre& P, double dX2, double dy2, double inter, SchedFactors fac,
                               double w_next) {
     S->passes = P.passes + 1;
+    S->fix = 0;   // the plan a restart picked has been formed before this pass, also where the pass ends the solve
     S->last_dX2 = dX2;
     S->last_dy2 = dy2;
     S->last_inter = inter;
@@ -575,7 +576,6 @@ __device__ void finalize_step(Ctrl* S, const StepPre& P, double dX2, double dy2,
         }
         return;
     }
-    S->fix = 0;   // the plan a restart picked has been formed before this pass
     if (P.lag) {
         // Deferred plan writes: this pass has applied the pending steps if
         // there were `lag` of them; an accepted step becomes pending.
