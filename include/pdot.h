@@ -393,11 +393,11 @@ pdot_status pdot_time_pass(pdot_handle *h, int64_t m, int64_t n, const void *C, 
                            int32_t *kernel_variant);
 
 /*
- * Self-test of the failure path of the shared-memory waits: on `device`,
- * one warp waits, with their bounded wait, for a transfer that is announced on
- * a shared-memory barrier but never issued.  The wait gives up after `polls`
- * polls (1 .. 2^24) and *device_status (host memory) receives the status a
- * pass sets when a wait gives up: PDOT_ERR_CUDA (3).  Returns PDOT_OK when the
+ * Self-test of the failure path of the solver's only wait on the device, the
+ * barrier between the CTAs of a cooperative launch: on `device`, a few CTAs
+ * wait in it for one arrival more than will come.  The wait gives up after
+ * `polls` polls (1 .. 2^24) and *device_status (host memory) receives the
+ * status a solve sets when a barrier gives up: PDOT_ERR_CUDA (3).  Returns PDOT_OK when the
  * self-test ran, PDOT_ERR_ARG for a bad device, poll count or null pointer,
  * PDOT_ERR_CUDA on a CUDA error.  Nothing on the device traps or waits without
  * bound, and the CUDA context stays usable.

@@ -1882,6 +1882,9 @@ pdot_status pdot_create(const pdot_options* opt, int device, void* cuda_stream, 
         const int per = setup_persist();
         if (per > 0) throw CudaError{(cudaError_t)per};
         h->cfg.coop_blocks = coop_ok ? h->sm_count * (-per) : 0;
+        h->cfg.barrier_polls = BARRIER_POLLS;
+        const char* bp = getenv("PDOT_BARRIER_POLLS");   // (tests of the failure path)
+        if (bp && atoi(bp) >= 1 && atoi(bp) < BARRIER_POLLS) h->cfg.barrier_polls = atoi(bp);
         const char* pe = getenv("PDOT_COOP");   // 0: an iteration as two kernels (comparison runs)
         if (pe && atoi(pe) == 0) h->cfg.coop_blocks = 0;
         CK(cudaMalloc(&h->d_gs, sizeof(GridSync)));
@@ -2292,9 +2295,10 @@ pdot_status pdot_watchdog_selftest(int device, int64_t polls, int32_t* device_st
     if (cudaGetDeviceCount(&ndev) != cudaSuccess || device < 0 || device >= ndev) return PDOT_ERR_ARG;
     if (cudaSetDevice(device) != cudaSuccess) return PDOT_ERR_CUDA;
     int* d = nullptr;
-    if (cudaMalloc(&d, sizeof(int)) != cudaSuccess) return PDOT_ERR_CUDA;
+    if (cudaMalloc(&d, 2 * sizeof(int)) != cudaSuccess) return PDOT_ERR_CUDA;   // the status, the barrier's counter
     int hs = -1;
-    bool ok = cudaMemset(d, 0xff, sizeof(int)) == cudaSuccess && launch_watchdog_selftest(polls, d, nullptr) == 0 &&
+    bool ok = cudaMemset(d, 0xff, sizeof(int)) == cudaSuccess && cudaMemset(d + 1, 0, sizeof(int)) == cudaSuccess &&
+              launch_watchdog_selftest((int)polls, d, reinterpret_cast<unsigned*>(d + 1), nullptr) == 0 &&
               cudaMemcpy(&hs, d, sizeof(int), cudaMemcpyDeviceToHost) == cudaSuccess;
     cudaFree(d);
     if (!ok) return PDOT_ERR_CUDA;

@@ -173,6 +173,8 @@ struct Inst {
     int nstrips, nchunks, tile_rows, ntiles, nvt;
 };
 
+constexpr int BARRIER_POLLS = 1 << 23;   // (a poll takes about a microsecond)
+
 // Barrier counters of the cooperative kernel, one pair per instance (zeroed
 // once; launches take them in turn and each zeroes the other).
 struct GridSync {
@@ -218,6 +220,7 @@ struct LaunchCfg {
     int pdl;              // 1: launch with programmatic dependent launch
     int gen_dims;         // largest coordinate count of the generated costs in flight (TT_GEN)
     int comp;             // 1: plan passes of FP32 plans form the compensated reduced cost
+    int barrier_polls;    // polls of the cooperative kernel's barrier before it gives up
     int kkt_blocks;       // CTAs of the bulk-copy KKT pass (0: the register KKT pass)
 };
 
@@ -255,8 +258,9 @@ bool resident_fits(long long m, long long n);
 int setup_resident();
 // out = a + d elementwise (count a multiple of 4; xtype 0 FP32, 2 FP64).
 int launch_combine(int xtype, const void* a, const void* d, void* out, long long count, void* stream);
-// One warp's bounded wait on a transfer that never comes; *d_status <- ST_DEVICE.
-int launch_watchdog_selftest(long long limit, int* d_status, void* stream);
+// The cooperative kernel's barrier with an arrival that never comes (*d_count: 0);
+// *d_status <- ST_DEVICE.
+int launch_watchdog_selftest(int polls, int* d_status, unsigned* d_count, void* stream);
 int occupancy_tile_blocks_per_sm(int ttype);
 int occupancy_vec_blocks_per_sm();
 // Opt the bulk-copy pass kernel into its shared-memory size; returns minus

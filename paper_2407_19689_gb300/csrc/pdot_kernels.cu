@@ -404,42 +404,7 @@ k_pass(const Inst* __restrict__ insts, const TileRef* __restrict__ tmap, const i
     }
 }
 
-// ---------------------------------------------------------------------------
-// Bulk copies (cp.async.bulk) with completion counted on mbarriers.
-// ---------------------------------------------------------------------------
-namespace bulk {
-
 __device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void mbar_init(unsigned bar, unsigned count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(unsigned bar, unsigned bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void g2s(unsigned dst, const void* src, unsigned bytes, unsigned bar) {
-    asm volatile("cp.async.bulk.shared::cta.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-                 "l"(src), "r"(bytes), "r"(bar)
-                 : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(unsigned bar, unsigned parity) {
-    unsigned ok;
-    asm volatile(
-        "{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-__device__ __forceinline__ void fence_mbar_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
-
-// Bounded wait: a copy that never lands must not hang the GPU.
-constexpr long long WAIT_LIMIT = 1LL << 24;
-__device__ __forceinline__ bool wait_stage(unsigned bar, unsigned parity, long long limit = WAIT_LIMIT) {
-    for (long long it = 0; it < limit; ++it)
-        if (mbar_try_wait(bar, parity)) return true;
-    return false;
-}
 
 // Row duals staged per window of PWIN rows (the KKT pass).
 constexpr int PWIN = 128;
@@ -448,8 +413,6 @@ struct RowRef {       // what a stage holds
     int tile;         // global tile index (into tmap), -1 = none
     int row;          // matrix row
 };
-
-}  // namespace bulk
 
 }  // namespace pdot
 
@@ -988,7 +951,7 @@ constexpr int KS = 4;                     // stages per warp (two CTAs per SM: 6
 constexpr int KSTAGE = 4 * STRIP * 4;     // C (<= 512 B), X, Xbar, anchor (512 B each)
 constexpr int KACC = TP + 8;              // FP64 accumulators per lane kept in shared memory (6 scalars, 2 x 4 columns)
 __host__ __device__ constexpr int kkt_warp_smem() {
-    return KS * KSTAGE + KS * 16 + bulk::PWIN * 8 + KACC * 32 * 8;
+    return KS * KSTAGE + KS * 16 + PWIN * 8 + KACC * 32 * 8;
 }
 constexpr int kkt_smem() { return TWARPS * kkt_warp_smem(); }
 
@@ -996,7 +959,6 @@ template <typename TC>
 __global__ void __launch_bounds__(TWARPS * 32, 2)
 k_kkt_bulk(const Inst* __restrict__ insts, const TileRef* __restrict__ tmap, const int* __restrict__ Tp,
            unsigned* wctr, int wc, int mode) {
-    using namespace bulk;
     const int T = *Tp;   // host-written: read before the wait
     extern __shared__ __align__(128) unsigned char dsm[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1006,7 +968,7 @@ k_kkt_bulk(const Inst* __restrict__ insts, const TileRef* __restrict__ tmap, con
     // The lane's FP64 accumulators (kept out of registers): [k * 32 + lane],
     // k < TP the tile scalars, then 4 column sums (average / initial plan), 4
     // column sums (current plan).
-    double* sacc = reinterpret_cast<double*>(wbase + KS * KSTAGE + KS * 16 + bulk::PWIN * 8);
+    double* sacc = reinterpret_cast<double*>(wbase + KS * KSTAGE + KS * 16 + PWIN * 8);
     const unsigned wbase_s = smem_u32(wbase);
     prefetch_first_tile(insts, tmap, T);
     pdl_enter();
@@ -1667,28 +1629,6 @@ __global__ void k_snapshot(const Inst* __restrict__ insts, const int* __restrict
     }
 }
 
-// ---------------------------------------------------------------------------
-// Watchdog self-test: one warp waits, with the pipelines' bounded wait, for a
-// 16-byte transfer that is announced on an mbarrier but never issued.  The
-// wait gives up after `limit` polls and the kernel reports the status a pass
-// would set (ST_DEVICE).  Nothing traps and nothing waits without bound; no
-// copy is in flight when the CTA exits.
-// ---------------------------------------------------------------------------
-__global__ void k_watchdog_selftest(long long limit, int* status) {
-    __shared__ __align__(8) unsigned long long bar_mem;
-    const unsigned bar = bulk::smem_u32(&bar_mem);
-    const int lane = threadIdx.x & 31;
-    if (lane == 0) {
-        bulk::mbar_init(bar, 1);
-        bulk::fence_mbar_init();
-    }
-    __syncwarp();
-    if (lane == 0) bulk::mbar_expect_tx(bar, 16u);   // the arrival happens; the bytes never come
-    __syncwarp();
-    const bool done = bulk::wait_stage(bar, 0u, limit);
-    if (lane == 0) *status = done ? ST_OK : ST_DEVICE;
-}
-
 }  // namespace pdot
 
 #include "pdot_resident.cuh"
@@ -1838,8 +1778,8 @@ int launch_combine(int xtype, const void* a, const void* d, void* out, long long
             static_cast<const float*>(a), static_cast<const float*>(d), static_cast<float*>(out), count);
     return err(cudaGetLastError());
 }
-int launch_watchdog_selftest(long long limit, int* d_status, void* stream) {
-    k_watchdog_selftest<<<1, 32, 0, (cudaStream_t)stream>>>(limit, d_status);
+int launch_watchdog_selftest(int polls, int* d_status, unsigned* d_count, void* stream) {
+    k_watchdog_selftest<<<4, 64, 0, (cudaStream_t)stream>>>(d_count, polls, d_status);
     return err(cudaGetLastError());
 }
 
@@ -1983,8 +1923,8 @@ static int launch_pers(const Inst* d_insts, const CtaRef* refs, int ctas, GridSy
     c.attrs = attr;
     c.numAttrs = 1;
     const int ro = cfg.pass_bulk == 1 ? 1 : 0;
-    return err(cfg.comp ? cudaLaunchKernelEx(&c, k_persist<TC, true>, d_insts, refs, gs, epoch, npass, ro)
-                        : cudaLaunchKernelEx(&c, k_persist<TC, false>, d_insts, refs, gs, epoch, npass, ro));
+    return err(cfg.comp ? cudaLaunchKernelEx(&c, k_persist<TC, true>, d_insts, refs, gs, epoch, npass, ro, cfg.barrier_polls)
+                        : cudaLaunchKernelEx(&c, k_persist<TC, false>, d_insts, refs, gs, epoch, npass, ro, cfg.barrier_polls));
 }
 int launch_persist(int ttype, const Inst* d_insts, const CtaRef* refs, int ctas, bool on_chip, GridSync* gs, int epoch,
                    int npass, const LaunchCfg& cfg, void* stream) {

@@ -231,7 +231,6 @@ template <typename TC, bool CP, bool FINAL>
 __global__ void __launch_bounds__(TWARPS * 32, 2)
 k_pass_lag(const Inst* __restrict__ insts, const TileRef* __restrict__ tmap, const int* __restrict__ Tp,
            unsigned* wctr, int wc, int dir_xor, int roworder) {
-    using namespace bulk;
     using namespace lagp;
     constexpr int DM = GenDims<TC>::value;
     constexpr bool GEN = DM > 0;                         // C generated, not copied

@@ -59,13 +59,12 @@ struct Lay {
 };
 
 constexpr int HALVE_MIN = 32;               // partial sums per column from which a vector tile is halved
-constexpr int SPIN_LIMIT = 1 << 23;          // polls of a barrier before it gives up (seconds)
-
 constexpr unsigned FAIL = 0x40000000u;       // set in a barrier's counter when someone gave up
 
-// Grid barrier: thread 0 of a CTA adds and polls.  Returns false (in every
-// thread of the CTA) when it, or another CTA, gave up.
-__device__ __forceinline__ bool grid_sync(unsigned* c, unsigned target, int* s_ok) {
+// Grid barrier: thread 0 of a CTA adds and polls, `polls` times at most (the
+// library's BARRIER_POLLS: seconds).  Returns false (in every thread of the
+// CTA) when it, or another CTA, gave up.
+__device__ __forceinline__ bool grid_sync(unsigned* c, unsigned target, int* s_ok, int polls) {
     __syncthreads();
     if (threadIdx.x == 0) {
         asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(c) : "memory");
@@ -73,7 +72,7 @@ __device__ __forceinline__ bool grid_sync(unsigned* c, unsigned target, int* s_o
         int it = 0;
         do {
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(c) : "memory");
-        } while (v < target && ++it < SPIN_LIMIT);
+        } while (v < target && ++it < polls);
         if (v < target) atomicOr(c, FAIL);
         *s_ok = v >= target && v < FAIL;
     }
@@ -254,8 +253,8 @@ __device__ __forceinline__ void dual_part(const Inst& I, const Ctrl& S, int lvt,
 // (ctype 3: the entries are computed once, when a tile is loaded).
 template <typename TC, bool CP>
 __global__ void __launch_bounds__(TWARPS * 32, 2)
-k_persist(const Inst* __restrict__ insts, const CtaRef* __restrict__ refs, GridSync* gs, int epoch, int npass, int roworder) {
-    using namespace bulk;
+k_persist(const Inst* __restrict__ insts, const CtaRef* __restrict__ refs, GridSync* gs, int epoch, int npass, int roworder,
+          int polls) {
     using namespace pers;
     using pers::pack; using lagp::unpack; using lagp::widen;
     constexpr int DM = GenDims<TC>::value;
@@ -687,7 +686,7 @@ k_persist(const Inst* __restrict__ insts, const CtaRef* __restrict__ refs, GridS
         }
         DualPre d;
         if (warp < 4 && vt0 < I.nvt) dual_pre(I, S, vt0, HALVES ? s_half : -1, d);   // (arrives during the barrier)
-        if (!grid_sync(bar_count, (unsigned)(me.count * (2 * ps + 1)), &s_ok)) { ok = false; break; }
+        if (!grid_sync(bar_count, (unsigned)(me.count * (2 * ps + 1)), &s_ok, polls)) { ok = false; break; }
         if (vt0 < I.nvt) dual_part(I, S, vt0, HALVES ? s_half : -1, d, s_sl[0], s_sl[1], dsm + L::SCR, L::WARP);
         if (threadIdx.x == 5 * 32) {
             // What the controller needs besides the sums, by a warp that has
@@ -702,7 +701,7 @@ k_persist(const Inst* __restrict__ insts, const CtaRef* __restrict__ refs, GridS
             dual_part(I, S, vt, -1, d, (int)((long long)I.ntiles * vt / I.nvt), (int)((long long)I.ntiles * (vt + 1) / I.nvt), dsm + L::SCR,
                       L::WARP);
         }
-        if (!grid_sync(bar_count, (unsigned)(me.count * (2 * ps + 2)), &s_ok)) { ok = false; break; }
+        if (!grid_sync(bar_count, (unsigned)(me.count * (2 * ps + 2)), &s_ok, polls)) { ok = false; break; }
         // The step scalars, one warp each; meanwhile all warps request what
         // the next pass starts with, for either decision.
         const int h_old = (S.h0 + S.npend) % YRING, np_old = S.npend;
@@ -788,6 +787,15 @@ k_persist(const Inst* __restrict__ insts, const CtaRef* __restrict__ refs, GridS
     for (int w = threadIdx.x; w < (int)(sizeof(Ctrl) / 4); w += blockDim.x)
         if (w != sw || S.status != ST_RUNNING)
             reinterpret_cast<int*>(I.ctrl)[w] = reinterpret_cast<const int*>(&S)[w];
+}
+
+// Self-test of the barrier's failure path: every CTA waits for one arrival
+// more than there are CTAs, gives up after `polls` polls or when another one
+// has, and records the status k_persist records then.
+__global__ void k_watchdog_selftest(unsigned* count, int polls, int* status) {
+    __shared__ int s_ok;
+    const bool ok = pers::grid_sync(count, gridDim.x + 1, &s_ok, polls);
+    if (threadIdx.x == 0) atomicExch(status, ok ? ST_OK : ST_DEVICE);
 }
 
 }  // namespace pdot
