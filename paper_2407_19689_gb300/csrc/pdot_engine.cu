@@ -2113,7 +2113,11 @@ pdot_status pdot_pdhg_steps(pdot_handle* h, int64_t m, int64_t n, const void* C,
         CK(cudaMemcpyAsync(S, w.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, h->stream));
         CK(cudaStreamSynchronize(h->stream));
         if (S->status == ST_ARG) throw ArgError{"invalid marginals"};
-        if (S->status == ST_NUMERIC) return PDOT_ERR_NUMERIC;
+        // (a step that is not finite, a barrier that gave up: the caller's state stays as it was)
+        if (S->status != ST_RUNNING) {
+            h->last_error = S->status == ST_NUMERIC ? "a step is not finite" : "a wait on the device gave up";
+            return map_status(S->status);
+        }
         const int cur = S->cur, bar = k > 0 ? S->bar : S->cur;   // vector sets
         const int xcur = plan_slot(*S);
         copy_plan_out(h, xcur, X, cudaMemcpyDeviceToDevice);

@@ -50,3 +50,19 @@ def test_batch(monkeypatch):
     for i, (big, one) in enumerate(out):
         assert big.status == (pdot.MAX_ITER if i < 2 else pdot.ERR_CUDA)
         assert one.status == out[0][1].status and torch.equal(one.X, out[0][1].X) and torch.equal(one.p, out[0][1].p)
+
+
+def test_constant_steps_leave_the_state(monkeypatch):
+    m, n = 2100, 2000
+    C, f, g = _instance(m, n)
+    f, g = (torch.tensor(v, device="cuda:0") for v in (f, g))
+    state = [(f[:, None] * g[None]).float(), torch.zeros_like(f), torch.zeros_like(g)]
+    before = [v.clone() for v in state]
+    monkeypatch.setenv("PDOT_BARRIER_POLLS", "1")
+    s = pdot.Solver(device=0)
+    st = pdot.pdot_pdhg_steps(s.h, m, n, C.data_ptr(), pdot.F32, n, f.data_ptr(), g.data_ptr(), 20, 0.01, 1.0,
+                              *(v.data_ptr() for v in state))
+    s.close()
+    assert st == pdot.ERR_CUDA
+    for a, b in zip(state, before):
+        assert torch.equal(a, b)
