@@ -119,6 +119,13 @@ struct __align__(8) Acc<double> {
     __device__ __forceinline__ double get() const { return s; }
 };
 
+// min(b / s, 1), 1 for a sum of zero; a marginal that is not a number makes its
+// scale one too (fmin would return 1 and leave the rest of the plan finite).
+__device__ __forceinline__ double scale_to(double b, double s) {
+    const double t = b / s;
+    return !(s > 0.0) ? 1.0 : t > 1.0 ? 1.0 : t;
+}
+
 template <typename T>
 __device__ __forceinline__ void warp_merge(Acc<T>& a) {
 #pragma unroll
@@ -291,7 +298,7 @@ __device__ __noinline__ void cols_wide(const T* X, long long r0, long long r1, l
         if (j + e * es >= n) break;
         double c = 0.0;
         for (long long i = r0; i < r1; ++i)
-            c += (double)X[i * ldx + j + e * es] * (r_sum[i] > 0.0 ? fmin(f[i] / r_sum[i], 1.0) : 1.0);
+            c += (double)X[i * ldx + j + e * es] * scale_to(f[i], r_sum[i]);
         part[j + e * es] = c;
     }
 }
@@ -315,8 +322,7 @@ __global__ void __launch_bounds__(RB) k_round_cols(const T* __restrict__ X, long
         const int cnt = (int)(b + 64 < r1 ? 64 : r1 - b);
         __syncthreads();
         if ((int)threadIdx.x < cnt) {
-            const double s = r_sum[b + threadIdx.x];
-            const double x = s > 0.0 ? fmin(f[b + threadIdx.x] / s, 1.0) : 1.0;
+            const double x = scale_to(f[b + threadIdx.x], r_sum[b + threadIdx.x]);
             sx[threadIdx.x].set(x);
             if (blockIdx.x == 0) xs[b + threadIdx.x] = x;
         }
@@ -369,7 +375,7 @@ __global__ void __launch_bounds__(64) k_round_colscale(const Acc<T>* __restrict_
         }
         c = a.get();
     }
-    const double y = c > 0.0 ? fmin(g[j] / c, 1.0) : 1.0;
+    const double y = scale_to(g[j], c);
     const double e = g[j] - y * c;
     ys[j].set(y);
     ec[j].set(e);

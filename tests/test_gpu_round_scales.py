@@ -42,3 +42,16 @@ def test_round_with_tiny_scales(kind, m, n):
     # FP32 number); the sums behind it differ by about 1e-12 of their terms'.
     scale = np.minimum(np.abs(want).max(axis=1, keepdims=True), np.abs(want).max(axis=0, keepdims=True))
     assert (np.abs(got - want) <= 1e-7 * scale + 1e-45).all()
+
+
+@pytest.mark.parametrize("xt", [pdot.F32, pdot.F64])
+@pytest.mark.parametrize("where", ["f", "g"])
+def test_round_with_a_marginal_that_is_not_a_number(xt, where):
+    """min(f / r, 1) of a NaN is NaN: it reaches the error terms of every row
+    and column, so no entry of the plan looks like a rounded one."""
+    X, f, g = _case("plain", 40, 300)
+    (f if where == "f" else g)[7] = np.nan
+    s = pdot.Solver(device=0, x_dtype=xt)
+    got = s.round(torch.tensor(X, device="cuda:0"), f, g)
+    s.close()
+    assert got.isnan().all()
