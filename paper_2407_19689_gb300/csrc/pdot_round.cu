@@ -26,8 +26,9 @@
 // that follow take FP64 arithmetic and the FP64 scales, which are kept beside
 // the pairs: row sums of 1e30 and more or not finite, and scales below RTINY
 // that are multiplied by more than 1 (a pair's absolute error is 2^-150, so a
-// product with at most 1 is as exact as an FP32 entry can be).  FP64 plans use
-// FP64 throughout.
+// product with at most 1 is as exact as an FP32 entry can be).  The objective
+// <C, plan> is an FP64 sum of FP64 products (once per solve that asks for it).
+// FP64 plans use FP64 throughout.
 #include <cuda_runtime.h>
 #include <math_constants.h>
 
@@ -498,7 +499,6 @@ __global__ void __launch_bounds__(RB) k_round_write(const T* X, long long m, lon
             }
             __syncthreads();
             if (j >= n) continue;
-            Acc<T> acc;
             for (int rb = 0; rb < cnt; rb += RU) {
 #pragma unroll
                 for (int u = 0; u < RU; ++u) {
@@ -524,21 +524,11 @@ __global__ void __launch_bounds__(RB) k_round_write(const T* X, long long m, lon
                     }
                     if (C.on()) {
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            if (j + e * ES >= n) continue;
-                            if constexpr (sizeof(T) == 4) {
-                                Scale<float> k;
-                                k.h = C.f32(b + r, j + e * ES);
-                                k.l = 0.f;
-                                acc.add(w[e], k);
-                            } else {
-                                obj += C(b + r, j + e * ES) * w[e];
-                            }
-                        }
+                        for (int e = 0; e < 4; ++e)
+                            if (j + e * ES < n) obj += C(b + r, j + e * ES) * (double)w[e];
                     }
                 }
             }
-            if (sizeof(T) == 4) obj += acc.get();
         }
     }
     if (!C.on()) return;

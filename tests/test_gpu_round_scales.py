@@ -55,3 +55,22 @@ def test_round_with_a_marginal_that_is_not_a_number(xt, where):
     got = s.round(torch.tensor(X, device="cuda:0"), f, g)
     s.close()
     assert got.isnan().all()
+
+
+def test_rounded_objective_of_equal_terms():
+    """<C, plan> of a constant plan and cost: the terms' rounding errors all have
+    the same sign.  In FP64 a thread adds at most 264 terms (67 rows of four
+    columns), a warp, block and the host 5 + 8 + 608 more sums, each of relative
+    error 2^-53 at most."""
+    m, n = 40000, 256
+    f, g = np.full(m, 1 / m), np.full(n, 1 / n)
+    X0 = torch.full((m, n), 1 / (m * n), dtype=torch.float32, device="cuda:0")
+    s = pdot.Solver(device=0, round_plan=1)
+    for c in (0.2718282, 0.5405107, 0.7697867, 0.8889214, 1.1231872, 1.4127556):
+        C = torch.full((m, n), c, dtype=torch.float32, device="cuda:0")
+        sol = s.solve(C, f, g, tol=1e9, X0=X0)   # (the start is accepted as it is)
+        assert sol.result["passes"] == 0
+        values, counts = sol.X.double().unique(return_counts=True)
+        want = float(C[0, 0].double()) * float((values * counts).sum())
+        assert abs(sol.result["rounded_obj"] - want) <= 900 * 2.0 ** -53 * want
+    s.close()
