@@ -257,6 +257,7 @@ struct pdot_handle {
     int res_clusters = 0;        // resident-kernel clusters the device holds at once (0: not available)
     GridSync* d_gs = nullptr;    // barrier counters of the cooperative kernel
     int coop_epoch = 0;
+    int coop_passes = 0;         // most passes of a cooperative launch
     bool persist_on = false;     // the current single-instance call runs its passes in the cooperative kernel
     int* d_res1 = nullptr;       // {0, 1}: the list and count of a single-instance resident launch
     bool res_on = false;         // the current single-instance call runs in the resident kernel
@@ -548,13 +549,15 @@ int coop_ctas(pdot_handle* h, long long ntiles) {
     return (int)((ntiles + per - 1) / per);
 }
 
-// `npass` passes and the final write in one launch.
-void run_persist(pdot_handle* h, int ttype, int npass) {
+// `npass` passes, each launch's with its final write (which changes no bits).
+void run_persist(pdot_handle* h, int ttype, int64_t npass) {
     const Work& w = h->ws;
-    CKL(launch_persist(ttype, h->d_inst, nullptr, coop_ctas(h, w.ntiles),
-                       w.tile_rows <= persist_rows(h->cfg.comp != 0), h->d_gs, h->coop_epoch, npass, h->cfg, h->stream));
-    h->coop_epoch ^= 1;
-    launch_count(h, 1);
+    for (int64_t s = 0; s < npass; s += h->coop_passes) {
+        CKL(launch_persist(ttype, h->d_inst, nullptr, coop_ctas(h, w.ntiles), w.tile_rows <= persist_rows(h->cfg.comp != 0),
+                           h->d_gs, h->coop_epoch, (int)std::min<int64_t>(h->coop_passes, npass - s), h->cfg, h->stream));
+        h->coop_epoch ^= 1;
+        launch_count(h, 1);
+    }
 }
 
 void launch_chunk(pdot_handle* h, int ttype, int K) {
@@ -1418,10 +1421,13 @@ void batch_issue_chunk(pdot_handle* h, int types) {
         launch_count(h, 1);
     }
     for (int c = 0; c < checks; ++c) {
-        if (!B->coop.empty()) CK(cudaMemsetAsync(B->gs, 0, sizeof(GridSync) * B->live.size(), st));
-        for (const BatchEngine::Coop& w : B->coop) {
-            CKL(launch_persist(w.ttype, B->insts.d, B->refs.d + w.first, w.ctas, false, B->gs, 0, K, h->cfg, st));
-            launch_count(h, 1);
+        for (int64_t s = 0; s < K && !B->coop.empty(); s += h->coop_passes) {
+            CK(cudaMemsetAsync(B->gs, 0, sizeof(GridSync) * B->live.size(), st));
+            for (const BatchEngine::Coop& w : B->coop) {
+                CKL(launch_persist(w.ttype, B->insts.d, B->refs.d + w.first, w.ctas, false, B->gs, 0,
+                                   (int)std::min<int64_t>(h->coop_passes, K - s), h->cfg, st));
+                launch_count(h, 1);
+            }
         }
         for (int s = 0; s < K && B->coop.empty(); ++s) {
             for (int t = 0; t < NTT; ++t) {
@@ -1887,6 +1893,10 @@ pdot_status pdot_create(const pdot_options* opt, int device, void* cuda_stream, 
         if (bp && atoi(bp) >= 1 && atoi(bp) < BARRIER_POLLS) h->cfg.barrier_polls = atoi(bp);
         const char* pe = getenv("PDOT_COOP");   // 0: an iteration as two kernels (comparison runs)
         if (pe && atoi(pe) == 0) h->cfg.coop_blocks = 0;
+        // Two arrivals of every CTA per pass stay below the counter's fail bit.
+        h->coop_passes = (int)((BARRIER_FAIL - 1) / (2u * (unsigned)std::max(1, h->cfg.coop_blocks)));
+        const char* cp = getenv("PDOT_COOP_PASSES");   // fewer passes per launch (comparison runs)
+        if (cp && atoi(cp) >= 1 && atoi(cp) < h->coop_passes) h->coop_passes = atoi(cp);
         CK(cudaMalloc(&h->d_gs, sizeof(GridSync)));
         CK(cudaMemset(h->d_gs, 0, sizeof(GridSync)));
         const int kb = setup_kkt_bulk();
@@ -2103,8 +2113,7 @@ pdot_status pdot_pdhg_steps(pdot_handle* h, int64_t m, int64_t n, const void* C,
             }
         } else {
             if (lag && persist_for(h, m, n, ttype, w.tile_rows)) {
-                constexpr int64_t MOST = 1 << 20;   // (the barrier counter's range)
-                for (int64_t s = 0; s < k; s += MOST) run_persist(h, ttype, (int)std::min(MOST, k - s));
+                run_persist(h, ttype, k);
             } else {
                 for (int64_t s = 0; s < k; ++s) run_step(h, ttype);
                 if (lag) run_final(h, ttype);

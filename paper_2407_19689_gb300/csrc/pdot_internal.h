@@ -174,6 +174,7 @@ struct Inst {
 };
 
 constexpr int BARRIER_POLLS = 1 << 23;   // (a poll takes about a microsecond)
+constexpr unsigned BARRIER_FAIL = 0x40000000u;   // set in a barrier's counter when someone gave up
 
 // Barrier counters of the cooperative kernel, one pair per instance (zeroed
 // once; launches take them in turn and each zeroes the other).

@@ -59,8 +59,6 @@ struct Lay {
 };
 
 constexpr int HALVE_MIN = 32;               // partial sums per column from which a vector tile is halved
-constexpr unsigned FAIL = 0x40000000u;       // set in a barrier's counter when someone gave up
-
 // Grid barrier: thread 0 of a CTA adds and polls, `polls` times at most (the
 // library's BARRIER_POLLS: seconds).  Returns false (in every thread of the
 // CTA) when it, or another CTA, gave up.
@@ -73,8 +71,8 @@ __device__ __forceinline__ bool grid_sync(unsigned* c, unsigned target, int* s_o
         do {
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(c) : "memory");
         } while (v < target && ++it < polls);
-        if (v < target) atomicOr(c, FAIL);
-        *s_ok = v >= target && v < FAIL;
+        if (v < target) atomicOr(c, BARRIER_FAIL);
+        *s_ok = v >= target && v < BARRIER_FAIL;
     }
     __syncthreads();
     return *s_ok != 0;
