@@ -2226,7 +2226,15 @@ pdot_status pdot_dual_bound(pdot_handle* h, int64_t m, int64_t n, const void* C,
         double* val = nullptr;
         GenSpec gs{};
         if (c_dtype == PDOT_POINTS) gs = gen_spec_of(C);
-        CKL(launch_dual_bound(C, (int)c_dtype, ldc, &gs, p, f, g, m, n, h->round_scratch, q_out, &val, h->sm_count, h->stream));
+        // q is written while p, f and g are still read: where it overlaps one
+        // of them, it is formed in the scratch and copied last.
+        auto overlaps = [&](const double* v, int64_t k) {
+            return q_out && (uintptr_t)q_out < (uintptr_t)(v + k) && (uintptr_t)v < (uintptr_t)(q_out + n);
+        };
+        const bool last = overlaps(p, m) || overlaps(f, m) || overlaps(g, n);
+        double* q = last ? h->round_scratch : q_out;
+        CKL(launch_dual_bound(C, (int)c_dtype, ldc, &gs, p, f, g, m, n, h->round_scratch, q, &val, h->sm_count, h->stream));
+        if (last) CK(cudaMemcpyAsync(q_out, q, sizeof(double) * (size_t)n, cudaMemcpyDeviceToDevice, h->stream));
         launch_count(h, c_dtype == PDOT_F64 ? 2 : 3);
         double* hv = reinterpret_cast<double*>(h->h_status);   // (pinned, 8 bytes)
         CK(cudaMemcpyAsync(hv, val, sizeof(double), cudaMemcpyDeviceToHost, h->stream));

@@ -680,10 +680,10 @@ __global__ void __launch_bounds__(RB) k_bound_cols64(CA C, const double* __restr
 
 // q from its keys (into q_out, where wanted) and out[0] = f^T p + g^T q: fixed
 // runs per block, the last block adds the blocks' sums in order.  ticket starts
-// as all ones.
+// as all ones.  (q_out may be the keys' own memory: an entry has one thread.)
 __global__ void __launch_bounds__(RB) k_bound_value(const double* __restrict__ f, const double* __restrict__ p, long long m,
                                                     const double* __restrict__ g,
-                                                    const unsigned long long* __restrict__ qkey, double* q_out, long long n,
+                                                    const unsigned long long* qkey, double* q_out, long long n,
                                                     double* part, double* out, unsigned* ticket) {
     __shared__ double red[RB / 32];
     __shared__ unsigned last;
