@@ -544,16 +544,20 @@ bool persist_for(pdot_handle* h, long long m, long long n, int ttype, int tile_r
 // per warp), or as few as four while that needs no second CTA on an SM (64 x
 // 64: 5.7K -> 4.5K cycles per traversal; 300 x 517: 5.4K -> 4.7K.  Two CTAs on
 // an SM take turns at the controller's FP64: 4.5K -> 5.4K cycles at 300 x 517).
-int coop_ctas(pdot_handle* h, long long ntiles) {
+// A plan of a few long rows has more vector tiles than such CTAs; each vector
+// tile then gets a CTA of its own as far as the device holds them, with or
+// without plan tiles (us per iteration, tiles only -> with this: 1 x 5000 41 ->
+// 13.6, 1 x 100000 83 -> 62, 40 x 4096 16.5 -> 14.2; two kernels 19, 60, 20).
+int coop_ctas(pdot_handle* h, long long ntiles, long long nvt) {
     const long long per = std::min<long long>(TWARPS, std::max<long long>(4, (ntiles + h->sm_count - 1) / h->sm_count));
-    return (int)((ntiles + per - 1) / per);
+    return (int)std::max((ntiles + per - 1) / per, std::min<long long>(nvt, h->cfg.coop_blocks));
 }
 
 // `npass` passes, each launch's with its final write (which changes no bits).
 void run_persist(pdot_handle* h, int ttype, int64_t npass) {
     const Work& w = h->ws;
     for (int64_t s = 0; s < npass; s += h->coop_passes) {
-        CKL(launch_persist(ttype, h->d_inst, nullptr, coop_ctas(h, w.ntiles), w.tile_rows <= persist_rows(h->cfg.comp != 0),
+        CKL(launch_persist(ttype, h->d_inst, nullptr, coop_ctas(h, w.ntiles, w.nvt), w.tile_rows <= persist_rows(h->cfg.comp != 0),
                            h->d_gs, h->coop_epoch, (int)std::min<int64_t>(h->coop_passes, npass - s), h->cfg, h->stream));
         h->coop_epoch ^= 1;
         launch_count(h, 1);
