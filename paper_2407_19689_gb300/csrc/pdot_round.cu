@@ -32,6 +32,7 @@
 #include <cuda_runtime.h>
 #include <math_constants.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <type_traits>
 
@@ -723,25 +724,41 @@ __global__ void __launch_bounds__(RB) k_bound_value(const double* __restrict__ f
 // 2000 x 2000 59.4 -> 69.2.
 constexpr long long BOUND_DIRECT = 1LL << 21;
 
+// Row groups of a sweep over `cb` blocks of columns: four blocks per SM, of at
+// least 16 rows.
+long long bound_parts(long long cb, long long m, int sm) {
+    long long parts = (4LL * sm + cb - 1) / cb;
+    if (parts > (m + 15) / 16) parts = (m + 15) / 16;
+    return parts > 65535 ? 65535 : parts;
+}
+
+// (Row groups as above, but up to 64 of any size: a thread's FP64 differences
+// are one chain.  With 64 groups at most, 100000 x 10 from 8 coordinates took
+// 632 us; here 119.)
 template <typename CA>
-void launch_bound_cols64(CA C, const double* p, long long m, long long n, unsigned long long* qkey, cudaStream_t st) {
-    const long long parts = 64 < m ? 64 : m;
+void launch_bound_cols64(CA C, const double* p, long long m, long long n, unsigned long long* qkey, int sm, cudaStream_t st) {
+    const long long parts = std::max(bound_parts((n + RB - 1) / RB, m, sm), std::min(64LL, m));
     k_bound_cols64<CA><<<dim3((unsigned)((n + RB - 1) / RB), (unsigned)parts), RB, 0, st>>>(C, p, m, n, qkey);
 }
+
+// Costs generated from 4 or 8 coordinates take one sweep at any size: the
+// columns' coordinates are then 16 or 32 bytes apart, a warp's loads of them
+// conflict in the banks, and the screen's second sweep reads them again (8191 x
+// 8191, direct / screened: 4 coordinates 460 / 467 us, 8 602 / 1056; 3: 464 /
+// 333, 6: 465 / 400).
+bool bound_direct(const PointsCost& C) { return C.g.d % 4 == 0; }
+template <typename CA>
+bool bound_direct(const CA&) { return false; }
 
 template <typename CA>
 void launch_bound_cols(CA C, bool vec, const double* p, long long m, long long n, unsigned* qmin, unsigned* pmax,
                        unsigned long long* qkey, int sm, cudaStream_t st) {
-    if (m * n < BOUND_DIRECT) {
-        launch_bound_cols64(C, p, m, n, qkey, st);
+    if (m * n < BOUND_DIRECT || bound_direct(C)) {
+        launch_bound_cols64(C, p, m, n, qkey, sm, st);
         return;
     }
-    // Row groups: four blocks per SM, of at least 16 rows.
     const long long cb = (n + 4 * RB - 1) / (4 * RB);
-    long long parts = (4LL * sm + cb - 1) / cb;
-    if (parts > (m + 15) / 16) parts = (m + 15) / 16;
-    if (parts > 65535) parts = 65535;
-    const dim3 grid((unsigned)cb, (unsigned)parts);
+    const dim3 grid((unsigned)cb, (unsigned)bound_parts(cb, m, sm));
     if (vec) {
         k_bound_cols<false, true, CA><<<grid, RB, 0, st>>>(C, p, m, n, qmin, pmax, qkey);
         k_bound_cols<true, true, CA><<<grid, RB, 0, st>>>(C, p, m, n, qmin, pmax, qkey);
@@ -777,7 +794,7 @@ int launch_dual_bound(const void* C, int ctype, long long ldc, const GenSpec* ge
     if (ctype == 3) {
         launch_bound_cols(PointsCost{*gen}, false, p, m, n, qmin, pmax, qkey, sm, st);
     } else if (ctype == 2) {
-        launch_bound_cols64(StoredCost<double>{(const double*)C, ldc}, p, m, n, qkey, st);
+        launch_bound_cols64(StoredCost<double>{(const double*)C, ldc}, p, m, n, qkey, sm, st);
     } else if (ctype == 1) {
         launch_bound_cols(StoredCost<Bf16>{(const Bf16*)C, ldc}, a16 && ldc % 4 == 0, p, m, n, qmin, pmax, qkey, sm, st);
     } else {
