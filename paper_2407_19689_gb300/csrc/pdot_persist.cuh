@@ -376,14 +376,22 @@ k_persist(const Inst* __restrict__ insts, const CtaRef* __restrict__ refs, GridS
         }
     }
     if (gen_fill && active) {
+        // (The columns' coordinates are read once: eight floats apart, a warp's
+        // loads of them conflict in every bank.  Read for each row, a launch at
+        // 1500 x 1400 from 8 coordinates took 52 us more.)
         const GenSpec gp = I.gen;
+        float y[4][GEN_DMAX];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+#pragma unroll
+            for (int k = 0; k < GEN_DMAX; ++k)
+                y[e][k] = (k < gp.d && j0 + e < n) ? __ldg(gp.ys + (long long)(j0 + e) * gp.d + k) : 0.f;
+        }
         for (int r = 0; r < nrows; ++r) {
+            const float* x = gp.xs + (long long)(r0 + r) * gp.d;
             float c[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e)
-                c[e] = j0 + e < n ? gen_cost<GEN_DMAX>(gp.kind, gp.d, gp.xs + (long long)(r0 + r) * gp.d,
-                                                       gp.ys + (long long)(j0 + e) * gp.d, gp.div, gp.inv)
-                                  : 0.f;
+            for (int e = 0; e < 4; ++e) c[e] = j0 + e < n ? gen_cost<GEN_DMAX>(gp.kind, gp.d, x, y[e], gp.div, gp.inv) : 0.f;
             st4(reinterpret_cast<float*>(wbase + (r / R) * SB + ARR + (r % R) * (STRIP * 4)) + lane * 4, c);
         }
         __syncwarp();
