@@ -40,7 +40,7 @@ int launch_round(const void* X, int xtype, long long m, long long n, long long l
 long long bound_scratch_bytes(long long n);
 int launch_dual_bound(const void* C, int ctype, long long ldc, const GenSpec* gen, const double* p,
                       const double* f, const double* g, long long m, long long n, void* scratch, double* q_out,
-                      double** value, int sm, void* stream);
+                      double** value, int sm, int* launches, void* stream);
 }  // namespace pdot
 
 namespace {
@@ -2237,9 +2237,11 @@ pdot_status pdot_dual_bound(pdot_handle* h, int64_t m, int64_t n, const void* C,
         };
         const bool last = overlaps(p, m) || overlaps(f, m) || overlaps(g, n);
         double* q = last ? h->round_scratch : q_out;
-        CKL(launch_dual_bound(C, (int)c_dtype, ldc, &gs, p, f, g, m, n, h->round_scratch, q, &val, h->sm_count, h->stream));
+        int launches = 0;
+        CKL(launch_dual_bound(C, (int)c_dtype, ldc, &gs, p, f, g, m, n, h->round_scratch, q, &val, h->sm_count, &launches,
+                              h->stream));
         if (last) CK(cudaMemcpyAsync(q_out, q, sizeof(double) * (size_t)n, cudaMemcpyDeviceToDevice, h->stream));
-        launch_count(h, c_dtype == PDOT_F64 ? 2 : 3);
+        launch_count(h, launches);
         double* hv = reinterpret_cast<double*>(h->h_status);   // (pinned, 8 bytes)
         CK(cudaMemcpyAsync(hv, val, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
         CK(cudaStreamSynchronize(h->stream));

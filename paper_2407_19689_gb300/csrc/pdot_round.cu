@@ -750,12 +750,13 @@ bool bound_direct(const PointsCost& C) { return C.g.d % 4 == 0; }
 template <typename CA>
 bool bound_direct(const CA&) { return false; }
 
+// Returns the number of launches.
 template <typename CA>
-void launch_bound_cols(CA C, bool vec, const double* p, long long m, long long n, unsigned* qmin, unsigned* pmax,
-                       unsigned long long* qkey, int sm, cudaStream_t st) {
+int launch_bound_cols(CA C, bool vec, const double* p, long long m, long long n, unsigned* qmin, unsigned* pmax,
+                      unsigned long long* qkey, int sm, cudaStream_t st) {
     if (m * n < BOUND_DIRECT || bound_direct(C)) {
         launch_bound_cols64(C, p, m, n, qkey, sm, st);
-        return;
+        return 1;
     }
     const long long cb = (n + 4 * RB - 1) / (4 * RB);
     const dim3 grid((unsigned)cb, (unsigned)bound_parts(cb, m, sm));
@@ -766,6 +767,7 @@ void launch_bound_cols(CA C, bool vec, const double* p, long long m, long long n
         k_bound_cols<false, false, CA><<<grid, RB, 0, st>>>(C, p, m, n, qmin, pmax, qkey);
         k_bound_cols<true, false, CA><<<grid, RB, 0, st>>>(C, p, m, n, qmin, pmax, qkey);
     }
+    return 2;
 }
 
 constexpr int BOUND_BLOCKS = 64;
@@ -778,10 +780,10 @@ long long bound_scratch_bytes(long long n) { return 8 * n + 4 * ((n + 1) / 2 * 2
 
 // The bound above: q_out (n, or null) and *value = f^T p + g^T q.
 // ctype: 0 FP32, 1 BF16, 2 FP64 (row-major with leading dimension ldc), 3
-// generated (gen).
+// generated (gen).  *launches: how many kernels it took.
 int launch_dual_bound(const void* C, int ctype, long long ldc, const GenSpec* gen, const double* p,
                       const double* f, const double* g, long long m, long long n, void* scratch, double* q_out,
-                      double** value, int sm, void* stream) {
+                      double** value, int sm, int* launches, void* stream) {
     const cudaStream_t st = (cudaStream_t)stream;
     unsigned long long* qkey = static_cast<unsigned long long*>(scratch);
     unsigned* qmin = reinterpret_cast<unsigned*>(qkey + n);
@@ -791,15 +793,17 @@ int launch_dual_bound(const void* C, int ctype, long long ldc, const GenSpec* ge
     const cudaError_t e = cudaMemsetAsync(scratch, 0xff, (size_t)(reinterpret_cast<char*>(part) - static_cast<char*>(scratch)), st);
     if (e != cudaSuccess) return (int)e;
     const bool a16 = reinterpret_cast<uintptr_t>(C) % 16 == 0;
+    int k = 1;
     if (ctype == 3) {
-        launch_bound_cols(PointsCost{*gen}, false, p, m, n, qmin, pmax, qkey, sm, st);
+        k = launch_bound_cols(PointsCost{*gen}, false, p, m, n, qmin, pmax, qkey, sm, st);
     } else if (ctype == 2) {
         launch_bound_cols64(StoredCost<double>{(const double*)C, ldc}, p, m, n, qkey, sm, st);
     } else if (ctype == 1) {
-        launch_bound_cols(StoredCost<Bf16>{(const Bf16*)C, ldc}, a16 && ldc % 4 == 0, p, m, n, qmin, pmax, qkey, sm, st);
+        k = launch_bound_cols(StoredCost<Bf16>{(const Bf16*)C, ldc}, a16 && ldc % 4 == 0, p, m, n, qmin, pmax, qkey, sm, st);
     } else {
-        launch_bound_cols(StoredCost<float>{(const float*)C, ldc}, a16 && ldc % 4 == 0, p, m, n, qmin, pmax, qkey, sm, st);
+        k = launch_bound_cols(StoredCost<float>{(const float*)C, ldc}, a16 && ldc % 4 == 0, p, m, n, qmin, pmax, qkey, sm, st);
     }
+    *launches = k + 1;
     // One block per 256 entries where that is fewer.
     long long vb = (m + n + RB - 1) / RB;
     if (vb > BOUND_BLOCKS) vb = BOUND_BLOCKS;

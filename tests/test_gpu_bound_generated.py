@@ -26,3 +26,14 @@ def test_bound_is_exact(m, n, d):
     np.testing.assert_array_equal(q.cpu().numpy(), want)
     terms = np.concatenate([f * p, g * want])
     assert abs(lower - terms.sum()) <= 1e-13 * np.abs(terms).sum()
+
+
+@pytest.mark.parametrize("m,n,d,launches", [(300, 200, 2, 2), (1500, 1501, 2, 3), (1500, 1501, 4, 2)])
+def test_launches_are_counted_as_they_are_made(m, n, d, launches):
+    """One sweep or two (see above), and the value."""
+    s = pdot.Solver(device=0)
+    xs, ys = (torch.rand((k, d), device="cuda:0") for k in (m, n))
+    n0 = s.launch_count()
+    s.dual_bound(pdot.Points(xs, ys), np.full(m, 1 / m), np.full(n, 1 / n), np.zeros(m))
+    assert s.launch_count() - n0 == launches
+    s.close()
