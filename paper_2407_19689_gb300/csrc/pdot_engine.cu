@@ -2186,7 +2186,11 @@ pdot_status pdot_kkt(pdot_handle* h, int64_t m, int64_t n, const void* C, pdot_d
         run_check(h, ttype, MODE_INIT);
         CK(cudaMemcpyAsync(S, w.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, h->stream));
         CK(cudaStreamSynchronize(h->stream));
-        if (S->status == ST_ARG) throw ArgError{"invalid marginals"};
+        if (S->status == ST_ARG) {   // the host's test says which of them, and why
+            double norm_b = 0.0;
+            validate_marginals(h, m, n, f, g, false, &norm_b);
+            throw ArgError{"invalid marginals"};
+        }
         out->rp2 = S->r_rp2; out->rd2 = S->r_rd2; out->cx = S->r_cx; out->dual = S->r_dual; out->gap = S->r_gap;
         out->kkt = S->r_kkt; out->rel_p = S->r_rel_p; out->rel_d = S->r_rel_d; out->rel_gap = S->r_rel_gap;
         out->rel_kkt = S->r_rel;
