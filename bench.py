@@ -31,7 +31,9 @@ sys.path.insert(0, ROOT)
 METRIC = "time-to-1e-6 KKT & HBM GB/s per iter; batched solves/s, p99 latency vs plain"
 PEAKS = os.path.join(ROOT, "MEASURED_PEAKS.json")
 TRAFFIC = os.path.join(ROOT, "profiles", "pass_kernel_traffic.json")
-KERNEL_SRC = os.path.join(ROOT, "paper_2407_19689_gb300", "csrc", "pdot_kernels.cu")
+# What the pass kernels are compiled from.
+KERNEL_SRC = [os.path.join(ROOT, "paper_2407_19689_gb300", "csrc", name)
+              for name in ("pdot_internal.h", "pdot_kernels.cu", "pdot_pass.cuh", "pdot_persist.cuh")]
 
 
 def parse():
@@ -161,15 +163,23 @@ def measured_peak():
         return 6800.0, "fallback"
 
 
+def kernel_source_sha256() -> str:
+    """SHA-256 of the pass kernels' source files, one after the other."""
+    h = hashlib.sha256()
+    for path in [KERNEL_SRC] if isinstance(KERNEL_SRC, str) else KERNEL_SRC:
+        with open(path, "rb") as fh:
+            h.update(fh.read())
+    return h.hexdigest()
+
+
 def recorded_traffic(cost_dtype: str, grid: int, variant: int):
     """Per-launch DRAM bytes of the pass kernel from the committed ncu summary
     for this cost storage, grid and kernel variant, or None when there is no
-    such record or the kernel source changed since it was captured."""
+    such record or a source file changed since it was captured."""
     try:
         with open(TRAFFIC) as fh:
             recs = json.load(fh)["records"]
-        with open(KERNEL_SRC, "rb") as fh:
-            sha = hashlib.sha256(fh.read()).hexdigest()
+        sha = kernel_source_sha256()
         for rec in recs:
             if (rec["cost_dtype"], rec["grid"], rec["kernel_variant"]) == (cost_dtype, grid, variant):
                 if rec.get("kernel_source_sha256") != sha:
