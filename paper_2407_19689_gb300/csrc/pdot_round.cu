@@ -24,7 +24,7 @@
 // written entries; measured against 64 bits the plan's error is unchanged
 // (2.5e-8).  Where FP32's range would not hold a sum or a scale, the sweeps
 // that follow take FP64 arithmetic and the FP64 scales, which are kept beside
-// the pairs: row sums of 1e30 and more or not finite, and scales below RTINY
+// the pairs: row sums or errors of 1e30 and more or not finite, and scales below RTINY
 // that are multiplied by more than 1 (a pair's absolute error is 2^-150, so a
 // product with at most 1 is as exact as an FP32 entry can be).  The objective
 // <C, plan> is an FP64 sum of FP64 products (once per solve that asks for it).
@@ -46,7 +46,7 @@ constexpr int RB = 256;           // threads per block
 constexpr int RPARTS = 64;        // most row groups of the column sums
 constexpr int RU = 4;             // rows a thread of the write has in flight
 constexpr int RROWS = 64;         // rows whose scales a block of the write holds at a time
-constexpr double RWIDE = 1e30;    // row sums from here on: FP64 arithmetic
+constexpr double RWIDE = 1e30;    // row sums and column errors from here on: FP64 arithmetic
 constexpr double RTINY = 0x1p-100;   // scales below: an FP32 pair has lost bits (its low part is subnormal from 2^-102 on)
 
 // Words of RoundScratch::state: the ticket; FP32's range does not hold a row
@@ -385,7 +385,10 @@ __global__ void __launch_bounds__(64) k_round_colscale(const Acc<T>* __restrict_
         yd[j] = y;
         ed[j] = e;
         if (from_one(c) && y > 0.0 && y < RTINY) atomicOr(state + RS_LATE, 1u);
-        if (from_one(e)) atomicOr(state + RS_ERR, 1u);
+        if (from_one(e)) {
+            atomicOr(state + RS_ERR, 1u);
+            if (!(e < RWIDE)) atomicOr(state + RS_LATE, 1u);
+        }
     }
 }
 

@@ -1,6 +1,8 @@
 """Rounding of FP32 plans whose scales leave the range of an FP32 pair: row
 scales f_i / (X 1)_i, column scales and error scales far below FP32's smallest
-numbers, with entries so large that the products are ordinary numbers."""
+numbers, with entries so large that the products are ordinary numbers; column
+errors beyond its largest.  And marginals that are not finite, and the FP64 sum
+of the objective."""
 import numpy as np
 import pytest
 import torch
@@ -26,11 +28,14 @@ def _case(kind, m, n):
     elif kind == "errors":      # err_r of one row against all: about 1e-45
         X, f, g = X * 1e-30, f * 1e-25, g * 1e20
         f[m // 2] = 1e20
+    elif kind == "beyond":      # column errors beyond FP32, entries within it
+        g = np.full(n, 1e39)
+        f = np.full(m, n * 1e39 / m)
     X = X.astype(np.float32).astype(np.float64)
     return X, f, g
 
 
-@pytest.mark.parametrize("kind", ["rows", "one_row", "columns", "errors"])
+@pytest.mark.parametrize("kind", ["rows", "one_row", "columns", "errors", "beyond"])
 @pytest.mark.parametrize("m,n", [(6, 6), (70, 1030), (2500, 36)])
 def test_round_with_tiny_scales(kind, m, n):
     X, f, g = _case(kind, m, n)
@@ -74,3 +79,16 @@ def test_rounded_objective_of_equal_terms():
         want = float(C[0, 0].double()) * float((values * counts).sum())
         assert abs(sol.result["rounded_obj"] - want) <= 900 * 2.0 ** -53 * want
     s.close()
+
+
+def test_round_with_an_infinite_marginal():
+    """Its column has an infinite error and infinite entries, as in FP64 (a pair's
+    low part, inf - inf, made them not a number)."""
+    X, f, g = _case("plain", 40, 300)
+    g[7] = np.inf
+    s = pdot.Solver(device=0)
+    got = s.round(torch.tensor(X, device="cuda:0"), f, g).cpu().numpy()
+    s.close()
+    want = oracle.round_plan(X, f, g)
+    np.testing.assert_array_equal(np.isnan(got), np.isnan(want))
+    np.testing.assert_array_equal(np.isinf(got), np.isinf(want))
