@@ -252,7 +252,7 @@ struct pdot_handle {
     int* h_status = nullptr;     // pinned [2]
     Graph chunk;                 // K x (pass, dual) + (kkt, checkvec)
     long long chunk_key[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    int autotune = 1;            // order of the pass's sums and tile height by shape (0: the handle's fixed choice)
+    int by_shape = 1;            // order of the pass's sums and tile height by shape (0: the handle's fixed choice)
     int batch_min_rows = 16;     // smallest tile height of a batched instance (even)
     int res_clusters = 0;        // resident-kernel clusters the device holds at once (0: not available)
     GridSync* d_gs = nullptr;    // barrier counters of the cooperative kernel
@@ -373,7 +373,7 @@ int tile_rows_for(pdot_handle* h, long long m, long long n, int ttype, int kerne
         // nearly alone at the end of a batch or in a sparse stream), but no
         // fewer than batch_min_rows rows (in a crowded batch, per-tile costs
         // stay small) and no more than 64.
-        long long tr = tile_rows_for(h, m, n, ttype, ttype == TT_F64 ? 0 : h->cfg_base.pass_bulk, false, true);
+        long long tr = tile_rows_for(h, m, n, ttype, ttype == TT_F64 ? 0 : h->cfg_base.pass_form, false, true);
         tr = std::max<long long>(tr, h->batch_min_rows);
         tr = std::min<long long>(tr, 64);
         return (int)tr;
@@ -383,7 +383,7 @@ int tile_rows_for(pdot_handle* h, long long m, long long n, int ttype, int kerne
     // each (the last wave of a dynamic queue would leave a tail), as tall as
     // that allows (fewer column partials).
     const long long blocks = ttype == TT_F64 ? h->cfg.tile_blocks_f64
-                             : kernel >= 1   ? h->cfg.bulk_blocks
+                             : kernel >= 1   ? h->cfg.lag_blocks
                                              : h->cfg.tile_blocks;
     const long long warps = blocks * TWARPS;
     long long nch = warps / nstrips;
@@ -402,8 +402,8 @@ int gen_dims_of(const void* C, int ctype) {
 // Tile height of a call: by shape when the library picks the kernel (one tile
 // per resident warp), else the explicit kernel's.
 int pick_tile_rows(pdot_handle* h, long long m, long long n, int ttype, bool batch = false) {
-    const bool by_shape = !batch && h->autotune && h->opt.pass_kernel == 0;
-    return tile_rows_for(h, m, n, ttype, by_shape ? 1 : h->cfg.pass_bulk, batch);
+    const bool by_shape = !batch && h->by_shape && h->opt.pass_kernel == 0;
+    return tile_rows_for(h, m, n, ttype, by_shape ? 1 : h->cfg.pass_form, batch);
 }
 
 const void* prepare_C(pdot_handle* h, long long m, long long n, const void* C, int ctype, long long ldc,
@@ -506,7 +506,7 @@ void run_avgfix(pdot_handle* h, int ttype) {
 
 // Whether the pass kernel of the current configuration defers plan writes
 // (every FP32-plan pass but the register pipeline).
-bool lag_for(pdot_handle* h, int ttype) { return ttype != TT_F64 && h->cfg.pass_bulk != 0; }
+bool lag_for(pdot_handle* h, int ttype) { return ttype != TT_F64 && h->cfg.pass_form != 0; }
 
 // Apply and write the pending steps of deferred plan writes.
 void run_final(pdot_handle* h, int ttype) {
@@ -584,7 +584,7 @@ void launch_chunk(pdot_handle* h, int ttype, int K) {
                               w.n,
                               K,
                               (long long)h->cfg.comp * 1000 + (long long)h->cfg.pdl * 100 +
-                                  (long long)h->cfg.pass_bulk * 10 + (long long)h->cfg.pass_u,
+                                  (long long)h->cfg.pass_form * 10 + (long long)h->cfg.pass_u,
                               w.tile_rows,
                               h->cfg.gen_dims};
     if (!h->opt.use_graph) {
@@ -738,20 +738,20 @@ void choose_pass(pdot_handle* h, long long m, long long n, const void* C, int ct
     if (h->opt.pass_kernel > 0) {
         int v = h->opt.pass_kernel - 1;
         if (ttype == TT_GEN && gen_d > 4 && v == 2) v = 1;   // rows in order beyond 4 coordinates
-        h->cfg.pass_bulk = v;
+        h->cfg.pass_form = v;
         return;
     }
     if (ttype == TT_GEN && gen_d > 4) {
-        h->cfg.pass_bulk = h->cfg_base.pass_bulk ? 1 : 0;
+        h->cfg.pass_form = h->cfg_base.pass_form ? 1 : 0;
         return;
     }
-    if (ttype == TT_F64 || h->opt.tile_rows > 0 || !h->cfg_base.pass_bulk) return;
-    if (!h->autotune) {
-        h->cfg.pass_bulk = h->cfg_base.pass_bulk;
+    if (ttype == TT_F64 || h->opt.tile_rows > 0 || !h->cfg_base.pass_form) return;
+    if (!h->by_shape) {
+        h->cfg.pass_form = h->cfg_base.pass_form;
         return;
     }
     const bool rows = m * n < (1LL << 22) || (ttype == TT_F32 && m * n > 30000000LL);
-    h->cfg.pass_bulk = rows ? 1 : 2;
+    h->cfg.pass_form = rows ? 1 : 2;
 }
 
 // ---------------------------------------------------------------------------
@@ -871,7 +871,7 @@ pdot_status solve_impl(pdot_handle* h, long long m, long long n, const void* C, 
     validate_marginals(h, m, n, f, g, false, &norm_b);
     const int ttype = ttype_of(ctype);
     {
-        const Range r_("autotune");
+        const Range r_("autotune");   // (the phase's name in profiles; the choice is a rule)
         choose_pass(h, m, n, C, ctype);
     }
     h->res_on = h->opt.pass_kernel == 0 && resident_for(h, m, n, ttype);
@@ -1239,7 +1239,7 @@ void batch_plan_coop(pdot_handle* h, const std::vector<char>& active) {
     for (int i : order) {
         const BSlot* s = B->live[(size_t)i];
         const int ctas = (int)((s->w.ntiles + TWARPS - 1) / TWARPS);
-        if (s->ttype == TT_F64 || h->cfg_base.pass_bulk == 0 || h->opt.pass_kernel != 0 || h->opt.tile_rows != 0 || ctas > cap ||
+        if (s->ttype == TT_F64 || h->cfg_base.pass_form == 0 || h->opt.pass_kernel != 0 || h->opt.tile_rows != 0 || ctas > cap ||
             (s->ttype == TT_GEN && B->gen_dims > 4))
             return;
         size_t k = 0;
@@ -1468,7 +1468,7 @@ void batch_launch_chunk(pdot_handle* h) {
     const int types = B->types;
     h->cfg.gen_dims = B->gen_dims;
     h->cfg.comp = h->opt.compensated_cost != 0 ? 1 : 0;
-    h->cfg.pass_bulk = h->cfg_base.pass_bulk;   // the batch engine's pass kernel (its tiles were sized for it)
+    h->cfg.pass_form = h->cfg_base.pass_form;   // the batch engine's pass kernel (its tiles were sized for it)
     long long tmaps = 0;
     for (int t = 0; t < NTT; ++t) tmaps ^= (long long)(uintptr_t)B->tmap[t].d << t;
     const long long key[8] = {(long long)(uintptr_t)B->insts.d, (long long)(uintptr_t)B->cnt.d,
@@ -1640,7 +1640,7 @@ bool batch_admit(pdot_handle* h) {
         // controller
         Ctrl* S = &B->ctrl_stage.h[B->live.size()];
         init_ctrl(h, S, r.m, r.n, r.tol > 0.0 ? r.tol : h->opt.tol, 0.0, 0.0, false, 0.0, 0.0,
-                  !s->resident && s->ttype != TT_F64 && h->cfg_base.pass_bulk != 0);
+                  !s->resident && s->ttype != TT_F64 && h->cfg_base.pass_form != 0);
         CK(cudaMemcpyAsync(s->w.ctrl, S, sizeof(Ctrl), cudaMemcpyHostToDevice, h->stream));
         CK(cudaMemsetAsync(s->w.ticket, 0, sizeof(unsigned), h->stream));
         CK(cudaMemsetAsync(s->w.X, 0, (size_t)s->w.m * s->w.ldx * xsize_of(s->w.xtype), h->stream));
@@ -1876,9 +1876,9 @@ pdot_status pdot_create(const pdot_options* opt, int device, void* cuda_stream, 
         h->cfg.pass_u = 2;
         const char* pu = getenv("PDOT_PASS_U");
         if (pu && atoi(pu) == 4) h->cfg.pass_u = 4;
-        const int bulk = setup_bulk_pass();
-        if (bulk > 0) throw CudaError{(cudaError_t)bulk};
-        h->cfg.bulk_blocks = h->sm_count * (-bulk);
+        const int lag = setup_lag_pass();
+        if (lag > 0) throw CudaError{(cudaError_t)lag};
+        h->cfg.lag_blocks = h->sm_count * (-lag);
         const int rc = setup_resident();
         if (rc > 0) throw CudaError{(cudaError_t)rc};
         h->res_clusters = -rc;
@@ -1903,24 +1903,24 @@ pdot_status pdot_create(const pdot_options* opt, int device, void* cuda_stream, 
         if (cp && atoi(cp) >= 1 && atoi(cp) < h->coop_passes) h->coop_passes = atoi(cp);
         CK(cudaMalloc(&h->d_gs, sizeof(GridSync)));
         CK(cudaMemset(h->d_gs, 0, sizeof(GridSync)));
-        const int kb = setup_kkt_bulk();
+        const int kb = setup_kkt_staged();
         if (kb > 0) throw CudaError{(cudaError_t)kb};
         h->cfg.kkt_blocks = h->sm_count * (-kb);
         const char* kk = getenv("PDOT_KKT_BULK");
         if (kk && atoi(kk) == 0) h->cfg.kkt_blocks = 0;   // the register KKT pass (comparison)
-        h->cfg.pass_bulk = 1;
+        h->cfg.pass_form = 1;
         const char* pb = getenv("PDOT_PASS_BULK");
         if (pb) {
             const int v = atoi(pb);
             if (v >= 0 && v <= 2) {
-                h->cfg.pass_bulk = v;
-                h->autotune = 0;   // an explicit choice replaces the rule
+                h->cfg.pass_form = v;
+                h->by_shape = 0;   // an explicit choice replaces the rule
             }
         }
         const char* bm = getenv("PDOT_BATCH_MIN_ROWS");   // comparison runs only
         if (bm && atoi(bm) >= 2 && atoi(bm) <= 64 && atoi(bm) % 2 == 0) h->batch_min_rows = atoi(bm);
-        const char* at = getenv("PDOT_AUTOTUNE");
-        if (at && atoi(at) == 0) h->autotune = 0;
+        const char* at = getenv("PDOT_AUTOTUNE");   // 0: the fixed choice at every shape (comparison runs)
+        if (at && atoi(at) == 0) h->by_shape = 0;
         // Programmatic dependent launch: on (PDOT_PDL=0 turns it off).
         const char* pp = getenv("PDOT_PDL");
         h->cfg.pdl = (pp && atoi(pp) == 0) ? 0 : 1;
@@ -2435,7 +2435,7 @@ pdot_status pdot_time_pass(pdot_handle* h, int64_t m, int64_t n, const void* C, 
             *bytes_per_pass = (double)m * (double)n *
                               pass_bytes(lag, (double)csize_of(c_dtype), (double)xsize_of(w.xtype));
         if (kernel_variant) {
-            int v = ttype == TT_F64 ? 0 : h->cfg.pass_bulk;
+            int v = ttype == TT_F64 ? 0 : h->cfg.pass_form;
             if (ttype == TT_GEN && v == 2 && h->cfg.gen_dims > 4) v = 1;   // no grouped kernel beyond 4 coordinates
             *kernel_variant = v;
         }

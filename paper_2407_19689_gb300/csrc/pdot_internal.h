@@ -11,7 +11,8 @@
 //          [p (m) | q (n) | r = X1 (m) | c = X^T1 (n)].
 //   rowpart[nstrips][m], colpart[nchunks][ldx]: FP64 partial row/column sums
 //          written by the plan-tile kernels and reduced in a fixed order (a
-//          pass writes sums of X+ - X; the check, sums of the average);
+//          pass writes sums of X+ - X; the check, sums of the average); the
+//          cooperative kernel's row sums are FP32 values and stay FP32 there;
 //          rowpart2 / colpart2: the check's sums of the current plan.
 //   tpart[ntiles][TP], vpart[nvt][VP]: FP64 per-tile scalar partials
 //          (nvt = ceil((m+n)/VE) vector tiles).
@@ -176,8 +177,9 @@ struct Inst {
 constexpr int BARRIER_POLLS = 1 << 23;   // (a poll takes about a microsecond)
 constexpr unsigned BARRIER_FAIL = 0x40000000u;   // set in a barrier's counter when someone gave up
 
-// Barrier counters of the cooperative kernel, one pair per instance (zeroed
-// once; launches take them in turn and each zeroes the other).
+// Barrier counters of the cooperative kernel, one pair per instance.  A single
+// instance's are zeroed once; its launches take them in turn and each zeroes
+// the other.  A batch zeroes its instances' before every round of launches.
 struct GridSync {
     unsigned int count[2];
 };
@@ -215,14 +217,14 @@ struct LaunchCfg {
     int tile_blocks_f64;  // CTAs of the FP64-plan tile kernels
     int vec_blocks;       // CTAs of the vector kernels (256 threads each)
     int pass_u;           // rows per load batch in the FP32-plan register pass (2 or 4)
-    int pass_bulk;        // FP32-plan pass: 0 register pipeline, 1 / 2 deferred writes (rows / groups in order)
-    int bulk_blocks;      // CTAs of the deferred-write pass kernel
+    int pass_form;        // FP32-plan pass: 0 register pipeline, 1 / 2 deferred writes (rows / groups in order)
+    int lag_blocks;      // CTAs of the deferred-write pass kernel
     int coop_blocks;      // CTAs of the cooperative kernel that fit at once (0: no cooperative launch)
     int pdl;              // 1: launch with programmatic dependent launch
     int gen_dims;         // largest coordinate count of the generated costs in flight (TT_GEN)
     int comp;             // 1: plan passes of FP32 plans form the compensated reduced cost
     int barrier_polls;    // polls of the cooperative kernel's barrier before it gives up
-    int kkt_blocks;       // CTAs of the bulk-copy KKT pass (0: the register KKT pass)
+    int kkt_blocks;       // CTAs of the staged KKT pass (0: the register KKT pass)
 };
 
 // Tile and vector-tile counts are read from device memory, so one captured
@@ -264,9 +266,9 @@ int launch_combine(int xtype, const void* a, const void* d, void* out, long long
 int launch_watchdog_selftest(int polls, int* d_status, unsigned* d_count, void* stream);
 int occupancy_tile_blocks_per_sm(int ttype);
 int occupancy_vec_blocks_per_sm();
-// Opt the bulk-copy pass kernel into its shared-memory size; returns minus
+// Opt the deferred-write pass kernel into its shared-memory size; returns minus
 // the CTAs per SM it can hold, or a positive cudaError_t code.
-int setup_bulk_pass();
+int setup_lag_pass();
 int setup_persist();
 // Passes of FP32-plan instances (one tile per warp, all resident) and the
 // final write of their pending steps, in one cooperative launch of `ctas`
@@ -276,6 +278,6 @@ int launch_persist(int ttype, const Inst* d_insts, const CtaRef* refs, int ctas,
                    int npass, const LaunchCfg& cfg, void* stream);
 // Tallest tile that stays in the cooperative kernel's shared memory.
 int persist_rows(bool comp);
-int setup_kkt_bulk();
+int setup_kkt_staged();
 
 }  // namespace pdot

@@ -822,7 +822,7 @@ __device__ __forceinline__ void kkt_tile(const Inst& I, const Ctrl& S, int lt, i
     // FP32 plans accumulate in FP32 over KKT_FLUSH_ROWS rows before adding
     // into the FP64 partials (an FP64 add per batch of two rows would make
     // this pass bound by the narrow FP64 pipe) -- the same grouping as
-    // k_kkt_bulk, so both give the same bits.
+    // k_kkt_staged, so both give the same bits.
     constexpr int KFLUSH = sizeof(A) == 4 ? KKT_FLUSH_ROWS / KU : 1;
     A t[TP] = {A(0), A(0), A(0), A(0), A(0), A(0)};
     A csa[4] = {A(0), A(0), A(0), A(0)}, csa2[4] = {A(0), A(0), A(0), A(0)};
@@ -940,7 +940,7 @@ k_kkt(const Inst* __restrict__ insts, const TileRef* __restrict__ tmap, const in
 }
 
 // ---------------------------------------------------------------------------
-// KKT pass, copy pipeline (FP32 plans with a stored FP32 or BF16 cost): the
+// KKT pass, staged (FP32 plans with a stored FP32 or BF16 cost): the
 // arithmetic of kkt_tile, with each warp streaming its tile's rows of C, X, D
 // and the restart anchor through KS shared-memory stages.  Every lane copies
 // the 16 bytes it reads itself (cp.async; by bulk copies the rows took 40
@@ -957,7 +957,7 @@ constexpr int kkt_smem() { return TWARPS * kkt_warp_smem(); }
 
 template <typename TC>
 __global__ void __launch_bounds__(TWARPS * 32, 2)
-k_kkt_bulk(const Inst* __restrict__ insts, const TileRef* __restrict__ tmap, const int* __restrict__ Tp,
+k_kkt_staged(const Inst* __restrict__ insts, const TileRef* __restrict__ tmap, const int* __restrict__ Tp,
            unsigned* wctr, int wc, int mode) {
     const int T = *Tp;   // host-written: read before the wait
     extern __shared__ __align__(128) unsigned char dsm[];
@@ -1544,9 +1544,6 @@ __global__ void __launch_bounds__(VT) k_checkvec(const Inst* __restrict__ insts,
 }
 
 // ---------------------------------------------------------------------------
-// Snapshot of every resident instance's controller (one D2H copy per chunk)
-// ---------------------------------------------------------------------------
-// ---------------------------------------------------------------------------
 // After every check: where the check picked the running average (a restart to
 // it, or the reported point), write X[fix_dst] = X[fix_x] + X[fix_d] -- the
 // current plan plus the stored deviation, with the rounding the checks used
@@ -1619,6 +1616,7 @@ __global__ void k_combine(const TX* __restrict__ a, const TX* __restrict__ d, TX
     }
 }
 
+// Snapshot of every live instance's controller (one D2H copy per chunk).
 __global__ void k_snapshot(const Inst* __restrict__ insts, const int* __restrict__ count, Ctrl* out) {
     pdl_enter();
     const int n = *count;
@@ -1668,8 +1666,8 @@ template <bool CP, bool FINAL>
 static int launch_lag(int ttype, const Inst* d_insts, const TileRef* d_tmap, const int* T, unsigned* wctr, int wc,
                       int dir_xor, const LaunchCfg& cfg, cudaStream_t st) {
     const bool pdl = cfg.pdl != 0;
-    const unsigned nb = (unsigned)cfg.bulk_blocks, th = TWARPS * 32;
-    const int ro = cfg.pass_bulk == 1 ? 1 : 0;
+    const unsigned nb = (unsigned)cfg.lag_blocks, th = TWARPS * 32;
+    const int ro = cfg.pass_form == 1 ? 1 : 0;
     constexpr int sm = lagp::smem_bytes();
     if (ttype == TT_BF16)
         return launch_k(pdl, k_pass_lag<unsigned short, CP, FINAL>, nb, th, sm, st, d_insts, d_tmap, T, wctr, wc, dir_xor, ro);
@@ -1692,7 +1690,7 @@ static int launch_pass_t(int ttype, const Inst* d_insts, const TileRef* d_tmap, 
     if (ttype == TT_F64)
         return launch_k(pdl, k_pass<double, double, 2, CP>, (unsigned)cfg.tile_blocks_f64, th, 0, st, d_insts, d_tmap, T,
                         wctr, wc, dir_xor);
-    if (cfg.pass_bulk)
+    if (cfg.pass_form)
         return launch_lag<CP, false>(ttype, d_insts, d_tmap, T, wctr, wc, dir_xor, cfg, st);
     if (ttype == TT_GEN)
         return launch_k(pdl, k_pass<GenC8, float, 2, CP>, tb, th, 0, st, d_insts, d_tmap, T, wctr, wc, dir_xor);
@@ -1738,11 +1736,11 @@ int launch_kkt(int ttype, const Inst* d_insts, const TileRef* d_tmap, const int*
     if (ttype == TT_GEN)
         return launch_k(pdl, k_kkt<GenC8, float>, (unsigned)cfg.tile_blocks, th, 0, st, d_insts, d_tmap, T, wctr, wc,
                         mode);
-    if (cfg.kkt_blocks > 0) {   // bulk-copy pipeline for stored FP32 / BF16 costs
+    if (cfg.kkt_blocks > 0) {   // stored FP32 / BF16 costs
         if (ttype == TT_BF16)
-            return launch_k(pdl, k_kkt_bulk<unsigned short>, (unsigned)cfg.kkt_blocks, th, kkt_smem(), st, d_insts,
+            return launch_k(pdl, k_kkt_staged<unsigned short>, (unsigned)cfg.kkt_blocks, th, kkt_smem(), st, d_insts,
                             d_tmap, T, wctr, wc, mode);
-        return launch_k(pdl, k_kkt_bulk<float>, (unsigned)cfg.kkt_blocks, th, kkt_smem(), st, d_insts, d_tmap, T, wctr,
+        return launch_k(pdl, k_kkt_staged<float>, (unsigned)cfg.kkt_blocks, th, kkt_smem(), st, d_insts, d_tmap, T, wctr,
                         wc, mode);
     }
     if (ttype == TT_BF16)
@@ -1876,8 +1874,8 @@ int launch_resident(int ttype, const Inst* d_insts, const int* list, const int* 
     return err(cudaGetLastError());
 }
 
-int setup_kkt_bulk() {
-    const void* fns[] = {(const void*)k_kkt_bulk<float>, (const void*)k_kkt_bulk<unsigned short>};
+int setup_kkt_staged() {
+    const void* fns[] = {(const void*)k_kkt_staged<float>, (const void*)k_kkt_staged<unsigned short>};
     return setup_dyn(fns, 2, kkt_smem());
 }
 
@@ -1887,7 +1885,7 @@ static int setup_lag() {
                          (const void*)k_pass_lag<TC, true, true>, (const void*)k_pass_lag<TC, false, true>};
     return setup_dyn(fns, 4, lagp::smem_bytes());
 }
-int setup_bulk_pass() {
+int setup_lag_pass() {
     const int r[] = {setup_lag<float>(), setup_lag<unsigned short>(), setup_lag<GenC<2>>(), setup_lag<GenC4>(),
                      setup_lag<GenC8>()};
     int worst = r[0];
@@ -1922,7 +1920,7 @@ static int launch_pers(const Inst* d_insts, const CtaRef* refs, int ctas, GridSy
     attr[0].val.cooperative = 1;
     c.attrs = attr;
     c.numAttrs = 1;
-    const int ro = cfg.pass_bulk == 1 ? 1 : 0;
+    const int ro = cfg.pass_form == 1 ? 1 : 0;
     return err(cfg.comp ? cudaLaunchKernelEx(&c, k_persist<TC, true>, d_insts, refs, gs, epoch, npass, ro, cfg.barrier_polls)
                         : cudaLaunchKernelEx(&c, k_persist<TC, false>, d_insts, refs, gs, epoch, npass, ro, cfg.barrier_polls));
 }

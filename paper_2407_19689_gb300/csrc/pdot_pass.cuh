@@ -27,9 +27,7 @@
 // took 40 cycles of an SM's bulk-copy engine per 512-byte row, 3.9 TB/s for
 // the device whatever the kernel did besides.  The same 12 KB hold three
 // stages of C and X, or two of C, X and D.  The group's row duals come with
-// its copies, so no load is waited for between groups.  The arithmetic is
-// issued as packed FP32 pairs (fma.f32x2), which round like the scalar
-// instructions and take half the issue slots.
+// its copies, so no load is waited for between groups.
 #pragma once
 
 namespace pdot {

@@ -9,10 +9,9 @@
 //   tile    as pdot_pass.cuh (deferred plan writes, the same sums), but the
 //           ring of shared-memory stages is not refilled at a pass's end: the
 //           passes alternate their row order, so the next pass starts with the
-//           groups the last one ended with.  A tile of up to 12 rows stays in
-//           shared memory for the whole launch, a taller one saves 12 rows of
-//           C and X per pass and has its next rows in flight while the dual
-//           update runs;
+//           groups the last one ended with.  A tile of up to 12 rows (8 with
+//           the compensated reduced cost) stays in shared memory for the whole
+//           launch, a taller one saves as many rows of C and X per pass;
 //   barrier (all row and column partial sums are written);
 //   dual    the arithmetic of dual_tile, one CTA per vector tile;
 //   barrier (the tiles' step scalars are written);

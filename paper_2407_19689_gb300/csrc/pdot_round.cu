@@ -13,7 +13,7 @@
 //   write  the plan, and <C, plan> when a cost is given
 // All scalars stay on the device: the old form copied them to the host and
 // back three times and took the write through 64 blocks (1313 us at 4096 x
-// 4096, FP32; here 139 us; 2 x 67 MB take 20 us).
+// 4096, FP32; here 133 us; 2 x 67 MB take 20 us).
 //
 // FP64 is a narrow pipe on this part (two lanes per cycle and SM: one FP64
 // operation per entry of a 4096 x 4096 plan takes 27 us), so FP32 plans are
@@ -26,7 +26,7 @@
 // that follow take FP64 arithmetic and the FP64 scales, which are kept beside
 // the pairs: row sums or errors of 1e30 and more or not finite, and scales below RTINY
 // that are multiplied by more than 1 (a pair's absolute error is 2^-150, so a
-// product with at most 1 is as exact as an FP32 entry can be).  The objective
+// product with at most 1 is off by one or two of FP32's smallest steps).  The objective
 // <C, plan> is an FP64 sum of FP64 products (once per solve that asks for it).
 // FP64 plans use FP64 throughout.
 #include <cuda_runtime.h>
