@@ -301,7 +301,12 @@ pdot_status pdot_kkt(pdot_handle *h, int64_t m, int64_t n, const void *C, pdot_d
 
 /* Algorithm 3: write into X_out (device, m x n, x_dtype) the rounding of the
  * device plan X onto {X >= 0, X1 = f, X^T1 = g}.  X and X_out may alias.
- * A zero row/column sum keeps scale 1; a zero ||err_r||_1 skips the rank-one term. */
+ * A zero row/column sum keeps scale 1; a zero ||err_r||_1 skips the rank-one term.
+ * FP64 plans are rounded in FP64.  FP32 plans: sums and scales are unevaluated
+ * FP32 pairs (48 bits; relative error of a sum about 1e-13), or FP64 where
+ * FP32's range would not hold them, and each entry is rounded to FP32 once: the
+ * error against 64 bits is that of the entries' FP32 rounding.  The objective of
+ * a solve with round_plan = 1 (rounded_obj) is an FP64 sum. */
 pdot_status pdot_round(pdot_handle *h, int64_t m, int64_t n, const void *X, const double *f, const double *g,
                        void *X_out);
 
@@ -351,7 +356,8 @@ pdot_status pdot_batch_pending(pdot_handle *h, int *queued, int *running);
  * device memory when they need it (memory owned by another allocator, a
  * serving loop that forbids cudaMalloc/cudaFree after warm-up because they
  * synchronise the device, a plug-in inside an application that owns all
- * allocations).  Same result as pdot_round, but no handle and no allocation:
+ * allocations).  The rounding of pdot_round (its sums in FP64 throughout and in
+ * another order), but no handle and no allocation:
  * the scratch is a 3.7 MB array in the library's device image, held by every
  * GPU that loads the library until the process exits.  This entry point has
  * no counterpart in the paper.
@@ -375,12 +381,14 @@ pdot_status pdot_round_noalloc(int device, void *cuda_stream, int64_t m, int64_t
 /* Kernel launches issued by this handle since creation (diagnostics). */
 int64_t pdot_launch_count(pdot_handle *h);
 
-/* Diagnostics for roofline measurement: set up the instance, take three
- * PDHG steps (so the running average is read), then launch the fused plan
- * pass `reps` times back to back on the handle's stream between two CUDA
- * events, each launch reading the plans the previous one wrote (as accepted
- * passes of a solve do; the dual update is left out, so every launch moves
- * the same bytes).  *ms_per_pass receives the mean device time of one pass;
+/* Diagnostics for roofline measurement: set up the instance, take a few
+ * PDHG steps (so the running average is read), then launch the plan pass of
+ * an iteration of two kernels `reps` times back to back on the handle's stream
+ * between two CUDA events, each launch reading the plans the previous ones
+ * wrote (as accepted passes of a solve do; the dual update is left out).  A
+ * solve whose tiles are resident at once runs its passes in the cooperative
+ * kernel instead, with the same arithmetic; this call does not time that
+ * kernel.  *ms_per_pass receives the mean device time of one pass;
  * *bytes_per_pass (nullable) the algorithmic bytes one pass moves:
  * m n (sizeof C + 2 sizeof X) with deferred plan writes (read C and X; every
  * third pass also reads Xbar and writes X+ and Xbar+), m n (sizeof C + 4
